@@ -38,8 +38,8 @@
 
 #include <algorithm>
 #include <cstddef>
-#include <vector>
 
+#include "grid_split.cuh"
 #include "progot_internal.h"
 #include "sweep_epilogue.cuh"
 #include "tc_common.cuh"
@@ -87,23 +87,24 @@ struct Layout {
   uint32_t a0, a_stride, a_lo_off, a_bias, bias0, bias_slot, stage0, stage_bytes, b_lo_off, ctrl, total;
 };
 
-// A buffers, the ones of the bias product, the bias-row ring, then the stages (B hi, B lo).
-__host__ __device__ inline Layout layout(int bn, int nkb, int split3, int stages, int a_bufs) {
+// A buffers, the ones of the bias product, the bias-row ring, then the stages: B hi and lo
+// of one K block, or with the grid split (three parts) one part of one K block.
+__host__ __device__ inline Layout layout(int bn, int nkb, int split3, int stages, int a_bufs, bool grid) {
   Layout L;
   uint32_t off = 0;
   L.a0 = off;
   L.a_lo_off = nkb * A_TILE_BYTES;
-  L.a_stride = nkb * A_TILE_BYTES * (split3 ? 2 : 1);
+  L.a_stride = nkb * A_TILE_BYTES * (grid ? kGridParts : split3 ? 2 : 1);
   off += a_bufs * L.a_stride;
   L.a_bias = off;
-  off += A_BIAS_BYTES;
+  off += A_BIAS_BYTES * (grid ? 2 : 1);
   L.bias0 = off;
   L.bias_slot = (uint32_t)bn * 32;
   off += BIAS_SLOTS * L.bias_slot;
   off = (off + 1023) & ~1023u;  // 128-byte swizzled stages start on 1024-byte boundaries
   L.stage0 = off;
   L.b_lo_off = (uint32_t)bn * KB * 2;
-  L.stage_bytes = L.b_lo_off * (split3 ? 2 : 1);
+  L.stage_bytes = L.b_lo_off * (!grid && split3 ? 2 : 1);
   off += stages * L.stage_bytes;
   L.ctrl = off;
   off += (uint32_t)sizeof(Shared);
@@ -126,12 +127,13 @@ struct Side {
   unsigned long long* cnt;  // [R] arrivals per row block (monotonic over the loop)
   unsigned long long* done; // finished row blocks (monotonic over the loop)
   float2* partial;          // [G * maxseg][2][128] (max, sum) per segment slot, LSE warpgroup and row
-  // the work split (host-built): CTA c's segments segs[c maxseg + k] = (row block, first
-  // tile, end tile), k < nseg[c]; row block r's contributors are the partial slots
-  // cslot[cptr[r] .. cptr[r + 1]) (slot = CTA * maxseg + segment), in combine order
+  // the work split (tables of the operand preparation's launch): CTA c's segments
+  // segs[c maxseg + k] = (row block, first tile, end tile), k < nseg[c]; row block r's
+  // contributors are the partial slots cslot[off .. off + count), (off, count) = crow[r]
+  // (slot = CTA * maxseg + segment), in combine order
   const int4* segs;
   const int32_t* nseg;
-  const int32_t* cptr;
+  const int2* crow;
   const int32_t* cslot;
   int32_t R, T;
   int64_t nA, nB;
@@ -144,6 +146,7 @@ struct Params {
   int32_t* fault;           // grid-wide abort / fault word
   unsigned long long wait_ns;
   int32_t nkb, split3, stages, a_bufs, G, maxseg;
+  const float* gscale;      // grid split: {2^(ex + ey), 2^-(ex + ey)} (device)
   int32_t seq0, niter;      // iterations seq0 .. seq0 + niter - 1 of the loop
 };
 
@@ -233,6 +236,12 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return r;
 }
 
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -242,32 +251,6 @@ __device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// beta split into three bf16 terms (hi, mid, lo) in the first three of 16 slots
-// (-inf in the first slot for a non-finite beta).
-__device__ __forceinline__ void write_bias_row(__nv_bfloat16* row16, float beta) {
-  __nv_bfloat16 h1, h2, h3;
-  if (isfinite(beta)) {
-    h1 = __float2bfloat16_rn(beta);
-    const float r1 = beta - __bfloat162float(h1);
-    h2 = __float2bfloat16_rn(r1);
-    h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
-  } else {
-    h1 = __float2bfloat16_rn(-INFINITY);
-    h2 = __float2bfloat16_rn(0.f);
-    h3 = __float2bfloat16_rn(0.f);
-  }
-  uint4 lo4;
-  lo4.x = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
-  lo4.y = (uint32_t)__bfloat16_as_ushort(h3);
-  lo4.z = 0u;
-  lo4.w = 0u;
-  uint4* dst = reinterpret_cast<uint4*>(row16);
-  dst[0] = lo4;
-  dst[1] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// Poll the ready flags of row blocks [r0, r1) until each is at least `want` (acquire);
-// bounded. Called by one lane.
 // Whole warp: lane l polls the ready flag of row block r0 + l (r1 - r0 <= 32), so the
 // flags under a tile are read in parallel rather than one after another; returns once
 // every flag carries want (the lanes' acquires are ordered before the caller's later
@@ -306,6 +289,18 @@ __device__ __forceinline__ bool wait_flags_warp(const uint32_t* flags, int r0, i
   return ok;
 }
 
+// Whole warp: lane l polls flag l of count (<= 32) until flag 0 carries want; returns the
+// number of leading flags seen ready (their acquires ordered as above), 0 on abort.
+__device__ __forceinline__ int wait_flags_ahead(const uint32_t* flags, int count, uint32_t want,
+                                                volatile int32_t* abort_flag, const Params& P) {
+  const int lane = threadIdx.x & 31;
+  if (!wait_flags_warp(flags, 0, 1, want, abort_flag, P)) return 0;
+  const bool seen = lane < count && ld_acquire_u32(flags + lane) >= want;
+  const uint32_t ready = __ballot_sync(0xffffffffu, seen);
+  __syncwarp();
+  return ready == 0xffffffffu ? 32 : max(1, __ffs(~ready) - 1);
+}
+
 // New potential of row i from its log2-sum-exp L (Alg. 1's update, the row constant
 // |a_i|^2 included): f_i = eps log w_i + |a_i|^2 - eps ln2 L, in float32 with the
 // product eps ln2 L folded into FMAs on a hi/lo split of eps ln2, so that |a_i|^2 - eps
@@ -325,6 +320,35 @@ __device__ __forceinline__ float loop_row_potential(const Side& Sd, int sd, int6
   } else {
     fnew = (t + Sd.w_lo) + Sd.w_hi;
   }
+  out[i] = fnew;
+  *val = fnew;
+  if (sd != 0) return 0.f;
+  float dlt = (in.pot - fnew) * Sd.p.inv_eps_f;
+  if (dlt > 80.f) dlt = 80.f;
+  return in.w * fabsf(expm1f(dlt));
+}
+
+// The same from the row's (max, sum) of an integer-grid sweep, every step carried in two
+// floats and rounded once: f = eps log w + |a|^2 - eps ln2 (max + log2 sum).
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  const float s = a + b, bb = s - a;
+  return make_float2(s, (a - (s - bb)) + (b - bb));
+}
+__device__ __forceinline__ float loop_row_potential_grid(const Side& Sd, int sd, int64_t i, float2 ms, const RowIn& in,
+                                                         float* out, float* val) {
+  const float2 L = two_sum(ms.x, log2f(ms.y));
+  const float p = Sd.c_hi * L.x;
+  const float pe = fmaf(Sd.c_hi, L.x, -p) + fmaf(Sd.c_lo, L.x, Sd.c_hi * L.y);
+  float wh = Sd.w_hi, wl = Sd.w_lo;
+  if (Sd.p.wA) {
+    const float lw = logf(in.w);
+    wh = Sd.e_hi * lw;
+    wl = fmaf(Sd.e_hi, lw, -wh) + Sd.e_lo * lw;
+  }
+  const float2 a = two_sum(in.an, -p);
+  const float2 b = two_sum(a.x, wh);
+  float fnew = b.x + ((b.y + a.y) + (wl - pe));
+  if (!isfinite(b.x)) fnew = b.x;  // zero weights, empty or overflowing rows
   out[i] = fnew;
   *val = fnew;
   if (sd != 0) return 0.f;
@@ -364,19 +388,29 @@ __device__ __forceinline__ Seg seg_at(const Side& Sd, int c, int k, int maxseg) 
 // ------------------------------------------------------------------ kernel
 // NKB: the operands' K blocks when fixed at compile time (1: d <= 64, the MMA warp's issue
 // path then has no runtime K loop), 0 when read from P.nkb.
-template <int BN, int NKB>
+// GRID: 0 bf16 operands; else the float32 path's integer-grid split (grid_split.cuh): three operand parts, one
+// part of one K block per stage (so that seven 16 KB stages fit next to two A buffers at
+// d <= 64), two accumulators per tile: leading products and the bias's integer part at
+// TMEM columns [0, 256), the rest at [256, 512). GRID = 1..4 is the number of K = 16 steps
+// that hold coordinates (d <= 64), so that a tile's products are issued without a loop
+// (56.7 -> 46 us per sweep at 8192^2, d = 64, where the CUDA-core sweep takes 238).
+template <int BN, int NKB, int GRID>
 __global__ void __launch_bounds__(NTHREADS, 1)
     sinkhorn_loop_tc(const __grid_constant__ CUtensorMap mXh_a, const __grid_constant__ CUtensorMap mXl_a,
                      const __grid_constant__ CUtensorMap mYh_a, const __grid_constant__ CUtensorMap mYl_a,
                      const __grid_constant__ CUtensorMap mXh_b, const __grid_constant__ CUtensorMap mXl_b,
                      const __grid_constant__ CUtensorMap mYh_b, const __grid_constant__ CUtensorMap mYl_b,
+                     const __grid_constant__ CUtensorMap mXr_a, const __grid_constant__ CUtensorMap mYr_a,
+                     const __grid_constant__ CUtensorMap mXr_b, const __grid_constant__ CUtensorMap mYr_b,
                      const __grid_constant__ CUtensorMap mXb0, const __grid_constant__ CUtensorMap mXb1,
                      const __grid_constant__ CUtensorMap mYb0, const __grid_constant__ CUtensorMap mYb1,
                      const Params P) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const Layout L = layout(BN, P.nkb, P.split3, P.stages, P.a_bufs);
+  static_assert(!GRID || (BN == 128 && NKB == 1 && GRID <= KB / 16),
+                "the grid split has two accumulators per 128-column tile");
+  const Layout L = layout(BN, P.nkb, P.split3, P.stages, P.a_bufs, GRID != 0);
   Shared& sh = *reinterpret_cast<Shared*>(smem + L.ctrl);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkb = NKB > 0 ? NKB : P.nkb;
@@ -419,11 +453,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   // A side of the bias product: all ones (bf16 0x3F80), so that the K = 16 step adds
   // beta_hi + beta_mid + beta_lo whatever the order of the 16-byte chunks in a row
-  {
+  if constexpr (GRID) {
+    fill_bias_ones_grid(smem + L.a_bias, threadIdx.x, NTHREADS);
+  } else {
     uint32_t* ab = reinterpret_cast<uint32_t*>(smem + L.a_bias);
     for (int i = threadIdx.x; i < A_BIAS_BYTES / 4; i += NTHREADS) ab[i] = 0x3F803F80u;
-    fence_async_smem();
   }
+  fence_async_smem();
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)),
                  "r"(TMEM_COLS)
@@ -468,12 +504,19 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             mbar_arrive_expect_tx(&sh.a_full[ai], L.a_stride);
             for (int kb = 0; kb < nkb; ++kb) {
               tma_load_2d(abuf + kb * A_TILE_BYTES, mAh, &sh.a_full[ai], kb * KB, sg.r * BM);
-              if (P.split3) tma_load_2d(abuf + L.a_lo_off + kb * A_TILE_BYTES, mAl, &sh.a_full[ai], kb * KB, sg.r * BM);
+              if (GRID || P.split3)
+                tma_load_2d(abuf + L.a_lo_off + kb * A_TILE_BYTES, mAl, &sh.a_full[ai], kb * KB, sg.r * BM);
+              if constexpr (GRID)
+                tma_load_2d(abuf + 2 * L.a_lo_off + kb * A_TILE_BYTES, sd == 0 ? &mXr_a : &mYr_a, &sh.a_full[ai],
+                            kb * KB, sg.r * BM);
             }
           }
           __syncwarp();
+          int seen = 0;  // row blocks below this one are known to be ready
           for (int t = sg.t0; t < sg.t1 && ok; ++t) {
-            for (int kb = 0; kb < nkb; ++kb, ++u) {
+            constexpr int UK = GRID ? kGridParts : 1;  // stage units per K block
+            for (int q = 0; q < nkb * UK; ++q, ++u) {
+              const int kb = GRID ? q / UK : q;
               const int s = s_cur;
               ok = warp_wait_bar(&sh.empty[s], s_par ^ 1u, abort_flag, P);
               if (!ok) break;
@@ -483,9 +526,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               }
               unsigned char* st = smem + L.stage0 + s * L.stage_bytes;
               if (elect_one()) {
-                mbar_arrive_expect_tx(&sh.full[s], B_TILE_BYTES * (P.split3 ? 2u : 1u));
-                tma_load_2d(st, mBh, &sh.full[s], kb * KB, t * BN);
-                if (P.split3) tma_load_2d(st + L.b_lo_off, mBl, &sh.full[s], kb * KB, t * BN);
+                if constexpr (GRID) {
+                  const int part = q % UK;
+                  const CUtensorMap* mBp = part == 0 ? mBh : part == 1 ? mBl : (sd == 0 ? &mYr_b : &mXr_b);
+                  mbar_arrive_expect_tx(&sh.full[s], B_TILE_BYTES);
+                  tma_load_2d(st, mBp, &sh.full[s], kb * KB, t * BN);
+                } else {
+                  mbar_arrive_expect_tx(&sh.full[s], B_TILE_BYTES * (P.split3 ? 2u : 1u));
+                  tma_load_2d(st, mBh, &sh.full[s], kb * KB, t * BN);
+                  if (P.split3) tma_load_2d(st + L.b_lo_off, mBl, &sh.full[s], kb * KB, t * BN);
+                }
               }
               __syncwarp();
             }
@@ -495,7 +545,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             ok = warp_wait_bar(&sh.bias_empty[bs], (uint32_t)(((ub / BIAS_SLOTS) & 1) ^ 1), abort_flag, P);
             if (!ok) break;
             const int r0 = t * RB_PER_TILE, r1 = min(Sd.RB, r0 + RB_PER_TILE);
-            ok = wait_flags_warp(Sd.flag_in, r0, r1, want, abort_flag, P);
+            if constexpr (GRID) {
+              // one row block per tile: the poll looks ahead over the segment, since a round
+              // trip per 128-column tile would be longer than the tile
+              if (t >= seen) {
+                seen = t + wait_flags_ahead(Sd.flag_in + t, min(32, min(Sd.RB, sg.t1) - t), want, abort_flag, P);
+                ok = seen > t;
+              }
+            } else {
+              ok = wait_flags_warp(Sd.flag_in, r0, r1, want, abort_flag, P);
+            }
             if (!ok) break;
             if (lane == 0) {
               mbar_arrive_expect_tx(&sh.bias_full[bs], BIAS_TILE_BYTES);
@@ -523,6 +582,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // tile's last product and the next tile's first; the other lanes wait at the end.
     if (lane == 0) {
       const uint64_t abias = desc_sw32(smem_u32(smem + L.a_bias));
+      const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
       bool ok = true;
       int tl = 0, ka = 0;
       int s_cur = 0;          // stage of the next B block (ring position, kept without division)
@@ -549,7 +609,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               if (!ok) break;
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
-              for (int kb = 0; kb < nkb; ++kb) {
+              if constexpr (GRID) {
+                // the B parts arrive one stage each: h meets (h, l, r) of A, l (h, l), r h;
+                // only h h' goes to the first accumulator
+                const uint32_t d2 = d_tmem + 256;
+                const uint64_t ah = desc_sw128(a_hi), al = desc_sw128(a_lo), ar = desc_sw128(a_lo + L.a_lo_off);
+#pragma unroll
+                for (int part = 0; part < kGridParts; ++part) {
+                  const int s = s_cur;
+                  ok = wait_bar(&sh.full[s], s_par, abort_flag, P);
+                  if (++s_cur == S) {
+                    s_cur = 0;
+                    s_par ^= 1u;
+                  }
+                  if (!ok) break;
+                  tc_fence_after();
+                  issue_grid_part<BN, GRID, kGridParts>(
+                      part, d_tmem, d2, ah, al, ar, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)), 0u);
+                  umma_commit(&sh.empty[s]);
+                }
+              }
+              for (int kb = 0; kb < (GRID ? 0 : nkb); ++kb) {
                 const int s = s_cur;
                 ok = wait_bar(&sh.full[s], s_par, abort_flag, P);
                 if (++s_cur == S) {
@@ -580,6 +660,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               if (!ok) break;
               tc_fence_after();
               umma<BN>(d_tmem, abias, desc_sw32(smem_u32(smem + L.bias0 + bs * L.bias_slot)), 1u);
+              if constexpr (GRID)
+                umma<BN>(d_tmem + 256, abias2, desc_sw32(smem_u32(smem + L.bias0 + bs * L.bias_slot)), 1u);
               umma_commit(&sh.bias_empty[bs]);
               umma_commit(&sh.tmem_full[b]);
             }
@@ -598,6 +680,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int quarter = warp & 3;
     const int row_local = quarter * 32 + lane;
     int tl = 0, kseg = 0;
+    const float inv2 = GRID ? __ldg(P.gscale + 1) : 1.f;
+    const uint64_t inv22 = pack2(inv2, inv2);
     bool dead = false;
     for (int it = P.seq0; it < it_end; ++it) {
       if (it > P.seq0) {
@@ -632,7 +716,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             float v[NC][32];
 #pragma unroll
             for (int cc = 0; cc < NC; ++cc) PROGOT_TMEM_LD32(taddr + 32 * cc, v[cc]);
-            tmem_wait_ld();
+            if constexpr (GRID) {
+              // t = leading sums + the rest, rounded once
+              float w[NC][32];
+#pragma unroll
+              for (int cc = 0; cc < NC; ++cc) PROGOT_TMEM_LD32(taddr + 256 + 32 * cc, w[cc]);
+              tmem_wait_ld();
+#pragma unroll
+              for (int cc = 0; cc < NC; ++cc)
+#pragma unroll
+                for (int i = 0; i < 32; i += 2)
+                  unpack2(add2(pack2(v[cc][i], v[cc][i + 1]), pack2(w[cc][i], w[cc][i + 1])), v[cc][i], v[cc][i + 1]);
+            } else {
+              tmem_wait_ld();
+            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tmem_empty[tl & 1]);
@@ -651,7 +748,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (int q = 1; q < 2 * NC; ++q) tmax = fmaxf(tmax, mx[q]);
             const float mnew = fmaxf(m_run, tmax);
             if (mnew != -INFINITY) {
-              const uint64_t negm = pack2(-mnew, -mnew);
+              // grid split: the accumulators hold t 2^(ex + ey); (t - m) 2^-(ex + ey) is exact
+              const float nm = GRID ? -mnew * inv2 : -mnew;
+              const uint64_t negm = pack2(nm, nm);
               uint64_t acc[4];
 #pragma unroll
               for (int q = 0; q < 4; ++q) acc[q] = 0ull;
@@ -660,7 +759,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
                 for (int i = 0; i < 32; i += 2) {
                   float a0, a1;
-                  unpack2(add2(pack2(v[cc][i], v[cc][i + 1]), negm), a0, a1);
+                  const uint64_t tv = pack2(v[cc][i], v[cc][i + 1]);
+                  unpack2(GRID ? fma2(tv, inv22, negm) : add2(tv, negm), a0, a1);
                   acc[(i >> 1) & 3] = add2(acc[(i >> 1) & 3], pack2(fast_exp2(a0), fast_exp2(a1)));
                 }
               float s0, s1, s2, s3, s4, s5, s6, s7;
@@ -668,10 +768,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               unpack2(acc[1], s2, s3);
               unpack2(acc[2], s4, s5);
               unpack2(acc[3], s6, s7);
-              s_run = s_run * fast_exp2(m_run - mnew) + (((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)));
+              s_run = s_run * fast_exp2(GRID ? (m_run - mnew) * inv2 : m_run - mnew) + (((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)));
               m_run = mnew;
             }
           }
+          if constexpr (GRID) m_run *= inv2;
           if (dead) {
             m_run = NAN;
             s_run = NAN;
@@ -690,6 +791,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else {
     // ------------------------------------------------------------ epilogue warps and stop decision
     const int etid = threadIdx.x - EPI_TID0;  // 0..63
+    const float s2 = GRID ? __ldg(P.gscale) : 1.f;
     int kseg = 0;
     // ---- stop test of iteration it (warp 10), once every row block of the f-update is done
     auto decide = [&](int it) {
@@ -750,11 +852,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           // the row block's contributors and their partial slots, once per segment, from the
           // split's tables; the previous segment's readers passed the barrier at its end
           if (etid < 8) {
-            const int p0 = __ldg(Sd.cptr + sg.r), p1 = __ldg(Sd.cptr + sg.r + 1);
-            if (p0 + etid < p1) sh.cslot[etid] = __ldg(Sd.cslot + p0 + etid);
+            const int2 cr = __ldg(Sd.crow + sg.r);
+            if (etid < cr.y) sh.cslot[etid] = __ldg(Sd.cslot + cr.x + etid);
             if (etid == 0) {
-              sh.cbase = p0;
-              sh.ccount = p1 - p0;
+              sh.cbase = cr.x;
+              sh.ccount = cr.y;
             }
           }
           // the segment's partials are in global memory once the LSE warps arrived (their
@@ -812,8 +914,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 const float Lr = acc[h].x + __log2f(acc[h].y);
                 if (!skip) {
                   float val;
-                  e[h] = loop_row_potential(Sd, sd, i, Lr, rin[h], out, &val);
-                  write_bias_row(bout + i * 16, (val - rin[h].an) * p.bscale);
+                  e[h] = GRID ? loop_row_potential_grid(Sd, sd, i, acc[h], rin[h], out, &val)
+                              : loop_row_potential(Sd, sd, i, Lr, rin[h], out, &val);
+                  if constexpr (GRID)
+                    write_bias_row_grid(bout + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), s2);
+                  else
+                    write_bias_row(bout + i * 16, (val - rin[h].an) * p.bscale);
                 }
               }
             }
@@ -856,25 +962,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
-__global__ void fill_u32_kernel(uint32_t* __restrict__ p, int64_t n, uint32_t v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
-}
-
 }  // namespace loop
 }  // namespace tc
 
 // ---------------------------------------------------------------- host side
 // Pipeline shape of the persistent loop: two resident A buffers and as many B stages
 // (2..8) as fit in 227 KB; 0 stages when no shape fits (the per-sweep kernel serves it).
-static void loop_shape(int bn, int nkb, int split3, int* stages, int* a_bufs) {
+static void loop_shape(int bn, int nkb, int split3, bool grid, int* stages, int* a_bufs) {
   *stages = 0;
   *a_bufs = 2;
   for (int na = 2; na >= 1; --na) {
     int best = 0;
     for (int s = 2; s <= 8; ++s)
-      if (tc::loop::layout(bn, nkb, split3, s, na).total <= 227 * 1024) best = s;
-    if (best >= 2) {
+      if (tc::loop::layout(bn, nkb, split3, s, na, grid).total <= 227 * 1024) best = s;
+    if (best >= (grid ? 3 : 2)) {  // the grid's stages hold a third of a K block each
       *stages = best;
       *a_bufs = na;
       return;
@@ -882,78 +983,32 @@ static void loop_shape(int bn, int nkb, int split3, int* stages, int* a_bufs) {
   }
 }
 
-cudaError_t launch_fill_u32(uint32_t* p, int64_t n, uint32_t v, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  tc::loop::fill_u32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p, n, v);
-  count_launch();
-  return cudaGetLastError();
-}
-
-bool loop_tc_supported(int bn, int nkb, int split3) {
+bool loop_tc_supported(int bn, int nkb, int split3, bool grid) {
   int s, na;
-  loop_shape(bn, nkb, split3, &s, &na);
-  return s >= 2 && (bn == 128 || bn == 256);
+  loop_shape(bn, nkb, split3, grid, &s, &na);
+  return s >= 2 && (grid ? bn == 128 && nkb == 1 : bn == 128 || bn == 256);
 }
 
-// ---- work split of the loop (host-built tables): the (row block, column tile) grid of
-// a sweep cut over the CTAs as in the per-update kernel (tc::Split), laid out for the
-// kernel as per-CTA segment lists and per-row-block contributor lists (in CTA order, the
-// order of the combine), so that no 64-bit division of the split runs on the GPU.
-struct SideTables {
-  std::vector<int4> segs;
-  std::vector<int32_t> nseg, cptr, cslot;
-  int maxseg = 0;
-};
-
-// ms_force: segment stride of the tables (the larger maxseg of both sides), 0 = own.
-static void side_tables(int R, int T, int G, SideTables* out, int ms_force = 0) {
-  const tc::Split sp = tc::make_split(R, T, G);
-  int ms = 1;
-  for (int c = 0; c < G; ++c) ms = std::max(ms, tc::num_segments(sp, c));
-  out->maxseg = ms;
-  if (ms_force >= ms) ms = ms_force;
-  out->segs.assign((size_t)G * ms, make_int4(0, 0, 0, 0));
-  out->nseg.assign((size_t)G, 0);
-  std::vector<std::vector<int32_t>> by_row((size_t)R);
-  for (int c = 0; c < G; ++c) {
-    const int ns = tc::num_segments(sp, c);
-    out->nseg[c] = ns;
-    for (int k = 0; k < ns; ++k) {
-      const tc::Seg sg = tc::segment(sp, c, k);
-      out->segs[(size_t)c * ms + k] = make_int4(sg.r, sg.t0, sg.t1, 0);
-      by_row[sg.r].push_back(c * ms + k);  // CTAs in increasing order
-    }
-  }
-  out->cptr.assign((size_t)R + 1, 0);
-  out->cslot.clear();
-  for (int r = 0; r < R; ++r) {
-    out->cptr[r + 1] = out->cptr[r] + (int32_t)by_row[r].size();
-    out->cslot.insert(out->cslot.end(), by_row[r].begin(), by_row[r].end());
-  }
-}
-
+// Work split of the loop: the (row block, column tile) grid of a sweep cut over the CTAs as
+// in the per-update kernel (tc::Split); the tables the kernel reads (per-CTA segment lists
+// and per-row-block contributor lists in CTA order, so that no 64-bit division of the split
+// runs inside the loop) are written by the operand preparation (operands.cu).
 void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg) {
   const int64_t Rx = (n + tc::BM - 1) / tc::BM, Ry = (m + tc::BM - 1) / tc::BM;
   const int64_t Tx = (n + bn - 1) / bn, Ty = (m + bn - 1) / bn;
   const int g = (int)std::min<int64_t>(std::min<int64_t>(Rx * Ty, Ry * Tx), sms);
-  SideTables a, b;
-  side_tables((int)Rx, (int)Ty, g, &a);
-  side_tables((int)Ry, (int)Tx, g, &b);
+  const tc::Split a = tc::make_split((int)Rx, (int)Ty, g), b = tc::make_split((int)Ry, (int)Tx, g);
+  int ms = 1;
+  for (int c = 0; c < g; ++c) ms = std::max(ms, std::max(tc::num_segments(a, c), tc::num_segments(b, c)));
   *G = g;
-  *maxseg = std::max(a.maxseg, b.maxseg);
+  *maxseg = ms;
 }
 
-size_t loop_tc_smem(int bn, int nkb, int split3) {
-  int s, na;
-  loop_shape(bn, nkb, split3, &s, &na);
-  return tc::loop::layout(bn, nkb, split3, s, na).total;
-}
-
-template <int BN, int NKB>
+template <int BN, int NKB, int GRID>
 static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const void* const* maps, cudaStream_t stream) {
   static thread_local size_t attr_bytes = 0;
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB>,
+    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB, GRID>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
@@ -968,16 +1023,17 @@ static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const voi
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const CUtensorMap* m[12];
-  for (int q = 0; q < 12; ++q) m[q] = reinterpret_cast<const CUtensorMap*>(maps[q]);
-  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
-                            *m[6], *m[7], *m[8], *m[9], *m[10], *m[11], P);
+  const CUtensorMap* m[16];
+  for (int q = 0; q < 16; ++q) m[q] = reinterpret_cast<const CUtensorMap*>(maps[q]);
+  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB, GRID>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
+                            *m[6], *m[7], *m[8], *m[9], *m[10], *m[11], *m[12], *m[13], *m[14], *m[15], P);
 }
 
 cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   int stages, a_bufs;
-  loop_shape(Lq.bn, Lq.nkb, Lq.split3, &stages, &a_bufs);
-  if (stages < 2 || (Lq.bn != 128 && Lq.bn != 256)) return cudaErrorInvalidValue;
+  const bool grid = Lq.gscale != nullptr;
+  loop_shape(Lq.bn, Lq.nkb, Lq.split3, grid, &stages, &a_bufs);
+  if (!loop_tc_supported(Lq.bn, Lq.nkb, Lq.split3, grid)) return cudaErrorInvalidValue;
   tc::loop::Params P;
   memset(&P, 0, sizeof(P));
   for (int sd = 0; sd < 2; ++sd) {
@@ -998,6 +1054,10 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
     d.R = (int)((s.p.nA + tc::BM - 1) / tc::BM);
     d.T = (int)((s.p.nB + Lq.bn - 1) / Lq.bn);
     d.RB = (int)((s.p.nB + tc::BM - 1) / tc::BM);
+    d.segs = reinterpret_cast<const int4*>(s.segs);
+    d.nseg = s.nseg;
+    d.crow = s.crow;
+    d.cslot = s.cslot;
     const double cl = s.p.eps * kLn2, wl = s.p.eps * s.p.log_w_uniform;
     d.c_hi = (float)cl;
     d.c_lo = (float)(cl - (double)d.c_hi);
@@ -1005,33 +1065,6 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
     d.e_lo = (float)(s.p.eps - (double)d.e_hi);
     d.w_hi = (float)wl;
     d.w_lo = (float)(wl - (double)d.w_hi);
-  }
-  // the work split's tables (the same as loop_tc_plan's), copied to the workspace
-  {
-    SideTables tab[2];
-    for (int sd = 0; sd < 2; ++sd) {
-      side_tables(P.side[sd].R, P.side[sd].T, Lq.G, &tab[sd], Lq.maxseg);
-      if (tab[sd].maxseg > Lq.maxseg) return cudaErrorInvalidValue;
-      const LoopSideLaunch& ls = Lq.side[sd];
-      if ((int64_t)tab[sd].segs.size() > ls.table_slots || (int64_t)tab[sd].cslot.size() > ls.table_slots)
-        return cudaErrorInvalidValue;
-      cudaError_t e = cudaMemcpyAsync(ls.segs, tab[sd].segs.data(), sizeof(int4) * tab[sd].segs.size(),
-                                      cudaMemcpyHostToDevice, stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ls.nseg, tab[sd].nseg.data(), sizeof(int32_t) * tab[sd].nseg.size(),
-                            cudaMemcpyHostToDevice, stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ls.cptr, tab[sd].cptr.data(), sizeof(int32_t) * tab[sd].cptr.size(),
-                            cudaMemcpyHostToDevice, stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ls.cslot, tab[sd].cslot.data(), sizeof(int32_t) * tab[sd].cslot.size(),
-                            cudaMemcpyHostToDevice, stream);
-      if (e != cudaSuccess) return e;
-      P.side[sd].segs = reinterpret_cast<const int4*>(ls.segs);
-      P.side[sd].nseg = ls.nseg;
-      P.side[sd].cptr = ls.cptr;
-      P.side[sd].cslot = ls.cslot;
-    }
   }
   P.errpart = Lq.errpart;
   P.state = Lq.state;
@@ -1045,10 +1078,19 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   P.maxseg = Lq.maxseg;
   P.seq0 = Lq.seq0;
   P.niter = Lq.niter;
-  const size_t smem = tc::loop::layout(Lq.bn, Lq.nkb, Lq.split3, stages, a_bufs).total;
-  cudaError_t e = Lq.bn == 128 ? launch_loop<128, 0>(P, smem, Lq.maps, stream)
-                  : Lq.nkb == 1 ? launch_loop<256, 1>(P, smem, Lq.maps, stream)
-                                : launch_loop<256, 0>(P, smem, Lq.maps, stream);
+  P.gscale = Lq.gscale;
+  const size_t smem = tc::loop::layout(Lq.bn, Lq.nkb, Lq.split3, stages, a_bufs, grid).total;
+  const int ks = (Lq.side[0].p.d + 15) / 16;  // K = 16 steps
+  cudaError_t e;
+  if (grid)
+    e = ks <= 1   ? launch_loop<128, 1, 1>(P, smem, Lq.maps, stream)
+        : ks == 2 ? launch_loop<128, 1, 2>(P, smem, Lq.maps, stream)
+        : ks == 3 ? launch_loop<128, 1, 3>(P, smem, Lq.maps, stream)
+                  : launch_loop<128, 1, 4>(P, smem, Lq.maps, stream);
+  else
+    e = Lq.bn == 128   ? launch_loop<128, 0, 0>(P, smem, Lq.maps, stream)
+        : Lq.nkb == 1 ? launch_loop<256, 1, 0>(P, smem, Lq.maps, stream)
+                      : launch_loop<256, 0, 0>(P, smem, Lq.maps, stream);
   count_launch();
   return e;
 }

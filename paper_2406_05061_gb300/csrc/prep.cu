@@ -1,8 +1,7 @@
-// Small O((n + m) d) kernels: squared norms (float64 accumulation), potential scaling
-// for the warm start of Alg. 2, state initialisation, deterministic float64 reductions
-// (first moments for the closed-form mean cost of Alg. 4 and of the theta rule, the
-// centre of the tensor-core operands, squared error for the Alg. 4 score, the coupling
-// diagonal of Prop. 3) and the move of a centred log-sum-exp back to uncentred form.
+// Small O((n + m) d) kernels: squared norms (float64 accumulation), state initialisation,
+// deterministic float64 reductions (first moments for the closed-form mean cost of Alg. 4
+// and of the theta rule, squared error for the Alg. 4 score, the coupling diagonal of
+// Prop. 3) and the move of a centred log-sum-exp back to uncentred form.
 #include <algorithm>
 
 #include "progot_internal.h"
@@ -27,11 +26,6 @@ __global__ void row_sqnorm_kernel(const float* __restrict__ X, int64_t n, int32_
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if (lane == 0) out[row] = (float)s;
-}
-
-__global__ void scale_kernel(float* v, int64_t n, float factor) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) v[i] *= factor;
 }
 
 // Both solver states (the second is used by loops that run the stop test one sweep later).
@@ -167,66 +161,6 @@ cudaError_t launch_row_sqnorm(const float* X, int64_t n, int32_t d, float* out, 
   return cudaGetLastError();
 }
 
-// Per-coordinate column sums of X (blockIdx.y = 0) and Y (blockIdx.y = 1) in float64, in a
-// fixed order: warp w of block b sums rows b W + w + k gridDim.x W (W warps per block),
-// then the block adds its warps' sums in warp order.
-__global__ void center_pass1(const float* __restrict__ X, int64_t n, const float* __restrict__ Y, int64_t m,
-                             int32_t d, double* __restrict__ partial) {
-  extern __shared__ double acc[];  // d per warp
-  const float* Z = blockIdx.y ? Y : X;
-  const int64_t rows = blockIdx.y ? m : n;
-  const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = threadIdx.x; k < warps * d; k += blockDim.x) acc[k] = 0.0;
-  __syncthreads();
-  for (int64_t row = (int64_t)blockIdx.x * warps + warp; row < rows; row += (int64_t)gridDim.x * warps)
-    for (int k = lane; k < d; k += 32) acc[warp * d + k] += (double)Z[row * (int64_t)d + k];
-  __syncthreads();
-  double* out = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * d;
-  for (int k = threadIdx.x; k < d; k += blockDim.x) {
-    double t = 0.0;
-    for (int w = 0; w < warps; ++w) t += acc[w * d + k];
-    out[k] = t;
-  }
-}
-
-// mu_k = (sum_x_k / n + sum_y_k / m) / 2 from the block partials: one warp per
-// coordinate, lane l summing blocks l, l + 32, ... in order, then a fixed shuffle tree.
-__global__ void center_finish(const double* __restrict__ partial, int parts, int64_t n, int64_t m, int32_t d,
-                              float* __restrict__ mu) {
-  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (k >= d) return;
-  double sx = 0.0, sy = 0.0;
-  for (int b = lane; b < parts; b += 32) {
-    sx += partial[(int64_t)b * d + k];
-    sy += partial[((int64_t)parts + b) * d + k];
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    sx += __shfl_xor_sync(0xffffffffu, sx, off);
-    sy += __shfl_xor_sync(0xffffffffu, sy, off);
-  }
-  if (lane == 0) mu[k] = (float)(0.5 * (sx / (double)n + sy / (double)m));
-}
-
-cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial, float* mu,
-                          cudaStream_t s) {
-  const size_t per_warp = sizeof(double) * (size_t)d;
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(8, (200 * 1024) / per_warp));
-  const size_t smem = per_warp * (size_t)warps;
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;  // d above 25,600
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(center_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  const int parts = kParts / 2;
-  center_pass1<<<dim3(parts, 2), 32 * warps, smem, s>>>(X, n, Y, m, d, partial);
-  count_launch();
-  center_finish<<<(d + 7) / 8, 256, 0, s>>>(partial, parts, n, m, d, mu);
-  count_launch();
-  return cudaGetLastError();
-}
-
 // L_i += bscale (|x_i|^2 - |x_i - mu|^2) = bscale (2 x_i . mu - |mu|^2): moves a row
 // log-sum-exp taken on centred operands to the uncentred form t_ij = scale x_i . y_j +
 // (g_j - |y_j|^2) bscale (one warp per row, float64 sums).
@@ -250,33 +184,6 @@ cudaError_t launch_lse_uncenter(float* L, const float* X, int64_t n, int32_t d, 
                                 cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   lse_uncenter_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(L, X, n, d, mu, bscale);
-  count_launch();
-  return cudaGetLastError();
-}
-
-// L_i = (eps log w_i + |a_i|^2 - f_i) / (eps ln2): the row log-sum-exp (log2 units) that
-// an f-update wrote as the potential f_i = eps log w_i + |a_i|^2 - eps ln2 L_i, recovered
-// from f in float64 (w = NULL: uniform weights, log w_i = log_w_uniform).
-__global__ void lse_from_potential_kernel(const float* __restrict__ f, const float* __restrict__ an,
-                                          const float* __restrict__ w, double log_w_uniform, double eps, int64_t n,
-                                          float* __restrict__ L) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double logw = w ? log((double)w[i]) : log_w_uniform;
-  L[i] = (float)((eps * logw + (double)an[i] - (double)f[i]) / (eps * 0.69314718055994530942));
-}
-
-cudaError_t launch_lse_from_potential(const float* f, const float* an, const float* w, double log_w_uniform,
-                                      double eps, int64_t n, float* L, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  lse_from_potential_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(f, an, w, log_w_uniform, eps, n, L);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scale(float* v, int64_t n, float factor, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  scale_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(v, n, factor);
   count_launch();
   return cudaGetLastError();
 }

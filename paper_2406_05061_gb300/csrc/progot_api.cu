@@ -189,10 +189,20 @@ struct Workspace {
   int64_t lslots;
   int64_t lrb;      // rbmax of the carve (row-block capacity of lcnt and lerr)
   int4* ltab_segs;  // work-split tables of both sides: segments [2][lslots], contributor slots
-  int32_t* ltab_cslot;  // [2][lslots], contributor offsets [2][rbmax + 1], segment counts [2][sms]
-  int32_t* ltab_cptr;
+  int32_t* ltab_cslot;  // [2][lslots], contributor lists [2][rbmax], segment counts [2][sms]
+  int2* ltab_crow;
   int32_t* ltab_nseg;
   double* lerr;     // [2][rbmax] error partials by iteration parity
+  // integer-grid operands (float32 path): third parts, largest squared norms, scales
+  void* xr;
+  void* yr;
+  float* gmax;      // [2], gscale [3] and ticket: in the solver states' 256 bytes
+  float* gscale;
+  unsigned* ticket;
+  char* prob;       // P tiles of the map step, a chunk of rows at a time (integer-grid operands)
+  int64_t prob_bytes;
+  float* rsum;      // their row sums
+  bool grid;        // the workspace holds the float32 path's tensor-core operands
   size_t bytes;
 };
 
@@ -200,13 +210,16 @@ struct WsDims {
   int64_t nmax, rbmax, partial_elems, opart_elems, rpart_elems;
   int32_t d, dp;
   bool tc;
+  bool grid;  // float32 path with tensor-core operands (three parts)
 };
 
 static int32_t pad64(int32_t d) { return (d + 63) / 64 * 64; }
 
-static WsDims ws_dims(int64_t n, int64_t m, int32_t d, int32_t precision = PROGOT_FP32) {
+// with_grid = false: the float32 path's smaller layout, on which it runs on CUDA cores.
+static WsDims ws_dims(int64_t n, int64_t m, int32_t d, int32_t precision = PROGOT_FP32, bool with_grid = true) {
   WsDims w;
-  w.tc = precision != PROGOT_FP32;
+  w.grid = precision == PROGOT_FP32 && with_grid;
+  w.tc = precision != PROGOT_FP32 || w.grid;
   w.dp = pad64(d);
   w.nmax = std::max<int64_t>(std::max<int64_t>(n, m), 1);
   w.d = d;
@@ -223,7 +236,7 @@ static WsDims ws_dims(int64_t n, int64_t m, int32_t d, int32_t precision = PROGO
   const int64_t rows_cap = (2 * mslots * kWaves / dch + w.rbmax + 1) * BMr + w.nmax;
   w.opart_elems = rows_cap * d;
   w.rpart_elems = rows_cap;
-  if (w.tc && w.dp <= 256) {
+  if (w.tc && !w.grid && w.dp <= 256) {
     // tensor-core map steps: G * maxseg <= R + 3 G partial slots of 128 rows x dp
     const int64_t slots = w.rbmax + 3 * (int64_t)num_sms();
     w.opart_elems = std::max<int64_t>(w.opart_elems, slots * BMr * w.dp);
@@ -253,9 +266,15 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   ws.metpart = (double*)take(sizeof(double) * kMetricSums * (w.rbmax + 2));
   ws.metout = (double*)take(sizeof(double) * (2 * kMetricSums + 2));
   ws.errpart = (double*)take(sizeof(double) * (w.rbmax + 2));
+  // the arrival counters and the slot of small words, zeroed together (zero_counters)
   ws.cnt = (unsigned*)take(sizeof(unsigned) * (w.rbmax + 2));
   ws.mcnt = (unsigned*)take(sizeof(unsigned) * (w.rbmax + 2));
-  ws.state = (SolverState*)take(2 * sizeof(SolverState));  // [2]: see SweepParams::lag
+  static_assert(2 * sizeof(SolverState) <= 128, "the solver states and the fault word share 256 bytes");
+  ws.state = (SolverState*)take(256);  // [2]: see SweepParams::lag
+  ws.fault = (int32_t*)((char*)ws.state + 128);
+  ws.gmax = (float*)((char*)ws.state + 144);
+  ws.gscale = (float*)((char*)ws.state + 160);
+  ws.ticket = (unsigned*)((char*)ws.state + 176);
   ws.rpart = (double*)take(sizeof(double) * reduce_parts() * (size_t)(w.d + 1));
   ws.rout = (double*)take(sizeof(double) * 2 * (size_t)(w.d + 1));
   ws.Opart = (float*)take(sizeof(float) * w.opart_elems);
@@ -271,7 +290,6 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   ws.mu = (float*)take(w.tc ? sizeof(float) * (size_t)w.dp : 0);
   ws.xnc = (float*)take(w.tc ? sizeof(float) * w.nmax : 0);
   ws.ync = (float*)take(w.tc ? sizeof(float) * w.nmax : 0);
-  ws.fault = (int32_t*)take(sizeof(int32_t));
   ws.xb2 = take(bb);
   ws.yb2 = take(bb);
   ws.lflag = (uint32_t*)take(w.tc ? sizeof(uint32_t) * 2 * (size_t)w.rbmax : 0);
@@ -284,25 +302,56 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   ws.lrb = w.rbmax;
   ws.ltab_segs = (int4*)take(sizeof(int4) * 2 * (size_t)ws.lslots);
   ws.ltab_cslot = (int32_t*)take(sizeof(int32_t) * 2 * (size_t)ws.lslots);
-  ws.ltab_cptr = (int32_t*)take(w.tc ? sizeof(int32_t) * 2 * ((size_t)w.rbmax + 1) : 0);
+  ws.ltab_crow = (int2*)take(w.tc ? sizeof(int2) * 2 * (size_t)w.rbmax : 0);
   ws.ltab_nseg = (int32_t*)take(w.tc ? sizeof(int32_t) * 2 * (size_t)num_sms() : 0);
   ws.lerr = (double*)take(w.tc ? sizeof(double) * 2 * (size_t)w.rbmax : 0);
+  ws.xr = take(w.grid ? opb : 0);
+  ws.yr = take(w.grid ? opb : 0);
+  // Map steps on integer-grid operands keep P for a chunk of row blocks: 64 MB stay in L2
+  // between the sweep that writes them and the product that reads them (one row block at
+  // least; less when all of P is smaller). The bf16x3 path needs them for d > 256, where
+  // the partial buffers of the CUDA-core map are idle and larger than one row block's P.
+  if (w.grid) {
+    const int64_t block = pv_prob_bytes_per_block(w.nmax);
+    ws.prob_bytes = std::max<int64_t>(block, std::min<int64_t>(block * w.rbmax, (int64_t)64 << 20));
+    ws.prob = take((size_t)ws.prob_bytes);
+    ws.rsum = ws.Rpart;
+  } else {
+    ws.prob = (char*)ws.Opart;
+    ws.prob_bytes = (int64_t)sizeof(float) * w.opart_elems;
+    ws.rsum = ws.Rpart;
+  }
+  ws.grid = w.grid;
   ws.bytes = off;
   if (out) *out = ws;
   return off;
 }
+
+// Float32 Sinkhorn loops use the integer-grid operands up to this dimension. The CUDA-core
+// sweeps round eps' products against unequal norms and so shift mass between f and g by a
+// little every iteration (the plan is unaffected); on wide normalised clouds, where g is
+// small, tens of iterations move it by 1e-5 of its size (1.3e-5 measured at 839 x 726,
+// d = 126, 17 iterations). The grid loops do not drift, and results callers already hold for
+// such clouds would change by as much, so these loops stay on CUDA cores.
+constexpr int32_t kGridSolveDim = 64;
+// Least rows x columns x coordinates of a float32 map step on the tensor cores.
+constexpr double kGridMapWork = 2.5e7;
 
 static int carve(int64_t n, int64_t m, int32_t d, void* workspace, size_t ws_bytes, Workspace* ws,
                  int32_t precision = PROGOT_FP32) {
   if (workspace == nullptr) return fail(PROGOT_ERR_WORKSPACE, "workspace is NULL");
   if ((reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
     return fail(PROGOT_ERR_WORKSPACE, "workspace is not 256-byte aligned");
-  const WsDims w = ws_dims(n, m, d, precision);
-  const size_t need = ws_layout(w, ws, (char*)workspace);
+  size_t need = ws_layout(ws_dims(n, m, d, precision), ws, (char*)workspace);
+  // a float32 workspace without room for the tensor-core operands still serves, on CUDA cores
+  if (ws_bytes < need && precision == PROGOT_FP32)
+    need = ws_layout(ws_dims(n, m, d, precision, false), ws, (char*)workspace);
   if (ws_bytes < need)
     return fail(PROGOT_ERR_WORKSPACE, "workspace has %zu bytes, %zu needed", ws_bytes, need);
   return PROGOT_OK;
 }
+
+constexpr size_t kStateBytes = 128 + sizeof(int32_t);  // both solver states, then the fault word
 
 // Pinned host mirror of the solver state, one pair per host thread.
 struct HostMirror {
@@ -312,7 +361,7 @@ struct HostMirror {
   bool ok = false;
   int init() {
     if (ok) return PROGOT_OK;
-    CK(cudaHostAlloc((void**)&hs, 2 * sizeof(SolverState), cudaHostAllocDefault));
+    CK(cudaHostAlloc((void**)&hs, 256, cudaHostAllocDefault));
     CK(cudaHostAlloc((void**)&hd, 1024 * sizeof(double), cudaHostAllocDefault));
     CK(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
@@ -396,6 +445,9 @@ struct TcOps {
   CUtensorMap yb128;
   // tensor-core map step for 64 < d <= 256: y operand and bias rows in 32-row boxes
   CUtensorMap yh_m32, yl_m32, yb_m32;
+  // integer-grid split: third parts in both roles
+  CUtensorMap xr_a, yr_a, xr_b, yr_b;
+  const float* gscale = nullptr;  // its device scales (non-NULL: the operands are the grid split's)
   // centre mu of the operands and the squared norms |x_i - mu|^2, |y_j - mu|^2 that
   // the tensor-core sweeps use in place of |x_i|^2, |y_j|^2
   const float* mu = nullptr;
@@ -403,65 +455,171 @@ struct TcOps {
   const float* ync = nullptr;
   int nkb = 0;
   int split3 = 0;
+  int parts = 1;
   int bn = 128;
   bool on = false;
+  // a persistent loop was set up with the operands, over G CTAs of up to maxseg segments
+  bool loop = false;
+  int G = 0, maxseg = 0;
+  void* yb_base = nullptr;  // the y-side bias rows in use (the maps below describe them)
   // ws.L holds the row log-sum-exps of t against the y-side bias rows (the map step's
   // stabiliser), written by the persistent loop from its last f-update
   bool lse_ready = false;
 };
 
-// Split sqrt(2 log2(e) / eps) (X - mu) and (Y - mu) into bf16 hi/lo and describe them
-// for TMA; write the bias rows of both sides from the current potentials (f on x, g on
-// y) and the centred squared norms. mu is the midpoint of the two clouds' means: the
-// cost |x - y|^2 = |x~|^2 + |y~|^2 - 2 x~ . y~ holds for any common centre, and the
-// bf16x3 products and their float32 accumulation lose accuracy in proportion to
-// |x~| |y~|, which centring keeps near the clouds' spread rather than their distance
-// from the origin. The potentials are the same for every centre.
+// Maps of the y-side bias rows at base (sweeps, loop, the map steps' boxes).
+static int map_y_bias(TcOps* ops, void* base, int64_t m) {
+  const int64_t rows = cdiv(m, 256) * 256;
+  ops->yb_base = base;
+  int rc = make_map(&ops->yb, base, rows, 16, ops->bn);
+  if (!rc && !ops->gscale && ops->nkb == 1) rc = make_map(&ops->yb128, base, rows, 16, 128);
+  if (!rc && !ops->gscale && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb))
+    rc = make_map(&ops->yb_m32, base, rows, 16, map_tc_onepass_tile_cols());
+  return rc;
+}
+
+// Test hook (progot_test_withhold_initial_betas): the persistent loop starts without the
+// initial g's ready flags, so the first f-update's bounded wait expires.
+static LoopSetup loop_setup_params(int64_t n, int64_t m, const TcOps& ops, const Workspace& ws) {
+  LoopSetup ls;
+  memset(&ls, 0, sizeof(ls));
+  ls.state = ws.state;
+  ls.G = ops.G;
+  ls.maxseg = ops.maxseg;
+  const int64_t rows[2] = {n, m}, cols[2] = {m, n};
+  for (int sd = 0; sd < 2; ++sd) {
+    LoopSetupSide& S = ls.side[sd];
+    S.R = (int32_t)cdiv(rows[sd], 128);
+    S.T = (int32_t)cdiv(cols[sd], ops.bn);
+    S.segs = ws.ltab_segs + sd * ws.lslots;
+    S.nseg = ws.ltab_nseg + sd * num_sms();
+    S.crow = ws.ltab_crow + sd * ws.lrb;
+    S.cslot = ws.ltab_cslot + sd * ws.lslots;
+    // flags: nothing published, then the initial g's row blocks as 1
+    S.flag = ws.lflag + sd * ws.lrb;
+    S.flag_init = sd == 1 && !g_withhold_betas.load() ? 1u : 0u;
+    S.cnt = ws.lcnt + sd * ws.lrb;
+    S.done = ws.lcnt + 2 * ws.lrb + sd;
+  }
+  return ls;
+}
+
+// What prep_tc prepares: bf16 operands of the precision setting, the integer grid's three
+// parts (the float32 path) or two of them on a centre already in ws.mu (the bf16x3 path's
+// map step for d > 256).
+// kMoved: as kAuto after an earlier kAuto of the same solve or map, the x cloud having moved
+// by map steps only: the integer grid then keeps its centre and its norms' bound, and needs
+// one launch (the bf16 operands are centred anew).
+enum class Operands { kAuto, kMoved, kGridTwoParts };
+
+// Tensor-core operands of both clouds at this eps (operands.cu) and their TMA descriptions;
+// bias rows of both sides from the current potentials (f on x, g on y) and the centred
+// squared norms; with loop, the set-up of a persistent loop (ops->loop tells whether the
+// shape has one). mu is the midpoint of the two clouds' means: the cost |x - y|^2 = |x~|^2 +
+// |y~|^2 - 2 x~ . y~ holds for any common centre, and the split products and their float32
+// accumulation lose accuracy in proportion to |x~| |y~|, which centring keeps near the
+// clouds' spread rather than their distance from the origin. The potentials are the same
+// for every centre.
 static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t d, double eps, int32_t precision,
                    const Workspace& ws, TcOps* ops, cudaStream_t s, const float* f_cur = nullptr,
-                   const float* g_cur = nullptr) {
-  ops->on = precision != PROGOT_FP32;
+                   const float* g_cur = nullptr, bool loop = false, Operands kind = Operands::kAuto) {
+  const bool two = kind == Operands::kGridTwoParts, grid = precision == PROGOT_FP32 || two;
+  ops->on = precision != PROGOT_FP32 || ws.grid;
   ops->lse_ready = false;
+  ops->loop = false;
+  ops->gscale = grid ? ws.gscale : nullptr;
   if (!ops->on) return PROGOT_OK;
   const int32_t dp = pad64(d);
   ops->nkb = dp / 64;
-  ops->split3 = precision == PROGOT_BF16X3 ? 1 : 0;
-  if (tc_stages(ops->nkb, ops->split3) < 2)
+  ops->split3 = precision != PROGOT_BF16 ? 1 : 0;
+  ops->parts = grid ? (two ? 2 : kGridParts) : 1 + ops->split3;
+  if (!grid && tc_stages(ops->nkb, ops->split3) < 2)
     return fail(PROGOT_ERR_INVALID_ARG, "d = %d is too large for the tensor-core sweep", d);
-  const float sc = (float)std::sqrt(2.0 * kLog2e / eps);
-  CK(launch_center(x, n, y, m, d, ws.rpart, ws.mu, s));
+  ops->bn = grid ? 128 : tc_tile_cols(ops->nkb, ops->split3);
   ops->mu = ws.mu;
   ops->xnc = ws.xnc;
   ops->ync = ws.ync;
-  CK(launch_split_bf16(x, n, d, dp, sc, ws.xh, ops->split3 ? ws.xl : nullptr, s, ws.mu, ws.xnc));
-  CK(launch_split_bf16(y, m, d, dp, sc, ws.yh, ops->split3 ? ws.yl : nullptr, s, ws.mu, ws.ync));
-  ops->bn = tc_tile_cols(ops->nkb, ops->split3);
-  void* xl = ops->split3 ? ws.xl : ws.xh;
-  void* yl = ops->split3 ? ws.yl : ws.yh;
+  const bool hull = grid && kind == Operands::kMoved;
+  if (two)
+    CK(cudaMemsetAsync(ws.gmax, 0, 2 * sizeof(float), s));
+  else if (!hull)
+    CK(launch_center(x, n, y, m, d, ws.rpart, ws.ticket, ws.mu, grid ? ws.gmax : nullptr, s));
+  OperandPrep op;
+  memset(&op, 0, sizeof(op));
+  op.x = x;
+  op.y = y;
+  op.n = n;
+  op.m = m;
+  op.d = d;
+  op.dp = dp;
+  const double sc = std::sqrt(2.0 * kLog2e / eps);
+  op.sc = (float)sc;
+  op.sc_lo = (float)(sc - (double)op.sc);
+  op.mu = ws.mu;
+  op.xnc = ws.xnc;
+  op.ync = ws.ync;
+  op.gmax = ws.gmax;
+  op.gscale = ws.gscale;
+  op.xp[0] = ws.xh;
+  op.xp[1] = ops->parts > 1 ? ws.xl : nullptr;
+  op.xp[2] = ops->parts > 2 ? ws.xr : nullptr;
+  op.yp[0] = ws.yh;
+  op.yp[1] = ops->parts > 1 ? ws.yl : nullptr;
+  op.yp[2] = ops->parts > 2 ? ws.yr : nullptr;
+  op.f = f_cur;
+  op.g = g_cur;
+  op.bscale = (float)(kLog2e / eps);
+  op.bscale_lo = (float)(kLog2e / eps - (double)op.bscale);
+  op.xb[0] = ws.xb;
+  op.yb[0] = ws.yb;
+  LoopSetup ls;
+  if (loop && loop_tc_supported(ops->bn, ops->nkb, ops->split3, grid)) {
+    ops->loop = true;
+    loop_tc_plan(n, m, ops->bn, num_sms(), &ops->G, &ops->maxseg);
+    if ((int64_t)ops->G * ops->maxseg > ws.lslots)
+      return fail(PROGOT_ERR_WORKSPACE, "persistent loop needs %lld partial slots, the workspace has %lld",
+                  (long long)ops->G * ops->maxseg, (long long)ws.lslots);
+    ls = loop_setup_params(n, m, *ops, ws);
+    // the loop's second bias buffers: their padding rows (-inf) matter, the others are
+    // written by the sweeps before any tile reads them
+    op.xb[1] = ws.xb2;
+    op.yb[1] = ws.yb2;
+  }
+  CK(launch_operands(op, hull ? OperandKind::kGridHull : grid ? OperandKind::kGrid : OperandKind::kBf16,
+                     ops->loop ? &ls : nullptr, s));
+  // absent parts alias the one before: their maps are never read
+  void* xl = ops->parts > 1 ? ws.xl : ws.xh;
+  void* yl = ops->parts > 1 ? ws.yl : ws.yh;
   int rc = make_map(&ops->xh_a, ws.xh, n, dp, 128);
   if (!rc) rc = make_map(&ops->xl_a, xl, n, dp, 128);
   if (!rc) rc = make_map(&ops->yh_a, ws.yh, m, dp, 128);
   if (!rc) rc = make_map(&ops->yl_a, yl, m, dp, 128);
-  if (!rc) rc = make_map(&ops->xh_b, ws.xh, n, dp, ops->bn);
-  if (!rc) rc = make_map(&ops->xl_b, xl, n, dp, ops->bn);
-  if (!rc) rc = make_map(&ops->yh_b, ws.yh, m, dp, ops->bn);
-  if (!rc) rc = make_map(&ops->yl_b, yl, m, dp, ops->bn);
-  if (!rc) rc = make_map(&ops->xb, ws.xb, cdiv(n, 256) * 256, 16, ops->bn);
-  if (!rc) rc = make_map(&ops->yb, ws.yb, cdiv(m, 256) * 256, 16, ops->bn);
-  if (!rc && dp == 64) {
-    rc = make_map(&ops->yb128, ws.yb, cdiv(m, 256) * 256, 16, 128);
+  if (!rc && grid) {
+    rc = make_map(&ops->xr_a, ops->parts > 2 ? ws.xr : xl, n, dp, 128);
+    if (!rc) rc = make_map(&ops->yr_a, ops->parts > 2 ? ws.yr : yl, m, dp, 128);
   }
-  if (!rc && dp > 64 && map_tc_onepass_supported(ops->nkb)) {
+  if (ops->bn == 128) {
+    // the same boxes serve both roles
+    ops->xh_b = ops->xh_a;
+    ops->xl_b = ops->xl_a;
+    ops->xr_b = ops->xr_a;
+    ops->yh_b = ops->yh_a;
+    ops->yl_b = ops->yl_a;
+    ops->yr_b = ops->yr_a;
+  } else {
+    if (!rc) rc = make_map(&ops->xh_b, ws.xh, n, dp, ops->bn);
+    if (!rc) rc = make_map(&ops->xl_b, xl, n, dp, ops->bn);
+    if (!rc) rc = make_map(&ops->yh_b, ws.yh, m, dp, ops->bn);
+    if (!rc) rc = make_map(&ops->yl_b, yl, m, dp, ops->bn);
+  }
+  if (!rc) rc = make_map(&ops->xb, ws.xb, cdiv(n, 256) * 256, 16, ops->bn);
+  if (!rc) rc = map_y_bias(ops, ws.yb, m);
+  if (!rc && !grid && dp > 64 && map_tc_onepass_supported(ops->nkb)) {
     const int bt = map_tc_onepass_tile_cols();
     rc = make_map(&ops->yh_m32, ws.yh, m, dp, bt);
     if (!rc) rc = make_map(&ops->yl_m32, yl, m, dp, bt);
-    if (!rc) rc = make_map(&ops->yb_m32, ws.yb, cdiv(m, 256) * 256, 16, bt);
   }
-  if (rc) return rc;
-  const float bscale = (float)(kLog2e / eps);
-  if (g_cur != nullptr) CK(launch_bias_prep(g_cur, ws.ync, m, cdiv(m, 256) * 256, bscale, ws.yb, s));
-  if (f_cur != nullptr) CK(launch_bias_prep(f_cur, ws.xnc, n, cdiv(n, 256) * 256, bscale, ws.xb, s));
-  return PROGOT_OK;
+  return rc;
 }
 
 // One sweep description for "update the potential of A from the potential of B".
@@ -482,6 +640,7 @@ static SweepParams make_sweep(const float* A, int64_t nA, const float* B, int64_
   p.splits = (int)cdiv(ct, p.tiles_per_split);  // drop empty splits
   p.scale = (float)(2.0 * kLog2e / eps);
   p.bscale = (float)(kLog2e / eps);
+  p.bscale_lo = (float)(kLog2e / eps - (double)p.bscale);
   p.eps = eps;
   p.inv_eps_f = (float)(1.0 / eps);
   p.inv_nA = 1.0 / (double)nA;
@@ -524,16 +683,19 @@ static void apply_cost(SweepParams& sp, const Cost& c, double eps) {
 
 // Launch one log-sum-exp sweep: float32 CUDA cores, or tcgen05 on the prepared split
 // operands (a_is_x: rows of the sweep are the x cloud).
-static int lse_sweep(const SweepParams& p, int32_t precision, cudaStream_t s, const TcOps* ops = nullptr,
+static int lse_sweep(const SweepParams& p, cudaStream_t s, const TcOps* ops = nullptr,
                      bool a_is_x = true, const Workspace* ws = nullptr, bool in_loop = false) {
   ProfRec r;
   const bool rec = !in_loop && prof_begin(r, s, kProfLse);
-  if (precision != PROGOT_FP32 && ops != nullptr && ops->on) {
-    const CUtensorMap* ah = a_is_x ? &ops->xh_a : &ops->yh_a;
-    const CUtensorMap* al = a_is_x ? &ops->xl_a : &ops->yl_a;
-    const CUtensorMap* bh = a_is_x ? &ops->yh_b : &ops->xh_b;
-    const CUtensorMap* bl = a_is_x ? &ops->yl_b : &ops->xl_b;
-    const CUtensorMap* bb = a_is_x ? &ops->yb : &ops->xb;
+  if (ops != nullptr && ops->on) {
+    TcMaps maps;
+    maps.a[0] = a_is_x ? &ops->xh_a : &ops->yh_a;
+    maps.a[1] = a_is_x ? &ops->xl_a : &ops->yl_a;
+    maps.a[2] = ops->gscale ? (a_is_x ? &ops->xr_a : &ops->yr_a) : maps.a[1];
+    maps.b[0] = a_is_x ? &ops->yh_b : &ops->xh_b;
+    maps.b[1] = a_is_x ? &ops->yl_b : &ops->xl_b;
+    maps.b[2] = ops->gscale ? (a_is_x ? &ops->yr_b : &ops->xr_b) : maps.b[1];
+    maps.bias = a_is_x ? &ops->yb : &ops->xb;
     void* bias_out = (p.mode == kModePotential && ws) ? (a_is_x ? ws->xb : ws->yb) : nullptr;
     int G = 0, maxseg = 0;
     tc_plan(p.nA, p.nB, ops->bn, num_sms(), &G, &maxseg);
@@ -542,8 +704,8 @@ static int lse_sweep(const SweepParams& p, int32_t precision, cudaStream_t s, co
     // the operands are centred: the row constants of the epilogue are the centred norms
     if (q.An != nullptr) q.An = a_is_x ? ops->xnc : ops->ync;
     if (q.Bn != nullptr) q.Bn = a_is_x ? ops->ync : ops->xnc;
-    CK(launch_lse_sweep_tc(q, ah, al, bh, bl, bb, ops->nkb, ops->split3, ops->bn, G, maxseg,
-                           ws ? ws->fault : nullptr, bias_out, s));
+    CK(launch_lse_sweep_tc(q, maps, ops->nkb, ops->parts, ops->gscale, ops->bn, G, maxseg, ws ? ws->fault : nullptr,
+                           bias_out, s));
   } else {
     CK(launch_lse_sweep_fp32(p, s));
   }
@@ -555,28 +717,19 @@ static int lse_sweep(const SweepParams& p, int32_t precision, cudaStream_t s, co
 // Sinkhorn loop (Alg. 1) as one persistent tensor-core launch (loop_tc.cu): the bias rows
 // of each update's potential pass between the GPU's CTAs behind per-row-block ready
 // flags, the stop test runs inside the kernel. pf and pg are the f- and g-update
-// descriptions built by sinkhorn_core; ops describes the prepared operands, whose bias
-// rows (ws.xb from f, ws.yb from g) prep_tc has written. On return the current f is in
-// f_a, g in g, and the y-side bias rows (ws.yb) hold g for a map step at the same eps.
+// descriptions built by sinkhorn_core; ops describes the prepared operands, with whose
+// bias rows prep_tc has written the loop's tables, flags and state. On return the current f
+// is in f_a, g in g, and (map_follows) the y-side bias rows ops describes hold g for a map
+// step at the same eps, ws.L its row log-sum-exps.
 static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, int64_t m, int32_t max_iter,
                                     double tau, float* f_a, float* f_b, float* g, const Workspace& ws,
-                                    TcOps& ops, int32_t* iters_out, double* err_out, cudaStream_t s) {
+                                    TcOps& ops, bool map_follows, int32_t* iters_out, double* err_out,
+                                    cudaStream_t s) {
   pf.An = ops.xnc;
   pf.Bn = ops.ync;
   pg.An = ops.ync;
   pg.Bn = ops.xnc;
   const int64_t rb = ws.lrb;
-  // the second bias buffers: their padding rows (-inf) matter, the others are written
-  // by the sweeps before any tile reads them
-  CK(launch_bias_prep(f_a, ops.xnc, n, cdiv(n, 256) * 256, pf.bscale, ws.xb2, s));
-  CK(launch_bias_prep(g, ops.ync, m, cdiv(m, 256) * 256, pf.bscale, ws.yb2, s));
-  // ready flags: nothing published, then the initial g's row blocks (in ws.yb) as flag 1,
-  // which the first f-update waits for. The test hook leaves them unpublished, so the
-  // first f-update's bounded wait expires.
-  CK(cudaMemsetAsync(ws.lflag, 0, sizeof(uint32_t) * 2 * (size_t)rb, s));
-  if (!g_withhold_betas.load()) CK(launch_fill_u32(ws.lflag + rb, cdiv(m, 128), 1u, s));
-  CK(cudaMemsetAsync(ws.lcnt, 0, sizeof(unsigned long long) * (2 * (size_t)rb + 2), s));
-  CK(launch_init_state(ws.state, s));
   CUtensorMap xb2_map, yb2_map;
   int rc = make_map(&xb2_map, ws.xb2, cdiv(n, 256) * 256, 16, ops.bn);
   if (!rc) rc = make_map(&yb2_map, ws.yb2, cdiv(m, 256) * 256, 16, ops.bn);
@@ -597,9 +750,8 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   F.partial = ws.lpart;
   F.segs = ws.ltab_segs;
   F.cslot = ws.ltab_cslot;
-  F.cptr = ws.ltab_cptr;
+  F.crow = ws.ltab_crow;
   F.nseg = ws.ltab_nseg;
-  F.table_slots = ws.lslots;
   Gs.p = pg;
   Gs.out0 = g;
   Gs.out1 = nullptr;
@@ -612,12 +764,16 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   Gs.partial = ws.lpart + ws.lslots * 2 * 128;
   Gs.segs = ws.ltab_segs + ws.lslots;
   Gs.cslot = ws.ltab_cslot + ws.lslots;
-  Gs.cptr = ws.ltab_cptr + (rb + 1);
+  Gs.crow = ws.ltab_crow + rb;
   Gs.nseg = ws.ltab_nseg + num_sms();
-  Gs.table_slots = ws.lslots;
-  const CUtensorMap* maps[12] = {&ops.xh_a, &ops.xl_a, &ops.yh_a, &ops.yl_a, &ops.xh_b, &ops.xl_b,
-                                 &ops.yh_b, &ops.yl_b, &ops.xb,   &xb2_map,   &ops.yb,   &yb2_map};
-  for (int q = 0; q < 12; ++q) L.maps[q] = maps[q];
+  const bool grid = ops.gscale != nullptr;
+  const CUtensorMap* maps[16] = {&ops.xh_a, &ops.xl_a, &ops.yh_a, &ops.yl_a, &ops.xh_b, &ops.xl_b,
+                                 &ops.yh_b, &ops.yl_b,
+                                 grid ? &ops.xr_a : &ops.xl_a, grid ? &ops.yr_a : &ops.yl_a,
+                                 grid ? &ops.xr_b : &ops.xl_b, grid ? &ops.yr_b : &ops.yl_b,
+                                 &ops.xb,   &xb2_map,   &ops.yb,   &yb2_map};
+  for (int q = 0; q < 16; ++q) L.maps[q] = maps[q];
+  L.gscale = ops.gscale;
   L.errpart = ws.lerr;
   L.state = ws.state;
   L.fault = ws.fault;
@@ -625,10 +781,8 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   L.nkb = ops.nkb;
   L.split3 = ops.split3;
   L.bn = ops.bn;
-  loop_tc_plan(n, m, ops.bn, num_sms(), &L.G, &L.maxseg);
-  if ((int64_t)L.G * L.maxseg > ws.lslots)
-    return fail(PROGOT_ERR_WORKSPACE, "persistent loop needs %lld partial slots, the workspace has %lld",
-                (long long)L.G * L.maxseg, (long long)ws.lslots);
+  L.G = ops.G;
+  L.maxseg = ops.maxseg;
   L.seq0 = 0;
   // max_iter + 1 f-updates always reach the stop test's max_iter branch; the tags of
   // sweep k are 2 k + 1 and 2 k + 2, so iterations stay below 2^30
@@ -645,11 +799,11 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   if (t_prof.on) CK(cudaEventRecord(pr.b, s));
   rc = t_host.init();
   if (rc) return rc;
-  int32_t fault = 0;
-  CK(cudaMemcpyAsync(&t_host.hs[0], ws.state, sizeof(SolverState), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(&fault, ws.fault, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  // the states and the fault word sit in one block of the workspace
+  CK(cudaMemcpyAsync(t_host.hs, ws.state, kStateBytes, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   const SolverState fin = t_host.hs[0];
+  const int32_t fault = *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(t_host.hs) + 128);
   if (fault) return fail(PROGOT_ERR_TIMEOUT, "the persistent Sinkhorn loop hit its bounded wait and aborted");
   // every iteration up to the stop ran both sweeps (the last g-update without writes)
   const int64_t sweeps = 2 * ((int64_t)fin.it + 1);
@@ -664,14 +818,19 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   // The loop stops after an f-update whose result it does not adopt (f stays the iterate
   // the stop test measured, g is unchanged): that update formed f_new from exactly the
   // t_ij = c x~.y~ + beta(g) of a map step that follows, so its row log-sum-exps, read
-  // back from f_new, are the map step's L and spare it a sweep.
-  if (fin.status != kNumeric) {
-    CK(launch_lse_from_potential(fin.fcur == 0 ? f_b : f_a, ops.xnc, pf.wA, pf.log_w_uniform, pf.eps, n, ws.L, s));
+  // back from f_new, are the map step's L and spare it a sweep. The bias rows of that g
+  // are in the buffer of the stopping iteration's parity.
+  if (map_follows && fin.status != kNumeric) {
+    CK(launch_loop_finish(fin.fcur == 0 ? f_b : f_a, ops.xnc, pf.wA, pf.log_w_uniform, pf.eps, n, ws.L, f_b,
+                          fin.fcur == 1 ? f_a : nullptr, s));
     ops.lse_ready = true;
+    if (fin.it & 1) {
+      rc = map_y_bias(&ops, ws.yb2, m);
+      if (rc) return rc;
+    }
+  } else if (fin.fcur == 1) {
+    CK(cudaMemcpyAsync(f_a, f_b, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
   }
-  if (fin.fcur == 1) CK(cudaMemcpyAsync(f_a, f_b, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
-  // the map step that may follow reads g through the y-side bias rows
-  CK(launch_bias_prep(g, ops.ync, m, cdiv(m, 256) * 256, pf.bscale, ws.yb, s));
   if (iters_out) *iters_out = fin.it;
   if (err_out) *err_out = fin.err;
   switch (fin.status) {
@@ -700,20 +859,21 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
                          int32_t d, double eps, double tau, int32_t max_iter, int32_t precision, float* f_a, float* f_b,
                          float* g, const float* xn, const float* yn, const Workspace& ws, int32_t* iters_out,
                          double* err_out, cudaStream_t s, TcOps* ops_out = nullptr, bool symmetric = false,
-                         const Cost& cost = Cost()) {
+                         const Cost& cost = Cost(), Operands kind = Operands::kAuto) {
   int rc = t_host.init();
   if (rc) return rc;
   TcOps ops_local;
   TcOps& ops = ops_out ? *ops_out : ops_local;
   if (cost.pnorm()) {
-    ops.on = false;  // the p-norm cost runs on CUDA cores (float32)
+    ops.on = ops.loop = false;  // the p-norm cost runs on CUDA cores (float32)
     precision = PROGOT_FP32;
   } else {
-    rc = prep_tc(x, n, y, m, d, eps, precision, ws, &ops, s, f_a, symmetric ? f_a : g);
+    rc = prep_tc(x, n, y, m, d, eps, precision, ws, &ops, s, f_a, symmetric ? f_a : g,
+                 !symmetric && g_loop_tc.load() != 0, kind);
     if (rc) return rc;
   }
   const int cps = ops.on ? 1 : 2;
-  CK(launch_init_state(ws.state, s));
+  if (!ops.loop) CK(launch_init_state(ws.state, s));
   SweepParams pf = make_sweep(x, n, y, m, d, xn, yn, eps, ws, cps);
   pf.wA = a;
   pf.potB = symmetric ? f_a : g;
@@ -742,9 +902,10 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
   // sweep-level arrival and finish
   const bool lag = ops.on && !symmetric;
   pf.lag = pg.lag = lag ? 1 : 0;
-  if (lag && g_loop_tc.load() && loop_tc_supported(ops.bn, ops.nkb, ops.split3)) {
+  if (ops.loop) {
     pf.lag = pg.lag = 0;
-    return sinkhorn_loop_persistent(pf, pg, n, m, max_iter, tau, f_a, f_b, g, ws, ops, iters_out, err_out, s);
+    return sinkhorn_loop_persistent(pf, pg, n, m, max_iter, tau, f_a, f_b, g, ws, ops, ops_out != nullptr, iters_out,
+                                    err_out, s);
   }
 
   int64_t sym_sweeps = 0;
@@ -755,15 +916,15 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
         // alternate the operand roles so that the tensor-core sweep reads the bias rows
         // of the current f from one side's buffer while it writes the next f's rows
         // into the other side's buffer (x and y are the same cloud)
-        int r = lse_sweep(pf, precision, s, &ops, (sym_sweeps & 1) == 0, &ws, true);
+        int r = lse_sweep(pf, s, &ops, (sym_sweeps & 1) == 0, &ws, true);
         if (r) return r;
         ++sym_sweeps;
         continue;
       }
       pf.seq = pg.seq = (int32_t)(launched + i);
-      int r = lse_sweep(pf, precision, s, &ops, true, &ws, true);
+      int r = lse_sweep(pf, s, &ops, true, &ws, true);
       if (r) return r;
-      r = lse_sweep(pg, precision, s, &ops, false, &ws, true);
+      r = lse_sweep(pg, s, &ops, false, &ws, true);
       if (r) return r;
     }
     return PROGOT_OK;
@@ -868,6 +1029,54 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
   }
 }
 
+// The map step on integer-grid operands, in place on X: for every chunk of row blocks that
+// ws.prob holds, a sweep writes P and its row sums (ws.L the stabiliser), then P Y.
+static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, double alpha, const Workspace& ws,
+                         cudaStream_t s, const TcOps& ops) {
+  CUtensorMap ymap[3];
+  void* const yparts[3] = {ws.yh, ws.yl, ops.parts > 2 ? ws.yr : ws.yl};
+  for (int q = 0; q < 3; ++q) {
+    const int rc = make_map(&ymap[q], yparts[q], m, pad64(d), 64);
+    if (rc) return rc;
+  }
+  const int64_t blocks = cdiv(n, 128);
+  int64_t cb = std::min<int64_t>(blocks, ws.prob_bytes / pv_prob_bytes_per_block(m));
+  if (cb < 1) return fail(PROGOT_ERR_WORKSPACE, "no room for one row block of P");
+  cb = cdiv(blocks, cdiv(blocks, cb));  // equal chunks
+  ProfRec r;
+  const bool rec = prof_begin(r, s, kProfMap);
+  for (int64_t b0 = 0; b0 < blocks; b0 += cb) {
+    const int64_t row0 = b0 * 128, rows = std::min<int64_t>(n - row0, cb * 128);
+    SweepParams p = make_sweep(X, rows, X, m, d, nullptr, nullptr, eps, ws, 1);
+    p.mode = kModeProb;
+    p.out = ws.rsum + row0;
+    TcMaps maps = {{&ops.xh_a, &ops.xl_a, &ops.xr_a}, {&ops.yh_b, &ops.yl_b, &ops.yr_b}, &ops.yb};
+    int G = 0, maxseg = 0;
+    tc_plan(rows, m, ops.bn, num_sms(), &G, &maxseg);
+    CK(launch_lse_sweep_tc(p, maps, ops.nkb, ops.parts, ops.gscale, ops.bn, G, maxseg, ws.fault, nullptr, s,
+                           ws.L + row0, ws.prob, row0));
+    PvLaunch pv;
+    pv.X = X + row0 * d;
+    pv.out = X + row0 * d;
+    pv.rsum = ws.rsum + row0;
+    pv.prob = ws.prob;
+    for (int q = 0; q < 3; ++q) pv.mapY[q] = &ymap[q];
+    pv.gscale = ops.gscale;
+    pv.mu = ops.mu;
+    pv.rows = rows;
+    pv.m = m;
+    pv.d = d;
+    pv.parts = ops.parts;
+    pv.alpha = (float)alpha;
+    pv.inv_sc = (float)std::sqrt(eps / (2.0 * kLog2e));
+    pv.fault = ws.fault;
+    CK(launch_pv_tc(pv, num_sms(), s));
+  }
+  if (rec) prof_end(r, s, kProfMap, (double)n * (double)m);
+  if (t_prof.on) t_prof.worked[kProfMap] += 1;
+  return PROGOT_OK;
+}
+
 // One barycentric displacement X <- X + alpha (T(X) - X) (Alg. 2 / Alg. 3), in place on X.
 // The log-sum-exp pass runs on the tensor cores when `ops` describes X, Y and the y-side
 // bias rows of g at this eps; the map sweep itself normalises by its own row sums, so
@@ -883,10 +1092,10 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
   apply_cost(pl, cost, eps);
   // the persistent loop that produced g may already have left L in ws.L
   int rc = (tc && ops->lse_ready) ? PROGOT_OK
-           : tc                   ? lse_sweep(pl, precision, s, ops, true, &ws)
-                                  : lse_sweep(pl, PROGOT_FP32, s);
+           : tc                   ? lse_sweep(pl, s, ops, true, &ws)
+                                  : lse_sweep(pl, s);
   if (rc) return rc;
-  if (tc && ops->nkb == 1 && g_map_tc.load()) {
+  if (tc && !ops->gscale && ops->nkb == 1 && g_map_tc.load()) {
     // d <= 64: S and P Y both on the tensor cores (P Y reuses the centred, scaled y operand)
     int G = 0, maxseg = 0;
     tc_plan(n, m, 128, num_sms(), &G, &maxseg);
@@ -899,7 +1108,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
   }
-  if (tc && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb) && g_map_tc.load()) {
+  if (tc && !ops->gscale && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb) && g_map_tc.load()) {
     // 64 < d <= 256: one launch, S once per tile, all output coordinates in TMEM
     int G = 0, maxseg = 0;
     tc_plan(n, m, map_tc_onepass_tile_cols(), num_sms(), &G, &maxseg);
@@ -911,6 +1120,19 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (rec) prof_end(r, s, kProfMap, (double)n * (double)m);
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
+  }
+  if (tc && g_map_tc.load()) {
+    // float32 path, and the bf16x3 path for d > 256 (its operands give way to the
+    // integer-grid ones, whose accuracy the CUDA-core map it replaces had): P a chunk of
+    // row blocks at a time, then P Y
+    TcOps gops;
+    const TcOps* go = ops;
+    if (!ops->gscale) {
+      rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g, false, Operands::kGridTwoParts);
+      if (rc) return rc;
+      go = &gops;
+    }
+    return grid_map_step(X, n, m, d, eps, alpha, ws, s, *go);
   }
   if (tc) {
     // the float32 map sweep below forms t_ij from the uncentred X and Y: move L there
@@ -954,10 +1176,10 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
   return PROGOT_OK;
 }
 
-static int zero_counters(const Workspace& ws, int64_t rbmax, cudaStream_t s) {
-  CK(cudaMemsetAsync(ws.cnt, 0, sizeof(unsigned) * (rbmax + 2), s));
-  CK(cudaMemsetAsync(ws.mcnt, 0, sizeof(unsigned) * (rbmax + 2), s));
-  CK(cudaMemsetAsync(ws.fault, 0, sizeof(int32_t), s));  // raised by a tensor-core kernel's expired wait
+static int zero_counters(const Workspace& ws, cudaStream_t s) {
+  // cnt, mcnt and the small words (fault, raised by a tensor-core kernel's expired wait)
+  // follow one another
+  CK(cudaMemsetAsync(ws.cnt, 0, (size_t)((char*)ws.state + 256 - (char*)ws.cnt), s));
   return PROGOT_OK;
 }
 
@@ -1043,6 +1265,7 @@ static int mean_cost_dev(const float* x, int64_t n, const float* y, int64_t m, i
   return PROGOT_OK;
 }
 
+
 // Alg. 2 with eps_k from `eps` (host, K) or, when eps is NULL, from the theta rule
 // eps_k = theta mean cost(X^(k), Y) / 20 on the cloud each solve transports.
 static int solve_impl(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m, int32_t d,
@@ -1053,25 +1276,20 @@ static int solve_impl(const float* x, const float* a, int64_t n, const float* y,
   Workspace ws;
   int rc = carve(n, m, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
-  rc = zero_counters(ws, ws_dims(n, m, d).rbmax, s);
+  if (d > kGridSolveDim) ws.grid = false;
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   if (x_out != x) CK(cudaMemcpyAsync(x_out, x, sizeof(float) * n * d, cudaMemcpyDeviceToDevice, s));
-  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
-  CK(cudaMemsetAsync(ws.f0, 0, sizeof(float) * n, s));
+  // the tensor-core operands carry centred norms of their own
+  const bool tc = !cost.pnorm() && (precision != PROGOT_FP32 || ws.grid);
+  if (!tc || !g_map_tc.load()) CK(launch_row_sqnorm(y, m, d, ws.yn, s));
   if (eps == nullptr && !cost.pnorm()) CK(launch_moments(y, m, d, ws.rpart, reduce_parts(), ws.rout + (d + 1), s));
   int worst = PROGOT_OK;
   std::string worst_msg;
   for (int k = 0; k < K; ++k) {
     float* gk = g_all + (int64_t)k * m;
-    if (k == 0) {
-      CK(cudaMemsetAsync(gk, 0, sizeof(float) * m, s));
-    } else {
-      // warm start of Alg. 2: (1 - alpha_k) f, (1 - alpha_k) g^(k-1)
-      const float c = (float)(1.0 - alpha[k]);
-      CK(cudaMemcpyAsync(gk, gk - m, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
-      CK(launch_scale(gk, m, c, s));
-      CK(launch_scale(ws.f0, n, c, s));
-    }
+    // warm start of Alg. 2: (1 - alpha_k) f, (1 - alpha_k) g^(k-1), zero at the first step
+    CK(launch_warm_start(gk, k == 0 ? nullptr : gk - m, m, ws.f0, n, k == 0 ? 0.f : (float)(1.0 - alpha[k]), s));
     if (x_last != nullptr && k == K - 1)
       CK(cudaMemcpyAsync(x_last, x_out, sizeof(float) * n * d, cudaMemcpyDeviceToDevice, s));
     double eps_k = 0.0;
@@ -1086,12 +1304,12 @@ static int solve_impl(const float* x, const float* a, int64_t n, const float* y,
         return fail(PROGOT_ERR_NUMERIC, "step %d: theta rule gave eps = %g (mean cost %g)", k + 1, eps_k, cbar);
     }
     if (eps_out) eps_out[k] = eps_k;
-    CK(launch_row_sqnorm(x_out, n, d, ws.xn, s));
+    if (!tc) CK(launch_row_sqnorm(x_out, n, d, ws.xn, s));
     int32_t it = 0;
     double err = 0.0;
     TcOps ops;
     rc = sinkhorn_core(x_out, a, n, y, b, m, d, eps_k, tau[k], max_iter, precision, ws.f0, ws.f1, gk, ws.xn, ws.yn,
-                       ws, &it, &err, s, &ops, false, cost);
+                       ws, &it, &err, s, &ops, false, cost, k ? Operands::kMoved : Operands::kAuto);
     if (iters) iters[k] = it;
     if (errs) errs[k] = err;
     if (rc == PROGOT_ERR_NOT_CONVERGED) {
@@ -1125,6 +1343,15 @@ extern "C" {
 const char* progot_last_error_string(void) { return t_last_error.c_str(); }
 
 const char* progot_version(void) { return "0.1.0"; }
+
+}  // extern "C"
+
+size_t progot::workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision) {
+  if (n <= 0 || m <= 0 || d <= 0) return 0;
+  return ws_layout(ws_dims(n, m, d, precision, false), nullptr, nullptr);
+}
+
+extern "C" {
 
 size_t progot_workspace_size(int64_t n, int64_t m, int32_t d, int32_t precision) {
   if (n <= 0 || m <= 0 || d <= 0) return 0;
@@ -1200,14 +1427,17 @@ int sinkhorn_potentials(const float* x, const float* a, int64_t n, const float* 
   rc = carve(n, m, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(n, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   if (init_zero) {
     CK(cudaMemsetAsync(f, 0, sizeof(float) * n, s));
     CK(cudaMemsetAsync(g, 0, sizeof(float) * m, s));
   }
-  CK(launch_row_sqnorm(x, n, d, ws.xn, s));
-  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  if (d > kGridSolveDim) ws.grid = false;
+  if (precision == PROGOT_FP32 && !ws.grid) {
+    CK(launch_row_sqnorm(x, n, d, ws.xn, s));
+    CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  }
   return sinkhorn_core(x, a, n, y, b, m, d, eps, tau, max_iter, precision, f, ws.f1, g, ws.xn, ws.yn, ws, iters_out,
                        err_out, s);
 }
@@ -1229,15 +1459,21 @@ int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, i
   rc = carve(nq, m, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(nq, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   if (out != xq) CK(cudaMemcpyAsync(out, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
-  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  // Small queries of the float32 path stay on CUDA cores, whose two launches a step cost less
+  // than the grid's four: 28 us against 35 a step at 500 x 500, d = 2; both 39 at 1000 x 2048,
+  // d = 16; 69 against 40 at 1000 x 2048, d = 64; 94 against 62 at 3000 x 3000, d = 16.
+  if (precision == PROGOT_FP32 && (double)nq * (double)m * (double)std::max<int32_t>(d, 16) < kGridMapWork)
+    ws.grid = false;
+  if ((precision == PROGOT_FP32 && !ws.grid) || !g_map_tc.load()) CK(launch_row_sqnorm(y, m, d, ws.yn, s));
   for (int k = 0; k < K; ++k) {
     const double al = (k == K - 1) ? 1.0 : alpha[k];
     const float* gk = g_all + (int64_t)k * m;
     TcOps ops;
-    rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk);
+    rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
+                 k ? Operands::kMoved : Operands::kAuto);
     if (rc) return rc;
     rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
     if (rc) return rc;
@@ -1259,34 +1495,40 @@ int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int
   rc = t_host.init();
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  const WsDims w = ws_dims(n, m, d);
-  rc = zero_counters(ws, w.rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
-  CK(launch_row_sqnorm(x, n, d, ws.xn, s));
-  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
-  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws);
+  if (!ws.grid) {
+    CK(launch_row_sqnorm(x, n, d, ws.xn, s));
+    CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  }
+  // float32 accuracy at every precision setting: the integer-grid operands where the
+  // workspace has room for them, else CUDA cores
+  TcOps ops;
+  rc = prep_tc(x, n, y, m, d, eps, PROGOT_FP32, ws, &ops, s, f, g);
+  if (rc) return rc;
+  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws, ops.on ? 1 : 2);
   pr.wA = a;
   pr.potB = g;
   pr.potA_old = f;
   pr.out = row;
   pr.mode = kModeMarginal;
-  rc = lse_sweep(pr, precision, s);
+  rc = lse_sweep(pr, s, &ops, true, &ws);
   if (rc) return rc;
   const int64_t rbr = cdiv(n, fp32_tile_rows());
   CK(cudaMemcpyAsync(&t_host.hd[0], ws.errpart + rbr, sizeof(double), cudaMemcpyDeviceToHost, s));
-  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws);
+  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws, ops.on ? 1 : 2);
   pc.wA = b;
   pc.potB = f;
   pc.potA_old = g;
   pc.out = col;
   pc.mode = kModeMarginal;
-  rc = lse_sweep(pc, precision, s);
+  rc = lse_sweep(pc, s, &ops, false, &ws);
   if (rc) return rc;
   const int64_t rbc = cdiv(m, fp32_tile_rows());
   CK(cudaMemcpyAsync(&t_host.hd[1], ws.errpart + rbc, sizeof(double), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (err_l1_out) *err_l1_out = t_host.hd[0] + t_host.hd[1];
-  return PROGOT_OK;
+  return ops.on ? check_fault(ws, s) : PROGOT_OK;
 }
 
 int progot_solve(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m, int32_t d,
@@ -1354,7 +1596,7 @@ int coupling_metrics(const float* x, const float* a, int64_t n, const float* y, 
   rc = carve(n, m, d, workspace, ws_bytes, &ws);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(n, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   CK(launch_row_sqnorm(x, n, d, ws.xn, s));
   CK(launch_row_sqnorm(y, m, d, ws.yn, s));
@@ -1375,6 +1617,7 @@ int sinkhorn_divergence(const float* x, const float* a, int64_t n, const float* 
   Workspace ws;
   rc = carve(nmax, nmax, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
+  if (d > kGridSolveDim) ws.grid = false;
   cudaStream_t s = (cudaStream_t)stream;
   struct Side {
     const float* p;
@@ -1388,7 +1631,7 @@ int sinkhorn_divergence(const float* x, const float* a, int64_t n, const float* 
   for (int q = 0; q < 3; ++q) {
     const Side& A = pairs[q][0];
     const Side& B = pairs[q][1];
-    rc = zero_counters(ws, ws_dims(nmax, nmax, d).rbmax, s);
+    rc = zero_counters(ws, s);
     if (rc) return rc;
     CK(launch_row_sqnorm(A.p, A.k, d, ws.xn, s));
     CK(launch_row_sqnorm(B.p, B.k, d, ws.yn, s));
@@ -1464,7 +1707,7 @@ int sinkhorn_potentials_pnorm(const float* x, const float* a, int64_t n, const f
   rc = carve(n, m, d, workspace, ws_bytes, &ws);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(n, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   if (init_zero) {
     CK(cudaMemsetAsync(f, 0, sizeof(float) * n, s));
@@ -1519,7 +1762,7 @@ int entropic_map_apply_pnorm(const float* xq, int64_t nq, const float* y, int64_
   rc = carve(nq, m, d, workspace, ws_bytes, &ws);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(nq, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   if (out != xq) CK(cudaMemcpyAsync(out, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
   for (int k = 0; k < K; ++k) {
@@ -1546,7 +1789,7 @@ int coupling_metrics_pnorm(const float* x, const float* a, int64_t n, const floa
   rc = carve(n, m, d, workspace, ws_bytes, &ws);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
-  rc = zero_counters(ws, ws_dims(n, m, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   return metrics_core(x, a, n, y, b, m, d, f, g, eps, ws, s, out, cost, x_cost);
 }
@@ -1611,6 +1854,7 @@ int progot_schedule_eps(const float* x, int64_t n, const float* y, const float* 
   Workspace ws;
   rc = carve(nmax, nmax, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
+  if (d > kGridSolveDim) ws.grid = false;
   cudaStream_t s = (cudaStream_t)stream;
   double mc_xy = 0.0, mc_yy = 0.0;
   rc = progot_mean_cost(x, n, y, m, d, &mc_xy, workspace, ws_bytes, stream);
@@ -1618,7 +1862,7 @@ int progot_schedule_eps(const float* x, int64_t n, const float* y, const float* 
   rc = progot_mean_cost(y, m, y, m, d, &mc_yy, workspace, ws_bytes, stream);
   if (rc) return rc;
   const double eps0 = mc_xy / 20.0, sigma = mc_yy / 20.0;
-  rc = zero_counters(ws, ws_dims(nmax, nmax, d).rbmax, s);
+  rc = zero_counters(ws, s);
   if (rc) return rc;
   CK(launch_row_sqnorm(y, m, d, ws.yn, s));
   std::vector<double> errors(P);

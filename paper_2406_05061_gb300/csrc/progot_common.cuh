@@ -8,6 +8,7 @@ namespace progot {
 
 constexpr double kLog2e = 1.4426950408889634;  // log2(e)
 constexpr double kLn2 = 0.6931471805599453;    // ln(2)
+constexpr int kGridParts = 3;  // operand parts of the integer-grid split (grid_split.cuh)
 
 // Epilogue of a row log-sum-exp sweep, applied once per row after the
 // deterministic combine of the column splits. L_i = log2 sum_j 2^{t_ij}.
@@ -16,6 +17,7 @@ enum SweepMode : int32_t {
   kModeLse = 1,        // out_i = L_i (log2 units)
   kModeMarginal = 2,   // out_i = exp((pot_i - |a_i|^2)/eps + ln2 L_i)  (row sums of P)
   kModeMetrics = 3,    // marginal plus the per-row-block sums of the coupling metrics
+  kModeProb = 4,       // integer-grid sweeps: P_ij = 2^{t_ij - L_i + 14} to memory, out_i = sum_j P_ij
 };
 
 // Per-row-block float64 sums written by a kModeMetrics sweep (metpart[block * kMetricSums + q]).
@@ -86,6 +88,7 @@ struct SweepParams {
   int32_t seq;         // iteration of this sweep in its Sinkhorn loop (lag = 1)
   float scale;         // 2 log2(e) / eps: multiplies x . y
   float bscale;        // log2(e) / eps: multiplies (potB_j - |b_j|^2)
+  float bscale_lo;     // what bscale's rounding left (integer-grid sweeps)
   double eps;
   float inv_eps_f;     // 1 / eps in float32 (the per-row error terms)
   double tau;

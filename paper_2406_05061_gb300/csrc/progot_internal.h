@@ -47,17 +47,8 @@ int map_dchunk();
 
 // small kernels (prep.cu)
 cudaError_t launch_row_sqnorm(const float* X, int64_t n, int32_t d, float* out, cudaStream_t s);
-// mu = (mean of the rows of X + mean of the rows of Y) / 2 (fixed-order float64 sums);
-// partial: reduce_parts() * 2 * d doubles of scratch.
-cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial, float* mu,
-                          cudaStream_t s);
-// L_i = (eps log w_i + |a_i|^2 - f_i) / (eps ln2) from a potential an f-update wrote
-// (w = NULL: log w_i = log_w_uniform).
-cudaError_t launch_lse_from_potential(const float* f, const float* an, const float* w, double log_w_uniform,
-                                      double eps, int64_t n, float* L, cudaStream_t s);
 cudaError_t launch_lse_uncenter(float* L, const float* X, int64_t n, int32_t d, const float* mu, float bscale,
                                 cudaStream_t s);
-cudaError_t launch_scale(float* v, int64_t n, float factor, cudaStream_t s);
 cudaError_t launch_init_state(SolverState* st, cudaStream_t s);
 // out[0] = sum_i |x_i|^2, out[1 + k] = sum_i x_ik (float64; partial buffer of
 // `parts` x (d + 1) doubles, deterministic two-pass reduction)
@@ -77,16 +68,93 @@ cudaError_t launch_mean_cost_closed(const double* mx, const double* my, int64_t 
 // out[k] = sum_b partial[b * width + k], b = 0..parts-1 in order
 cudaError_t launch_sum_parts(const double* partial, int parts, int width, double* out, cudaStream_t s);
 
-// tcgen05 sweeps (sweep_tc.cu): operands pre-scaled by sqrt(2 log2(e) / eps), split into
-// bf16 hi/lo with K padded to a multiple of 64; map* point at CUtensorMap objects.
-cudaError_t launch_split_bf16(const float* X, int64_t n, int32_t d, int32_t dp, float scale, void* hi, void* lo,
-                              cudaStream_t s, const float* mu = nullptr, float* norm = nullptr);
-// mapBbias: (nB padded to 128) x 16 bf16 rows [beta_hi, beta_mid, beta_lo, 0...] of the
+// tcgen05 sweeps (sweep_tc.cu) on the operands of operands.cu; maps point at CUtensorMap objects.
+// bias map: (nB padded to 128) x 16 bf16 rows [beta_hi, beta_mid, beta_lo, 0...] of the
 // B side; bias_out (optional): the same rows for the A side, written from the updated
 // potential in potential mode (the next sweep's B bias).
-cudaError_t launch_lse_sweep_tc(const SweepParams& p, const void* mapAh, const void* mapAl, const void* mapBh,
-                                const void* mapBl, const void* mapBbias, int nkb, int split3, int bn, int G,
-                                int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream);
+struct TcMaps {
+  const void* a[3];   // operand maps of the rows' side (128-row boxes): hi, lo, (grid split) third part
+  const void* b[3];   // of the columns' side (bn-row boxes)
+  const void* bias;   // bias rows of the columns' side (bn-row boxes)
+};
+// parts: operand parts in use (1 bf16, 2 bf16x3); gscale non-NULL: the integer-grid split
+// (grid_split.cuh; parts 2 or 3, bn = 128) with its device scales.
+cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const float* gscale,
+                                int bn, int G, int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream,
+                                const float* lrow = nullptr, void* prob = nullptr, int64_t a_row0 = 0);
+// x <- x + alpha (T(x) - x) for rows [row0, row0 + rows) from the P tiles and row sums a
+// kModeProb sweep left (pv_tc.cu); mapY: the parts of the y operand in 64-row boxes.
+struct PvLaunch {
+  const float* X;      // row row0 of the points (may alias out)
+  float* out;
+  const float* rsum;   // [rows]
+  const void* prob;
+  const void* mapY[3];
+  const float* gscale;
+  const float* mu;
+  int64_t rows, m;
+  int32_t d, parts;
+  float alpha, inv_sc; // inv_sc = 1 / sqrt(c)
+  int32_t* fault;
+};
+int64_t pv_prob_bytes_per_block(int64_t m);  // P bytes of one 128-row block
+cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream);
+// Tensor-core operands (operands.cu).
+// mu = (mean of the rows of X + mean of the rows of Y) / 2, the sums carried beyond float64
+// rounding of their order; partial: reduce_parts() * d doubles of scratch; ticket: a zero
+// word, zero again afterwards; gmax (or NULL): two words zeroed for launch_operands.
+cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial,
+                          unsigned* ticket, float* mu, float* gmax, cudaStream_t s);
+// Both clouds: parts of sqrt(c) (x - mu), rows of dp 16-bit elements (zeros past d): bf16
+// hi, lo, or the integer grid's two or three half-precision parts (grid_split.cuh); unused
+// parts are NULL. Centred squared norms, and bias rows of both sides from the potentials f
+// (x side) and g (y side) where given, into one or two buffers each, rows padded to a
+// multiple of 256. Grid: gmax = the largest squared norms, gscale = {2^(ex + ey),
+// 2^-(ex + ey), 2^-ey}.
+struct OperandPrep {
+  const float* x;
+  const float* y;
+  int64_t n, m;
+  int32_t d, dp;
+  float sc, sc_lo;          // sqrt(c) = sc + sc_lo (bf16: sc alone)
+  const float* mu;
+  float* xnc;
+  float* ync;
+  float* gmax;
+  float* gscale;
+  void* xp[3];
+  void* yp[3];
+  const float* f;           // NULL: no x-side bias rows
+  const float* g;
+  float bscale, bscale_lo;  // log2(e) / eps = bscale + bscale_lo
+  void* xb[2];
+  void* yb[2];
+};
+// What a persistent loop finds when it starts: its work-split tables, ready flags, counters
+// and state.
+struct LoopSetupSide {
+  void* segs;               // int4 [G * maxseg]
+  int32_t* nseg;            // [G]
+  int2* crow;               // [R] (offset, count) into cslot
+  int32_t* cslot;
+  uint32_t* flag;           // [R]
+  unsigned long long* cnt;  // [R]
+  unsigned long long* done;
+  int32_t R, T;
+  uint32_t flag_init;
+};
+struct LoopSetup {
+  LoopSetupSide side[2];
+  SolverState* state;       // [2]
+  int32_t G, maxseg;
+};
+// kGridHull: the integer grid for clouds inside the hull of the two that the last kGrid call
+// on this workspace saw (same mu and gmax).
+enum class OperandKind { kBf16, kGrid, kGridHull };
+cudaError_t launch_operands(const OperandPrep& op, OperandKind kind, const LoopSetup* loop, cudaStream_t s);
+cudaError_t launch_loop_finish(const float* f_new, const float* an, const float* w, double log_w_uniform, double eps,
+                               int64_t n, float* L, const float* f_cur, float* f_out, cudaStream_t s);
+cudaError_t launch_warm_start(float* g, const float* g_prev, int64_t m, float* f, int64_t n, float c, cudaStream_t s);
 cudaError_t launch_bias_prep(const float* potB, const float* Bn, int64_t nB, int64_t nB_pad, float bscale, void* out,
                              cudaStream_t s);
 void tc_plan(int64_t nA, int64_t nB, int bn, int sms, int* G, int* maxseg);
@@ -128,19 +196,19 @@ struct LoopSideLaunch {
   unsigned long long* cnt;   // [row blocks] arrival counters, zero at the loop's start
   unsigned long long* done;  // finished row blocks, zero at the loop's start
   float2* partial;           // (max, sum) slots of this side's sweeps
-  // device buffers for the work split's tables (filled by the launch): segs (int4) and
-  // cslot hold table_slots entries each, cptr row blocks + 1, nseg one entry per CTA
-  void* segs;
-  int32_t* nseg;
-  int32_t* cptr;
-  int32_t* cslot;
-  int64_t table_slots;
+  // the work split's tables (LoopSetupSide)
+  const void* segs;
+  const int32_t* nseg;
+  const int2* crow;
+  const int32_t* cslot;
 };
 struct LoopLaunch {
   LoopSideLaunch side[2];
   // CUtensorMap: X hi, X lo, Y hi, Y lo (128-row boxes); X hi, X lo, Y hi, Y lo (bn-row
-  // boxes); bias rows X[0], X[1], Y[0], Y[1] (bn-row boxes)
-  const void* maps[12];
+  // boxes); third parts of the grid split: X, Y (128-row), X, Y (bn-row; any map without
+  // the grid split); bias rows X[0], X[1], Y[0], Y[1] (bn-row boxes)
+  const void* maps[16];
+  const float* gscale;       // grid split: its device scales (NULL: bf16 operands)
   double* errpart;           // [2][row blocks of X]
   SolverState* state;
   int32_t* fault;
@@ -157,11 +225,11 @@ int encode_operand_map(void* map, void* base, int64_t rows, int32_t dp, int box_
 int32_t stall_window_setting();
 unsigned long long wait_limit_setting();
 int device_sm_count();
+// Least workspace a solve accepts (the float32 path then runs on CUDA cores).
+size_t workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision);
 int fail_message(int code, const char* msg);  // sets the last-error text, returns code
-cudaError_t launch_fill_u32(uint32_t* p, int64_t n, uint32_t v, cudaStream_t s);
-bool loop_tc_supported(int bn, int nkb, int split3);
+bool loop_tc_supported(int bn, int nkb, int split3, bool grid);
 
 void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg);
-size_t loop_tc_smem(int bn, int nkb, int split3);
 
 }  // namespace progot

@@ -241,6 +241,7 @@ struct Request {
   int32_t status = PROGOT_OK;
   bool done = false;
   size_t bytes = 0;
+  size_t ws_bytes = 0;  // of which the solve's workspace
 };
 
 }  // namespace progot
@@ -265,15 +266,14 @@ struct progot_server {
 namespace progot {
 
 // Device bytes of one request: inputs, outputs and its solve workspace (each 256-aligned).
-static size_t request_bytes(const progot_problem& p, int32_t precision) {
+static size_t request_bytes(const progot_problem& p, size_t solve_ws) {
   const size_t f = sizeof(float);
   size_t b = 0;
   b += round_up256(f * (size_t)p.n * p.d) + round_up256(f * (size_t)p.m * p.d);             // x, y
   if (p.a) b += round_up256(f * (size_t)p.n);
   if (p.b) b += round_up256(f * (size_t)p.m);
   b += round_up256(f * (size_t)p.n * p.d) + round_up256(f * (size_t)p.K * p.m) + round_up256(f * (size_t)p.n);
-  b += round_up256(progot_workspace_size(p.n, p.m, p.d, precision));
-  return b;
+  return b + solve_ws;
 }
 
 static void serve(progot_server* S) {
@@ -324,7 +324,7 @@ static void serve(progot_server* S) {
     float* x_out = (float*)take(f * hp.n * hp.d);
     float* g_all = (float*)take(f * hp.K * hp.m);
     float* f_last = (float*)take(f * hp.n);
-    const size_t wsb = round_up256(progot_workspace_size(hp.n, hp.m, hp.d, S->precision));
+    const size_t wsb = rq->ws_bytes;
     void* ws = take(wsb);
     int32_t rc = PROGOT_OK;
     if (cudaMemcpyAsync(x, hp.x, f * hp.n * hp.d, cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -390,7 +390,11 @@ int64_t progot_server_submit(progot_server* S, const progot_problem* req) {
     set_last_error_message("invalid server or request");
     return -PROGOT_ERR_INVALID_ARG;
   }
-  const size_t bytes = progot::request_bytes(*req, S->precision);
+  // a request that fits the budget only with the smallest workspace runs with that
+  size_t wsb = progot::round_up256(progot_workspace_size(req->n, req->m, req->d, S->precision));
+  if (progot::request_bytes(*req, wsb) > S->arena->size())
+    wsb = progot::round_up256(progot::workspace_size_min(req->n, req->m, req->d, S->precision));
+  const size_t bytes = progot::request_bytes(*req, wsb);
   if (bytes > S->arena->size()) {
     set_last_error_message("request needs more device memory than the server's budget");
     return -PROGOT_ERR_OOM;
@@ -403,6 +407,7 @@ int64_t progot_server_submit(progot_server* S, const progot_problem* req) {
     r.prob = *req;
     r.t_submit = std::chrono::steady_clock::now();
     r.bytes = bytes;
+    r.ws_bytes = wsb;
     S->queue.push_back(id);
   }
   S->cv_work.notify_one();

@@ -95,7 +95,8 @@ __device__ __forceinline__ RowIn row_inputs(const SweepParams& p, int64_t i, con
   return r;
 }
 
-// Epilogue for one row given L = log2 sum_j 2^{t_ij}. Writes the row's output, returns
+// Epilogue for one row given L = log2 sum_j 2^{t_ij} (a float in the float32 and bf16
+// sweeps, float64 in the integer-grid sweeps). Writes the row's output, returns
 // its error term and the written value in *val. The error terms are float32 (they only
 // feed the stop test against tau): on GB300 every float64 instruction of this epilogue
 // sits on the sweep's critical path at a small fraction of the float32 rate.
@@ -105,11 +106,11 @@ __device__ __forceinline__ RowIn row_inputs(const SweepParams& p, int64_t i, con
 //              average (f_old + f_new) / 2 and measures the error at f_old;
 //   marginal:  r_i = exp((pot_i - |a_i|^2)/eps + ln2 L), the exponent formed in float64
 //              (it is a difference of large terms) and exponentiated in float32.
-__device__ __forceinline__ float row_epilogue(const SweepParams& p, int64_t i, float L, const RowIn& in,
+__device__ __forceinline__ float row_epilogue(const SweepParams& p, int64_t i, double L, const RowIn& in,
                                               float* out_target, float* val) {
   if (p.mode == kModePotential) {
     const double logw = p.wA ? (double)__logf(in.w) : p.log_w_uniform;
-    const float fnew = (float)(p.eps * logw + (double)in.an - p.eps * kLn2 * (double)L);
+    const float fnew = (float)(p.eps * logw + (double)in.an - p.eps * kLn2 * L);
     const float fout = (p.role == 3) ? 0.5f * (in.pot + fnew) : fnew;
     out_target[i] = fout;
     *val = fout;
@@ -124,12 +125,12 @@ __device__ __forceinline__ float row_epilogue(const SweepParams& p, int64_t i, f
     return 0.f;
   }
   if (p.mode == kModeLse) {
-    out_target[i] = L;
-    *val = L;
+    out_target[i] = (float)L;
+    *val = (float)L;
     return 0.f;
   }
   // marginal
-  const double arg = ((double)in.pot - (double)in.an) / p.eps + kLn2 * (double)L;
+  const double arg = ((double)in.pot - (double)in.an) / p.eps + kLn2 * L;
   const float r = expf((float)arg);
   if (out_target) out_target[i] = r;
   *val = r;

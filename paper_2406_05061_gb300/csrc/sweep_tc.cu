@@ -32,6 +32,7 @@
 
 #include <algorithm>
 
+#include "grid_split.cuh"
 #include "progot_internal.h"
 #include "sweep_epilogue.cuh"
 #include "tc_common.cuh"
@@ -65,6 +66,7 @@ struct TcShared {
   int32_t stop;           // the previous sweep already stopped the Sinkhorn loop
   float red[4];
   float ered[4];
+  int32_t slots[32], eslots[32];  // partial slots of the row block being combined, by group
   float2 ms[2][128];   // (max, sum) of LSE warpgroup 1 by segment parity, merged by warpgroup 0
   float2 seg[2][128];  // merged (max, sum) of a handed-off segment, by segment parity
 };
@@ -78,7 +80,7 @@ struct TcShared {
 struct TcParams {
   SweepParams p;
   int32_t nkb;        // K blocks of 64
-  int32_t split3;     // 1: bf16x3 (hi and lo operands), 0: bf16 (hi only)
+  int32_t parts;      // operand parts: 1 bf16 (hi only), 2 bf16x3 (hi, lo), or the grid split's 2 or 3
   int32_t stages;     // B pipeline depth (units of one K block of one tile)
   int32_t a_bufs;     // 1 or 2 resident A-operand buffers, or 0: A K blocks stream with B
   int32_t G;          // CTAs
@@ -87,28 +89,36 @@ struct TcParams {
   int32_t maxseg;     // partial slots per CTA
   int32_t* fault;     // set to 1 by a CTA whose bounded wait expired
   __nv_bfloat16* bias_out;  // potential mode: beta rows of the updated side (rows x 16), or nullptr
+  const float* gscale;      // grid split: {2^(ex + ey), 2^-(ex + ey)} (device)
+  // kModeProb: row L (log2 units) of this launch's rows, which start at operand row a_row0,
+  // and the P tiles (see pv_tc.cu): [row block][64-column unit][hi, lo][128 rows x 64]
+  const float* lrow;
+  unsigned char* prob;
+  int64_t a_row0;
 };
 
 struct SmemLayout {
   uint32_t a0, a_stride, a_lo_off, a_bias, stage0, stage_bytes, b_lo_off, bias_off, a_stage_off, ctrl, total;
 };
 
-__host__ __device__ inline SmemLayout smem_layout(int bn, int nkb, int split3, int stages, int a_bufs) {
+// Offsets of an operand's part q: q * a_lo_off in a resident A buffer, q * b_lo_off in a
+// stage, q * A_TILE_BYTES in a stage's streamed A block. The grid split has two ones tiles.
+__host__ __device__ inline SmemLayout smem_layout(int bn, int nkb, int parts, int stages, int a_bufs, bool grid) {
   SmemLayout L;
   const uint32_t b_tile = (uint32_t)bn * KB * 2, bias_tile = (uint32_t)bn * 32;
   uint32_t off = 0;
   L.a0 = off;
   L.a_lo_off = nkb * A_TILE_BYTES;
-  L.a_stride = nkb * A_TILE_BYTES * (split3 ? 2 : 1);
+  L.a_stride = nkb * A_TILE_BYTES * parts;
   off += a_bufs * L.a_stride;
   L.a_bias = off;
-  off += A_BIAS_BYTES;
+  off += A_BIAS_BYTES * (grid ? 2 : 1);
   L.stage0 = off;
   L.b_lo_off = b_tile;
-  L.bias_off = b_tile * (split3 ? 2 : 1);
-  // streamed A (a_bufs = 0): the A K block (hi, then lo) follows the bias rows in the stage
+  L.bias_off = b_tile * parts;
+  // streamed A (a_bufs = 0): the A K block (its parts in order) follows the bias rows in the stage
   L.a_stage_off = L.bias_off + bias_tile;
-  L.stage_bytes = L.a_stage_off + (a_bufs == 0 ? A_TILE_BYTES * (split3 ? 2u : 1u) : 0u);
+  L.stage_bytes = L.a_stage_off + (a_bufs == 0 ? A_TILE_BYTES * (uint32_t)parts : 0u);
   off += stages * L.stage_bytes;
   L.ctrl = off;
   off += sizeof(TcShared);
@@ -147,28 +157,23 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 
-// beta_j split into three bf16 terms (hi, mid, lo) in the first three of 16 slots.
-__device__ __forceinline__ void write_bias_row(__nv_bfloat16* row16, float beta) {
-  __nv_bfloat16 h1, h2, h3;
-  if (isfinite(beta)) {
-    h1 = __float2bfloat16_rn(beta);
-    const float r1 = beta - __bfloat162float(h1);
-    h2 = __float2bfloat16_rn(r1);
-    h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
-  } else {
-    h1 = __float2bfloat16_rn(-INFINITY);
-    h2 = __float2bfloat16_rn(0.f);
-    h3 = __float2bfloat16_rn(0.f);
+// Two 16-byte chunks (w[0..3], w[4..7]) as one 32-byte store, in swapped order on odd rows.
+__device__ __forceinline__ void store_pair32(unsigned char* dst, const uint32_t (&w)[8], int swap) {
+  uint32_t q[8];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    q[e] = swap ? w[e + 4] : w[e];
+    q[e + 4] = swap ? w[e] : w[e + 4];
   }
-  uint4 lo4;
-  lo4.x = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
-  lo4.y = (uint32_t)__bfloat16_as_ushort(h3);
-  lo4.z = 0u;
-  lo4.w = 0u;
-  uint4* dst = reinterpret_cast<uint4*>(row16);
-  dst[0] = lo4;
-  dst[1] = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "r"(q[0]), "r"(q[1]), "r"(q[2]),
+               "r"(q[3]), "r"(q[4]), "r"(q[5]), "r"(q[6]), "r"(q[7])
+               : "memory");
 }
 
 static_assert(sizeof(SolverState) % 16 == 0, "the solver state is loaded in 16-byte pieces");
@@ -199,10 +204,10 @@ __device__ __forceinline__ SolverState sweep_state(const SweepParams& p) {
 // 32 rows, then (q0 + q1) + (q2 + q3)); the last row block of the sweep finishes it.
 // The g-update of a Sinkhorn loop (role 2) measures no error and changes no solver
 // state, so its row blocks skip the sweep-level arrival altogether.
-template <int NT>
+template <int NT, int GRID>
 __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int k, const Seg& sg, const Split& sp,
                                                  int tid, int row0, const float2 (&mv)[BM / NT], int fcur,
-                                                 int32_t& s_last, int32_t& s_fin, float* red) {
+                                                 int32_t& s_last, int32_t& s_fin, float* red, int32_t* slots) {
   constexpr int RPT = BM / NT;
   const SweepParams& p = tp.p;
   const float* potA_cur = p.potA_old;
@@ -227,6 +232,16 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
   }
   int c_first, c_last;
   contributors(sp, sg.r, &c_first, &c_last);
+  const int nc = c_last - c_first + 1;
+  // partial slots of the row block's CTAs (32 at a time), one thread each: a division per
+  // contributor and row would sit between the arrival and the loads
+  auto fill_slots = [&](int base) {
+    if (tid < 32 && base + tid < nc) {
+      const int cc = c_first + base + tid;
+      slots[tid] = cc * tp.maxseg + seg_of(sp, sg.r, cc);
+    }
+  };
+  fill_slots(0);
   seg_bar<NT>();  // the partial stores of all rows happen before the arrival below
   if (tid == 0) {
     const unsigned prev = atomic_add_acq_rel_gpu(&p.cnt[sg.r], 1u);
@@ -235,37 +250,55 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
   seg_bar<NT>();  // ... and the other CTAs' partials are visible after it
   if (!s_last) return;
   float e[RPT];
+  float2 accs[RPT];
+#pragma unroll
+  for (int h = 0; h < RPT; ++h) accs[h] = make_float2(-INFINITY, 0.f);
+  for (int base = 0; base < nc; base += 32) {
+    if (base > 0) {
+      seg_bar<NT>();
+      fill_slots(base);
+      seg_bar<NT>();
+    }
+    // the loads of eight contributors back to back, then combined in CTA order
+    for (int q0 = base; q0 < min(nc, base + 32); q0 += 8) {
+      float2 pv[RPT][8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int h = 0; h < RPT; ++h)
+          if (q0 + q < nc) pv[h][q] = __ldcg(&p.partial[(int64_t)slots[q0 + q - base] * BM + row0 + NT * h]);
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int h = 0; h < RPT; ++h)
+          if (q0 + q < nc) accs[h] = lse_combine(accs[h], pv[h][q]);
+    }
+  }
 #pragma unroll
   for (int h = 0; h < RPT; ++h) {
     e[h] = 0.f;
     const int rl = row0 + NT * h;
     const int64_t i = (int64_t)sg.r * BM + rl;
     if (i < p.nA) {
-      // issue the partial loads back to back, then combine them in CTA order
-      constexpr int kMaxC = 8;
-      const int nc = c_last - c_first + 1;
-      float2 pv[kMaxC];
-#pragma unroll
-      for (int q = 0; q < kMaxC; ++q) {
-        if (q < nc) {
-          const int cc = c_first + q;
-          pv[q] = __ldcg(&p.partial[((int64_t)cc * tp.maxseg + seg_of(sp, sg.r, cc)) * BM + rl]);
-        }
+      const float2 acc = accs[h];
+      const double Lr = GRID ? (double)acc.x + (double)log2f(acc.y) : (double)(acc.x + __log2f(acc.y));
+      if (GRID && p.mode == kModeProb) {
+        out_target[i] = acc.y;
+        continue;
       }
-      float2 acc = make_float2(-INFINITY, 0.f);
-#pragma unroll
-      for (int q = 0; q < kMaxC; ++q)
-        if (q < nc) acc = lse_combine(acc, pv[q]);
-      for (int cc = c_first + kMaxC; cc <= c_last; ++cc)
-        acc = lse_combine(acc, __ldcg(&p.partial[((int64_t)cc * tp.maxseg + seg_of(sp, sg.r, cc)) * BM + rl]));
-      const float Lr = acc.x + __log2f(acc.y);
       float val;
       e[h] = row_epilogue(p, i, Lr, rin[h], out_target, &val);
-      if (tp.bias_out != nullptr && p.mode == kModePotential)
-        write_bias_row(tp.bias_out + i * 16, (val - rin[h].an) * p.bscale);
+      if (tp.bias_out != nullptr && p.mode == kModePotential) {
+        if constexpr (GRID)
+          write_bias_row_grid(tp.bias_out + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), __ldg(tp.gscale));
+        else
+          write_bias_row(tp.bias_out + i * 16, (val - rin[h].an) * p.bscale);
+      }
     }
   }
-  if (p.role == 2) {
+  // a g-update and the passes of a map step measure no error
+  if (p.role == 2 || (p.state == nullptr && (p.mode == kModeLse || p.mode == kModeProb))) {
+    seg_bar<NT>();  // the slots are free for the next segment
     if (tid == 0) p.cnt[sg.r] = 0;
     return;  // the counter is read again only by the next sweep, after this grid ends
   }
@@ -298,10 +331,14 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
   seg_bar<NT>();
 }
 
-template <int BN>
+// GRID = 0: bf16 operands, one accumulator (two buffers of BN columns). GRID = 1: the
+// integer-grid split (grid_split.cuh), BN = 128, two accumulators per tile (leading
+// products at TMEM columns [0, 256), the others at [256, 512)).
+template <int BN, int GRID>
 __global__ void __launch_bounds__(NTHREADS, 1)
     lse_sweep_tc(const __grid_constant__ CUtensorMap mapAh, const __grid_constant__ CUtensorMap mapAl,
-                 const __grid_constant__ CUtensorMap mapBh, const __grid_constant__ CUtensorMap mapBl,
+                 const __grid_constant__ CUtensorMap mapAr, const __grid_constant__ CUtensorMap mapBh,
+                 const __grid_constant__ CUtensorMap mapBl, const __grid_constant__ CUtensorMap mapBr,
                  const __grid_constant__ CUtensorMap mapBbias, TcParams tp) {
   const SweepParams& p = tp.p;
   // Programmatic dependent launch: let the next sweep's CTAs be scheduled as soon as
@@ -310,7 +347,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const SmemLayout L = smem_layout(BN, tp.nkb, tp.split3, tp.stages, tp.a_bufs);
+  const SmemLayout L = smem_layout(BN, tp.nkb, tp.parts, tp.stages, tp.a_bufs, GRID != 0);
+  const int parts = tp.parts;
   constexpr uint32_t B_TILE_BYTES = (uint32_t)BN * KB * 2, BIAS_TILE_BYTES = (uint32_t)BN * 32;
   TcShared& sh = *reinterpret_cast<TcShared*>(smem + L.ctrl);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -344,11 +382,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
   // A-side bias operand: all ones (bf16 0x3F80), so that the K = 16 bias step adds
   // beta_hi + beta_mid + beta_lo whatever the order of the 16-byte chunks in a row.
-  {
+  if constexpr (GRID) {
+    fill_bias_ones_grid(smem + L.a_bias, threadIdx.x, NTHREADS);
+  } else {
     uint32_t* ab = reinterpret_cast<uint32_t*>(smem + L.a_bias);
     for (int i = threadIdx.x; i < A_BIAS_BYTES / 4; i += NTHREADS) ab[i] = 0x3F803F80u;
-    fence_async_smem();
   }
+  fence_async_smem();
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)),
                  "r"(TMEM_COLS)
@@ -371,9 +411,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     int u = 0;  // B stage units issued
     bool ok = true;
     const uint32_t abytes = (uint32_t)L.a_stride;
-    const uint32_t bbytes = B_TILE_BYTES * (tp.split3 ? 2u : 1u);
+    const uint32_t bbytes = B_TILE_BYTES * (uint32_t)parts;
     // streamed A: each stage also carries the A K block (hi and lo) of its tile
-    const uint32_t sabytes = NA == 0 ? A_TILE_BYTES * (tp.split3 ? 2u : 1u) : 0u;
+    const uint32_t sabytes = NA == 0 ? A_TILE_BYTES * (uint32_t)parts : 0u;
     int a_issued = 0;
     bool waited = false, stopped = false;
     int pend_s[8], pend_t[8], npend = 0;  // stages whose bias rows wait for the previous sweep
@@ -399,6 +439,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     };
     for (int k = 0; k < nseg && ok && !stopped; ++k) {
       const Seg sg = segment(sp, c, k);
+      const int a_row = sg.r * BM + (GRID ? (int)tp.a_row0 : 0);
       if (NA > 0) {
         const int ai = k % NA;
         // reusing an A buffer waits for the MMA warp, which waits for the pending bias
@@ -413,9 +454,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (elect_one()) {
           mbar_arrive_expect_tx(&sh.a_full[ai], abytes);
           for (int kb = 0; kb < nkb; ++kb) {
-            tma_load_2d(abuf + kb * A_TILE_BYTES, &mapAh, &sh.a_full[ai], kb * KB, sg.r * BM);
-            if (tp.split3)
-              tma_load_2d(abuf + L.a_lo_off + kb * A_TILE_BYTES, &mapAl, &sh.a_full[ai], kb * KB, sg.r * BM);
+            tma_load_2d(abuf + kb * A_TILE_BYTES, &mapAh, &sh.a_full[ai], kb * KB, a_row);
+            if (parts > 1)
+              tma_load_2d(abuf + L.a_lo_off + kb * A_TILE_BYTES, &mapAl, &sh.a_full[ai], kb * KB, a_row);
+            if (GRID && parts > 2)
+              tma_load_2d(abuf + 2 * L.a_lo_off + kb * A_TILE_BYTES, &mapAr, &sh.a_full[ai], kb * KB, a_row);
           }
         }
         __syncwarp();
@@ -438,11 +481,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const bool bias_now = waited && kb == 0;
             mbar_arrive_expect_tx(&sh.full[s], bbytes + sabytes + (bias_now ? BIAS_TILE_BYTES : 0u));
             tma_load_2d(st, &mapBh, &sh.full[s], kb * KB, t * BN);
-            if (tp.split3) tma_load_2d(st + L.b_lo_off, &mapBl, &sh.full[s], kb * KB, t * BN);
+            if (parts > 1) tma_load_2d(st + L.b_lo_off, &mapBl, &sh.full[s], kb * KB, t * BN);
+            if (GRID && parts > 2) tma_load_2d(st + 2 * L.b_lo_off, &mapBr, &sh.full[s], kb * KB, t * BN);
             if (bias_now) tma_load_2d(st + L.bias_off, &mapBbias, &sh.full[s], 0, t * BN);
             if (NA == 0) {
-              tma_load_2d(st + L.a_stage_off, &mapAh, &sh.full[s], kb * KB, sg.r * BM);
-              if (tp.split3) tma_load_2d(st + L.a_stage_off + A_TILE_BYTES, &mapAl, &sh.full[s], kb * KB, sg.r * BM);
+              tma_load_2d(st + L.a_stage_off, &mapAh, &sh.full[s], kb * KB, a_row);
+              if (parts > 1) tma_load_2d(st + L.a_stage_off + A_TILE_BYTES, &mapAl, &sh.full[s], kb * KB, a_row);
+              if (GRID && parts > 2)
+                tma_load_2d(st + L.a_stage_off + 2 * A_TILE_BYTES, &mapAr, &sh.full[s], kb * KB, a_row);
             }
             if (waited || kb != 0) mbar_arrive(&sh.bias_full[s]);
           }
@@ -466,6 +512,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
     const uint64_t abias = desc_sw32(smem_u32(smem + L.a_bias));
+    const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
     bool ok = true;
     int u = 0, tl = 0;
     for (int k = 0; k < nseg && ok; ++k) {
@@ -495,13 +542,31 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const uint64_t ah = NA > 0 ? desc_sw128(a_hi + kb * A_TILE_BYTES) : desc_sw128(sa);
           const uint64_t al = NA > 0 ? desc_sw128(a_lo + kb * A_TILE_BYTES) : desc_sw128(sa + A_TILE_BYTES);
           const uint64_t bb = desc_sw32(st + L.bias_off);
-          if (elect_one()) {
+          if constexpr (GRID) {
+            // K = 16 steps that hold coordinates (the padding up to 64 multiplies zeros)
+            const int ksteps = min(KB / 16, (p.d - kb * KB + 15) / 16);
+            const uint64_t ar = NA > 0 ? desc_sw128(a_hi + 2 * L.a_lo_off + kb * A_TILE_BYTES)
+                                       : desc_sw128(sa + 2 * A_TILE_BYTES);
+            const uint64_t br = desc_sw128(st + 2 * L.b_lo_off);
+            const uint32_t d2 = d_tmem + 256;
+            if (elect_one()) {
+              const uint32_t more = kb > 0 ? 1u : 0u;
+              if (parts > 2) {
+                issue_grid_part<BN, 3>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
+                issue_grid_part<BN, 3>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
+                issue_grid_part<BN, 3>(ksteps, 2, d_tmem, d2, ah, al, ar, br, more);
+              } else {
+                issue_grid_part<BN, 2>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
+                issue_grid_part<BN, 2>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
+              }
+            }
+          } else if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < KB / 16; ++kk) {
               // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
               const uint64_t adv = (uint64_t)(kk * 2);
               umma<BN>(d_tmem, ah + adv, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
-              if (tp.split3) {
+              if (parts > 1) {
                 umma<BN>(d_tmem, ah + adv, bl + adv, 1u);
                 umma<BN>(d_tmem, al + adv, bh + adv, 1u);
               }
@@ -521,7 +586,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             tc_fence_after();
           }
           if (elect_one()) {
-            if (kb == 0) umma<BN>(d_tmem, abias, bb, 1u);
+            if (kb == 0) {
+              umma<BN>(d_tmem, abias, bb, 1u);
+              if constexpr (GRID) umma<BN>(d_tmem + 256, abias2, bb, 1u);
+            }
             umma_commit(&sh.empty[s]);
           }
           __syncwarp();
@@ -546,7 +614,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int quarter = warp & 3;  // TMEM lane quarter this warp may access
     const int row_local = quarter * 32 + lane;
     const int ltid = threadIdx.x - 64;  // 0..127 in warpgroup 0
+    constexpr int CW = GRID ? 64 : 128;  // columns folded at a time (registers)
+    constexpr int NC = CW / 32;
     int tl = 0, jt = 0;
+    const float inv2 = GRID ? __ldg(tp.gscale + 1) : 1.f;
+    const uint64_t inv22 = pack2(inv2, inv2);
+    const bool prob = GRID && p.mode == kModeProb;
     // potentials, weights and the solver state below are the previous sweep's results
     asm volatile("griddepcontrol.wait;" ::: "memory");
     SolverState st0{};
@@ -558,7 +631,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     bool dead = false;
     for (int k = 0; k < (stopped ? 0 : nseg); ++k) {
       const Seg sg = segment(sp, c, k);
-      float m_run = -INFINITY, s_run = 0.f;
+      float m_run = prob ? 0.f : -INFINITY, s_run = 0.f;
+      const bool row_ok = (int64_t)sg.r * BM + row_local < p.nA;
+      const float Lr = (prob && row_ok) ? __ldg(tp.lrow + (int64_t)sg.r * BM + row_local) : 0.f;
       for (int t = sg.t0; t < sg.t1; ++t, ++tl) {
         if ((tl & 1) != wg) continue;
         const uint32_t ph = (uint32_t)(jt & 1);
@@ -574,44 +649,90 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tc_fence_after();
         const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(wg * BN);
 #pragma unroll 1
-        for (int half = 0; half < BN / 128; ++half) {
-          const uint32_t taddr = taddr0 + (uint32_t)(half * 128);
-          float v[4][32];
-          PROGOT_TMEM_LD32(taddr + 0, v[0]);
-          PROGOT_TMEM_LD32(taddr + 32, v[1]);
-          PROGOT_TMEM_LD32(taddr + 64, v[2]);
-          PROGOT_TMEM_LD32(taddr + 96, v[3]);
-          tmem_wait_ld();
-          if (half == BN / 128 - 1) {
+        for (int half = 0; half < BN / CW; ++half) {
+          const uint32_t taddr = taddr0 + (uint32_t)(half * CW);
+          float v[NC][32];
+#pragma unroll
+          for (int cc = 0; cc < NC; ++cc) PROGOT_TMEM_LD32(taddr + 32 * cc, v[cc]);
+          if constexpr (GRID) {
+            // t = leading sums + the rest, rounded once
+            float w[NC][32];
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) PROGOT_TMEM_LD32(taddr + 256 + 32 * cc, w[cc]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc)
+#pragma unroll
+              for (int i = 0; i < 32; i += 2)
+                unpack2(add2(pack2(v[cc][i], v[cc][i + 1]), pack2(w[cc][i], w[cc][i + 1])), v[cc][i], v[cc][i + 1]);
+          } else {
+            tmem_wait_ld();
+          }
+          if (half == BN / CW - 1) {
             // the whole accumulator is in registers: hand the TMEM buffer back to the MMA warp
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tmem_empty[wg]);
           }
-          // maximum: 8 independent chains of three-input max
-          float mx[8];
+          if constexpr (GRID) {
+            if (prob) {
+              // P = 2^{t - L + 14} as half-precision hi + lo, in the shared-memory image
+              // of a 128-byte-swizzled K-major tile (32-byte pieces: full sectors)
+              unsigned char* tile = tp.prob + ((int64_t)sg.r * (2 * T) + 2 * t + half) * 32768 + row_local * 128;
+              const uint64_t neg = pack2(14.f - Lr, 14.f - Lr);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) mx[q] = v[q >> 1][(q & 1) * 16];
+              for (int cp = 0; cp < 4; ++cp) {
+                uint32_t hw[8], lw[8];
 #pragma unroll
-          for (int cc = 0; cc < 4; ++cc)
+                for (int e = 0; e < 8; ++e) {
+                  const int cc = cp >> 1, i = (cp & 1) * 16 + 2 * e;
+                  float a0, a1;
+                  unpack2(fma2(pack2(v[cc][i], v[cc][i + 1]), inv22, neg), a0, a1);
+                  const float p0 = row_ok ? fast_exp2(a0) : 0.f, p1 = row_ok ? fast_exp2(a1) : 0.f;
+                  s_run += p0 + p1;
+                  const __half2 h = __floats2half2_rn(p0, p1);
+                  const float2 hf = __half22float2(h);
+                  const __half2 l = __floats2half2_rn(p0 - hf.x, p1 - hf.y);
+                  hw[e] = *reinterpret_cast<const uint32_t*>(&h);
+                  lw[e] = *reinterpret_cast<const uint32_t*>(&l);
+                }
+                unsigned char* dst = tile + (((2 * cp) ^ (row_local & 6)) * 16);
+                store_pair32(dst, hw, row_local & 1);
+                store_pair32(dst + 16384, lw, row_local & 1);
+              }
+              m_run = 0.f;
+              continue;
+            }
+          }
+          // maximum: 2 NC independent chains of three-input max
+          float mx[2 * NC];
+#pragma unroll
+          for (int q = 0; q < 2 * NC; ++q) mx[q] = v[q >> 1][(q & 1) * 16];
+#pragma unroll
+          for (int cc = 0; cc < NC; ++cc)
 #pragma unroll
             for (int i = 1; i < 16; i += 2) {
               mx[cc * 2] = max3(mx[cc * 2], v[cc][i], v[cc][i + 1 < 16 ? i + 1 : i]);
               mx[cc * 2 + 1] = max3(mx[cc * 2 + 1], v[cc][16 + i], v[cc][16 + (i + 1 < 16 ? i + 1 : i)]);
             }
-          const float tmax = max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), fmaxf(mx[6], mx[7]));
+          float tmax = mx[0];
+#pragma unroll
+          for (int q = 1; q < 2 * NC; ++q) tmax = fmaxf(tmax, mx[q]);
           const float mnew = fmaxf(m_run, tmax);
           if (mnew != -INFINITY) {
-            const uint64_t negm = pack2(-mnew, -mnew);
+            // grid split: the accumulators hold t 2^(ex + ey); (t - m) 2^-(ex + ey) is exact
+            const float nm = GRID ? -mnew * inv2 : -mnew;
+            const uint64_t negm = pack2(nm, nm);
             uint64_t acc[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[q] = 0ull;
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc)
+            for (int cc = 0; cc < NC; ++cc)
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 float a0, a1;
-                unpack2(add2(pack2(v[cc][i], v[cc][i + 1]), negm), a0, a1);
+                const uint64_t tv = pack2(v[cc][i], v[cc][i + 1]);
+                unpack2(GRID ? fma2(tv, inv22, negm) : add2(tv, negm), a0, a1);
                 acc[(i >> 1) & 3] = add2(acc[(i >> 1) & 3], pack2(fast_exp2(a0), fast_exp2(a1)));
               }
             float s0, s1, s2, s3, s4, s5, s6, s7;
@@ -619,11 +740,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             unpack2(acc[1], s2, s3);
             unpack2(acc[2], s4, s5);
             unpack2(acc[3], s6, s7);
-            s_run = s_run * fast_exp2(m_run - mnew) + (((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)));
+            s_run = s_run * fast_exp2(GRID ? (m_run - mnew) * inv2 : m_run - mnew) +
+                    (((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)));
             m_run = mnew;
           }
         }
       }
+      if constexpr (GRID) m_run *= inv2;
       if (dead) {
         m_run = NAN;
         s_run = NAN;
@@ -651,7 +774,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         continue;
       }
       const float2 mv[1] = {make_float2(m_run, s_run)};
-      segment_epilogue<128>(tp, c, k, sg, sp, ltid, row_local, mv, fcur, sh.s_last, sh.s_fin, sh.red);
+      segment_epilogue<128, GRID>(tp, c, k, sg, sp, ltid, row_local, mv, fcur, sh.s_last, sh.s_fin, sh.red, sh.slots);
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
@@ -674,7 +797,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mv[0] = okw ? sh.seg[sl][etid] : make_float2(NAN, NAN);
       mv[1] = okw ? sh.seg[sl][etid + 64] : make_float2(NAN, NAN);
       mbar_arrive(&sh.seg_empty[sl]);
-      segment_epilogue<64>(tp, c, k, sg, sp, etid, etid, mv, fcur, sh.e_last, sh.e_fin, sh.ered);
+      segment_epilogue<64, GRID>(tp, c, k, sg, sp, etid, etid, mv, fcur, sh.e_last, sh.e_fin, sh.ered, sh.eslots);
     }
   }
 
@@ -697,31 +820,6 @@ __global__ void bias_prep_kernel(const float* __restrict__ potB, const float* __
   write_bias_row(out + j * 16, beta);
 }
 
-// ---------------------------------------------------------------- operand prep
-// One warp per row: hi/lo bf16 split of sqrt(c) (x_i - mu) (mu = 0 when NULL), K padded
-// with zeros to dp (a multiple of 64), and (when norm is not NULL) |x_i - mu|^2 summed in
-// float64 from the float32 differences.
-__global__ void split_bf16_kernel(const float* __restrict__ X, int64_t n, int32_t d, int32_t dp, float scale,
-                                  const float* __restrict__ mu, __nv_bfloat16* __restrict__ hi,
-                                  __nv_bfloat16* __restrict__ lo, float* __restrict__ norm) {
-  const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (r >= n) return;
-  double s = 0.0;
-  for (int k = lane; k < dp; k += 32) {
-    const float u = (k < d) ? X[r * d + k] - (mu ? mu[k] : 0.f) : 0.f;
-    s += (double)u * (double)u;
-    const float v = u * scale;
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    hi[r * dp + k] = h;
-    if (lo) lo[r * dp + k] = __float2bfloat16_rn(v - __bfloat162float(h));
-  }
-  if (norm == nullptr) return;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if (lane == 0) norm[r] = (float)s;
-}
-
 }  // namespace tc
 
 // ---------------------------------------------------------------- host side
@@ -729,13 +827,13 @@ __global__ void split_bf16_kernel(const float* __restrict__ X, int64_t n, int32_
 // block resident in shared memory (two buffers when at least three B stages still fit
 // in 227 KB, else one), or, when no resident A leaves room for two B stages (large d),
 // streamed with B one K block per stage (a_bufs = 0); as many stages (<= 8) as fit.
-static void tc_shape(int bn, int nkb, int split3, int* stages, int* a_bufs) {
+static void tc_shape(int bn, int nkb, int parts, bool grid, int* stages, int* a_bufs) {
   *stages = 0;
   *a_bufs = 1;
   for (int na = 2; na >= 0; --na) {
     int best = 0;
     for (int s = 2; s <= 8; ++s)
-      if (tc::smem_layout(bn, nkb, split3, s, na).total <= 227 * 1024) best = s;
+      if (tc::smem_layout(bn, nkb, parts, s, na, grid).total <= 227 * 1024) best = s;
     if (best >= (na == 2 ? 3 : 2)) {
       *stages = best;
       *a_bufs = na;
@@ -749,27 +847,18 @@ static void tc_shape(int bn, int nkb, int split3, int* stages, int* a_bufs) {
 // streamed (or 128 when even that does not fit).
 int tc_tile_cols(int nkb, int split3) {
   int s, na;
-  tc_shape(256, nkb, split3, &s, &na);
+  tc_shape(256, nkb, 1 + split3, false, &s, &na);
   if (s >= 2 && na > 0) return 256;
-  tc_shape(128, nkb, split3, &s, &na);
+  tc_shape(128, nkb, 1 + split3, false, &s, &na);
   if (s >= 2 && na > 0) return 128;
-  tc_shape(256, nkb, split3, &s, &na);
+  tc_shape(256, nkb, 1 + split3, false, &s, &na);
   return s >= 2 ? 256 : 128;
 }
 
 int tc_stages(int nkb, int split3) {
   int s, na;
-  tc_shape(tc_tile_cols(nkb, split3), nkb, split3, &s, &na);
+  tc_shape(tc_tile_cols(nkb, split3), nkb, 1 + split3, false, &s, &na);
   return s;
-}
-
-cudaError_t launch_split_bf16(const float* X, int64_t n, int32_t d, int32_t dp, float scale, void* hi, void* lo,
-                              cudaStream_t s, const float* mu, float* norm) {
-  if (n <= 0) return cudaSuccess;
-  tc::split_bf16_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(X, n, d, dp, scale, mu, (__nv_bfloat16*)hi,
-                                                                (__nv_bfloat16*)lo, norm);
-  count_launch();
-  return cudaGetLastError();
 }
 
 cudaError_t launch_bias_prep(const float* potB, const float* Bn, int64_t nB, int64_t nB_pad, float bscale, void* out,
@@ -792,12 +881,12 @@ void tc_plan(int64_t nA, int64_t nB, int bn, int sms, int* G, int* maxseg) {
   *maxseg = ms;
 }
 
-template <int BN>
-static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const void* mapAh, const void* mapAl,
-                             const void* mapBh, const void* mapBl, const void* mapBbias, cudaStream_t stream) {
+template <int BN, int GRID>
+static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const TcMaps& m, cudaStream_t stream) {
   static thread_local size_t attr_bytes = 0;  // per host thread, see launch_map_sweep_fp32
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(tc::lse_sweep_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(tc::lse_sweep_tc<BN, GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
@@ -811,23 +900,24 @@ static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const void* ma
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc::lse_sweep_tc<BN>, *reinterpret_cast<const CUtensorMap*>(mapAh),
-                            *reinterpret_cast<const CUtensorMap*>(mapAl), *reinterpret_cast<const CUtensorMap*>(mapBh),
-                            *reinterpret_cast<const CUtensorMap*>(mapBl),
-                            *reinterpret_cast<const CUtensorMap*>(mapBbias), tp);
+  auto at = [](const void* p) -> const CUtensorMap& { return *reinterpret_cast<const CUtensorMap*>(p); };
+  return cudaLaunchKernelEx(&cfg, tc::lse_sweep_tc<BN, GRID>, at(m.a[0]), at(m.a[1]), at(m.a[2]), at(m.b[0]),
+                            at(m.b[1]), at(m.b[2]), at(m.bias), tp);
 }
 
-cudaError_t launch_lse_sweep_tc(const SweepParams& p, const void* mapAh, const void* mapAl, const void* mapBh,
-                                const void* mapBl, const void* mapBbias, int nkb, int split3, int bn, int G,
-                                int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream) {
+cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const float* gscale,
+                                int bn, int G, int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream,
+                                const float* lrow, void* prob, int64_t a_row0) {
+  const bool grid = gscale != nullptr;
   int stages, a_bufs;
-  tc_shape(bn, nkb, split3, &stages, &a_bufs);
-  if (stages < 2 || (bn != 128 && bn != 256)) return cudaErrorInvalidValue;
-  const size_t smem = tc::smem_layout(bn, nkb, split3, stages, a_bufs).total;
+  tc_shape(bn, nkb, parts, grid, &stages, &a_bufs);
+  if (stages < 2 || (bn != 128 && bn != 256) || (grid && (bn != 128 || parts < 2)) || parts < 1 || parts > 3)
+    return cudaErrorInvalidValue;
+  const size_t smem = tc::smem_layout(bn, nkb, parts, stages, a_bufs, grid).total;
   tc::TcParams tp;
   tp.p = p;
   tp.nkb = nkb;
-  tp.split3 = split3;
+  tp.parts = parts;
   tp.stages = stages;
   tp.a_bufs = a_bufs;
   tp.G = G;
@@ -836,8 +926,14 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const void* mapAh, const v
   tp.maxseg = maxseg;
   tp.fault = fault;
   tp.bias_out = (__nv_bfloat16*)bias_out;
-  cudaError_t e = (bn == 256) ? launch_tc<256>(tp, smem, mapAh, mapAl, mapBh, mapBl, mapBbias, stream)
-                              : launch_tc<128>(tp, smem, mapAh, mapAl, mapBh, mapBl, mapBbias, stream);
+  tp.gscale = gscale;
+  tp.lrow = lrow;
+  tp.prob = (unsigned char*)prob;
+  tp.a_row0 = a_row0;
+  if (p.mode == kModeProb && (!grid || prob == nullptr || lrow == nullptr)) return cudaErrorInvalidValue;
+  cudaError_t e = grid        ? launch_tc<128, 1>(tp, smem, maps, stream)
+                  : bn == 256 ? launch_tc<256, 0>(tp, smem, maps, stream)
+                              : launch_tc<128, 0>(tp, smem, maps, stream);
   count_launch();
   return e;
 }

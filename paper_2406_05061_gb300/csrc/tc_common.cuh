@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace progot {
@@ -118,6 +119,20 @@ __device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr) {
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// The same for half-precision operands (f16 x f16 -> fp32).
+__host__ __device__ constexpr uint32_t make_idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+// kind::f16 product with a run-time instruction descriptor.
+__device__ __forceinline__ void umma_id(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 template <int BN>
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   constexpr uint32_t kIdesc = make_idesc(BM, BN);
@@ -145,6 +160,30 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// beta split into three bf16 terms (hi, mid, lo) in the first three of 16 slots
+// (-inf in the first slot for a non-finite beta).
+__device__ __forceinline__ void write_bias_row(__nv_bfloat16* row16, float beta) {
+  __nv_bfloat16 h1, h2, h3;
+  if (isfinite(beta)) {
+    h1 = __float2bfloat16_rn(beta);
+    const float r1 = beta - __bfloat162float(h1);
+    h2 = __float2bfloat16_rn(r1);
+    h3 = __float2bfloat16_rn(r1 - __bfloat162float(h2));
+  } else {
+    h1 = __float2bfloat16_rn(-INFINITY);
+    h2 = __float2bfloat16_rn(0.f);
+    h3 = __float2bfloat16_rn(0.f);
+  }
+  uint4 lo4;
+  lo4.x = (uint32_t)__bfloat16_as_ushort(h1) | ((uint32_t)__bfloat16_as_ushort(h2) << 16);
+  lo4.y = (uint32_t)__bfloat16_as_ushort(h3);
+  lo4.z = 0u;
+  lo4.w = 0u;
+  uint4* dst = reinterpret_cast<uint4*>(row16);
+  dst[0] = lo4;
+  dst[1] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Persistent work split of the (row block, column tile) grid, R x T, over G CTAs.
 // Bands: the first nb G row blocks (nb = floor(R / G)) go whole to one CTA each, row
 // block b G + c to CTA c as its segment b, so that within a band all CTAs walk the
@@ -170,14 +209,20 @@ __host__ __device__ inline Split make_split(int R, int T, int G) {
   s.Gr = (int)(s.W < (int64_t)G ? s.W : (int64_t)G);
   return s;
 }
+// a / b for 0 <= a, 0 < b, in 32 bits where both fit: the kernels' segment ends run a dozen of
+// these on their critical path, and the GPU's 64-bit division is a routine of ~100 instructions.
+__host__ __device__ inline int64_t div_small(int64_t a, int64_t b) {
+  if ((((uint64_t)a | (uint64_t)b) >> 32) == 0) return (int64_t)((uint32_t)a / (uint32_t)b);
+  return a / b;
+}
 __host__ __device__ inline int64_t work_begin(const Split& s, int c) {
-  return c >= s.Gr ? s.W : (int64_t)c * s.W / s.Gr;
+  return c >= s.Gr ? s.W : div_small((int64_t)c * s.W, s.Gr);
 }
 // CTA owning remainder unit w (0 <= w < W): the largest c with floor(c W / Gr) <= w.
-__host__ __device__ inline int cta_of(const Split& s, int64_t w) { return (int)(((w + 1) * s.Gr - 1) / s.W); }
+__host__ __device__ inline int cta_of(const Split& s, int64_t w) { return (int)div_small((w + 1) * s.Gr - 1, s.W); }
 __host__ __device__ inline int num_segments(const Split& s, int c) {
   const int64_t w0 = work_begin(s, c), w1 = work_begin(s, c + 1);
-  return s.nb + (w1 <= w0 ? 0 : (int)((w1 - 1) / s.T - w0 / s.T + 1));
+  return s.nb + (w1 <= w0 ? 0 : (int)(div_small(w1 - 1, s.T) - div_small(w0, s.T) + 1));
 }
 __host__ __device__ inline Seg segment(const Split& s, int c, int k) {
   Seg sg;
@@ -188,7 +233,7 @@ __host__ __device__ inline Seg segment(const Split& s, int c, int k) {
     return sg;
   }
   const int64_t w0 = work_begin(s, c), w1 = work_begin(s, c + 1);
-  const int64_t rr = w0 / s.T + (k - s.nb);
+  const int64_t rr = div_small(w0, s.T) + (k - s.nb);
   const int64_t rb0 = rr * s.T;
   sg.r = s.nb * s.G + (int)rr;
   sg.t0 = (int)((w0 > rb0 ? w0 : rb0) - rb0);
@@ -208,7 +253,7 @@ __host__ __device__ inline void contributors(const Split& s, int r, int* c_first
 }
 __host__ __device__ inline int seg_of(const Split& s, int r, int cc) {
   if (r < s.nb * s.G) return r / s.G;
-  return s.nb + (r - s.nb * s.G) - (int)(work_begin(s, cc) / s.T);
+  return s.nb + (r - s.nb * s.G) - (int)div_small(work_begin(s, cc), s.T);
 }
 
 // Named barriers: 1 = both LSE warpgroups (256 threads), 2 = LSE warpgroup 0 (128).
