@@ -89,6 +89,7 @@ struct Layout {
 
 // A buffers, the ones of the bias product, the bias-row ring, then the stages: B hi and lo
 // of one K block, or with the grid split (three parts) one part of one K block.
+// a_bufs = 0: the A row block is in TMEM.
 __host__ __device__ inline Layout layout(int bn, int nkb, int split3, int stages, int a_bufs, bool grid) {
   Layout L;
   uint32_t off = 0;
@@ -126,6 +127,7 @@ struct Side {
   float c_hi, c_lo, e_hi, e_lo, w_hi, w_lo;
   unsigned long long* cnt;  // [R] arrivals per row block (monotonic over the loop)
   unsigned long long* done; // finished row blocks (monotonic over the loop)
+  const uint4* a_part[2];   // bf16 hi, lo rows of A (nA x 64 nkb), for the A row block in TMEM
   float2* partial;          // [G * maxseg][2][128] (max, sum) per segment slot, LSE warpgroup and row
   // the work split (tables of the operand preparation's launch): CTA c's segments
   // segs[c maxseg + k] = (row block, first tile, end tile), k < nseg[c]; row block r's
@@ -394,7 +396,16 @@ __device__ __forceinline__ Seg seg_at(const Side& Sd, int c, int k, int maxseg) 
 // TMEM columns [0, 256), the rest at [256, 512). GRID = 1..4 is the number of K = 16 steps
 // that hold coordinates (d <= 64), so that a tile's products are issued without a loop
 // (56.7 -> 46 us per sweep at 8192^2, d = 64, where the CUDA-core sweep takes 238).
-template <int BN, int NKB, int GRID>
+// ATM: the bf16 A row block sits in TMEM, hi at columns [256, 256 + 32 nkb), lo after it,
+// written by the LSE warpgroups (one part each) at every segment's start. Taken for 128 < d
+// <= 256, whose resident A left shared memory for two B stages only, fewer than a copy's
+// latency needs; now six fit, and the products read half as much shared memory.
+// CONV: how the MMA warp issues. N = 128 products are shorter than a single divergent lane
+// needs to put the next one's operands in place beside the LSE warps: with the converged
+// warp 16384^2 sweeps took 141 us instead of 164 (grid, d = 64) and 247 instead of 290 (d =
+// 256). N = 256 products are long enough, and a handful of tiles per sweep is paced by the
+// hand-over, where the single lane is faster (512^2: 7.4 against 8.3 us).
+template <int BN, int NKB, int GRID, int ATM, int CONV>
 __global__ void __launch_bounds__(NTHREADS, 1)
     sinkhorn_loop_tc(const __grid_constant__ CUtensorMap mXh_a, const __grid_constant__ CUtensorMap mXl_a,
                      const __grid_constant__ CUtensorMap mYh_a, const __grid_constant__ CUtensorMap mYl_a,
@@ -432,7 +443,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sh.tmem_full[b], 1);
       mbar_init(&sh.tmem_empty[b], 8);  // every LSE warp reads its columns of each tile
-      mbar_init(&sh.a_full[b], 1);
+      mbar_init(&sh.a_full[b], ATM ? 8 : 1);
       mbar_init(&sh.a_empty[b], 1);
     }
     for (int b = 0; b < SEG_RING; ++b) {
@@ -496,6 +507,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int nseg = __ldg(Sd.nseg + c);
         for (int k = 0; k < nseg && ok; ++k, ++ka) {
           const Seg sg = seg_at(Sd, c, k, P.maxseg);
+          if constexpr (!ATM) {
           const int ai = ka % NA;
           ok = warp_wait_bar(&sh.a_empty[ai], (uint32_t)(((ka / NA) & 1) ^ 1), abort_flag, P);
           if (!ok) break;
@@ -512,6 +524,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
           }
           __syncwarp();
+          }
           int seen = 0;  // row blocks below this one are known to be ready
           for (int t = sg.t0; t < sg.t1 && ok; ++t) {
             constexpr int UK = GRID ? kGridParts : 1;  // stage units per K block
@@ -577,10 +590,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    // One thread runs the whole issue loop (a product is issued by a single thread): no
-    // per-wait votes or elections between tiles, whose bookkeeping sits between one
-    // tile's last product and the next tile's first; the other lanes wait at the end.
-    if (lane == 0) {
+    // CONV = 0: one thread runs the whole issue loop (a product is issued by a single thread):
+    // no elections between tiles, whose bookkeeping sits between one tile's last product and
+    // the next tile's first; the other lanes wait at the end. CONV = 1: the whole warp runs
+    // it and elects the issuing lane, which keeps the products' descriptors in uniform
+    // registers.
+    auto wait = [&](uint64_t* bar, uint32_t parity, bool ignore_abort = false) {
+      const bool seen = wait_bar(bar, parity, abort_flag, P, ignore_abort);
+      // the warp leaves together when a wait ran out
+      return CONV ? __all_sync(0xffffffffu, seen) != 0 : seen;
+    };
+    auto issuer = []() { return !CONV || elect_one(); };
+    if (CONV || lane == 0) {
       const uint64_t abias = desc_sw32(smem_u32(smem + L.a_bias));
       const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
       bool ok = true;
@@ -589,7 +610,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       uint32_t s_par = 0;     // the parity of its fill
       for (int it = P.seq0; it < it_end && ok; ++it) {
         if (it > P.seq0) {
-          wait_bar(&sh.dec_full, (uint32_t)((it - 1 - P.seq0) & 1), abort_flag, P, true);
+          wait(&sh.dec_full, (uint32_t)((it - 1 - P.seq0) & 1), true);
           if (sh.dec_stop[(it - 1) & 1] || *abort_flag) break;
         }
         for (int sd = 0; sd < 2 && ok; ++sd) {
@@ -597,15 +618,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const int nseg = __ldg(Sd.nseg + c);
           for (int k = 0; k < nseg && ok; ++k, ++ka) {
             const Seg sg = seg_at(Sd, c, k, P.maxseg);
-            const int ai = ka % NA;
-            ok = wait_bar(&sh.a_full[ai], (uint32_t)((ka / NA) & 1), abort_flag, P);
+            const int ai = ATM ? 0 : ka % NA;
+            ok = wait(&sh.a_full[ai], (uint32_t)((ATM ? ka : ka / NA) & 1));
             if (!ok) break;
             tc_fence_after();
             const uint32_t a_hi = smem_u32(smem + L.a0 + ai * L.a_stride);
             const uint32_t a_lo = a_hi + L.a_lo_off;
             for (int t = sg.t0; t < sg.t1 && ok; ++t, ++tl) {
               const int b = tl & 1;
-              ok = wait_bar(&sh.tmem_empty[b], (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, P);
+              ok = wait(&sh.tmem_empty[b], (uint32_t)(((tl >> 1) & 1) ^ 1));
               if (!ok) break;
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
@@ -617,21 +638,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
                 for (int part = 0; part < kGridParts; ++part) {
                   const int s = s_cur;
-                  ok = wait_bar(&sh.full[s], s_par, abort_flag, P);
+                  ok = wait(&sh.full[s], s_par);
                   if (++s_cur == S) {
                     s_cur = 0;
                     s_par ^= 1u;
                   }
                   if (!ok) break;
                   tc_fence_after();
-                  issue_grid_part<BN, GRID, kGridParts>(
-                      part, d_tmem, d2, ah, al, ar, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)), 0u);
-                  umma_commit(&sh.empty[s]);
+                  if (issuer())
+                    issue_grid_part<BN, GRID, kGridParts>(
+                        part, d_tmem, d2, ah, al, ar, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)), 0u);
+                  if (issuer()) umma_commit(&sh.empty[s]);
                 }
               }
               for (int kb = 0; kb < (GRID ? 0 : nkb); ++kb) {
                 const int s = s_cur;
-                ok = wait_bar(&sh.full[s], s_par, abort_flag, P);
+                ok = wait(&sh.full[s], s_par);
                 if (++s_cur == S) {
                   s_cur = 0;
                   s_par ^= 1u;
@@ -641,37 +663,54 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 const uint32_t st = smem_u32(smem + L.stage0 + s * L.stage_bytes);
                 const uint64_t bh = desc_sw128(st), bl = desc_sw128(st + L.b_lo_off);
                 const uint64_t ah = desc_sw128(a_hi + kb * A_TILE_BYTES), al = desc_sw128(a_lo + kb * A_TILE_BYTES);
+                if (issuer()) {
+                  if constexpr (ATM) {
+                    const uint32_t th = tmem_base + 256 + (uint32_t)(kb * 32), tlo = th + (uint32_t)(nkb * 32);
 #pragma unroll
-                for (int kk = 0; kk < KB / 16; ++kk) {
-                  // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
-                  const uint64_t adv = (uint64_t)(kk * 2);
-                  umma<BN>(d_tmem, ah + adv, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
-                  if (P.split3) {
-                    umma<BN>(d_tmem, ah + adv, bl + adv, 1u);
-                    umma<BN>(d_tmem, al + adv, bh + adv, 1u);
+                    for (int kk = 0; kk < KB / 16; ++kk) {
+                      // K = 16 step: 8 TMEM columns of A, +32 bytes of B
+                      const uint64_t adv = (uint64_t)(kk * 2);
+                      umma_ta<BN>(d_tmem, th + kk * 8, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
+                      if (P.split3) {
+                        umma_ta<BN>(d_tmem, th + kk * 8, bl + adv, 1u);
+                        umma_ta<BN>(d_tmem, tlo + kk * 8, bh + adv, 1u);
+                      }
+                    }
+                  } else
+#pragma unroll
+                  for (int kk = 0; kk < KB / 16; ++kk) {
+                    // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
+                    const uint64_t adv = (uint64_t)(kk * 2);
+                    umma<BN>(d_tmem, ah + adv, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
+                    if (P.split3) {
+                      umma<BN>(d_tmem, ah + adv, bl + adv, 1u);
+                      umma<BN>(d_tmem, al + adv, bh + adv, 1u);
+                    }
                   }
                 }
-                umma_commit(&sh.empty[s]);
+                if (issuer()) umma_commit(&sh.empty[s]);
               }
               if (!ok) break;
               // bias: t_ij = c (a_i . b_j) + beta_j, once the producer has the row blocks' bias rows
               const int bs = tl % BIAS_SLOTS;  // one bias slot per tile, in tile order
-              ok = wait_bar(&sh.bias_full[bs], (uint32_t)((tl / BIAS_SLOTS) & 1), abort_flag, P);
+              ok = wait(&sh.bias_full[bs], (uint32_t)((tl / BIAS_SLOTS) & 1));
               if (!ok) break;
               tc_fence_after();
-              umma<BN>(d_tmem, abias, desc_sw32(smem_u32(smem + L.bias0 + bs * L.bias_slot)), 1u);
-              if constexpr (GRID)
-                umma<BN>(d_tmem + 256, abias2, desc_sw32(smem_u32(smem + L.bias0 + bs * L.bias_slot)), 1u);
-              umma_commit(&sh.bias_empty[bs]);
-              umma_commit(&sh.tmem_full[b]);
+              if (issuer()) {
+                const uint64_t brows = desc_sw32(smem_u32(smem + L.bias0 + bs * L.bias_slot));
+                umma<BN>(d_tmem, abias, brows, 1u);
+                if constexpr (GRID) umma<BN>(d_tmem + 256, abias2, brows, 1u);
+                umma_commit(&sh.bias_empty[bs]);
+                umma_commit(&sh.tmem_full[b]);
+              }
             }
             if (!ok) break;
-            umma_commit(&sh.a_empty[ai]);
+            if (issuer()) umma_commit(&sh.a_empty[ai]);
           }
         }
       }
-      umma_commit(&sh.drain);
-      wait_bar(&sh.drain, 0, abort_flag, P, true);
+      if (issuer()) umma_commit(&sh.drain);
+      wait(&sh.drain, 0, true);
     }
     __syncwarp();
   } else if (threadIdx.x < EPI_TID0) {
@@ -696,6 +735,21 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int nseg = __ldg(Sd.nseg + c);
         for (int k = 0; k < nseg; ++k, ++kseg) {
           const Seg sg = seg_at(Sd, c, k, P.maxseg);
+          if constexpr (ATM) {
+            // A's part wg of this segment's rows into TMEM once the previous segment's
+            // products have read theirs (with hi parts only warpgroup 1 just arrives)
+            if (!dead && !warp_wait_bar(&sh.a_empty[0], (uint32_t)((kseg & 1) ^ 1), abort_flag, P)) dead = true;
+            if (!dead) {
+              tc_fence_after();
+              const int64_t i = (int64_t)sg.r * BM + row_local;
+              if (wg == 0 || P.split3)
+                tmem_store_row(tmem_base + ((uint32_t)(quarter * 32) << 16) + 256 + (uint32_t)(wg * nkb * 32),
+                               Sd.a_part[wg] + i * (nkb * 8), nkb, i < Sd.nA);
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&sh.a_full[0]);
+            }
+          }
           float m_run = -INFINITY, s_run = 0.f;
           for (int t = sg.t0; t < sg.t1; ++t, ++tl) {
             // both warpgroups take every tile, warpgroup wg its columns wg BN / 2 ..: the
@@ -968,10 +1022,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // ---------------------------------------------------------------- host side
 // Pipeline shape of the persistent loop: two resident A buffers and as many B stages
 // (2..8) as fit in 227 KB; 0 stages when no shape fits (the per-sweep kernel serves it).
+// A in TMEM (a_bufs = 0): 128-column bf16 tiles of three or four K blocks, where hi and lo
+// fill the 256 TMEM columns beside the accumulators (16384^2, d = 256: 292 us per sweep with
+// a resident A and two stages).
+static bool loop_a_in_tmem(int bn, int nkb, bool grid) { return !grid && bn == 128 && nkb <= 4; }
+
 static void loop_shape(int bn, int nkb, int split3, bool grid, int* stages, int* a_bufs) {
   *stages = 0;
   *a_bufs = 2;
-  for (int na = 2; na >= 1; --na) {
+  const bool atm = loop_a_in_tmem(bn, nkb, grid);
+  for (int na = atm ? 0 : 2; na >= (atm ? 0 : 1); --na) {
     int best = 0;
     for (int s = 2; s <= 8; ++s)
       if (tc::loop::layout(bn, nkb, split3, s, na, grid).total <= 227 * 1024) best = s;
@@ -1004,11 +1064,11 @@ void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg) {
   *maxseg = ms;
 }
 
-template <int BN, int NKB, int GRID>
+template <int BN, int NKB, int GRID, int ATM = 0, int CONV = 0>
 static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const void* const* maps, cudaStream_t stream) {
   static thread_local size_t attr_bytes = 0;
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB, GRID>,
+    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
@@ -1025,7 +1085,7 @@ static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const voi
   cfg.numAttrs = 1;
   const CUtensorMap* m[16];
   for (int q = 0; q < 16; ++q) m[q] = reinterpret_cast<const CUtensorMap*>(maps[q]);
-  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB, GRID>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
+  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
                             *m[6], *m[7], *m[8], *m[9], *m[10], *m[11], *m[12], *m[13], *m[14], *m[15], P);
 }
 
@@ -1049,6 +1109,8 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
     d.cnt = s.cnt;
     d.done = s.done;
     d.partial = s.partial;
+    d.a_part[0] = reinterpret_cast<const uint4*>(s.a_part[0]);
+    d.a_part[1] = reinterpret_cast<const uint4*>(s.a_part[1]);
     d.nA = s.p.nA;
     d.nB = s.p.nB;
     d.R = (int)((s.p.nA + tc::BM - 1) / tc::BM);
@@ -1081,16 +1143,23 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   P.gscale = Lq.gscale;
   const size_t smem = tc::loop::layout(Lq.bn, Lq.nkb, Lq.split3, stages, a_bufs, grid).total;
   const int ks = (Lq.side[0].p.d + 15) / 16;  // K = 16 steps
+  const bool many = (int64_t)P.side[0].R * P.side[0].T >= 4 * (int64_t)Lq.G;  // tiles per CTA and sweep
   cudaError_t e;
-  if (grid)
+  if (grid && many)
+    e = ks <= 1   ? launch_loop<128, 1, 1, 0, 1>(P, smem, Lq.maps, stream)
+        : ks == 2 ? launch_loop<128, 1, 2, 0, 1>(P, smem, Lq.maps, stream)
+        : ks == 3 ? launch_loop<128, 1, 3, 0, 1>(P, smem, Lq.maps, stream)
+                  : launch_loop<128, 1, 4, 0, 1>(P, smem, Lq.maps, stream);
+  else if (grid)
     e = ks <= 1   ? launch_loop<128, 1, 1>(P, smem, Lq.maps, stream)
         : ks == 2 ? launch_loop<128, 1, 2>(P, smem, Lq.maps, stream)
         : ks == 3 ? launch_loop<128, 1, 3>(P, smem, Lq.maps, stream)
                   : launch_loop<128, 1, 4>(P, smem, Lq.maps, stream);
   else
-    e = Lq.bn == 128   ? launch_loop<128, 0, 0>(P, smem, Lq.maps, stream)
-        : Lq.nkb == 1 ? launch_loop<256, 1, 0>(P, smem, Lq.maps, stream)
-                      : launch_loop<256, 0, 0>(P, smem, Lq.maps, stream);
+    e = a_bufs == 0    ? launch_loop<128, 0, 0, 1, 1>(P, smem, Lq.maps, stream)
+        : Lq.bn == 128 ? launch_loop<128, 0, 0>(P, smem, Lq.maps, stream)
+        : Lq.nkb == 1  ? launch_loop<256, 1, 0>(P, smem, Lq.maps, stream)
+                       : launch_loop<256, 0, 0>(P, smem, Lq.maps, stream);
   count_launch();
   return e;
 }

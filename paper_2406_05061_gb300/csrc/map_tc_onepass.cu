@@ -162,17 +162,6 @@ __device__ __forceinline__ void op_umma_ta(uint32_t d_tmem, uint32_t a_tmem, uin
       "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// 32 lanes x 32 columns of 32 bits from registers (one row per thread).
-__device__ __forceinline__ void op_tmem_st32(uint32_t taddr, const uint32_t* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
-      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
-      "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
-      "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
-      : "memory");
-}
 __device__ __forceinline__ uint32_t op_bf2_bits(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 __device__ __forceinline__ void op_split8(const float* v, uint4& hi, uint4& lo) {
   uint32_t h[4], l[4];
@@ -435,20 +424,8 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
           dead = true;
         } else {
           tc_fence_after();
-          const uint4* src = reinterpret_cast<const uint4*>(mp.xh + i * (int64_t)(nkb * 32));
-          for (int kb = 0; kb < nkb; ++kb) {
-            uint32_t w[32];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const uint4 u4 = row_ok ? __ldg(src + kb * 8 + e) : make_uint4(0u, 0u, 0u, 0u);
-              w[4 * e] = u4.x;
-              w[4 * e + 1] = u4.y;
-              w[4 * e + 2] = u4.z;
-              w[4 * e + 3] = u4.w;
-            }
-            op_tmem_st32(tmem_base + ((uint32_t)(quarter * 32) << 16) + OP_X_COL + (uint32_t)(kb * 32), w);
-          }
-          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          tmem_store_row(tmem_base + ((uint32_t)(quarter * 32) << 16) + OP_X_COL,
+                         reinterpret_cast<const uint4*>(mp.xh + i * (int64_t)(nkb * 32)), nkb, row_ok);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&sh.x_full);

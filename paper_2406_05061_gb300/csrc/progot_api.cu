@@ -696,6 +696,9 @@ static int lse_sweep(const SweepParams& p, cudaStream_t s, const TcOps* ops = nu
     maps.b[1] = a_is_x ? &ops->yl_b : &ops->xl_b;
     maps.b[2] = ops->gscale ? (a_is_x ? &ops->yr_b : &ops->xr_b) : maps.b[1];
     maps.bias = a_is_x ? &ops->yb : &ops->xb;
+    const bool bf16 = ops->gscale == nullptr && ws != nullptr;
+    maps.a_part[0] = !bf16 ? nullptr : a_is_x ? ws->xh : ws->yh;
+    maps.a_part[1] = !bf16 ? nullptr : ops->parts < 2 ? maps.a_part[0] : a_is_x ? ws->xl : ws->yl;
     void* bias_out = (p.mode == kModePotential && ws) ? (a_is_x ? ws->xb : ws->yb) : nullptr;
     int G = 0, maxseg = 0;
     tc_plan(p.nA, p.nB, ops->bn, num_sms(), &G, &maxseg);
@@ -748,6 +751,8 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   F.cnt = ws.lcnt;
   F.done = ws.lcnt + 2 * rb;
   F.partial = ws.lpart;
+  F.a_part[0] = ws.xh;
+  F.a_part[1] = ops.parts > 1 ? ws.xl : ws.xh;
   F.segs = ws.ltab_segs;
   F.cslot = ws.ltab_cslot;
   F.crow = ws.ltab_crow;
@@ -762,6 +767,8 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   Gs.cnt = ws.lcnt + rb;
   Gs.done = ws.lcnt + 2 * rb + 1;
   Gs.partial = ws.lpart + ws.lslots * 2 * 128;
+  Gs.a_part[0] = ws.yh;
+  Gs.a_part[1] = ops.parts > 1 ? ws.yl : ws.yh;
   Gs.segs = ws.ltab_segs + ws.lslots;
   Gs.cslot = ws.ltab_cslot + ws.lslots;
   Gs.crow = ws.ltab_crow + rb;
@@ -1050,7 +1057,7 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
     SweepParams p = make_sweep(X, rows, X, m, d, nullptr, nullptr, eps, ws, 1);
     p.mode = kModeProb;
     p.out = ws.rsum + row0;
-    TcMaps maps = {{&ops.xh_a, &ops.xl_a, &ops.xr_a}, {&ops.yh_b, &ops.yl_b, &ops.yr_b}, &ops.yb};
+    TcMaps maps = {{&ops.xh_a, &ops.xl_a, &ops.xr_a}, {&ops.yh_b, &ops.yl_b, &ops.yr_b}, &ops.yb, {nullptr, nullptr}};
     int G = 0, maxseg = 0;
     tc_plan(rows, m, ops.bn, num_sms(), &G, &maxseg);
     CK(launch_lse_sweep_tc(p, maps, ops.nkb, ops.parts, ops.gscale, ops.bn, G, maxseg, ws.fault, nullptr, s,

@@ -76,6 +76,7 @@ struct TcMaps {
   const void* a[3];   // operand maps of the rows' side (128-row boxes): hi, lo, (grid split) third part
   const void* b[3];   // of the columns' side (bn-row boxes)
   const void* bias;   // bias rows of the columns' side (bn-row boxes)
+  const void* a_part[2];  // the rows' side bf16 hi, lo operand rows (NULL: grid operands)
 };
 // parts: operand parts in use (1 bf16, 2 bf16x3); gscale non-NULL: the integer-grid split
 // (grid_split.cuh; parts 2 or 3, bn = 128) with its device scales.
@@ -196,6 +197,7 @@ struct LoopSideLaunch {
   unsigned long long* cnt;   // [row blocks] arrival counters, zero at the loop's start
   unsigned long long* done;  // finished row blocks, zero at the loop's start
   float2* partial;           // (max, sum) slots of this side's sweeps
+  const void* a_part[2];     // operand rows of this side, hi and lo (read where A sits in TMEM)
   // the work split's tables (LoopSetupSide)
   const void* segs;
   const int32_t* nseg;

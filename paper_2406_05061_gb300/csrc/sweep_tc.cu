@@ -92,6 +92,7 @@ struct TcParams {
   const float* gscale;      // grid split: {2^(ex + ey), 2^-(ex + ey)} (device)
   // kModeProb: row L (log2 units) of this launch's rows, which start at operand row a_row0,
   // and the P tiles (see pv_tc.cu): [row block][64-column unit][hi, lo][128 rows x 64]
+  const uint4* a_part[2];   // A in TMEM: bf16 hi, lo rows of A (nA x 64 nkb)
   const float* lrow;
   unsigned char* prob;
   int64_t a_row0;
@@ -103,7 +104,8 @@ struct SmemLayout {
 
 // Offsets of an operand's part q: q * a_lo_off in a resident A buffer, q * b_lo_off in a
 // stage, q * A_TILE_BYTES in a stage's streamed A block. The grid split has two ones tiles.
-__host__ __device__ inline SmemLayout smem_layout(int bn, int nkb, int parts, int stages, int a_bufs, bool grid) {
+__host__ __device__ inline SmemLayout smem_layout(int bn, int nkb, int parts, int stages, int a_bufs, bool grid,
+                                                   bool atm = false) {
   SmemLayout L;
   const uint32_t b_tile = (uint32_t)bn * KB * 2, bias_tile = (uint32_t)bn * 32;
   uint32_t off = 0;
@@ -118,7 +120,7 @@ __host__ __device__ inline SmemLayout smem_layout(int bn, int nkb, int parts, in
   L.bias_off = b_tile * parts;
   // streamed A (a_bufs = 0): the A K block (its parts in order) follows the bias rows in the stage
   L.a_stage_off = L.bias_off + bias_tile;
-  L.stage_bytes = L.a_stage_off + (a_bufs == 0 ? A_TILE_BYTES * (uint32_t)parts : 0u);
+  L.stage_bytes = L.a_stage_off + (a_bufs == 0 && !atm ? A_TILE_BYTES * (uint32_t)parts : 0u);
   off += stages * L.stage_bytes;
   L.ctrl = off;
   off += sizeof(TcShared);
@@ -334,7 +336,9 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
 // GRID = 0: bf16 operands, one accumulator (two buffers of BN columns). GRID = 1: the
 // integer-grid split (grid_split.cuh), BN = 128, two accumulators per tile (leading
 // products at TMEM columns [0, 256), the others at [256, 512)).
-template <int BN, int GRID>
+// ATM: the bf16 A row block sits in TMEM (hi at columns [256, 256 + 32 nkb), lo after it),
+// as in the persistent loop: 128 < d <= 256.
+template <int BN, int GRID, int ATM>
 __global__ void __launch_bounds__(NTHREADS, 1)
     lse_sweep_tc(const __grid_constant__ CUtensorMap mapAh, const __grid_constant__ CUtensorMap mapAl,
                  const __grid_constant__ CUtensorMap mapAr, const __grid_constant__ CUtensorMap mapBh,
@@ -347,7 +351,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const SmemLayout L = smem_layout(BN, tp.nkb, tp.parts, tp.stages, tp.a_bufs, GRID != 0);
+  const SmemLayout L = smem_layout(BN, tp.nkb, tp.parts, tp.stages, tp.a_bufs, GRID != 0, ATM != 0);
   const int parts = tp.parts;
   constexpr uint32_t B_TILE_BYTES = (uint32_t)BN * KB * 2, BIAS_TILE_BYTES = (uint32_t)BN * 32;
   TcShared& sh = *reinterpret_cast<TcShared*>(smem + L.ctrl);
@@ -368,7 +372,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sh.tmem_full[b], 1);
       mbar_init(&sh.tmem_empty[b], 4);
-      mbar_init(&sh.a_full[b], 1);
+      mbar_init(&sh.a_full[b], ATM ? 8 : 1);
       mbar_init(&sh.a_empty[b], 1);
     }
     mbar_init(&sh.drain, 1);
@@ -413,7 +417,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const uint32_t abytes = (uint32_t)L.a_stride;
     const uint32_t bbytes = B_TILE_BYTES * (uint32_t)parts;
     // streamed A: each stage also carries the A K block (hi and lo) of its tile
-    const uint32_t sabytes = NA == 0 ? A_TILE_BYTES * (uint32_t)parts : 0u;
+    const uint32_t sabytes = !ATM && NA == 0 ? A_TILE_BYTES * (uint32_t)parts : 0u;
     int a_issued = 0;
     bool waited = false, stopped = false;
     int pend_s[8], pend_t[8], npend = 0;  // stages whose bias rows wait for the previous sweep
@@ -484,7 +488,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (parts > 1) tma_load_2d(st + L.b_lo_off, &mapBl, &sh.full[s], kb * KB, t * BN);
             if (GRID && parts > 2) tma_load_2d(st + 2 * L.b_lo_off, &mapBr, &sh.full[s], kb * KB, t * BN);
             if (bias_now) tma_load_2d(st + L.bias_off, &mapBbias, &sh.full[s], 0, t * BN);
-            if (NA == 0) {
+            if (!ATM && NA == 0) {
               tma_load_2d(st + L.a_stage_off, &mapAh, &sh.full[s], kb * KB, a_row);
               if (parts > 1) tma_load_2d(st + L.a_stage_off + A_TILE_BYTES, &mapAl, &sh.full[s], kb * KB, a_row);
               if (GRID && parts > 2)
@@ -518,8 +522,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int k = 0; k < nseg && ok; ++k) {
       const Seg sg = segment(sp, c, k);
       const int ai = NA > 0 ? k % NA : 0;
-      if (NA > 0) {
-        ok = warp_wait(&sh.a_full[ai], (uint32_t)((k / NA) & 1), abort_flag);
+      if (ATM || NA > 0) {
+        ok = warp_wait(&sh.a_full[ai], (uint32_t)((ATM ? k : k / NA) & 1), abort_flag);
         if (!ok) break;
         tc_fence_after();
       }
@@ -558,6 +562,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               } else {
                 issue_grid_part<BN, 2>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
                 issue_grid_part<BN, 2>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
+              }
+            }
+          } else if constexpr (ATM) {
+            const uint32_t th = tmem_base + 256 + (uint32_t)(kb * 32), tlo = th + (uint32_t)(nkb * 32);
+            if (elect_one()) {
+#pragma unroll
+              for (int kk = 0; kk < KB / 16; ++kk) {
+                // K = 16 step: 8 TMEM columns of A, +32 bytes of B
+                const uint64_t adv = (uint64_t)(kk * 2);
+                umma_ta<BN>(d_tmem, th + kk * 8, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
+                if (parts > 1) {
+                  umma_ta<BN>(d_tmem, th + kk * 8, bl + adv, 1u);
+                  umma_ta<BN>(d_tmem, tlo + kk * 8, bh + adv, 1u);
+                }
               }
             }
           } else if (elect_one()) {
@@ -599,7 +617,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         __syncwarp();
       }
       if (!ok) break;
-      if (NA > 0 && elect_one()) umma_commit(&sh.a_empty[ai]);
+      if ((ATM || NA > 0) && elect_one()) umma_commit(&sh.a_empty[ai]);
       __syncwarp();
     }
     // make sure no MMA is still writing TMEM when the CTA moves on
@@ -629,8 +647,26 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // A warp whose bounded wait failed turns "dead": it skips tile work but keeps
     // executing every named barrier below, so the other LSE warps never block on it.
     bool dead = false;
+    // a stopped sweep's MMA warp passes the A barrier (its products go nowhere) to the bias
+    // barriers, where it sees the stop
+    if (ATM && stopped && lane == 0) mbar_arrive(&sh.a_full[0]);
     for (int k = 0; k < (stopped ? 0 : nseg); ++k) {
       const Seg sg = segment(sp, c, k);
+      if constexpr (ATM) {
+        // A's part wg of this segment's rows into TMEM once the previous segment's products
+        // have read theirs (with hi parts only warpgroup 1 just arrives)
+        if (!dead && !warp_wait(&sh.a_empty[0], (uint32_t)((k & 1) ^ 1), abort_flag)) dead = true;
+        if (!dead) {
+          tc_fence_after();
+          const int64_t i = (int64_t)sg.r * BM + row_local;
+          if (wg == 0 || parts > 1)
+            tmem_store_row(tmem_base + ((uint32_t)(quarter * 32) << 16) + 256 + (uint32_t)(wg * nkb * 32),
+                           tp.a_part[wg] + i * (nkb * 8), nkb, i < p.nA);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.a_full[0]);
+        }
+      }
       float m_run = prob ? 0.f : -INFINITY, s_run = 0.f;
       const bool row_ok = (int64_t)sg.r * BM + row_local < p.nA;
       const float Lr = (prob && row_ok) ? __ldg(tp.lrow + (int64_t)sg.r * BM + row_local) : 0.f;
@@ -855,6 +891,13 @@ int tc_tile_cols(int nkb, int split3) {
   return s >= 2 ? 256 : 128;
 }
 
+static int tc_stages_atm(int nkb, int parts) {
+  int best = 0;
+  for (int s = 2; s <= 8; ++s)
+    if (tc::smem_layout(128, nkb, parts, s, 0, false, true).total <= 227 * 1024) best = s;
+  return best;
+}
+
 int tc_stages(int nkb, int split3) {
   int s, na;
   tc_shape(tc_tile_cols(nkb, split3), nkb, 1 + split3, false, &s, &na);
@@ -881,12 +924,12 @@ void tc_plan(int64_t nA, int64_t nB, int bn, int sms, int* G, int* maxseg) {
   *maxseg = ms;
 }
 
-template <int BN, int GRID>
+template <int BN, int GRID, int ATM = 0>
 static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const TcMaps& m, cudaStream_t stream) {
   static thread_local size_t attr_bytes = 0;  // per host thread, see launch_map_sweep_fp32
   if (smem > attr_bytes) {
     cudaError_t e =
-        cudaFuncSetAttribute(tc::lse_sweep_tc<BN, GRID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(tc::lse_sweep_tc<BN, GRID, ATM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
@@ -901,7 +944,7 @@ static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const TcMaps& 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   auto at = [](const void* p) -> const CUtensorMap& { return *reinterpret_cast<const CUtensorMap*>(p); };
-  return cudaLaunchKernelEx(&cfg, tc::lse_sweep_tc<BN, GRID>, at(m.a[0]), at(m.a[1]), at(m.a[2]), at(m.b[0]),
+  return cudaLaunchKernelEx(&cfg, tc::lse_sweep_tc<BN, GRID, ATM>, at(m.a[0]), at(m.a[1]), at(m.a[2]), at(m.b[0]),
                             at(m.b[1]), at(m.b[2]), at(m.bias), tp);
 }
 
@@ -911,9 +954,15 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
   const bool grid = gscale != nullptr;
   int stages, a_bufs;
   tc_shape(bn, nkb, parts, grid, &stages, &a_bufs);
+  // 128-column bf16 tiles of up to four K blocks: A in TMEM, all of shared memory for stages
+  const bool atm = !grid && bn == 128 && nkb <= 4 && maps.a_part[0] != nullptr;
+  if (atm) {
+    a_bufs = 0;
+    stages = tc_stages_atm(nkb, parts);
+  }
   if (stages < 2 || (bn != 128 && bn != 256) || (grid && (bn != 128 || parts < 2)) || parts < 1 || parts > 3)
     return cudaErrorInvalidValue;
-  const size_t smem = tc::smem_layout(bn, nkb, parts, stages, a_bufs, grid).total;
+  const size_t smem = tc::smem_layout(bn, nkb, parts, stages, a_bufs, grid, atm).total;
   tc::TcParams tp;
   tp.p = p;
   tp.nkb = nkb;
@@ -931,7 +980,10 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
   tp.prob = (unsigned char*)prob;
   tp.a_row0 = a_row0;
   if (p.mode == kModeProb && (!grid || prob == nullptr || lrow == nullptr)) return cudaErrorInvalidValue;
+  tp.a_part[0] = reinterpret_cast<const uint4*>(maps.a_part[0]);
+  tp.a_part[1] = reinterpret_cast<const uint4*>(maps.a_part[1]);
   cudaError_t e = grid        ? launch_tc<128, 1>(tp, smem, maps, stream)
+                  : atm       ? launch_tc<128, 0, 1>(tp, smem, maps, stream)
                   : bn == 256 ? launch_tc<256, 0>(tp, smem, maps, stream)
                               : launch_tc<128, 0>(tp, smem, maps, stream);
   count_launch();

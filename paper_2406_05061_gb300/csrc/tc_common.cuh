@@ -143,6 +143,17 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t b
       "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
       : "memory");
 }
+// The same with A read from TMEM (K-major: lane = row, two 16-bit elements per column).
+template <int BN>
+__device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t accumulate) {
+  constexpr uint32_t kIdesc = make_idesc(BM, BN);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(kIdesc), "r"(accumulate)
+      : "memory");
+}
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
@@ -157,6 +168,35 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
         "=f"(v[17]), "=f"(v[18]), "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]),     \
         "=f"(v[25]), "=f"(v[26]), "=f"(v[27]), "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])                   \
       : "r"(taddr))
+
+// 32 lanes x 32 columns of 32 bits from registers (one row per thread).
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+      "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]),
+      "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
+      "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+      : "memory");
+}
+// One row of a 16-bit operand (nkb blocks of 64) into TMEM at taddr, called by the 32 threads
+// of a warp for the rows of its lane quarter (zeros where !row_ok).
+__device__ __forceinline__ void tmem_store_row(uint32_t taddr, const uint4* __restrict__ src, int nkb, bool row_ok) {
+  for (int kb = 0; kb < nkb; ++kb) {
+    uint32_t w[32];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint4 u4 = row_ok ? __ldg(src + kb * 8 + e) : make_uint4(0u, 0u, 0u, 0u);
+      w[4 * e] = u4.x;
+      w[4 * e + 1] = u4.y;
+      w[4 * e + 2] = u4.z;
+      w[4 * e + 3] = u4.w;
+    }
+    tmem_st32(taddr + (uint32_t)(kb * 32), w);
+  }
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
