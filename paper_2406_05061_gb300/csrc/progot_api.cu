@@ -148,6 +148,20 @@ static int plan_splits(int64_t nA, int64_t nB, int ctas_per_sm, int extra_mult =
   return (int)cdiv(ct, tps);
 }
 
+// Float32 Sinkhorn loops use the integer-grid operands up to this dimension. The CUDA-core
+// sweeps round eps' products against unequal norms and so shift mass between f and g by a
+// little every iteration (the plan is unaffected); on wide normalised clouds, where g is
+// small, tens of iterations move it by 1e-5 of its size (1.3e-5 measured at 839 x 726,
+// d = 126, 17 iterations). The grid loops do not drift, and results callers already hold for
+// such clouds would change by as much, so these loops stay on CUDA cores.
+constexpr int32_t kGridSolveDim = 64;
+// Least rows x columns x coordinates of a float32 map step on the tensor cores.
+constexpr double kGridMapWork = 2.5e7;
+// P of a chunk of rows stays in L2 between the sweep that writes it and the product that
+// reads it; a p-norm cost up to about the size of L2 is kept for its loop.
+constexpr int64_t kProbChunk = (int64_t)64 << 20;
+constexpr int64_t kCostBytes = (int64_t)128 << 20;
+
 // Device workspace carved from the caller's buffer.
 struct Workspace {
   float* xn;        // nmax
@@ -307,13 +321,12 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   ws.lerr = (double*)take(w.tc ? sizeof(double) * 2 * (size_t)w.rbmax : 0);
   ws.xr = take(w.grid ? opb : 0);
   ws.yr = take(w.grid ? opb : 0);
-  // Map steps on integer-grid operands keep P for a chunk of row blocks: 64 MB stay in L2
-  // between the sweep that writes them and the product that reads them (one row block at
-  // least; less when all of P is smaller). The bf16x3 path needs them for d > 256, where
+  // Map steps on integer-grid operands keep P for a chunk of row blocks (kProbChunk; one row
+  // block at least, less when all of P is smaller); p-norm loops their cost (kCostBytes). The bf16x3 path needs them for d > 256, where
   // the partial buffers of the CUDA-core map are idle and larger than one row block's P.
   if (w.grid) {
     const int64_t block = pv_prob_bytes_per_block(w.nmax);
-    ws.prob_bytes = std::max<int64_t>(block, std::min<int64_t>(block * w.rbmax, (int64_t)64 << 20));
+    ws.prob_bytes = std::max<int64_t>(block, std::min<int64_t>(block * w.rbmax, kCostBytes));
     ws.prob = take((size_t)ws.prob_bytes);
     ws.rsum = ws.Rpart;
   } else {
@@ -326,16 +339,6 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   if (out) *out = ws;
   return off;
 }
-
-// Float32 Sinkhorn loops use the integer-grid operands up to this dimension. The CUDA-core
-// sweeps round eps' products against unequal norms and so shift mass between f and g by a
-// little every iteration (the plan is unaffected); on wide normalised clouds, where g is
-// small, tens of iterations move it by 1e-5 of its size (1.3e-5 measured at 839 x 726,
-// d = 126, 17 iterations). The grid loops do not drift, and results callers already hold for
-// such clouds would change by as much, so these loops stay on CUDA cores.
-constexpr int32_t kGridSolveDim = 64;
-// Least rows x columns x coordinates of a float32 map step on the tensor cores.
-constexpr double kGridMapWork = 2.5e7;
 
 static int carve(int64_t n, int64_t m, int32_t d, void* workspace, size_t ws_bytes, Workspace* ws,
                  int32_t precision = PROGOT_FP32) {
@@ -659,6 +662,8 @@ static SweepParams make_sweep(const float* A, int64_t nA, const float* B, int64_
 struct Cost {
   int32_t kind = kCostSqEuclid;
   float p = 2.f;
+  const float* C = nullptr;  // stored cost sums of the current clouds (keep_cost)
+  int64_t ldc = 0;
   bool pnorm() const { return kind != kCostSqEuclid; }
 };
 
@@ -676,9 +681,24 @@ static void apply_cost(SweepParams& sp, const Cost& c, double eps) {
   if (!c.pnorm()) return;
   sp.cost = c.kind;
   sp.cost_p = c.p;
+  sp.C = c.C;
+  sp.ldc = c.ldc;
   sp.scale = (float)(-kLog2e / (eps * (double)c.p));
   sp.An = nullptr;
   sp.Bn = nullptr;
+}
+
+// Form the p-norm cost of (x, y) in the workspace for the sweeps and map step that follow,
+// where it fits (n rows of whole 128-column tiles); otherwise they form it tile by tile.
+static int keep_cost(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const Workspace& ws, Cost* c,
+                     cudaStream_t s) {
+  const int64_t ld = cdiv(m, 128) * 128;
+  c->C = nullptr;
+  if (!c->pnorm() || !ws.grid || n > ws.prob_bytes / (int64_t)sizeof(float) / ld) return PROGOT_OK;
+  CK(launch_pnorm_cost(x, n, y, m, d, c->kind, c->p, (float*)ws.prob, ld, s));
+  c->C = (const float*)ws.prob;
+  c->ldc = ld;
+  return PROGOT_OK;
 }
 
 // Launch one log-sum-exp sweep: float32 CUDA cores, or tcgen05 on the prepared split
@@ -904,6 +924,7 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
   pg.tau = tau;
   pg.max_iter = max_iter;
   apply_cost(pg, cost, eps);
+  pg.c_cols = 1;
   // tensor-core loops run the stop test of an f-update in the g-update that follows it
   // (SweepParams::lag): the f-update's last row block then ends the sweep without a
   // sweep-level arrival and finish
@@ -1047,8 +1068,9 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
     if (rc) return rc;
   }
   const int64_t blocks = cdiv(n, 128);
-  int64_t cb = std::min<int64_t>(blocks, ws.prob_bytes / pv_prob_bytes_per_block(m));
-  if (cb < 1) return fail(PROGOT_ERR_WORKSPACE, "no room for one row block of P");
+  const int64_t room = std::max<int64_t>(std::min<int64_t>(ws.prob_bytes, kProbChunk), pv_prob_bytes_per_block(m));
+  int64_t cb = std::min<int64_t>(blocks, room / pv_prob_bytes_per_block(m));
+  if (cb < 1 || pv_prob_bytes_per_block(m) > ws.prob_bytes) return fail(PROGOT_ERR_WORKSPACE, "no room for one row block of P");
   cb = cdiv(blocks, cdiv(blocks, cb));  // equal chunks
   ProfRec r;
   const bool rec = prof_begin(r, s, kProfMap);
@@ -1170,6 +1192,8 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
   if (cost.pnorm()) {
     mp.cost = cost.kind;
     mp.cost_p = cost.p;
+    mp.C = cost.C;
+    mp.ldc = cost.ldc;
     mp.scale = (float)(-kLog2e / (eps * (double)cost.p));
   }
   ProfRec r;
@@ -1283,7 +1307,7 @@ static int solve_impl(const float* x, const float* a, int64_t n, const float* y,
   Workspace ws;
   int rc = carve(n, m, d, workspace, ws_bytes, &ws, precision);
   if (rc) return rc;
-  if (d > kGridSolveDim) ws.grid = false;
+  if (!cost.pnorm() && d > kGridSolveDim) ws.grid = false;
   rc = zero_counters(ws, s);
   if (rc) return rc;
   if (x_out != x) CK(cudaMemcpyAsync(x_out, x, sizeof(float) * n * d, cudaMemcpyDeviceToDevice, s));
@@ -1315,8 +1339,11 @@ static int solve_impl(const float* x, const float* a, int64_t n, const float* y,
     int32_t it = 0;
     double err = 0.0;
     TcOps ops;
+    Cost step = cost;  // of this step's x cloud
+    rc = keep_cost(x_out, n, y, m, d, ws, &step, s);
+    if (rc) return rc;
     rc = sinkhorn_core(x_out, a, n, y, b, m, d, eps_k, tau[k], max_iter, precision, ws.f0, ws.f1, gk, ws.xn, ws.yn,
-                       ws, &it, &err, s, &ops, false, cost, k ? Operands::kMoved : Operands::kAuto);
+                       ws, &it, &err, s, &ops, false, step, k ? Operands::kMoved : Operands::kAuto);
     if (iters) iters[k] = it;
     if (errs) errs[k] = err;
     if (rc == PROGOT_ERR_NOT_CONVERGED) {
@@ -1327,7 +1354,7 @@ static int solve_impl(const float* x, const float* a, int64_t n, const float* y,
     } else if (rc) {
       return rc;
     }
-    rc = map_step(x_out, n, y, m, d, gk, ws.yn, eps_k, alpha[k], precision, ws, s, &ops, cost);
+    rc = map_step(x_out, n, y, m, d, gk, ws.yn, eps_k, alpha[k], precision, ws, s, &ops, step);
     if (rc) return rc;
   }
   if (f_last) CK(cudaMemcpyAsync(f_last, ws.f0, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
@@ -1720,6 +1747,8 @@ int sinkhorn_potentials_pnorm(const float* x, const float* a, int64_t n, const f
     CK(cudaMemsetAsync(f, 0, sizeof(float) * n, s));
     CK(cudaMemsetAsync(g, 0, sizeof(float) * m, s));
   }
+  rc = keep_cost(x, n, y, m, d, ws, &cost, s);
+  if (rc) return rc;
   return sinkhorn_core(x, a, n, y, b, m, d, eps, tau, max_iter, PROGOT_FP32, f, ws.f1, g, ws.xn, ws.yn, ws, iters_out,
                        err_out, s, nullptr, false, cost);
 }
@@ -1774,6 +1803,8 @@ int entropic_map_apply_pnorm(const float* xq, int64_t nq, const float* y, int64_
   if (out != xq) CK(cudaMemcpyAsync(out, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
   for (int k = 0; k < K; ++k) {
     const double al = (k == K - 1) ? 1.0 : alpha[k];
+    rc = keep_cost(out, nq, y, m, d, ws, &cost, s);
+    if (rc) return rc;
     rc = map_step(out, nq, y, m, d, g_all + (int64_t)k * m, ws.yn, eps[k], al, PROGOT_FP32, ws, s, nullptr, cost);
     if (rc) return rc;
   }

@@ -97,6 +97,9 @@ struct SweepParams {
   int32_t cost;        // CostKind: kCostSqEuclid uses scale * (a . b) + bscale (potB - |b|^2);
                        // the p-norm costs use scale * sum_k |a_k - b_k|^p + bscale potB
   float cost_p;        // p of the p-norm cost
+  const float* C;      // p-norm: stored sums sum_k |x_ik - y_jk|^p (rows of ldc floats), or nullptr
+  int64_t ldc;
+  int32_t c_cols;      // 1: this sweep's rows are C's columns
 };
 
 // Cost of the sweeps. kCostSqEuclid: |x - y|^2 through the dot product (tensor cores or

@@ -26,6 +26,8 @@ struct MapParams {
   float alpha;
   int32_t cost;        // CostKind (the p-norm map moves x by grad h*(sum_j Q_ij grad h(x - y_j)))
   float cost_p;
+  const float* C;      // p-norm: stored cost sums (SweepParams::C), or nullptr
+  int64_t ldc;
 };
 
 void count_launch();
@@ -41,6 +43,9 @@ cudaError_t launch_map_sweep_pnorm(const MapParams& p, cudaStream_t stream);
 // reduce_parts() doubles)
 cudaError_t launch_pairwise_cost_sum(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, int32_t cost,
                                      float cost_p, double* partial, double* out, cudaStream_t s);
+// C[i ld + j] = sum_k |x_ik - y_jk|^p, zeros for m <= j < 128 ceil(m / 128) <= ld
+cudaError_t launch_pnorm_cost(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, int32_t cost, float cost_p,
+                              float* C, int64_t ld, cudaStream_t s);
 int fp32_tile_rows();
 int fp32_tile_cols();
 int map_dchunk();

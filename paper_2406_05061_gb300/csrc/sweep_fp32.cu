@@ -14,6 +14,8 @@
 // map_sweep_fp32: the barycentric projection of Alg. 2 / Alg. 3: with L_i known,
 //   T_i = sum_j 2^{t_ij - L_i} y_j / sum_j 2^{t_ij - L_i},
 //   x_i <- x_i + alpha (T_i - x_i).
+#include <algorithm>
+
 #include "progot_common.cuh"
 #include "progot_internal.h"
 #include "sweep_epilogue.cuh"
@@ -181,6 +183,58 @@ __device__ __forceinline__ float rescaled(float w, float mp, float M) {
   return (mp == -INFINITY) ? 0.f : w * exp2f(mp - M);
 }
 
+// ---- the end of a sweep's CTA (row block blockIdx.x, column split blockIdx.y)
+// Count the CTA's partials in; true in the row block's last CTA.
+__device__ __forceinline__ bool last_split(const SweepParams& p, int& s_last) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned prev = atomicAdd(&p.cnt[blockIdx.x], 1u);
+    s_last = (prev == (unsigned)(p.splits - 1));
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+// Combine the row block's splits in order and apply the epilogue (plain log-sum-exp sweeps);
+// returns the thread's error term.
+__device__ __forceinline__ double combine_rows(const SweepParams& p, int64_t row0, int fcur) {
+  const float* potA_cur = p.potA_old;
+  float* out_target = p.out;
+  if (p.role == 1 || p.role == 3) {
+    potA_cur = (fcur == 0) ? p.out : p.out_alt;
+    out_target = (fcur == 0) ? p.out_alt : p.out;
+  }
+  if (threadIdx.x >= BM) return 0.0;
+  const int64_t i = row0 + threadIdx.x;
+  if (i >= p.nA) return 0.0;
+  const RowIn in = row_inputs(p, i, potA_cur);
+  float2 v = make_float2(-INFINITY, 0.f);
+  for (int s = 0; s < p.splits; ++s) v = lse_combine(v, __ldcg(&p.partial[(int64_t)s * p.nA + i]));
+  const float L = v.x + __log2f(v.y);
+  float val;
+  return row_epilogue(p, i, L, in, out_target, &val);
+}
+// The row block's error, and in the sweep's last row block the solver state.
+__device__ __forceinline__ void finish_block(const SweepParams& p, double e, double* red, int& s_last) {
+  const double tot = block_sum_f64<NT>(e, red);
+  if (threadIdx.x == 0) {
+    p.errpart[blockIdx.x] = tot;
+    p.cnt[blockIdx.x] = 0;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned prev = atomicAdd(&p.cnt[gridDim.x], 1u);
+    s_last = (prev == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (s_last && threadIdx.x < 32) {
+    __threadfence();
+    finish_sweep_warp(p, gridDim.x);
+    if (threadIdx.x == 0) p.cnt[gridDim.x] = 0;
+  }
+}
+
 // kTilt adds the tilted sum W per row (coupling metrics) and, when p.Ac is given, the
 // plain sum V = sum_j 2^{t_ij - M} c(ac_i, b_j) of the cost from another cloud (the
 // cost tile is computed first and parked in dynamic shared memory, one entry per
@@ -327,22 +381,9 @@ __global__ void __launch_bounds__(NT, kTilt ? 1 : 2) lse_sweep_fp32(SweepParams 
       }
     }
   }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(&p.cnt[blockIdx.x], 1u);
-    s_last = (prev == (unsigned)(p.splits - 1));
-  }
-  __syncthreads();
-  if (!s_last) return;
+  if (!last_split(p, s_last)) return;
 
   // ---- last CTA of this row block: combine splits in order, epilogue
-  const float* potA_cur = p.potA_old;
-  float* out_target = p.out;
-  if (p.role == 1 || p.role == 3) {
-    potA_cur = (fcur == 0) ? p.out : p.out_alt;
-    out_target = (fcur == 0) ? p.out_alt : p.out;
-  }
   double e = 0.0;
   if constexpr (kTilt) {
     // coupling metrics of the rows of this block: with base_i = (pot_i - |a_i|^2) / eps,
@@ -352,7 +393,7 @@ __global__ void __launch_bounds__(NT, kTilt ? 1 : 2) lse_sweep_fp32(SweepParams 
     if (threadIdx.x < BM) {
       const int64_t i = row0 + threadIdx.x;
       if (i < p.nA) {
-        const RowIn in = row_inputs(p, i, potA_cur);
+        const RowIn in = row_inputs(p, i, p.potA_old);
         float3 v = make_float3(-INFINITY, 0.f, 0.f);
         float vc = 0.f;
         for (int s = 0; s < p.splits; ++s) {
@@ -371,7 +412,7 @@ __global__ void __launch_bounds__(NT, kTilt ? 1 : 2) lse_sweep_fp32(SweepParams 
           plogp = r * (base + kLn2 * tbar);
           pc = r * (double)vc / (double)v.y;
         }
-        if (out_target) out_target[i] = (float)r;
+        if (p.out) p.out[i] = (float)r;
         q[kSumErr] = fabs(r - (double)in.w);
         q[kSumMass] = r;
         q[kSumPotR] = (double)in.pot * r;
@@ -387,35 +428,9 @@ __global__ void __launch_bounds__(NT, kTilt ? 1 : 2) lse_sweep_fp32(SweepParams 
       if (threadIdx.x == 0) p.metpart[(int64_t)blockIdx.x * kMetricSums + k] = t;
     }
   } else {
-    if (threadIdx.x < BM) {
-      const int64_t i = row0 + threadIdx.x;
-      if (i < p.nA) {
-        const RowIn in = row_inputs(p, i, potA_cur);
-        float2 v = make_float2(-INFINITY, 0.f);
-        for (int s = 0; s < p.splits; ++s) v = lse_combine(v, __ldcg(&p.partial[(int64_t)s * p.nA + i]));
-        const float L = v.x + __log2f(v.y);
-        float val;
-        e = row_epilogue(p, i, L, in, out_target, &val);
-      }
-    }
+    e = combine_rows(p, row0, fcur);
   }
-  const double tot = block_sum_f64<NT>(e, red);
-  if (threadIdx.x == 0) {
-    p.errpart[blockIdx.x] = tot;
-    p.cnt[blockIdx.x] = 0;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(&p.cnt[gridDim.x], 1u);
-    s_last = (prev == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (s_last && threadIdx.x < 32) {
-    __threadfence();
-    finish_sweep_warp(p, gridDim.x);
-    if (threadIdx.x == 0) p.cnt[gridDim.x] = 0;
-  }
+  finish_block(p, e, red, s_last);
 }
 
 // ---------------------------------------------------------------- map sweep
@@ -657,7 +672,25 @@ __global__ void __launch_bounds__(NT, 1) map_sweep_pnorm(MapParams p) {
       const int kk = dch0 + k;
       sm.Ys[c][k] = (j < p.nB && kk < p.d) ? __ldg(p.B + j * (int64_t)p.d + kk) : 0.f;
     }
-    tile_accumulate<kCost>(sm.g, p.A, p.nA, p.B, p.nB, p.d, row0, col0, vec_ok, p.cost_p, acc);
+    if (p.C != nullptr) {
+      // the loop before this step kept the cost
+      __syncthreads();  // beta_s and Ys are written
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int64_t i = row0 + thread_row(r);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (i < p.nA) v = __ldg(reinterpret_cast<const float4*>(p.C + i * p.ldc + col0 + thread_col(4 * h)));
+          acc[r][4 * h + 0] = v.x;
+          acc[r][4 * h + 1] = v.y;
+          acc[r][4 * h + 2] = v.z;
+          acc[r][4 * h + 3] = v.w;
+        }
+      }
+    } else {
+      tile_accumulate<kCost>(sm.g, p.A, p.nA, p.B, p.nB, p.d, row0, col0, vec_ok, p.cost_p, acc);
+    }
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       const int rr = thread_row(r);
@@ -791,7 +824,176 @@ __global__ void __launch_bounds__(NT, 2) pairwise_cost_sum(const float* __restri
   if (threadIdx.x == 0) partial[blockIdx.x] = b;
 }
 
+// ------------------------------------------------------- p-norm cost kept for a loop
+// The p-norm cost of a pair takes d square roots (or d powers), at 16 a clock and SM the
+// bound of a sweep that forms it (321 us at 11000 x 2800, d = 47); it does not change over
+// the sweeps of a loop or the map step after it. Where it fits beside L2's size (128 MB of
+// the workspace: 33 million pairs), one pass writes sum_k |x_ik - y_jk|^p and every sweep
+// reads it, at about 25 us for the same pairs. Rows of ld = 128 ceil(m / 128) floats, zeros
+// past m.
+template <int kCost>
+__global__ void __launch_bounds__(NT, 2) pnorm_cost_kernel(const float* __restrict__ X, int64_t n,
+                                                           const float* __restrict__ Y, int64_t m, int32_t d,
+                                                           float cp, float* __restrict__ C, int64_t ld) {
+  __shared__ GemmSmem sm;
+  const int64_t row0 = (int64_t)blockIdx.y * BM, col0 = (int64_t)blockIdx.x * BN;
+  const bool vec_ok = ((d & 3) == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) &&
+                      ((reinterpret_cast<uintptr_t>(Y) & 15) == 0);
+  float acc[8][8];
+  tile_accumulate<kCost>(sm, X, n, Y, m, d, row0, col0, vec_ok, cp, acc);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int64_t i = row0 + thread_row(r);
+    if (i >= n) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t j = col0 + thread_col(4 * h);
+      float4 v;
+      v.x = j + 0 < m ? acc[r][4 * h + 0] : 0.f;
+      v.y = j + 1 < m ? acc[r][4 * h + 1] : 0.f;
+      v.z = j + 2 < m ? acc[r][4 * h + 2] : 0.f;
+      v.w = j + 3 < m ? acc[r][4 * h + 3] : 0.f;
+      *reinterpret_cast<float4*>(C + i * ld + j) = v;
+    }
+  }
+}
+
+// Fold four values into a running (max, sum) in log2 units.
+__device__ __forceinline__ void online4(float& m, float& s, float t0, float t1, float t2, float t3) {
+  const float mn = fmaxf(m, fmaxf(fmaxf(t0, t1), fmaxf(t2, t3)));
+  if (mn == -INFINITY) return;
+  s = s * fast_exp2(m - mn) + ((fast_exp2(t0 - mn) + fast_exp2(t1 - mn)) + (fast_exp2(t2 - mn) + fast_exp2(t3 - mn)));
+  m = mn;
+}
+
+// The log-sum-exp sweep over a stored cost. kCols = 0: the updated side's points are C's
+// rows; a warp takes 16 of the block's 128 rows, its lanes four columns each of a 128-column
+// tile, eight rows' loads in flight. kCols = 1: they are C's columns; a lane takes four of
+// the block's 128, a warp every eighth row, four in flight. Same partials, combine, epilogue
+// and stop test as lse_sweep_fp32.
+template <int kCols>
+__global__ void __launch_bounds__(NT) lse_sweep_cost(SweepParams p) {
+  if (p.state != nullptr && p.state->done) return;
+  __shared__ double red[NT / 32];
+  __shared__ int s_last;
+  __shared__ float2 part[kCols ? NT / 32 : 1][BM];
+  const int fcur = p.state ? p.state->fcur : 0;
+  const float* potB = (p.potB_alt && fcur == 1) ? p.potB_alt : p.potB;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row0 = (int64_t)blockIdx.x * BM;
+  const int ntiles = (int)((p.nB + BN - 1) / BN);
+  const int t_begin = blockIdx.y * p.tiles_per_split;
+  const int t_end = min(ntiles, t_begin + p.tiles_per_split);
+  if constexpr (kCols == 0) {
+    float m_run[16], s_run[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      m_run[r] = -INFINITY;
+      s_run[r] = 0.f;
+    }
+    for (int tile = t_begin; tile < t_end; ++tile) {
+      const int64_t j = (int64_t)tile * BN + 4 * lane;
+      float beta[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) beta[e] = j + e < p.nB ? __ldg(potB + j + e) * p.bscale : -INFINITY;
+#pragma unroll
+      for (int r0 = 0; r0 < 16; r0 += 8) {
+        float4 c[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int64_t i = row0 + warp * 16 + r0 + r;
+          c[r] = i < p.nA ? __ldg(reinterpret_cast<const float4*>(p.C + i * p.ldc + j)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          online4(m_run[r0 + r], s_run[r0 + r], fmaf(c[r].x, p.scale, beta[0]), fmaf(c[r].y, p.scale, beta[1]),
+                  fmaf(c[r].z, p.scale, beta[2]), fmaf(c[r].w, p.scale, beta[3]));
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      float M = m_run[r];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+      float sum = M == -INFINITY ? 0.f : s_run[r] * fast_exp2(m_run[r] - M);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      const int64_t i = row0 + warp * 16 + r;
+      if (lane == 0 && i < p.nA) p.partial[(int64_t)blockIdx.y * p.nA + i] = make_float2(M, sum);
+    }
+  } else {
+    float m_run[4], s_run[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      m_run[e] = -INFINITY;
+      s_run[e] = 0.f;
+    }
+    // C's rows are the points summed over; columns past nA hold zeros and are not written
+    const float* col = p.C + row0 + 4 * lane;
+    const int64_t r_end = min((int64_t)t_end * BN, p.nB);
+    for (int64_t r = (int64_t)t_begin * BN + warp; r < r_end; r += 4 * (NT / 32)) {
+      float4 c[4];
+      float beta[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t rr = r + q * (NT / 32);
+        const bool in = rr < r_end;
+        c[q] = in ? __ldg(reinterpret_cast<const float4*>(col + rr * p.ldc)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        beta[q] = in ? __ldg(potB + rr) * p.bscale : -INFINITY;
+      }
+      online4(m_run[0], s_run[0], fmaf(c[0].x, p.scale, beta[0]), fmaf(c[1].x, p.scale, beta[1]),
+              fmaf(c[2].x, p.scale, beta[2]), fmaf(c[3].x, p.scale, beta[3]));
+      online4(m_run[1], s_run[1], fmaf(c[0].y, p.scale, beta[0]), fmaf(c[1].y, p.scale, beta[1]),
+              fmaf(c[2].y, p.scale, beta[2]), fmaf(c[3].y, p.scale, beta[3]));
+      online4(m_run[2], s_run[2], fmaf(c[0].z, p.scale, beta[0]), fmaf(c[1].z, p.scale, beta[1]),
+              fmaf(c[2].z, p.scale, beta[2]), fmaf(c[3].z, p.scale, beta[3]));
+      online4(m_run[3], s_run[3], fmaf(c[0].w, p.scale, beta[0]), fmaf(c[1].w, p.scale, beta[1]),
+              fmaf(c[2].w, p.scale, beta[2]), fmaf(c[3].w, p.scale, beta[3]));
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) part[warp][4 * lane + e] = make_float2(m_run[e], s_run[e]);
+    __syncthreads();
+    if (threadIdx.x < BM) {
+      float2 v = part[0][threadIdx.x];
+      for (int w = 1; w < NT / 32; ++w) v = lse_combine(v, part[w][threadIdx.x]);
+      const int64_t i = row0 + threadIdx.x;
+      if (i < p.nA) p.partial[(int64_t)blockIdx.y * p.nA + i] = v;
+    }
+  }
+  if (!last_split(p, s_last)) return;
+  const double e = combine_rows(p, row0, fcur);
+  finish_block(p, e, red, s_last);
+}
+
+cudaError_t launch_pnorm_cost(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, int32_t cost, float cost_p,
+                              float* C, int64_t ld, cudaStream_t s) {
+  const dim3 grid((unsigned)((m + BN - 1) / BN), (unsigned)((n + BM - 1) / BM));
+  if (cost == kCostP15)
+    pnorm_cost_kernel<kCostP15><<<grid, NT, 0, s>>>(X, n, Y, m, d, cost_p, C, ld);
+  else
+    pnorm_cost_kernel<kCostPGeneral><<<grid, NT, 0, s>>>(X, n, Y, m, d, cost_p, C, ld);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// About six CTAs per SM, at least one tile each (the bound on splits * nA that sizes the
+// partial buffer holds: at most 6 * SMs / row blocks + 1 splits).
+static cudaError_t launch_lse_sweep_cost(SweepParams p, cudaStream_t stream) {
+  const int64_t rb = (p.nA + BM - 1) / BM, ct = (p.nB + BN - 1) / BN;
+  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(ct, (6 * (int64_t)device_sm_count() + rb - 1) / rb));
+  p.tiles_per_split = (int)((ct + want - 1) / want);
+  p.splits = (int)((ct + p.tiles_per_split - 1) / p.tiles_per_split);
+  const dim3 grid((unsigned)rb, (unsigned)p.splits);
+  if (p.c_cols)
+    lse_sweep_cost<1><<<grid, NT, 0, stream>>>(p);
+  else
+    lse_sweep_cost<0><<<grid, NT, 0, stream>>>(p);
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lse_sweep_fp32(const SweepParams& p, cudaStream_t stream) {
+  if (p.C != nullptr) return launch_lse_sweep_cost(p, stream);
   const int rb = (int)((p.nA + BM - 1) / BM);
   dim3 grid(rb, p.splits);
   const bool tilt = p.mode == kModeMetrics;

@@ -134,3 +134,33 @@ def test_coupling_metrics_pnorm_against_the_original_cloud(nat):
     xl, f, g = host(res.x_last), host(res.f_last), host(res.g_all[K - 1])
     met = nat.coupling_metrics_pnorm(res.x_last, dev(pr.y), 1.5, res.f_last, res.g_all[K - 1], e0, x_cost=dev(pr.x))
     assert met["transport_cost"] == pytest.approx(O.coupling_cost(xl, pr.y, f, g, e0, P15, X_cost=pr.x), rel=TOL_FP32)
+
+
+@pytest.mark.parametrize("n,m,d,p", [(1, 1, 1, 1.5), (127, 129, 3, 1.5), (128, 128, 16, 1.5), (257, 384, 5, 3.0),
+                                     (700, 65, 47, 1.25), (130, 1500, 8, 1.5)])
+def test_stored_cost_loop_matches_tiled_loop(nat, n, m, d, p):
+    """The cost kept in the workspace against the sweeps that form it tile by tile (a workspace
+    without room for it): both fold the same float32 costs, so potentials and maps agree to
+    the rounding of t (2^-22 of the largest |cost / eps|) and of the potentials per iteration."""
+    pr = W.gmm_pair(n, m, d, seed=n + m, k=2)
+    C = (np.abs(pr.x[:, None, :].astype(np.float64) - pr.y[None, :, :]) ** p).sum(-1) / p
+    eps, its = 0.1 * float(C.mean()) + 1e-3, 6
+    x, y = torch.from_numpy(pr.x).cuda(), torch.from_numpy(pr.y).cuda()
+    a = torch.from_numpy(np.full(n, 1.0 / n, np.float32)).cuda()
+    full = nat.sinkhorn_potentials_pnorm(x, y, p, eps, 0.0, its, a=a)
+    size = nat.workspace_size(n, m, d) - 1  # one byte short of the layout that holds the cost
+    buf = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+    ws = nat.Workspace.__new__(nat.Workspace)
+    ws.buf, ws.bytes, ws.ptr = buf, size, (buf.data_ptr() + 255) & ~255
+    ws.covers = lambda *args: True
+    tiled = nat.sinkhorn_potentials_pnorm(x, y, p, eps, 0.0, its, a=a, workspace=ws)
+    torch.cuda.synchronize()
+    tol = 2.0 ** -20 * float(C.max()) * its + 2.0 ** -20 * eps * 16
+    np.testing.assert_allclose(full.f.cpu().numpy(), tiled.f.cpu().numpy(), rtol=0, atol=tol)
+    np.testing.assert_allclose(full.g.cpu().numpy(), tiled.g.cpu().numpy(), rtol=0, atol=tol)
+    assert abs(full.err - tiled.err) <= 2.0 ** -20 * (float(C.max()) / eps + 16)
+    m1 = nat.entropic_map_apply_pnorm(x, y, p, full.g, [eps], [1.0])
+    m2 = nat.entropic_map_apply_pnorm(x, y, p, full.g, [eps], [1.0], workspace=ws)
+    spread = float(np.abs(pr.y[:, None, :] - pr.x[None, :, :]).max()) if n * m < 50000 else float(np.abs(pr.y).max() * 2)
+    np.testing.assert_allclose(m1.cpu().numpy(), m2.cpu().numpy(), rtol=0,
+                               atol=2.0 ** -19 * spread * (float(C.max()) / eps + 16))
