@@ -1226,14 +1226,24 @@ static int check_fault(const Workspace& ws, cudaStream_t s) {
 
 // Coupling metrics (Sec. 5.2) of P = exp((f (+) g - C)/eps): a row sweep and a column
 // sweep in kModeMetrics, each followed by a fixed-order float64 reduction of its
-// per-row-block sums into ws.metout. ws.xn, ws.yn must hold |x|^2 and |y|^2 and the
-// arrival counters must be zero.
+// per-row-block sums into ws.metout. The arrival counters must be zero.
 static int metrics_core(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m,
                         int32_t d, const float* f, const float* g, double eps, const Workspace& ws, cudaStream_t s,
                         progot_coupling_metrics* out, const Cost& cost = Cost(), const float* x_cost = nullptr) {
   int rc = t_host.init();
   if (rc) return rc;
-  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws);
+  // the tensor cores where the workspace holds their operands; the p-norm cost and the cost
+  // of another cloud on CUDA cores
+  TcOps ops;
+  if (!cost.pnorm() && x_cost == nullptr) {
+    rc = prep_tc(x, n, y, m, d, eps, PROGOT_FP32, ws, &ops, s, f, g);
+    if (rc) return rc;
+  }
+  if (!ops.on && !cost.pnorm()) {
+    CK(launch_row_sqnorm(x, n, d, ws.xn, s));
+    CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  }
+  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws, ops.on ? 1 : 2);
   pr.wA = a;
   pr.potB = g;
   pr.potA_old = f;
@@ -1246,18 +1256,24 @@ static int metrics_core(const float* x, const float* a, int64_t n, const float* 
     pr.Acn = cost.pnorm() ? nullptr : ws.L;
     pr.cpart = ws.cpart;
   }
-  CK(launch_lse_sweep_fp32(pr, s));
+  rc = lse_sweep(pr, s, &ops, true, &ws, true);
+  if (rc) return rc;
   CK(launch_sum_parts(ws.metpart, (int)cdiv(n, fp32_tile_rows()), kMetricSums, ws.metout, s));
-  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws);
+  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws, ops.on ? 1 : 2);
   pc.wA = b;
   pc.potB = f;
   pc.potA_old = g;
   pc.mode = kModeMetrics;
   apply_cost(pc, cost, eps);
-  CK(launch_lse_sweep_fp32(pc, s));
+  rc = lse_sweep(pc, s, &ops, false, &ws, true);
+  if (rc) return rc;
   CK(launch_sum_parts(ws.metpart, (int)cdiv(m, fp32_tile_rows()), kMetricSums, ws.metout + kMetricSums, s));
   CK(cudaMemcpyAsync(t_host.hd, ws.metout, sizeof(double) * 2 * kMetricSums, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  if (ops.on) {
+    rc = check_fault(ws, s);
+    if (rc) return rc;
+  }
   const double* R = t_host.hd;                // row sweep: pot = f, w = a
   const double* Cs = t_host.hd + kMetricSums;  // column sweep: pot = g, w = b
   out->mass = R[kSumMass];
@@ -1632,8 +1648,6 @@ int coupling_metrics(const float* x, const float* a, int64_t n, const float* y, 
   cudaStream_t s = (cudaStream_t)stream;
   rc = zero_counters(ws, s);
   if (rc) return rc;
-  CK(launch_row_sqnorm(x, n, d, ws.xn, s));
-  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
   return metrics_core(x, a, n, y, b, m, d, f, g, eps, ws, s, out, Cost(), x_cost);
 }
 

@@ -133,11 +133,16 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     bool ok = true;
-    int u = 0;
+    int u = 0, s_cur = 0;  // ring position and fill parity kept without division
+    uint32_t s_par = 0;
     for (; u < nu; ++u) {
-      const int s = u % S;
-      ok = warp_wait(&sh.empty[s], (uint32_t)(((u / S) & 1) ^ 1), abort_flag);
+      const int s = s_cur;
+      ok = warp_wait(&sh.empty[s], s_par ^ 1u, abort_flag);
       if (!ok) break;
+      if (++s_cur == S) {
+        s_cur = 0;
+        s_par ^= 1u;
+      }
       unsigned char* st = smem + s * st_bytes;
       if (elect_one()) {
         mbar_arrive_expect_tx(&sh.full[s], st_bytes);
@@ -158,11 +163,17 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
     // ------------------------------------------------------------ MMA issuer
     constexpr uint32_t kId = make_idesc_f16(BM, N) | (1u << 16);  // A K-major, B MN-major
     bool ok = true;
+    int s_cur = 0;
+    uint32_t s_par = 0;
     for (int u = 0; u < nu && ok; ++u) {
-      const int s = u % S, b = u & 1;
+      const int s = s_cur, b = u & 1;
       ok = warp_wait(&sh.acc_empty[b], (uint32_t)(((u >> 1) & 1) ^ 1), abort_flag) &&
-           warp_wait(&sh.full[s], (uint32_t)((u / S) & 1), abort_flag);
+           warp_wait(&sh.full[s], s_par, abort_flag);
       if (!ok) break;
+      if (++s_cur == S) {
+        s_cur = 0;
+        s_par ^= 1u;
+      }
       tc_fence_after();
       const uint32_t st = smem_u32(smem + s * st_bytes);
       const uint64_t ph = desc_sw128(st), pl = desc_sw128(st + PV_P_BYTES / 2);

@@ -69,6 +69,8 @@ struct TcShared {
   int32_t slots[32], eslots[32];  // partial slots of the row block being combined, by group
   float2 ms[2][128];   // (max, sum) of LSE warpgroup 1 by segment parity, merged by warpgroup 0
   float2 seg[2][128];  // merged (max, sum) of a handed-off segment, by segment parity
+  float mw[2][128], segw[2][128];  // ... and their tilted sums (coupling metrics)
+  double mred[4][kMetricSums], emred[4][kMetricSums];
 };
 
 
@@ -206,10 +208,30 @@ __device__ __forceinline__ SolverState sweep_state(const SweepParams& p) {
 // 32 rows, then (q0 + q1) + (q2 + q3)); the last row block of the sweep finishes it.
 // The g-update of a Sinkhorn loop (role 2) measures no error and changes no solver
 // state, so its row blocks skip the sweep-level arrival altogether.
+// (max, sum, tilted sum) of two parts of a row in log2 units: with M the max, S = sum 2^{t - M}
+// and W = sum 2^{t - M} (t - M).
+__device__ __forceinline__ float3 tilt_merge(float3 p, float3 q) {
+  const float M = fmaxf(p.x, q.x);
+  if (M == -INFINITY) return make_float3(-INFINITY, 0.f, 0.f);
+  float s = 0.f, w = 0.f;
+  if (p.x != -INFINITY) {
+    const float c = exp2f(p.x - M);
+    s += p.y * c;
+    w += c * fmaf(p.y, p.x - M, p.z);
+  }
+  if (q.x != -INFINITY) {
+    const float c = exp2f(q.x - M);
+    s += q.y * c;
+    w += c * fmaf(q.y, q.x - M, q.z);
+  }
+  return make_float3(M, s, w);
+}
+
 template <int NT, int GRID>
 __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int k, const Seg& sg, const Split& sp,
-                                                 int tid, int row0, const float2 (&mv)[BM / NT], int fcur,
-                                                 int32_t& s_last, int32_t& s_fin, float* red, int32_t* slots) {
+                                                 int tid, int row0, const float2 (&mv)[BM / NT],
+                                                 const float (&mw)[BM / NT], int fcur, int32_t& s_last, int32_t& s_fin,
+                                                 float* red, int32_t* slots, double (*mred)[kMetricSums]) {
   constexpr int RPT = BM / NT;
   const SweepParams& p = tp.p;
   const float* potA_cur = p.potA_old;
@@ -229,6 +251,7 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
     rin[h].w = 0.f;
     if (i < p.nA) {
       p.partial[((int64_t)c * tp.maxseg + k) * BM + rl] = mv[h];
+      if constexpr (GRID == 2) p.wpart[((int64_t)c * tp.maxseg + k) * BM + rl] = mw[h];
       rin[h] = row_inputs(p, i, potA_cur);
     }
   }
@@ -253,8 +276,12 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
   if (!s_last) return;
   float e[RPT];
   float2 accs[RPT];
+  float accw[RPT];
 #pragma unroll
-  for (int h = 0; h < RPT; ++h) accs[h] = make_float2(-INFINITY, 0.f);
+  for (int h = 0; h < RPT; ++h) {
+    accs[h] = make_float2(-INFINITY, 0.f);
+    accw[h] = 0.f;
+  }
   for (int base = 0; base < nc; base += 32) {
     if (base > 0) {
       seg_bar<NT>();
@@ -264,18 +291,69 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
     // the loads of eight contributors back to back, then combined in CTA order
     for (int q0 = base; q0 < min(nc, base + 32); q0 += 8) {
       float2 pv[RPT][8];
+      float pw[RPT][8];
 #pragma unroll
       for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int h = 0; h < RPT; ++h)
-          if (q0 + q < nc) pv[h][q] = __ldcg(&p.partial[(int64_t)slots[q0 + q - base] * BM + row0 + NT * h]);
+          if (q0 + q < nc) {
+            pv[h][q] = __ldcg(&p.partial[(int64_t)slots[q0 + q - base] * BM + row0 + NT * h]);
+            if constexpr (GRID == 2) pw[h][q] = __ldcg(&p.wpart[(int64_t)slots[q0 + q - base] * BM + row0 + NT * h]);
+          }
 #pragma unroll
       for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int h = 0; h < RPT; ++h)
-          if (q0 + q < nc) accs[h] = lse_combine(accs[h], pv[h][q]);
+          if (q0 + q < nc) {
+            if constexpr (GRID == 2) {
+              const float3 v = tilt_merge(make_float3(accs[h].x, accs[h].y, accw[h]),
+                                          make_float3(pv[h][q].x, pv[h][q].y, pw[h][q]));
+              accs[h] = make_float2(v.x, v.y);
+              accw[h] = v.z;
+            } else {
+              accs[h] = lse_combine(accs[h], pv[h][q]);
+            }
+          }
     }
   }
+  if constexpr (GRID == 2) {
+    // with base_i = (pot_i - |a_i|^2) / eps: log P_ij = base_i + ln2 t_ij, r_i = exp(base_i +
+    // ln2 L_i), sum_j P_ij log P_ij = r_i (base_i + ln2 (M + W / S)); the row block's sums in
+    // a fixed order (a shuffle tree per 32 rows, then the four groups)
+    double q[RPT][kMetricSums];
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+#pragma unroll
+      for (int m = 0; m < kMetricSums; ++m) q[h][m] = 0.0;
+      const int64_t i = (int64_t)sg.r * BM + row0 + NT * h;
+      if (i < p.nA) {
+        double r = 0.0, plogp = 0.0;
+        // a NaN sum (an aborted CTA, a NaN input) stays NaN
+        if (!(accs[h].y <= 0.f)) {
+          const double base = ((double)rin[h].pot - (double)rin[h].an) / p.eps;
+          r = (double)expf((float)(base + kLn2 * ((double)accs[h].x + (double)log2f(accs[h].y))));
+          plogp = r * (base + kLn2 * ((double)accs[h].x + (double)accw[h] / (double)accs[h].y));
+        }
+        q[h][kSumErr] = fabs(r - (double)rin[h].w);
+        q[h][kSumMass] = r;
+        q[h][kSumPotR] = (double)rin[h].pot * r;
+        q[h][kSumPlogP] = plogp;
+        q[h][kSumPotW] = (double)rin[h].pot * (double)rin[h].w;
+      }
+#pragma unroll
+      for (int m = 0; m < kMetricSums; ++m) {
+        double v = q[h][m];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if ((tid & 31) == 0) mred[(row0 + NT * h) >> 5][m] = v;
+      }
+    }
+    seg_bar<NT>();
+    if (tid < kMetricSums)
+      p.metpart[(int64_t)sg.r * kMetricSums + tid] = (mred[0][tid] + mred[1][tid]) + (mred[2][tid] + mred[3][tid]);
+    if (tid == 0) p.cnt[sg.r] = 0;
+    seg_bar<NT>();
+  } else {
 #pragma unroll
   for (int h = 0; h < RPT; ++h) {
     e[h] = 0.f;
@@ -331,10 +409,11 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
     if (tid == 0) p.cnt[tp.R] = 0;
   }
   seg_bar<NT>();
+  }
 }
 
-// GRID = 0: bf16 operands, one accumulator (two buffers of BN columns). GRID = 1: the
-// integer-grid split (grid_split.cuh), BN = 128, two accumulators per tile (leading
+// GRID = 0: bf16 operands, one accumulator (two buffers of BN columns). GRID = 1, 2 (2 with
+// the tilted sums of the coupling metrics): the integer-grid split (grid_split.cuh), BN = 128, two accumulators per tile (leading
 // products at TMEM columns [0, 256), the others at [256, 512)).
 // ATM: the bf16 A row block sits in TMEM (hi at columns [256, 256 + 32 nkb), lo after it),
 // as in the persistent loop: 128 < d <= 256.
@@ -413,6 +492,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 0) {
     // ------------------------------------------------------------ producer (whole warp, one lane issues)
     int u = 0;  // B stage units issued
+    int s_cur = 0;       // ring position of unit u (kept without division)
+    uint32_t s_par = 0;  // parity of that stage's fills so far
     bool ok = true;
     const uint32_t abytes = (uint32_t)L.a_stride;
     const uint32_t bbytes = B_TILE_BYTES * (uint32_t)parts;
@@ -470,13 +551,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       for (int t = sg.t0; t < sg.t1 && ok && !stopped; ++t) {
         for (int kb = 0; kb < nkb; ++kb, ++u) {
-          const int s = u % S;
+          const int s = s_cur;
           if (!waited && u == S) {  // a stage is about to be reused: its bias must be on its way
             resolve();
             if (stopped) break;
           }
-          ok = warp_wait(&sh.empty[s], (uint32_t)(((u / S) & 1) ^ 1), abort_flag);
+          ok = warp_wait(&sh.empty[s], s_par ^ 1u, abort_flag);
           if (!ok) break;
+          if (++s_cur == S) {
+            s_cur = 0;
+            s_par ^= 1u;
+          }
           unsigned char* st = smem + L.stage0 + s * L.stage_bytes;
           if (elect_one()) {
             // after the wait the bias rows travel with the operands on full[s]; before it
@@ -519,6 +604,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
     bool ok = true;
     int u = 0, tl = 0;
+    int s_cur = 0;       // ring position and fill parity of unit u, kept without division
+    uint32_t s_par = 0;
     for (int k = 0; k < nseg && ok; ++k) {
       const Seg sg = segment(sp, c, k);
       const int ai = NA > 0 ? k % NA : 0;
@@ -536,9 +623,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
         for (int kb = 0; kb < nkb; ++kb, ++u) {
-          const int s = u % S;
-          ok = warp_wait(&sh.full[s], (uint32_t)((u / S) & 1), abort_flag);
+          const int s = s_cur;
+          ok = warp_wait(&sh.full[s], s_par, abort_flag);
           if (!ok) break;
+          if (++s_cur == S) {
+            s_cur = 0;
+            s_par ^= 1u;
+          }
           tc_fence_after();
           const uint32_t st = smem_u32(smem + L.stage0 + s * L.stage_bytes);
           const uint64_t bh = desc_sw128(st), bl = desc_sw128(st + L.b_lo_off);
@@ -595,7 +686,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // the first stages were loaded before the previous sweep finished: their bias
             // rows (its new potential) may follow on bias_full[s]; later stages carry them
             // on full[s]
-            ok = warp_wait(&sh.bias_full[s], (uint32_t)((u / S) & 1), abort_flag);
+            ok = warp_wait(&sh.bias_full[s], 0u, abort_flag);  // each stage's first fill
             if (!ok) break;
             if (*reinterpret_cast<volatile int32_t*>(&sh.stop) != 0) {
               ok = false;  // the loop had already stopped: wind down (not a fault)
@@ -667,7 +758,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           if (lane == 0) mbar_arrive(&sh.a_full[0]);
         }
       }
-      float m_run = prob ? 0.f : -INFINITY, s_run = 0.f;
+      float m_run = prob ? 0.f : -INFINITY, s_run = 0.f, w_run = 0.f;
       const bool row_ok = (int64_t)sg.r * BM + row_local < p.nA;
       const float Lr = (prob && row_ok) ? __ldg(tp.lrow + (int64_t)sg.r * BM + row_local) : 0.f;
       for (int t = sg.t0; t < sg.t1; ++t, ++tl) {
@@ -759,7 +850,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             // grid split: the accumulators hold t 2^(ex + ey); (t - m) 2^-(ex + ey) is exact
             const float nm = GRID ? -mnew * inv2 : -mnew;
             const uint64_t negm = pack2(nm, nm);
-            uint64_t acc[4];
+            uint64_t acc[4], wacc = 0ull;
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[q] = 0ull;
 #pragma unroll
@@ -769,13 +860,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 float a0, a1;
                 const uint64_t tv = pack2(v[cc][i], v[cc][i + 1]);
                 unpack2(GRID ? fma2(tv, inv22, negm) : add2(tv, negm), a0, a1);
-                acc[(i >> 1) & 3] = add2(acc[(i >> 1) & 3], pack2(fast_exp2(a0), fast_exp2(a1)));
+                const uint64_t ex = pack2(fast_exp2(a0), fast_exp2(a1));
+                acc[(i >> 1) & 3] = add2(acc[(i >> 1) & 3], ex);
+                // padded columns have t - m near -3e38 and e = 0: the clamp keeps 0 * inf out
+                if constexpr (GRID == 2) wacc = fma2(ex, pack2(fmaxf(a0, -256.f), fmaxf(a1, -256.f)), wacc);
               }
             float s0, s1, s2, s3, s4, s5, s6, s7;
             unpack2(acc[0], s0, s1);
             unpack2(acc[1], s2, s3);
             unpack2(acc[2], s4, s5);
             unpack2(acc[3], s6, s7);
+            if constexpr (GRID == 2) {
+              const float dm = (m_run - mnew) * inv2;
+              float w0, w1;
+              unpack2(wacc, w0, w1);
+              w_run = (m_run == -INFINITY ? 0.f : fast_exp2(dm) * fmaf(s_run, dm, w_run)) + (w0 + w1);
+            }
             s_run = s_run * fast_exp2(GRID ? (m_run - mnew) * inv2 : m_run - mnew) +
                     (((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7)));
             m_run = mnew;
@@ -790,12 +890,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // merge warpgroup 1's (max, sum) into warpgroup 0
       // (slots alternate by segment parity: warpgroup 1 can only reuse slot k & 1 after
       // the next 256-thread barrier, which warpgroup 0 reaches after reading it)
-      if (wg == 1) sh.ms[k & 1][row_local] = make_float2(m_run, s_run);
+      if (wg == 1) {
+        sh.ms[k & 1][row_local] = make_float2(m_run, s_run);
+        if constexpr (GRID == 2) sh.mw[k & 1][row_local] = w_run;
+      }
       lse_bar_all();
       if (wg == 1) continue;
       {
         const float2 o = sh.ms[k & 1][row_local];
-        const float2 mrg = lse_combine(make_float2(m_run, s_run), o);
+        float2 mrg;
+        if constexpr (GRID == 2) {
+          const float3 v = tilt_merge(make_float3(m_run, s_run, w_run), make_float3(o.x, o.y, sh.mw[k & 1][row_local]));
+          mrg = make_float2(v.x, v.y);
+          w_run = v.z;
+        } else {
+          mrg = lse_combine(make_float2(m_run, s_run), o);
+        }
         m_run = (isnan(o.y) || isnan(s_run)) ? NAN : mrg.x;
         s_run = (isnan(o.y) || isnan(s_run)) ? NAN : mrg.y;
       }
@@ -806,11 +916,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int sl = k & 1;
         mbar_wait(&sh.seg_empty[sl], (uint32_t)(((k >> 1) & 1) ^ 1), abort_flag);
         sh.seg[sl][row_local] = make_float2(m_run, s_run);
+        if constexpr (GRID == 2) sh.segw[sl][row_local] = w_run;
         mbar_arrive(&sh.seg_full[sl]);
         continue;
       }
       const float2 mv[1] = {make_float2(m_run, s_run)};
-      segment_epilogue<128, GRID>(tp, c, k, sg, sp, ltid, row_local, mv, fcur, sh.s_last, sh.s_fin, sh.red, sh.slots);
+      const float mw[1] = {w_run};
+      segment_epilogue<128, GRID>(tp, c, k, sg, sp, ltid, row_local, mv, mw, fcur, sh.s_last, sh.s_fin, sh.red,
+                                  sh.slots, sh.mred);
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
@@ -832,8 +945,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       float2 mv[2];
       mv[0] = okw ? sh.seg[sl][etid] : make_float2(NAN, NAN);
       mv[1] = okw ? sh.seg[sl][etid + 64] : make_float2(NAN, NAN);
+      float mw[2] = {0.f, 0.f};
+      if constexpr (GRID == 2) {
+        mw[0] = sh.segw[sl][etid];
+        mw[1] = sh.segw[sl][etid + 64];
+      }
       mbar_arrive(&sh.seg_empty[sl]);
-      segment_epilogue<64, GRID>(tp, c, k, sg, sp, etid, etid, mv, fcur, sh.e_last, sh.e_fin, sh.ered, sh.eslots);
+      segment_epilogue<64, GRID>(tp, c, k, sg, sp, etid, etid, mv, mw, fcur, sh.e_last, sh.e_fin, sh.ered, sh.eslots,
+                                 sh.emred);
     }
   }
 
@@ -979,10 +1098,12 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
   tp.lrow = lrow;
   tp.prob = (unsigned char*)prob;
   tp.a_row0 = a_row0;
+  if (p.mode == kModeMetrics && !grid) return cudaErrorInvalidValue;
   if (p.mode == kModeProb && (!grid || prob == nullptr || lrow == nullptr)) return cudaErrorInvalidValue;
   tp.a_part[0] = reinterpret_cast<const uint4*>(maps.a_part[0]);
   tp.a_part[1] = reinterpret_cast<const uint4*>(maps.a_part[1]);
-  cudaError_t e = grid        ? launch_tc<128, 1>(tp, smem, maps, stream)
+  cudaError_t e = grid && p.mode == kModeMetrics ? launch_tc<128, 2>(tp, smem, maps, stream)
+                  : grid      ? launch_tc<128, 1>(tp, smem, maps, stream)
                   : atm       ? launch_tc<128, 0, 1>(tp, smem, maps, stream)
                   : bn == 256 ? launch_tc<256, 0>(tp, smem, maps, stream)
                               : launch_tc<128, 0>(tp, smem, maps, stream);
