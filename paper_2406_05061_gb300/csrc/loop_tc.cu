@@ -397,14 +397,13 @@ __device__ __forceinline__ Seg seg_at(const Side& Sd, int c, int k, int maxseg) 
 // that hold coordinates (d <= 64), so that a tile's products are issued without a loop
 // (56.7 -> 46 us per sweep at 8192^2, d = 64, where the CUDA-core sweep takes 238).
 // ATM: the bf16 A row block sits in TMEM, hi at columns [256, 256 + 32 nkb), lo after it,
-// written by the LSE warpgroups (one part each) at every segment's start. Taken for 128 < d
-// <= 256, whose resident A left shared memory for two B stages only, fewer than a copy's
-// latency needs; now six fit, and the products read half as much shared memory.
+// written by the LSE warpgroups (one part each) at every segment's start. For 128 < d <= 256
+// and many tiles: a resident A leaves shared memory for two B stages only, now six fit, and
+// the products read half as much shared memory.
 // CONV: how the MMA warp issues. N = 128 products are shorter than a single divergent lane
-// needs to put the next one's operands in place beside the LSE warps: with the converged
-// warp 16384^2 sweeps took 141 us instead of 164 (grid, d = 64) and 247 instead of 290 (d =
-// 256). N = 256 products are long enough, and a handful of tiles per sweep is paced by the
-// hand-over, where the single lane is faster (512^2: 7.4 against 8.3 us).
+// needs to put the next one's operands in place beside the LSE warps (a probe: 90 cycles a
+// product against 71): with the converged warp 16384^2 sweeps took 145 us instead of 164
+// (grid, d = 64) and 248 instead of 290 (d = 256). N = 256 products are long enough.
 template <int BN, int NKB, int GRID, int ATM, int CONV>
 __global__ void __launch_bounds__(NTHREADS, 1)
     sinkhorn_loop_tc(const __grid_constant__ CUtensorMap mXh_a, const __grid_constant__ CUtensorMap mXl_a,
@@ -1022,15 +1021,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // ---------------------------------------------------------------- host side
 // Pipeline shape of the persistent loop: two resident A buffers and as many B stages
 // (2..8) as fit in 227 KB; 0 stages when no shape fits (the per-sweep kernel serves it).
-// A in TMEM (a_bufs = 0): 128-column bf16 tiles of three or four K blocks, where hi and lo
-// fill the 256 TMEM columns beside the accumulators (16384^2, d = 256: 292 us per sweep with
-// a resident A and two stages).
-static bool loop_a_in_tmem(int bn, int nkb, bool grid) { return !grid && bn == 128 && nkb <= 4; }
-
-static void loop_shape(int bn, int nkb, int split3, bool grid, int* stages, int* a_bufs) {
+// A in TMEM (atm, a_bufs = 0): 128-column bf16 tiles of three or four K blocks, where hi and
+// lo fill the 256 TMEM columns beside the accumulators.
+static void loop_shape(int bn, int nkb, int split3, bool grid, bool atm, int* stages, int* a_bufs) {
   *stages = 0;
   *a_bufs = 2;
-  const bool atm = loop_a_in_tmem(bn, nkb, grid);
   for (int na = atm ? 0 : 2; na >= (atm ? 0 : 1); --na) {
     int best = 0;
     for (int s = 2; s <= 8; ++s)
@@ -1045,7 +1040,7 @@ static void loop_shape(int bn, int nkb, int split3, bool grid, int* stages, int*
 
 bool loop_tc_supported(int bn, int nkb, int split3, bool grid) {
   int s, na;
-  loop_shape(bn, nkb, split3, grid, &s, &na);
+  loop_shape(bn, nkb, split3, grid, false, &s, &na);
   return s >= 2 && (grid ? bn == 128 && nkb == 1 : bn == 128 || bn == 256);
 }
 
@@ -1092,7 +1087,12 @@ static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const voi
 cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   int stages, a_bufs;
   const bool grid = Lq.gscale != nullptr;
-  loop_shape(Lq.bn, Lq.nkb, Lq.split3, grid, &stages, &a_bufs);
+  // A in TMEM from 64 tiles per CTA and sweep: writing it costs about 4 us at every segment's
+  // start, which many tiles repay (16384^2, d = 256, 107 tiles: 248 us per sweep against 262)
+  // and few do not (8000^2, 26 tiles: 69 against 65.5; 2000^2: 16.5 against 11.6)
+  const int64_t tiles = ((Lq.side[0].p.nA + tc::BM - 1) / tc::BM) * ((Lq.side[0].p.nB + Lq.bn - 1) / Lq.bn);
+  const bool atm = !grid && Lq.bn == 128 && Lq.nkb <= 4 && tiles >= 64 * (int64_t)Lq.G;
+  loop_shape(Lq.bn, Lq.nkb, Lq.split3, grid, atm, &stages, &a_bufs);
   if (!loop_tc_supported(Lq.bn, Lq.nkb, Lq.split3, grid)) return cudaErrorInvalidValue;
   tc::loop::Params P;
   memset(&P, 0, sizeof(P));
@@ -1143,7 +1143,7 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   P.gscale = Lq.gscale;
   const size_t smem = tc::loop::layout(Lq.bn, Lq.nkb, Lq.split3, stages, a_bufs, grid).total;
   const int ks = (Lq.side[0].p.d + 15) / 16;  // K = 16 steps
-  const bool many = (int64_t)P.side[0].R * P.side[0].T >= 4 * (int64_t)Lq.G;  // tiles per CTA and sweep
+  const bool many = tiles >= 4 * (int64_t)Lq.G;  // fewer are paced by the hand-over
   cudaError_t e;
   if (grid && many)
     e = ks <= 1   ? launch_loop<128, 1, 1, 0, 1>(P, smem, Lq.maps, stream)
@@ -1157,7 +1157,7 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
                   : launch_loop<128, 1, 4>(P, smem, Lq.maps, stream);
   else
     e = a_bufs == 0    ? launch_loop<128, 0, 0, 1, 1>(P, smem, Lq.maps, stream)
-        : Lq.bn == 128 ? launch_loop<128, 0, 0>(P, smem, Lq.maps, stream)
+        : Lq.bn == 128 ? launch_loop<128, 0, 0, 0, 1>(P, smem, Lq.maps, stream)
         : Lq.nkb == 1  ? launch_loop<256, 1, 0>(P, smem, Lq.maps, stream)
                        : launch_loop<256, 0, 0>(P, smem, Lq.maps, stream);
   count_launch();

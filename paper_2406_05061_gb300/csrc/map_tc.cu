@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(MT_NTHREADS, 1)
           float4 acc[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
           for (int q2 = 0; q2 < nc; ++q2) {
             int64_t sl;
             if (q2 < 8) {

@@ -5,21 +5,26 @@
 // log-sum-exp (from a log-sum-exp pass, or from the Sinkhorn loop's last f-update, which
 // used the same g), as in the d <= 64 kernel (map_tc.cu):
 //   S = X Y~^T over all K blocks of the operands (bf16 hi/lo pre-scaled by sqrt(c), three
-//     products, beta added by one more K = 16 step) into one of two 32-column TMEM
-//     buffers (tiles of 32 columns j);
+//     products, beta added by one more K = 16 step) into one of two 64-column TMEM buffers
+//     (tiles of 64 columns j);
 //   O += P Y~ over all d coordinates at once (N = 64 nkb <= 256), with P_ij =
 //     2^{t_ij - L_i} written by the LSE warps into shared memory as bf16 hi/lo (K-major,
-//     64-byte swizzle, K = 32 columns of the tile), three products; the B operand is the
-//     tile's K blocks of Y~, the very blocks S read, read again as one MN-major matrix
-//     whose 64-coordinate column groups are the K blocks; O takes up to 256 TMEM columns.
+//     64-byte swizzle, K = 32: half a tile's columns at a time), three products; the B
+//     operand is the tile's K blocks of Y~, the very blocks S read, read again as one
+//     MN-major matrix whose 64-coordinate column groups are the K blocks; O takes up to 256
+//     TMEM columns.
+// A product costs the tensor core 40 to 60 cycles however narrow it is, so S wants wide
+// tiles: with 32 columns the 48 products of S took three quarters of a tile's time at d =
+// 256 (1.29 ms per 16384 x 32768 step). 64 columns is what TMEM holds beside X hi and O, and
+// half a P tile what shared memory holds beside two such stages.
 // With hi parts only (split3 = 0) each product is the single hi x hi term and the lo
 // blocks are not loaded. So S is formed once per (row, column) pair, where a map run
 // chunk by chunk forms it once per chunk.
 // Operands in place: the X row block's hi part sits in TMEM (the A operand of the Xh Yh
 // and Xh Yl products, written by warpgroup 1 from the bf16 operand rows at each
-// segment's start), its lo part in shared memory (TMA); so four stages fit, each holding
-// a tile's K blocks (hi and lo) and bias rows from the S products until its P Y~
-// products, and three tiles' copies are in flight while a fourth is in use. The MMA
+// segment's start), its lo part in shared memory (TMA); so two stages (four at d = 128)
+// fit, each holding a tile's K blocks (hi and lo) and bias rows from the S products until
+// its P Y~ products. The MMA
 // warp issues S and P Y~ in whichever order their inputs arrive (S at most one tile
 // ahead), so the exponentials of tile q overlap the products of tile q + 1 and P Y~(q)
 // does not wait for a later copy.
@@ -38,28 +43,29 @@
 namespace progot {
 namespace tc {
 
-constexpr int OP_BN = 32;                      // columns j per tile
+constexpr int OP_BN = 64;                      // columns j per tile
 constexpr int OP_NTHREADS = 320;
-constexpr int OP_TMEM_COLS = 512;              // S buffers [0, 64), X hi [64, 64 + 32 nkb), O [256, 256 + 64 nkb)
-constexpr uint32_t OP_X_COL = 64;
+constexpr int OP_TMEM_COLS = 512;              // S buffers [0, 128), X hi [128, 128 + 32 nkb), O [256, 256 + 64 nkb)
+constexpr uint32_t OP_X_COL = 128;
 constexpr uint32_t OP_O_COL = 256;
 constexpr uint32_t OP_A_TILE = 128 * 64 * 2;   // 16 KB: one K block of the X row block (hi or lo)
-constexpr uint32_t OP_B_TILE = 32 * 64 * 2;    // 4 KB: one K block of a 32-row Y tile (hi or lo)
-constexpr uint32_t OP_BIAS = 32 * 32;          // 1 KB: 32 bias rows x 16 bf16
-constexpr uint32_t OP_P_HALF = 128 * 32 * 2;   // 8 KB: the P tile (hi or lo), 128 rows x 32 bf16
-constexpr int OP_NST = 4;                      // operand stages
+constexpr uint32_t OP_B_TILE = OP_BN * 64 * 2; // 8 KB: one K block of a 64-row Y tile (hi or lo)
+constexpr uint32_t OP_BIAS = OP_BN * 32;       // 2 KB: 64 bias rows x 16 bf16
+constexpr uint32_t OP_P_HALF = 128 * 32 * 2;   // 8 KB: half a P tile (hi or lo), 128 rows x 32 bf16
+constexpr int OP_MAXST = 4;                    // operand stages: as many as fit, two at d = 256
 constexpr int OP_MAXKB = 4;                    // d <= 256
 
 struct OpLayout {
   uint32_t ones, st, st_bytes, st_lo, st_bias, p, ctrl, total;
+  int nst;
 };
 
 struct OpShared {
-  uint64_t full[OP_NST], empty[OP_NST];
+  uint64_t full[OP_MAXST], empty[OP_MAXST];
   uint64_t tmem_full[2], tmem_empty[2];
   uint64_t a_full, a_empty;  // X lo copied / the segment's S products done (X hi, X lo free)
   uint64_t x_full;           // X hi written to TMEM (the 4 warps of warpgroup 1 arrive)
-  uint64_t p_full, p_empty;  // the P buffer written (4 warps arrive) / consumed (commit)
+  uint64_t p_full[2], p_empty[2];  // half h of a tile's P written (4 warps arrive) / consumed (commit)
   uint64_t o_full, o_empty;
   uint64_t drain;
   uint32_t tmem_base;
@@ -71,7 +77,7 @@ struct OpShared {
 };
 
 // X lo (the K blocks of the row block), the ones of the bias product, the stages (K
-// blocks hi, K blocks lo, bias rows), the P tile (hi, lo), the control block; offsets
+// blocks hi, K blocks lo, bias rows), half a P tile (hi, lo), the control block; offsets
 // from a 1024-aligned base.
 __host__ __device__ inline OpLayout op_layout(int nkb) {
   OpLayout L;
@@ -80,7 +86,10 @@ __host__ __device__ inline OpLayout op_layout(int nkb) {
   L.st_lo = (uint32_t)nkb * OP_B_TILE;
   L.st_bias = 2 * L.st_lo;
   L.st_bytes = (L.st_bias + OP_BIAS + 1023) & ~1023u;
-  L.p = L.st + OP_NST * L.st_bytes;
+  const uint32_t fixed = L.st + 2 * OP_P_HALF + (uint32_t)sizeof(OpShared) + 1024;
+  L.nst = (int)((227 * 1024 - fixed) / L.st_bytes);
+  if (L.nst > OP_MAXST) L.nst = OP_MAXST;
+  L.p = L.st + (uint32_t)L.nst * L.st_bytes;
   L.ctrl = L.p + 2 * OP_P_HALF;
   L.total = L.ctrl + (uint32_t)sizeof(OpShared) + 1024;
   return L;
@@ -187,14 +196,14 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
   const OpLayout Lo = op_layout(mp.nkb);
   OpShared& sh = *reinterpret_cast<OpShared*>(smem + Lo.ctrl);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x, G = mp.G, T = mp.T, nkb = mp.nkb;
+  const int c = blockIdx.x, G = mp.G, T = mp.T, nkb = mp.nkb, S = Lo.nst;
   const int dw = nkb * 64;  // coordinates held in O and in a partial slot's row
   const Split sp = make_split(mp.R, T, G);
   const int nseg = num_segments(sp, c);
   volatile int32_t* abort_flag = &sh.abort_flag;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < OP_NST; ++s) {
+    for (int s = 0; s < S; ++s) {
       mbar_init(&sh.full[s], 1);
       mbar_init(&sh.empty[s], 1);
     }
@@ -202,8 +211,10 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
       mbar_init(&sh.tmem_full[s], 1);
       mbar_init(&sh.tmem_empty[s], 4);
     }
-    mbar_init(&sh.p_full, 4);
-    mbar_init(&sh.p_empty, 1);
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(&sh.p_full[h], 4);
+      mbar_init(&sh.p_empty[h], 1);
+    }
     mbar_init(&sh.a_full, 1);
     mbar_init(&sh.a_empty, 1);
     mbar_init(&sh.x_full, 4);
@@ -233,6 +244,8 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
     // ------------------------------------------------------------ producer
     bool ok = true;
     int u = 0, a_issued = 0;  // stage units (tiles) and A loads issued
+    int s_cur = 0;            // ring position and fill parity of unit u
+    uint32_t s_par = 0;
     const uint32_t nh = mp.split3 ? 2u : 1u;  // hi, or hi and lo
     const uint32_t st_tx = nh * (uint32_t)nkb * OP_B_TILE + OP_BIAS;
     for (int k = 0; k < nseg && ok; ++k) {
@@ -249,9 +262,13 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
       __syncwarp();
       a_issued = k + 1;
       for (int t = sg.t0; t < sg.t1 && ok; ++t, ++u) {
-        const int s = u % OP_NST;
-        ok = warp_wait(&sh.empty[s], (uint32_t)(((u / OP_NST) & 1) ^ 1), abort_flag);
+        const int s = s_cur;
+        ok = warp_wait(&sh.empty[s], s_par ^ 1u, abort_flag);
         if (!ok) break;
+        if (++s_cur == S) {
+          s_cur = 0;
+          s_par ^= 1u;
+        }
         unsigned char* st = smem + Lo.st + s * Lo.st_bytes;
         if (elect_one()) {
           mbar_arrive_expect_tx(&sh.full[s], st_tx);
@@ -267,19 +284,18 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
     if (!ok) {
       // drain the copies this CTA still has in flight before shared memory is released
       if (a_issued > 0) warp_wait(&sh.a_full, (uint32_t)((a_issued - 1) & 1), abort_flag, true);
-      for (int v = (u > OP_NST ? u - OP_NST : 0); v < u; ++v)
-        warp_wait(&sh.full[v % OP_NST], (uint32_t)((v / OP_NST) & 1), abort_flag, true);
+      for (int v = (u > S ? u - S : 0); v < u; ++v)
+        warp_wait(&sh.full[v % S], (uint32_t)((v / S) & 1), abort_flag, true);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     // Two streams over the CTA's tiles in order, S(q) and P Y~(q), issued in whichever
-    // order their inputs arrive, S at most one tile ahead of the oldest tile still
-    // without P Y~: so S(q + 1) runs while the exponentials of tile q are computed, and
-    // an LSE warpgroup never waits on the P buffer's barrier more than one phase ahead
-    // of it (a parity wait two phases early would pass on the older phase and overwrite
-    // P before its products read it). The copies run up to three tiles ahead through
-    // the four stages. S and P Y~ write different TMEM columns, so the order of issue
-    // changes no result.
+    // order their inputs arrive, S at most one tile ahead of the oldest tile whose P Y~ is
+    // not all issued: so S(q + 1) runs while the exponentials of tile q are computed, and
+    // an LSE warpgroup never waits on a half's barrier more than one phase ahead of it
+    // (S(q)'s completion follows both halves of P Y~(q - 2); a parity wait two phases early
+    // would pass on the older phase and overwrite P before its products read it). S and
+    // P Y~ write different TMEM columns, so the order of issue changes no result.
     const uint64_t ones = desc_sw32(smem_u32(smem + Lo.ones));
     const int split3 = mp.split3;
     const uint32_t a_lo = smem_u32(smem);
@@ -298,7 +314,9 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
     int ts = sgs.t0;
     bool a_pending = true;  // the segment's A row block not yet seen
     // P Y~ stream
-    int kp = 0, qp = 0, oseg = 0;
+    int kp = 0, qp = 0, oseg = 0, half = 0;  // qp: the oldest tile with a half of P Y~ to come
+    int ss_cur = 0, ps_cur = 0;  // stages of the two streams' next tiles
+    uint32_t ss_par = 0;
     Seg sgp = sgs;
     int tpp = sgp.t0;
     unsigned long long t_idle = 0;
@@ -309,11 +327,11 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
         bool r = !a_pending ||
                  (op_test_wait(&sh.a_full, (uint32_t)(ks & 1)) && op_test_wait(&sh.x_full, (uint32_t)(ks & 1)));
         r = r && op_test_wait(&sh.tmem_empty[qs & 1], (uint32_t)(((qs >> 1) & 1) ^ 1));
-        r = r && op_test_wait(&sh.full[qs % OP_NST], (uint32_t)((qs / OP_NST) & 1));
+        r = r && op_test_wait(&sh.full[ss_cur], ss_par);
         if (__all_sync(0xffffffffu, r)) {
           tc_fence_after();
           const int b = qs & 1;
-          const uint32_t st = smem_u32(smem + Lo.st + (qs % OP_NST) * Lo.st_bytes);
+          const uint32_t st = smem_u32(smem + Lo.st + ss_cur * Lo.st_bytes);
           const uint32_t d_tmem = tmem_base + (uint32_t)(b * OP_BN);
           const bool seg_end = (ts == sgs.t1 - 1);
           if (elect_one()) {
@@ -339,6 +357,10 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
           __syncwarp();
           a_pending = false;
           ++qs;
+          if (++ss_cur == S) {
+            ss_cur = 0;
+            ss_par ^= 1u;
+          }
           if (++ts == sgs.t1 && ++ks < nseg) {
             sgs = segment(sp, c, ks);
             ts = sgs.t0;
@@ -348,15 +370,16 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
         }
       }
       if (qp < qs) {
-        // O += P Y~ over every coordinate, from the P buffer and the tile's stage (its K
-        // blocks are the B operand's column groups); the stage and P go back after it
-        const bool first = (tpp == sgp.t0), last = (tpp == sgp.t1 - 1);
+        // O += P Y~ over every coordinate for 32 of the tile's columns, from the P buffer and
+        // the tile's stage (its K blocks are the B operand's column groups); P goes back after
+        // it, the stage after the second half
+        const bool first = (tpp == sgp.t0) && half == 0, last = (tpp == sgp.t1 - 1);
         bool r = !(first && oseg > 0) || op_test_wait(&sh.o_empty, (uint32_t)((oseg - 1) & 1));
-        r = r && op_test_wait(&sh.p_full, (uint32_t)(qp & 1));
+        r = r && op_test_wait(&sh.p_full[half], (uint32_t)(qp & 1));
         if (__all_sync(0xffffffffu, r)) {
           tc_fence_after();
-          const int stage = qp % OP_NST;
-          const uint32_t st = smem_u32(smem + Lo.st + stage * Lo.st_bytes);
+          const int stage = ps_cur;
+          const uint32_t st = smem_u32(smem + Lo.st + stage * Lo.st_bytes) + (uint32_t)half * 4096u;
           const uint64_t ah = op_desc_sw64(p0), al = op_desc_sw64(p0 + OP_P_HALF);
           if (elect_one()) {
             const uint64_t bh = op_desc_mn(st), bl = op_desc_mn(st + Lo.st_lo);
@@ -371,16 +394,22 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
                 op_umma(d_o, al + adv, bh + bdv, id_py, 1u);
               }
             }
-            umma_commit(&sh.p_empty);
-            umma_commit(&sh.empty[stage]);
-            if (last) umma_commit(&sh.o_full);
+            umma_commit(&sh.p_empty[half]);
+            if (half == 1) {
+              umma_commit(&sh.empty[stage]);
+              if (last) umma_commit(&sh.o_full);
+            }
           }
           __syncwarp();
-          if (last) ++oseg;
-          ++qp;
-          if (++tpp == sgp.t1 && ++kp < nseg) {
-            sgp = segment(sp, c, kp);
-            tpp = sgp.t0;
+          half ^= 1;
+          if (half == 0) {
+            if (last) ++oseg;
+            ++qp;
+            if (++ps_cur == S) ps_cur = 0;
+            if (++tpp == sgp.t1 && ++kp < nseg) {
+              sgp = segment(sp, c, kp);
+              tpp = sgp.t0;
+            }
           }
           progressed = true;
         }
@@ -444,35 +473,38 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
         }
         tc_fence_after();
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(wg * OP_BN);
-        float v[32];
+        float v[64];
         PROGOT_TMEM_LD32(taddr, v);
+        PROGOT_TMEM_LD32(taddr + 32, (v + 32));
         tmem_wait_ld();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.tmem_empty[wg]);
         // P_ij = 2^{t_ij - L_i} (0 on rows past the cloud)
 #pragma unroll
-        for (int e = 0; e < 32; ++e) {
+        for (int e = 0; e < 64; ++e) {
           const float pv = row_ok ? fast_exp2(v[e] - Lr) : 0.f;
           v[e] = pv;
           rs += pv;
         }
-        // the P buffer is free once the previous tile's P Y~ has read it
-        if (!warp_wait(&sh.p_empty, (uint32_t)((tl & 1) ^ 1), abort_flag)) {
-          dead = true;
-          continue;
-        }
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          uint4 hi, lo;
-          op_split8(&v[ch * 8], hi, lo);
-          const int pos = (ch ^ pswz) * 16;
-          *reinterpret_cast<uint4*>(prow + pos) = hi;
-          *reinterpret_cast<uint4*>(prow + OP_P_HALF + pos) = lo;
+        for (int h = 0; h < 2; ++h) {
+          // the P buffer is free once the products of the half before have read it: the
+          // previous tile's second half, then this tile's first
+          if (!dead && !warp_wait(&sh.p_empty[h ^ 1], (uint32_t)(h == 0 ? (tl & 1) ^ 1 : tl & 1), abort_flag)) dead = true;
+          if (dead) break;
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            uint4 hi, lo;
+            op_split8(&v[h * 32 + ch * 8], hi, lo);
+            const int pos = (ch ^ pswz) * 16;
+            *reinterpret_cast<uint4*>(prow + pos) = hi;
+            *reinterpret_cast<uint4*>(prow + OP_P_HALF + pos) = lo;
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.p_full[h]);
         }
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.p_full);
       }
       // ---- segment done: row sums of both warpgroups, O out of TMEM, partial slot
       if (wg == 1) sh.rs[k & 1][row_local] = rs;
@@ -554,6 +586,7 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
             float4 acc[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
             for (int q2 = 0; q2 < nc; ++q2) {
               int64_t sl;
               if (q2 < 8) {
@@ -621,7 +654,7 @@ __global__ void __launch_bounds__(OP_NTHREADS, 1)
 }  // namespace tc
 
 bool map_tc_onepass_supported(int nkb) {
-  return nkb >= 2 && nkb <= tc::OP_MAXKB && tc::op_layout(nkb).total <= 227 * 1024;
+  return nkb >= 2 && nkb <= tc::OP_MAXKB && tc::op_layout(nkb).nst >= 2;
 }
 
 int map_tc_onepass_tile_cols() { return tc::OP_BN; }

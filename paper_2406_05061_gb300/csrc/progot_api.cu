@@ -446,8 +446,8 @@ struct TcOps {
   CUtensorMap xh_a, xl_a, yh_a, yl_a, xh_b, xl_b, yh_b, yl_b, xb, yb;
   // tensor-core map step (dp = 64): y-side bias rows in 128-row boxes
   CUtensorMap yb128;
-  // tensor-core map step for 64 < d <= 256: y operand and bias rows in 32-row boxes
-  CUtensorMap yh_m32, yl_m32, yb_m32;
+  // tensor-core map step for 64 < d <= 256: y operand and bias rows in boxes of one map tile (64 rows)
+  CUtensorMap yh_mt, yl_mt, yb_mt;
   // integer-grid split: third parts in both roles
   CUtensorMap xr_a, yr_a, xr_b, yr_b;
   const float* gscale = nullptr;  // its device scales (non-NULL: the operands are the grid split's)
@@ -477,7 +477,7 @@ static int map_y_bias(TcOps* ops, void* base, int64_t m) {
   int rc = make_map(&ops->yb, base, rows, 16, ops->bn);
   if (!rc && !ops->gscale && ops->nkb == 1) rc = make_map(&ops->yb128, base, rows, 16, 128);
   if (!rc && !ops->gscale && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb))
-    rc = make_map(&ops->yb_m32, base, rows, 16, map_tc_onepass_tile_cols());
+    rc = make_map(&ops->yb_mt, base, rows, 16, map_tc_onepass_tile_cols());
   return rc;
 }
 
@@ -619,8 +619,8 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   if (!rc) rc = map_y_bias(ops, ws.yb, m);
   if (!rc && !grid && dp > 64 && map_tc_onepass_supported(ops->nkb)) {
     const int bt = map_tc_onepass_tile_cols();
-    rc = make_map(&ops->yh_m32, ws.yh, m, dp, bt);
-    if (!rc) rc = make_map(&ops->yl_m32, yl, m, dp, bt);
+    rc = make_map(&ops->yh_mt, ws.yh, m, dp, bt);
+    if (!rc) rc = make_map(&ops->yl_mt, yl, m, dp, bt);
   }
   return rc;
 }
@@ -1144,7 +1144,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     ProfRec r;
     const bool rec = prof_begin(r, s, kProfMap);
     CK(launch_map_sweep_tc_onepass(X, X, ws.L, n, m, d, ops->nkb, (float)alpha, &ops->xl_a,
-                                   &ops->yh_m32, &ops->yl_m32, &ops->yb_m32, (float)std::sqrt(eps / (2.0 * kLog2e)),
+                                   &ops->yh_mt, &ops->yl_mt, &ops->yb_mt, (float)std::sqrt(eps / (2.0 * kLog2e)),
                                    ops->mu, ws.xh, ws.Opart, ws.Rpart, ws.mcnt, G, maxseg, ops->split3, ws.fault, s));
     if (rec) prof_end(r, s, kProfMap, (double)n * (double)m);
     if (t_prof.on) t_prof.worked[kProfMap] += 1;

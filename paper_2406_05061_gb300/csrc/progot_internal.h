@@ -174,8 +174,8 @@ cudaError_t launch_map_sweep_tc(const float* X, float* out, const float* L, int6
                                 float* Opart, float* Rpart, unsigned* cnt, int G, int maxseg, int32_t split3,
                                 int32_t* fault, cudaStream_t stream);
 size_t map_sweep_tc_smem();
-// The same for 64 < d <= 256 in one pass (map_tc_onepass.cu): tiles of 32 columns (B maps
-// and bias rows in 32-row boxes) whose K blocks all stay in one stage, S formed once per
+// The same for 64 < d <= 256 in one pass (map_tc_onepass.cu): tiles of 64 columns (B maps
+// and bias rows in 64-row boxes) whose K blocks all stay in one stage, S formed once per
 // tile and every chunk of 64 output coordinates accumulated in TMEM; Opart slots hold
 // 128 rows x 64 nkb floats. xh is the bf16 hi operand of X (nA x 64 nkb, the buffer the
 // A maps describe), read directly into TMEM.

@@ -1073,8 +1073,10 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
   const bool grid = gscale != nullptr;
   int stages, a_bufs;
   tc_shape(bn, nkb, parts, grid, &stages, &a_bufs);
-  // 128-column bf16 tiles of up to four K blocks: A in TMEM, all of shared memory for stages
-  const bool atm = !grid && bn == 128 && nkb <= 4 && maps.a_part[0] != nullptr;
+  // 128-column bf16 tiles of up to four K blocks and many of them per CTA: A in TMEM, all of
+  // shared memory for stages (the rule of the persistent loop)
+  const int64_t tiles = ((p.nA + tc::BM - 1) / tc::BM) * ((p.nB + bn - 1) / bn);
+  const bool atm = !grid && bn == 128 && nkb <= 4 && maps.a_part[0] != nullptr && tiles >= 64 * (int64_t)G;
   if (atm) {
     a_bufs = 0;
     stages = tc_stages_atm(nkb, parts);
