@@ -404,7 +404,8 @@ __device__ __forceinline__ Seg seg_at(const Side& Sd, int c, int k, int maxseg) 
 // needs to put the next one's operands in place beside the LSE warps (a probe: 90 cycles a
 // product against 71): with the converged warp 16384^2 sweeps took 145 us instead of 164
 // (grid, d = 64) and 248 instead of 290 (d = 256). N = 256 products are long enough.
-template <int BN, int NKB, int GRID, int ATM, int CONV>
+// KS: K = 16 steps of a bf16 K block when NKB = 1 (the padding up to 64 multiplies zeros).
+template <int BN, int NKB, int GRID, int ATM, int CONV, int KS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     sinkhorn_loop_tc(const __grid_constant__ CUtensorMap mXh_a, const __grid_constant__ CUtensorMap mXl_a,
                      const __grid_constant__ CUtensorMap mYh_a, const __grid_constant__ CUtensorMap mYl_a,
@@ -677,7 +678,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     }
                   } else
 #pragma unroll
-                  for (int kk = 0; kk < KB / 16; ++kk) {
+                  for (int kk = 0; kk < KS; ++kk) {
                     // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
                     const uint64_t adv = (uint64_t)(kk * 2);
                     umma<BN>(d_tmem, ah + adv, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
@@ -1059,11 +1060,11 @@ void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg) {
   *maxseg = ms;
 }
 
-template <int BN, int NKB, int GRID, int ATM = 0, int CONV = 0>
+template <int BN, int NKB, int GRID, int ATM = 0, int CONV = 0, int KS = 4>
 static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const void* const* maps, cudaStream_t stream) {
   static thread_local size_t attr_bytes = 0;
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV>,
+    cudaError_t e = cudaFuncSetAttribute(tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV, KS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
@@ -1080,7 +1081,7 @@ static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const voi
   cfg.numAttrs = 1;
   const CUtensorMap* m[16];
   for (int q = 0; q < 16; ++q) m[q] = reinterpret_cast<const CUtensorMap*>(maps[q]);
-  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
+  return cudaLaunchKernelEx(&cfg, tc::loop::sinkhorn_loop_tc<BN, NKB, GRID, ATM, CONV, KS>, *m[0], *m[1], *m[2], *m[3], *m[4], *m[5],
                             *m[6], *m[7], *m[8], *m[9], *m[10], *m[11], *m[12], *m[13], *m[14], *m[15], P);
 }
 
@@ -1158,7 +1159,10 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   else
     e = a_bufs == 0    ? launch_loop<128, 0, 0, 1, 1>(P, smem, Lq.maps, stream)
         : Lq.bn == 128 ? launch_loop<128, 0, 0, 0, 1>(P, smem, Lq.maps, stream)
-        : Lq.nkb == 1  ? launch_loop<256, 1, 0>(P, smem, Lq.maps, stream)
+        : Lq.nkb == 1  ? (ks <= 1   ? launch_loop<256, 1, 0, 0, 0, 1>(P, smem, Lq.maps, stream)
+                          : ks == 2 ? launch_loop<256, 1, 0, 0, 0, 2>(P, smem, Lq.maps, stream)
+                          : ks == 3 ? launch_loop<256, 1, 0, 0, 0, 3>(P, smem, Lq.maps, stream)
+                                    : launch_loop<256, 1, 0>(P, smem, Lq.maps, stream))
                        : launch_loop<256, 0, 0>(P, smem, Lq.maps, stream);
   count_launch();
   return e;

@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(MT_NTHREADS, 1)
     // ------------------------------------------------------------ MMA issuer
     const uint64_t ones = desc_sw32(smem_u32(smem + MT_OFF_ONES));
     const int split3 = mp.split3;
+    const int ksteps = (mp.d + 15) / 16;  // K = 16 steps that hold coordinates
     const uint32_t a_hi = smem_u32(smem + MT_OFF_A), a_lo = a_hi + MT_TILE;
     const uint32_t p0 = smem_u32(smem + MT_OFF_P);
     bool ok = true;
@@ -278,8 +279,7 @@ __global__ void __launch_bounds__(MT_NTHREADS, 1)
         const uint64_t bh = desc_sw128(st), bl = desc_sw128(st + MT_TILE), bb = desc_sw32(st + 2 * MT_TILE);
         const uint32_t d_tmem = tmem_base + (uint32_t)(b * MT_BN);
         if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
+          for (int kk = 0; kk < ksteps; ++kk) {
             const uint64_t adv = (uint64_t)(kk * 2);
             umma<MT_BN>(d_tmem, ah + adv, bh + adv, kk > 0 ? 1u : 0u);
             if (split3) {

@@ -670,8 +670,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               }
             }
           } else if (elect_one()) {
-#pragma unroll
-            for (int kk = 0; kk < KB / 16; ++kk) {
+            // K = 16 steps that hold coordinates (the padding up to 64 multiplies zeros)
+            const int ksteps = min(KB / 16, (p.d - kb * KB + 15) / 16);
+            for (int kk = 0; kk < ksteps; ++kk) {
               // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
               const uint64_t adv = (uint64_t)(kk * 2);
               umma<BN>(d_tmem, ah + adv, bh + adv, (kb > 0 || kk > 0) ? 1u : 0u);
