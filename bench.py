@@ -853,18 +853,20 @@ def main():
     sms = props.multi_processor_count
     avg_ms = lse["ms"] / max(1, lse["launches"])
     pairs_per_launch = lse["pairs"] / max(1, lse["launches"])
-    if args.precision == "fp32":
+    # the float32 path's loops run on the tensor cores up to d = 64 (six half-precision products)
+    cuda_cores = args.precision == "fp32" and p.d > 64
+    if cuda_cores:
         flops_pair = 2.0 * p.d
         peak = sms * 128 * 2 * sm_max_ghz * 1e9 / 1e12  # TFLOP/s, FP32 FMA pipe
         bound, peak_src = "alu", f"derived: {sms} SMs x 128 FP32 FMA/clk x 2 flop x {sm_max_ghz:.2f} GHz"
     else:
-        split = 3.0 if args.precision == "bf16x3" else 1.0
+        split = {"fp32": 6.0, "bf16x3": 3.0, "bf16": 1.0}[args.precision]
         flops_pair = 2.0 * p.d * split
         # burst: the sweeps are timed inside sub-second runs at full clock
         peak = float(peaks.get("bf16_tflops", 1900.0))
         bound, peak_src = "tensor", f"{peaks['source']} bf16_tflops (burst)"
     achieved = flops_pair * pairs_per_launch / (avg_ms / 1e3) / 1e12
-    kernel = "lse_sweep_fp32" if args.precision == "fp32" else "sinkhorn_loop_tc"
+    kernel = "lse_sweep_fp32" if cuda_cores else "sinkhorn_loop_tc"
     sweeps_per_solve = (lse["worked"] + mp["worked"]) / args.steps
     roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": captured_traffic(kernel, args.workload, args.precision),

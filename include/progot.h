@@ -25,11 +25,16 @@
  * - stream: a cudaStream_t (NULL = legacy default stream). Entry points that return
  *   host results (iteration counts, errors) synchronise that stream before
  *   returning; the others are asynchronous.
- * - precision: PROGOT_FP32 evaluates the cross term x . y with float32 FMAs on CUDA
- *   cores; PROGOT_BF16X3 uses tcgen05 tensor cores on a bf16 hi/lo split of both
- *   operands (x.y ~ xh.yh + xh.yl + xl.yh, float32 accumulation); PROGOT_BF16 uses the
- *   hi parts only. Log-sum-exps and potentials are float32 in every mode; squared norms
- *   and the marginal-error reduction accumulate in float64.
+ * - precision: PROGOT_FP32 has float32 accuracy throughout. Sinkhorn loops up to d = 64,
+ *   map steps, marginals and metrics form the cross term x . y on the tcgen05 tensor cores
+ *   from half-precision parts whose leading products add exactly (error at or below a
+ *   float32 FMA chain's); loops beyond d = 64, small map queries and workspaces smaller than
+ *   progot_workspace_size (down to what the CUDA cores need) use float32 FMAs.
+ *   PROGOT_BF16X3 uses tcgen05 tensor cores on a bf16 hi/lo split of both operands
+ *   (x.y ~ xh.yh + xh.yl + xl.yh, float32 accumulation; map steps beyond d = 256 as
+ *   PROGOT_FP32's); PROGOT_BF16 uses the hi parts only. Log-sum-exps and potentials are
+ *   float32 in every mode; squared norms and the marginal-error reduction accumulate in
+ *   float64 or without rounding loss.
  * - Return value: PROGOT_OK or an error code below. progot_last_error_string()
  *   describes the last error on the calling thread. On PROGOT_ERR_NOT_CONVERGED all
  *   outputs are still written (the last iterate).
@@ -383,8 +388,9 @@ typedef struct progot_coupling_metrics {
 } progot_coupling_metrics;
 
 /*
- * coupling_metrics - the metrics above from two float32 CUDA-core sweeps (one over rows,
- * one over columns) that never store P. The row sweep carries, besides the row
+ * coupling_metrics - the metrics above from two sweeps (one over rows, one over columns;
+ * on the tensor cores at float32 accuracy, on float32 CUDA cores with the p-norm, with
+ * x_cost, or in a workspace of the least size) that never store P. The row sweep carries, besides the row
  * log-sum-exp, the 2^t-weighted mean of t_ij (t_ij = log2 of the row's terms), which
  * gives sum_j P_ij log P_ij per row; then <P, C> = <f, P 1> + <g, P^T 1> - eps
  * sum P log P. All reductions are float64 in a fixed order (deterministic).
@@ -432,7 +438,8 @@ int coupling_diagonal(const float* x, const float* y, int64_t n, int32_t d, cons
  * The p-norm cost of the coupling experiments (Sec. 5.2): c(x, y) = h(x - y) with
  * h(z) = (1/p) sum_k |z_k|^p, 1 < p <= 8 (the paper uses p = 1.5, which has a
  * specialised kernel; other p go through 2^(p log2 |z|)). There is no product form, so
- * these entry points run on float32 CUDA cores: every pair term is summed coordinate by
+ * these entry points run on float32 CUDA cores (a loop keeps the cost in the workspace when
+ * it fits in 128 MB there): every pair term is summed coordinate by
  * coordinate, and the map step evaluates grad h(z)_k = sign(z_k) |z_k|^(p-1) for every
  * pair and coordinate and moves x by grad h*(w)_k = sign(w_k) |w_k|^(1/(p-1)):
  *   Z_i = grad h*(sum_j Q_ij grad h(x_i - y_j)), x_i <- x_i - alpha_k Z_i   (Alg. 2, Alg. 3).
@@ -475,13 +482,12 @@ int progot_mean_cost_pnorm(const float* x, int64_t n, const float* y, int64_t m,
 int progot_set_stall_window(int32_t iters);
 
 /*
- * progot_set_map_tc - choose the kernel of the map step (Alg. 2 / Alg. 3) on the
- * tensor-core paths (PROGOT_BF16X3, PROGOT_BF16) for d <= 256: 1 (default) runs S = X Y^T
- * and P Y on tcgen05 (P and the centred, scaled Y in bf16 hi/lo, three products with
- * PROGOT_BF16X3 and one with PROGOT_BF16, float32 accumulation in TMEM; for 64 < d <= 256
- * in one pass over Y with every output coordinate in TMEM); 0 runs P Y on float32 CUDA
- * cores after the tensor-core LSE pass (the path for d > 256 and PROGOT_FP32).
- * Process-wide setting.
+ * progot_set_map_tc - choose the kernel of the map step (Alg. 2 / Alg. 3) where the
+ * operands are on the tensor cores: 1 (default) runs S = X Y^T and P Y on tcgen05 (mixed
+ * precisions, d <= 256: P and the centred, scaled Y in bf16 hi/lo, three products with
+ * PROGOT_BF16X3 and one with PROGOT_BF16, in one kernel; PROGOT_FP32, and d > 256 at the
+ * mixed precisions: half-precision parts, P through memory a chunk of rows at a time); 0
+ * runs P Y on float32 CUDA cores after the tensor-core LSE pass. Process-wide setting.
  */
 int progot_set_map_tc(int32_t on);
 

@@ -1,6 +1,7 @@
 // Host orchestration of the ProgOT hot path and its C ABI (include/progot.h).
 //
-// The Sinkhorn loop of Alg. 1 runs without a host round trip per iteration: every
+// Where the operands are on the tensor cores (prep_tc), a Sinkhorn loop of Alg. 1 is one
+// persistent launch. Elsewhere it runs without a host round trip per iteration: every
 // f-sweep measures the row-marginal error of the current (f, g) in its epilogue and the
 // stop test runs on the device (SolverState): in the f-sweep's last CTA, or, in
 // tensor-core loops, in the g-sweep that follows (SweepParams::lag). Later sweeps of a

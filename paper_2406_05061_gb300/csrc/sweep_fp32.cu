@@ -14,6 +14,9 @@
 // map_sweep_fp32: the barycentric projection of Alg. 2 / Alg. 3: with L_i known,
 //   T_i = sum_j 2^{t_ij - L_i} y_j / sum_j 2^{t_ij - L_i},
 //   x_i <- x_i + alpha (T_i - x_i).
+//
+// With the squared cost these serve float32 loops beyond d = 64, small float32 queries and
+// workspaces without room for the tensor-core operands; the p-norm costs always run here.
 #include <algorithm>
 
 #include "progot_common.cuh"

@@ -531,8 +531,8 @@ def progot_schedule_eps(x, y, y_test, alpha, s_grid=None, beta0=5.0, tau=1e-6, m
 
 
 def set_map_tc(on: bool) -> None:
-    """Map step of the tensor-core paths (d <= 64) on tcgen05 (True, default) or with a
-    float32 CUDA-core P Y (False)."""
+    """Map step of the tensor-core paths on tcgen05 (True, default) or with a float32
+    CUDA-core P Y (False)."""
     _check(lib().progot_set_map_tc(1 if on else 0), allow_not_converged=False)
 
 
