@@ -150,12 +150,20 @@ __global__ void __launch_bounds__(32 * kCenterWarps)
 
 // Tables and initial words of a persistent loop (loop_tc.cu): CTA c's segments, a row
 // block's contributors (offset, count): row block r of the remainder starts at slot
-// first contributor + r, which leaves a gap of at most one slot between row blocks.
+// first contributor + r, which leaves a gap of at most one slot between row blocks; in an
+// aligned split CTA c's only segment has slot c.
 __device__ void loop_setup(const LoopSetup& ls, int64_t tid, int64_t nthreads) {
   for (int sd = 0; sd < 2; ++sd) {
     const LoopSetupSide& S = ls.side[sd];
     const tc::Split sp = tc::make_split(S.R, S.T, ls.G);
     for (int64_t c = tid; c < ls.G; c += nthreads) {
+      if (ls.aligned) {
+        const tc::Seg sg = tc::aligned_segment(S.R, S.T, ls.G, (int)c);
+        S.nseg[c] = 1;
+        reinterpret_cast<int4*>(S.segs)[c] = make_int4(sg.r, sg.t0, sg.t1, 0);
+        S.cslot[c] = (int)c;
+        continue;
+      }
       const int ns = tc::num_segments(sp, (int)c);
       S.nseg[c] = ns;
       int4* segs = reinterpret_cast<int4*>(S.segs) + c * ls.maxseg;
@@ -165,11 +173,16 @@ __device__ void loop_setup(const LoopSetup& ls, int64_t tid, int64_t nthreads) {
       }
     }
     for (int64_t r = tid; r < S.R; r += nthreads) {
-      int c0, c1;
-      tc::contributors(sp, (int)r, &c0, &c1);
-      const int off = r < (int64_t)sp.nb * sp.G ? (int)r : (int)r + c0;
-      S.crow[r] = make_int2(off, c1 - c0 + 1);
-      for (int cc = c0; cc <= c1; ++cc) S.cslot[off + cc - c0] = cc * ls.maxseg + tc::seg_of(sp, (int)r, cc);
+      if (ls.aligned) {
+        const int c0 = tc::aligned_begin(S.R, ls.G, (int)r);
+        S.crow[r] = make_int2(c0, tc::aligned_begin(S.R, ls.G, (int)r + 1) - c0);
+      } else {
+        int c0, c1;
+        tc::contributors(sp, (int)r, &c0, &c1);
+        const int off = r < (int64_t)sp.nb * sp.G ? (int)r : (int)r + c0;
+        S.crow[r] = make_int2(off, c1 - c0 + 1);
+        for (int cc = c0; cc <= c1; ++cc) S.cslot[off + cc - c0] = cc * ls.maxseg + tc::seg_of(sp, (int)r, cc);
+      }
       S.flag[r] = S.flag_init;
       S.cnt[r] = 0ull;
     }

@@ -464,7 +464,7 @@ struct TcOps {
   bool on = false;
   // a persistent loop was set up with the operands, over G CTAs of up to maxseg segments
   bool loop = false;
-  int G = 0, maxseg = 0;
+  int G = 0, maxseg = 0, aligned = 0;
   void* yb_base = nullptr;  // the y-side bias rows in use (the maps below describe them)
   // ws.L holds the row log-sum-exps of t against the y-side bias rows (the map step's
   // stabiliser), written by the persistent loop from its last f-update
@@ -490,6 +490,7 @@ static LoopSetup loop_setup_params(int64_t n, int64_t m, const TcOps& ops, const
   ls.state = ws.state;
   ls.G = ops.G;
   ls.maxseg = ops.maxseg;
+  ls.aligned = ops.aligned;
   const int64_t rows[2] = {n, m}, cols[2] = {m, n};
   for (int sd = 0; sd < 2; ++sd) {
     LoopSetupSide& S = ls.side[sd];
@@ -579,7 +580,7 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   LoopSetup ls;
   if (loop && loop_tc_supported(ops->bn, ops->nkb, ops->split3, grid)) {
     ops->loop = true;
-    loop_tc_plan(n, m, ops->bn, num_sms(), &ops->G, &ops->maxseg);
+    loop_tc_plan(n, m, ops->bn, num_sms(), &ops->G, &ops->maxseg, &ops->aligned);
     if ((int64_t)ops->G * ops->maxseg > ws.lslots)
       return fail(PROGOT_ERR_WORKSPACE, "persistent loop needs %lld partial slots, the workspace has %lld",
                   (long long)ops->G * ops->maxseg, (long long)ws.lslots);

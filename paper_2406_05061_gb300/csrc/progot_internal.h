@@ -153,6 +153,7 @@ struct LoopSetup {
   LoopSetupSide side[2];
   SolverState* state;       // [2]
   int32_t G, maxseg;
+  int32_t aligned;          // every CTA on one row block (tc::aligned_segment)
 };
 // kGridHull: the integer grid for clouds inside the hull of the two that the last kGrid call
 // on this workspace saw (same mu and gmax).
@@ -237,6 +238,6 @@ size_t workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision);
 int fail_message(int code, const char* msg);  // sets the last-error text, returns code
 bool loop_tc_supported(int bn, int nkb, int split3, bool grid);
 
-void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg);
+void loop_tc_plan(int64_t n, int64_t m, int bn, int sms, int* G, int* maxseg, int* aligned);
 
 }  // namespace progot

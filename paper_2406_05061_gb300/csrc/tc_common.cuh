@@ -296,6 +296,33 @@ __host__ __device__ inline int seg_of(const Split& s, int r, int cc) {
   return s.nb + (r - s.nb * s.G) - (int)div_small(work_begin(s, cc), s.T);
 }
 
+// Aligned split of the persistent loop, for R <= G <= R T: every CTA works on one row block.
+// Row block r belongs to CTAs aligned_begin(r) .. aligned_begin(r + 1) - 1 (floor or ceil of
+// G / R of them), which share its T tiles evenly.
+__host__ __device__ inline int aligned_begin(int R, int G, int r) { return (int)div_small((int64_t)r * G, R); }
+__host__ __device__ inline Seg aligned_segment(int R, int T, int G, int c) {
+  Seg sg;
+  sg.r = (int)div_small((int64_t)(c + 1) * R - 1, G);
+  const int c0 = aligned_begin(R, G, sg.r), k = aligned_begin(R, G, sg.r + 1) - c0;
+  sg.t0 = (int)div_small((int64_t)(c - c0) * T, k);
+  sg.t1 = (int)div_small((int64_t)(c - c0 + 1) * T, k);
+  return sg;
+}
+// The fewest CTAs (at most g) whose aligned splits of both sweeps, Rx x Ty and Ry x Tx, give no
+// CTA more tiles than the contiguous split's busiest one over g CTAs has; 0 where there is no such
+// number, or where the contiguous split is the better one: with five tiles or more a CTA streams
+// across a row block's end, and an aligned split whose busiest CTA has over half a tile more than
+// the mean costs more than the crossings (3500^2, d = 256, 128-column tiles, 6 against 5.2: 18.7
+// against 17.8 us per sweep; float32 d = 64: 14.2 against 13.85).
+inline int aligned_ctas(int64_t Rx, int64_t Ty, int64_t Ry, int64_t Tx, int64_t g) {
+  const int64_t px = (Rx * Ty + g - 1) / g, py = (Ry * Tx + g - 1) / g;
+  if (px > 4 && 2 * (px * g - Rx * Ty) > g) return 0;
+  if (py > 4 && 2 * (py * g - Ry * Tx) > g) return 0;
+  const int64_t gx = Rx * ((Ty + px - 1) / px), gy = Ry * ((Tx + py - 1) / py);
+  const int64_t G = gx > gy ? gx : gy;
+  return G <= g ? (int)G : 0;
+}
+
 // Named barriers: 1 = both LSE warpgroups (256 threads), 2 = LSE warpgroup 0 (128).
 // Arrival on a grid-wide counter with acquire-release semantics at GPU scope: orders
 // this CTA's prior writes (made visible to the calling thread by a CTA barrier) before

@@ -132,3 +132,32 @@ def test_persistent_loop_bounded_wait_expires_and_context_survives(nat):
     assert marginal_l1(p.x, p.y, host(r.f), host(r.g), eps) <= TOL_MIXED
     assert map_rms_rel(O.entropic_map(p.x, p.y, host(r.g), eps), O.entropic_map(p.x, p.y, ref.g, eps),
                        p.y) <= TOL_MIXED
+
+
+@pytest.mark.parametrize("n,m,d,prec", [(1777, 3001, 16, "bf16x3"), (3000, 1000, 17, "fp32"), (700, 2600, 64, "fp32"),
+                                        (2000, 1900, 256, "bf16x3"), (4700, 4700, 48, "bf16x3"),
+                                        (2049, 5000, 128, "bf16x3"), (3500, 3500, 33, "fp32")])
+def test_split_of_the_loop_matches_per_update_path(nat, n, m, d, prec):
+    """Sizes on both sides of the rule that gives each CTA one row block (uneven shares, a
+    partial last tile, more CTAs than one side needs), against one launch per update after as
+    many iterations. Both compute the same updates from the same clouds; each rounds t_ij
+    (|t| <= 4 T / ln 2 + 32, T = max |x~|^2 / eps) and its sums, a few 2^-23 each, per update,
+    and the float32 path's launches per update use uncentred norms, rounded at 2^-24."""
+    p = W.gmm_pair(n, m, d, seed=n + d, k=4)
+    eps, its = 0.05 * O.mean_cost(p.x[:500], p.y[:500]), 7
+    x64, y64 = p.x.astype(np.float64), p.y.astype(np.float64)
+    mu = 0.5 * (x64.mean(0) + y64.mean(0))
+    r2 = max(((x64 - mu) ** 2).sum(1).max(), ((y64 - mu) ** 2).sum(1).max())
+    tol = 2 * its * eps * 2.0 ** -21 * (4.0 * r2 / eps + 16.0) + \
+        2.0 ** -21 * float((x64 ** 2).sum(1).max() + (y64 ** 2).sum(1).max())
+    x, y = dev(p.x), dev(p.y)
+    out = []
+    try:
+        for on in (True, False):
+            nat.set_loop_tc(on)
+            out.append(nat.sinkhorn_potentials(x, y, eps, 0.0, max_iter=its, precision=prec))
+    finally:
+        nat.set_loop_tc(True)
+    assert out[0].iters == out[1].iters == its
+    np.testing.assert_allclose(host(out[0].f), host(out[1].f), rtol=0, atol=tol)
+    np.testing.assert_allclose(host(out[0].g), host(out[1].g), rtol=0, atol=tol)

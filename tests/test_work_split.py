@@ -22,3 +22,16 @@ def test_work_split_covers_every_unit_once(tmp_path):
     out = subprocess.run([exe], capture_output=True, text=True, timeout=600)
     assert out.returncode == 0, out.stdout + out.stderr
     assert "work split ok" in out.stdout
+
+
+def test_aligned_split_covers_every_row_block_once(tmp_path):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    exe = str(tmp_path / "aligned_split_check")
+    src = os.path.join(ROOT, "tests", "host", "aligned_split_check.cu")
+    subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-o", exe, src],
+                   check=True, capture_output=True, timeout=600)
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0, out.stdout + out.stderr
+    assert "aligned split ok" in out.stdout
