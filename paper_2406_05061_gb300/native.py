@@ -214,10 +214,11 @@ def sinkhorn_potentials(x, y, eps, tau, max_iter=10000, a=None, b=None, f=None, 
     n, d = x.shape
     m = y.shape[0]
     init_zero = 1 if (f is None and g is None) else 0
+    alloc = torch.empty if init_zero else torch.zeros  # the library zeroes both with init_zero
     if f is None:
-        f = torch.zeros(n, dtype=torch.float32, device=x.device)
+        f = alloc(n, dtype=torch.float32, device=x.device)
     if g is None:
-        g = torch.zeros(m, dtype=torch.float32, device=x.device)
+        g = alloc(m, dtype=torch.float32, device=x.device)
     ws = _ws(workspace, n, m, d, precision)
     it = ctypes.c_int32(0)
     err = ctypes.c_double(0.0)
@@ -400,10 +401,11 @@ def sinkhorn_potentials_pnorm(x, y, p, eps, tau, max_iter=10000, a=None, b=None,
     n, d = x.shape
     m = y.shape[0]
     init_zero = 1 if (f is None and g is None) else 0
+    alloc = torch.empty if init_zero else torch.zeros  # the library zeroes both with init_zero
     if f is None:
-        f = torch.zeros(n, dtype=torch.float32, device=x.device)
+        f = alloc(n, dtype=torch.float32, device=x.device)
     if g is None:
-        g = torch.zeros(m, dtype=torch.float32, device=x.device)
+        g = alloc(m, dtype=torch.float32, device=x.device)
     ws = _ws(workspace, n, m, d, "fp32")
     it = ctypes.c_int32(0)
     err = ctypes.c_double(0.0)
