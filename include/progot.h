@@ -111,6 +111,10 @@ int sinkhorn_potentials(const float* x, const float* a, int64_t n, const float* 
  *
  * xq (device, nq x d) query points; y (device, m x d); g_all (device, K x m) the stored
  * g^(k); eps (host, K) and alpha (host, K) float64; out (device, nq x d) may alias xq.
+ * Where tensor-core kernels run (the mixed precisions, and PROGOT_FP32 beyond small sizes)
+ * the call synchronises the stream to report a bounded wait that ran out
+ * (PROGOT_ERR_TIMEOUT). A PROGOT_FP32 call may be captured into a CUDA graph: it then runs on
+ * CUDA cores and reads nothing back.
  */
 int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, int32_t d, int32_t K,
                        const float* g_all, const double* eps, const double* alpha, int32_t precision, float* out,
@@ -519,7 +523,8 @@ int progot_set_wait_limit_ns(uint64_t ns);
  * persistent Sinkhorn loops that start afterwards never publish the initial g's betas
  * (their row blocks' ready flags stay at "nothing published"), so the first f-update
  * waits for words that no sweep provides until the bounded wait
- * (progot_set_wait_limit_ns) expires and the entry point returns PROGOT_ERR_TIMEOUT.
+ * (progot_set_wait_limit_ns) expires and the entry point returns PROGOT_ERR_TIMEOUT; a map
+ * step in two passes raises the fault word as if a wait had run out.
  * Nothing faults or hangs; the context stays usable. 0 (default) restores normal
  * operation. Process-wide setting.
  */

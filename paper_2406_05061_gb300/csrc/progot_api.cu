@@ -383,7 +383,8 @@ static std::atomic<int> g_loop_tc{1};
 constexpr unsigned long long kDefaultWaitNs = 2000000000ull;
 static std::atomic<unsigned long long> g_wait_ns{kDefaultWaitNs};
 // Test hook (progot_test_withhold_initial_betas): the persistent loop starts without the
-// initial betas of g, so its first tiles wait on words that no sweep writes.
+// initial betas of g, so its first tiles wait on words that no sweep writes; a map step in two
+// passes raises the fault word, as a wait of its kernels that ran out does.
 static std::atomic<int> g_withhold_betas{0};
 
 static int check_common(const float* x, int64_t n, const float* y, int64_t m, int32_t d, int32_t precision) {
@@ -1105,6 +1106,7 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
   }
   if (rec) prof_end(r, s, kProfMap, (double)n * (double)m);
   if (t_prof.on) t_prof.worked[kProfMap] += 1;
+  if (g_withhold_betas.load()) CK(cudaMemsetAsync(ws.fault, 1, sizeof(int32_t), s));
   return PROGOT_OK;
 }
 
@@ -1519,18 +1521,27 @@ int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, i
   // d = 16; 69 against 40 at 1000 x 2048, d = 64; 94 against 62 at 3000 x 3000, d = 16.
   if (precision == PROGOT_FP32 && (double)nq * (double)m * (double)std::max<int32_t>(d, 16) < kGridMapWork)
     ws.grid = false;
+  // A capture cannot read the fault word of the tensor-core kernels back; the CUDA cores wait
+  // for nothing.
+  if (precision == PROGOT_FP32 && ws.grid) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      (void)cudaGetLastError();
+      ws.grid = false;
+    }
+  }
   if ((precision == PROGOT_FP32 && !ws.grid) || !g_map_tc.load()) CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  TcOps ops;
   for (int k = 0; k < K; ++k) {
     const double al = (k == K - 1) ? 1.0 : alpha[k];
     const float* gk = g_all + (int64_t)k * m;
-    TcOps ops;
     rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
                  k ? Operands::kMoved : Operands::kAuto);
     if (rc) return rc;
     rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
     if (rc) return rc;
   }
-  return precision == PROGOT_FP32 ? PROGOT_OK : check_fault(ws, s);
+  return ops.on ? check_fault(ws, s) : PROGOT_OK;
 }
 
 int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const float* f,
