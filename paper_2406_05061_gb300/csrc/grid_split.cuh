@@ -39,23 +39,45 @@ __device__ __forceinline__ int grid_exp(float norm2_max, float sc, int cap) {
 }
 struct GridScale {
   int ex, ey;
-  float s2;   // 2^(ex + ey): units of the accumulators per log2 unit
+  float s2;   // 2^(ex + ey)
   float inv;  // 2^-(ex + ey)
 };
-// The larger of both clouds' norms bounds every point of their hull.
-__device__ __forceinline__ GridScale grid_scale(const float* __restrict__ norm2_max, float sc);
-__device__ __forceinline__ GridScale grid_scale_hull(const float* __restrict__ norm2_max, float sc) {
-  const float a = norm2_max[0], b = norm2_max[1];
-  const float both[2] = {__int_as_float(max(__float_as_int(a), __float_as_int(b))), b};
-  return grid_scale(both, sc);
-}
-__device__ __forceinline__ GridScale grid_scale(const float* __restrict__ norm2_max, float sc) {
+// hull: the x cloud moved inside the hull of both since its norms were taken; the larger of
+// both clouds' norms bounds every point of it.
+__device__ __forceinline__ GridScale grid_scale(const GridWords& w, float sc, bool hull) {
   GridScale g;
-  g.ex = grid_exp(norm2_max[0], sc, 9);
-  g.ey = grid_exp(norm2_max[1], sc, 10);
+  const float a = w.norm2_max[0], b = w.norm2_max[1];
+  g.ex = grid_exp(hull ? __int_as_float(max(__float_as_int(a), __float_as_int(b))) : a, sc, 9);
+  g.ey = grid_exp(b, sc, 10);
   g.s2 = ldexpf(1.f, g.ex + g.ey);
   g.inv = ldexpf(1.f, -(g.ex + g.ey));
   return g;
+}
+
+// Whether the split carries these clouds. A point's parts resolve 2^-25 units, 2^-36 of its cloud's
+// largest norm, so a pair of ordinary points has t to 2^-36 max|x~| |y~| c (and the same with the
+// sides swapped), where the CUDA cores' float32 chain has 2^-24 |x||y| c, uncentred: when far points
+// set the grid (or pull the centre away) by more than 2^10 the CUDA cores are the more exact. Norms
+// of ordinary points: geometric means (of powers of two). Below ex + ey = 0 t exceeds 2^22 and float32 log-sum-exps of it lose whole
+// units; a norm that is not finite has no grid at all. Such clouds are left to the CUDA cores.
+constexpr float kGridReach = 10.f;
+__device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const GridScale& g, bool hull) {
+  const float a = w.norm2_max[0], b = w.norm2_max[1];
+  if (!isfinite(a) || !isfinite(b) || g.ex + g.ey < 0) return true;
+  if (w.nonzero[0] == 0u || w.nonzero[1] == 0u || !(a > 0.f) || !(b > 0.f)) return false;
+  // log2 of: largest norms, ordinary norms about the centre and about the origin
+  float ax = 0.5f * (float)ilogbf(a);
+  const float ay = 0.5f * (float)ilogbf(b);
+  float cx = (float)(0.5 * (double)w.exp_sum[0] / (double)w.nonzero[0]);
+  const float cy = (float)(0.5 * (double)w.exp_sum[1] / (double)w.nonzero[1]);
+  float rx = (float)(0.5 * (double)w.raw_sum[0] / (double)w.nonzero[0]);
+  const float ry = (float)(0.5 * (double)w.raw_sum[1] / (double)w.nonzero[1]);
+  if (hull) {
+    ax = fmaxf(ax, ay);
+    cx = fmaxf(cx, cy);
+    rx = fminf(rx, ry);
+  }
+  return fmaxf(ax + cy, ay + cx) - (rx + ry) > kGridReach;
 }
 
 // beta = (pot - norm) bscale as an unevaluated sum of two floats (hi + lo): a float32 beta

@@ -148,7 +148,7 @@ struct Params {
   int32_t* fault;           // grid-wide abort / fault word
   unsigned long long wait_ns;
   int32_t nkb, split3, stages, a_bufs, G, maxseg;
-  const float* gscale;      // grid split: {2^(ex + ey), 2^-(ex + ey)} (device)
+  const GridWords* words;   // grid split: its words
   int32_t seq0, niter;      // iterations seq0 .. seq0 + niter - 1 of the loop
 };
 
@@ -416,6 +416,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                      const __grid_constant__ CUtensorMap mXb0, const __grid_constant__ CUtensorMap mXb1,
                      const __grid_constant__ CUtensorMap mYb0, const __grid_constant__ CUtensorMap mYb1,
                      const Params P) {
+  if constexpr (GRID)
+    if (__ldg(&P.words->bad) != 0) return;  // the host runs this loop on CUDA cores
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -719,7 +721,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int quarter = warp & 3;
     const int row_local = quarter * 32 + lane;
     int tl = 0, kseg = 0;
-    const float inv2 = GRID ? __ldg(P.gscale + 1) : 1.f;
+    const float inv2 = GRID ? __ldg(&P.words->inv) : 1.f;
     const uint64_t inv22 = pack2(inv2, inv2);
     bool dead = false;
     for (int it = P.seq0; it < it_end; ++it) {
@@ -845,7 +847,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   } else {
     // ------------------------------------------------------------ epilogue warps and stop decision
     const int etid = threadIdx.x - EPI_TID0;  // 0..63
-    const float s2 = GRID ? __ldg(P.gscale) : 1.f;
+    const float s2 = GRID ? __ldg(&P.words->s2) : 1.f;
     int kseg = 0;
     // ---- stop test of iteration it (warp 10), once every row block of the f-update is done
     auto decide = [&](int it) {
@@ -1099,7 +1101,7 @@ static cudaError_t launch_loop(const tc::loop::Params& P, size_t smem, const voi
 
 cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   int stages, a_bufs;
-  const bool grid = Lq.gscale != nullptr;
+  const bool grid = Lq.words != nullptr;
   // A in TMEM from 64 tiles per CTA and sweep: writing it costs about 4 us at every segment's
   // start, which many tiles repay (16384^2, d = 256, 107 tiles: 248 us per sweep against 262)
   // and few do not (8000^2, 26 tiles: 69 against 65.5; 2000^2: 16.5 against 11.6)
@@ -1153,7 +1155,7 @@ cudaError_t launch_sinkhorn_loop_tc(const LoopLaunch& Lq, cudaStream_t stream) {
   P.maxseg = Lq.maxseg;
   P.seq0 = Lq.seq0;
   P.niter = Lq.niter;
-  P.gscale = Lq.gscale;
+  P.words = Lq.words;
   const size_t smem = tc::loop::layout(Lq.bn, Lq.nkb, Lq.split3, stages, a_bufs, grid).total;
   const int ks = (Lq.side[0].p.d + 15) / 16;  // K = 16 steps
   const bool many = tiles >= 4 * (int64_t)Lq.G;  // fewer are paced by the hand-over

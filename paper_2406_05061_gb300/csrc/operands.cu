@@ -42,7 +42,7 @@ template <int CL>
 __global__ void __launch_bounds__(32 * kCenterWarps)
     center_kernel(const float* __restrict__ X, int64_t n, const float* __restrict__ Y, int64_t m, int32_t d,
                   double* __restrict__ partial, unsigned* __restrict__ ticket, float* __restrict__ mu,
-                  float* __restrict__ gmax) {
+                  GridWords* __restrict__ words) {
   __shared__ double acc[kCenterWarps][kCenterCols];
   __shared__ double tot[kCenterCols];
   __shared__ int s_last;
@@ -111,7 +111,11 @@ __global__ void __launch_bounds__(32 * kCenterWarps)
   }
   __syncthreads();
   if (!s_last) return;
-  if (gmax != nullptr && threadIdx.x < 2) gmax[threadIdx.x] = 0.f;  // for grid_norms_kernel
+  if (words != nullptr && threadIdx.x < 2) {  // for grid_norms_kernel
+    words->norm2_max[threadIdx.x] = 0.f;
+    words->nonzero[threadIdx.x] = 0u;
+    words->exp_sum[threadIdx.x] = words->raw_sum[threadIdx.x] = 0;
+  }
   // 256 coordinates at a time; where there are fewer, several threads share a coordinate's
   // blocks (slices added in order)
   const int cols = center_cols(d), slices = 32 * kCenterWarps / cols;
@@ -202,9 +206,11 @@ __device__ void loop_setup(const LoopSetup& ls, int64_t tid, int64_t nthreads) {
   }
 }
 
-// |x_i - mu|^2 of one row by one warp: exact differences and squares as float pairs.
-__device__ __forceinline__ float row_norm(const float* __restrict__ v, const float* __restrict__ mu, int d, int lane) {
-  float s = 0.f, e = 0.f;
+// |x_i - mu|^2 of one row by one warp: exact differences and squares as float pairs. raw (or
+// NULL): |x_i|^2, rounded.
+__device__ __forceinline__ float row_norm(const float* __restrict__ v, const float* __restrict__ mu, int d, int lane,
+                                          float* raw = nullptr) {
+  float s = 0.f, e = 0.f, r = 0.f;
   for (int k = lane; k < d; k += 32) {
     const float x = __ldg(v + k), c = __ldg(mu + k);
     const float u = x - c;
@@ -213,6 +219,12 @@ __device__ __forceinline__ float row_norm(const float* __restrict__ v, const flo
     const float p = u * u;
     acc2(s, e, p);
     e += fmaf(u, u, -p) + 2.f * u * ue;
+    if (raw) r = fmaf(x, x, r);
+  }
+  if (raw) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    *raw = r;
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -223,32 +235,53 @@ __device__ __forceinline__ float row_norm(const float* __restrict__ v, const flo
   return isfinite(s) ? s + e : s;
 }
 
-// Centred squared norms of both clouds and the largest of each, through an integer maximum
-// of the (non-negative) floats' bits, NaN above all.
+// Centred squared norms of both clouds; of each the largest, through an integer maximum of the
+// (non-negative) floats' bits, NaN above all, and the sums of exponents of GridWords.
 __global__ void grid_norms_kernel(OperandPrep op) {
-  __shared__ int red[2];
-  if (threadIdx.x < 2) red[threadIdx.x] = 0;
+  __shared__ int red[2], cnt[2], exps[2], raws[2];
+  if (threadIdx.x < 2) red[threadIdx.x] = cnt[threadIdx.x] = exps[threadIdx.x] = raws[threadIdx.x] = 0;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int best[2] = {0, 0};
+  int best[2] = {0, 0}, nz[2] = {0, 0}, ex[2] = {0, 0}, rex[2] = {0, 0};
+  float raw;
   for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < op.n + op.m; row += (int64_t)gridDim.x * 8) {
     const int side = row < op.n ? 0 : 1;
     const int64_t i = side ? row - op.n : row;
-    const float nv = row_norm((side ? op.y : op.x) + i * (int64_t)op.d, op.mu, op.d, lane);
+    const float nv = row_norm((side ? op.y : op.x) + i * (int64_t)op.d, op.mu, op.d, lane, &raw);
     if (lane == 0) (side ? op.ync : op.xnc)[i] = nv;
     best[side] = max(best[side], __float_as_int(nv));
+    if (nv > 0.f && isfinite(nv)) {
+      nz[side] += 1;
+      ex[side] += ilogbf(nv);
+      rex[side] += ilogbf(raw > 0.f && isfinite(raw) ? raw : nv);
+    }
   }
   if (lane == 0) {
-    if (best[0] > 0) atomicMax(&red[0], best[0]);
-    if (best[1] > 0) atomicMax(&red[1], best[1]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (best[q] > 0) atomicMax(&red[q], best[q]);
+      if (nz[q] > 0) {
+        atomicAdd(&cnt[q], nz[q]);
+        atomicAdd(&exps[q], ex[q]);
+        atomicAdd(&raws[q], rex[q]);
+      }
+    }
   }
   __syncthreads();
-  if (threadIdx.x < 2 && red[threadIdx.x] > 0) atomicMax(reinterpret_cast<int*>(op.gmax) + threadIdx.x, red[threadIdx.x]);
+  if (threadIdx.x < 2) {
+    const int q = threadIdx.x;
+    if (red[q] > 0) atomicMax(reinterpret_cast<int*>(op.words->norm2_max) + q, red[q]);
+    if (cnt[q] > 0) {
+      atomicAdd(&op.words->nonzero[q], (unsigned)cnt[q]);
+      atomicAdd(reinterpret_cast<unsigned long long*>(op.words->exp_sum) + q, (unsigned long long)(long long)exps[q]);
+      atomicAdd(reinterpret_cast<unsigned long long*>(op.words->raw_sum) + q, (unsigned long long)(long long)raws[q]);
+    }
+  }
 }
 
 // One warp per row (and per padding row of the bias buffers): parts, norm and bias row.
 // GRID: 0 bf16; 1 the integer grid, whose norms exist already; 2 the integer grid on clouds
-// that moved inside the hull of those whose largest norms gmax holds (a map step's), which
+// that moved inside the hull of those whose largest norms op.words holds (a map step's), which
 // bound theirs. Blocks past the rows set a loop up.
 template <int GRID>
 __global__ void operands_kernel(OperandPrep op, LoopSetup ls, int row_blocks) {
@@ -268,12 +301,13 @@ __global__ void operands_kernel(OperandPrep op, LoopSetup ls, int row_blocks) {
   GridScale gs;
   float pe = 1.f;
   if constexpr (GRID) {
-    gs = GRID == 2 ? grid_scale_hull(op.gmax, op.sc) : grid_scale(op.gmax, op.sc);
+    gs = grid_scale(*op.words, op.sc, GRID == 2);
     pe = ldexpf(1.f, side ? gs.ey : gs.ex);
     if (row == 0 && lane == 0) {
-      op.gscale[0] = gs.s2;
-      op.gscale[1] = gs.inv;
-      op.gscale[2] = ldexpf(1.f, -gs.ey);
+      op.words->s2 = gs.s2;
+      op.words->inv = gs.inv;
+      op.words->inv_ey = ldexpf(1.f, -gs.ey);
+      if (op.words->bad == 0 && grid_out_of_range(*op.words, gs, GRID == 2)) op.words->bad = op.step;
     }
   }
   float nv = 0.f;
@@ -349,14 +383,14 @@ __global__ void operands_kernel(OperandPrep op, LoopSetup ls, int row_blocks) {
 }
 
 cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial,
-                          unsigned* ticket, float* mu, float* gmax, cudaStream_t s) {
+                          unsigned* ticket, float* mu, GridWords* words, cudaStream_t s) {
   // at least four rows a warp (one load round); clusters of eight where the last block
   // would otherwise add more than two rounds of block sums a thread
   const int64_t rows = std::max<int64_t>(n, m);
   int parts = (int)std::max<int64_t>(1, std::min<int64_t>(reduce_parts() / 2, rows / (4 * kCenterWarps)));
   const int z = (d + kCenterCols - 1) / kCenterCols;
   if (parts * center_cols(d) <= 16 * 32 * kCenterWarps) {
-    center_kernel<1><<<dim3(parts, 2, z), 32 * kCenterWarps, 0, s>>>(X, n, Y, m, d, partial, ticket, mu, gmax);
+    center_kernel<1><<<dim3(parts, 2, z), 32 * kCenterWarps, 0, s>>>(X, n, Y, m, d, partial, ticket, mu, words);
     count_launch();
     return cudaGetLastError();
   }
@@ -372,7 +406,7 @@ cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, center_kernel<8>, X, n, Y, m, d, partial, ticket, mu, gmax);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, center_kernel<8>, X, n, Y, m, d, partial, ticket, mu, words);
   count_launch();
   return e;
 }

@@ -211,8 +211,7 @@ struct Workspace {
   // integer-grid operands (float32 path): third parts, largest squared norms, scales
   void* xr;
   void* yr;
-  float* gmax;      // [2], gscale [3] and ticket: in the solver states' 256 bytes
-  float* gscale;
+  GridWords* words; // and ticket: in the solver states' 256 bytes
   unsigned* ticket;
   char* prob;       // P tiles of the map step, a chunk of rows at a time (integer-grid operands)
   int64_t prob_bytes;
@@ -287,9 +286,9 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   static_assert(2 * sizeof(SolverState) <= 128, "the solver states and the fault word share 256 bytes");
   ws.state = (SolverState*)take(256);  // [2]: see SweepParams::lag
   ws.fault = (int32_t*)((char*)ws.state + 128);
-  ws.gmax = (float*)((char*)ws.state + 144);
-  ws.gscale = (float*)((char*)ws.state + 160);
-  ws.ticket = (unsigned*)((char*)ws.state + 176);
+  static_assert(144 + sizeof(GridWords) <= 240, "the small words share 256 bytes");
+  ws.words = (GridWords*)((char*)ws.state + 144);
+  ws.ticket = (unsigned*)((char*)ws.state + 240);
   ws.rpart = (double*)take(sizeof(double) * reduce_parts() * (size_t)(w.d + 1));
   ws.rout = (double*)take(sizeof(double) * 2 * (size_t)(w.d + 1));
   ws.Opart = (float*)take(sizeof(float) * w.opart_elems);
@@ -355,7 +354,8 @@ static int carve(int64_t n, int64_t m, int32_t d, void* workspace, size_t ws_byt
   return PROGOT_OK;
 }
 
-constexpr size_t kStateBytes = 128 + sizeof(int32_t);  // both solver states, then the fault word
+// Both solver states, the fault word and the integer grid's words, as the host reads them.
+constexpr size_t kStateBytes = 144 + sizeof(GridWords);
 
 // Pinned host mirror of the solver state, one pair per host thread.
 struct HostMirror {
@@ -372,6 +372,9 @@ struct HostMirror {
     ok = true;
     return PROGOT_OK;
   }
+  // of a copy of kStateBytes from ws.state to hs
+  int32_t fault() const { return *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(hs) + 128); }
+  const GridWords& words() const { return *reinterpret_cast<const GridWords*>(reinterpret_cast<const char*>(hs) + 144); }
 };
 static thread_local HostMirror t_host;
 
@@ -452,7 +455,7 @@ struct TcOps {
   CUtensorMap yh_mt, yl_mt, yb_mt;
   // integer-grid split: third parts in both roles
   CUtensorMap xr_a, yr_a, xr_b, yr_b;
-  const float* gscale = nullptr;  // its device scales (non-NULL: the operands are the grid split's)
+  const GridWords* words = nullptr;  // its device words (non-NULL: the operands are the grid split's)
   // centre mu of the operands and the squared norms |x_i - mu|^2, |y_j - mu|^2 that
   // the tensor-core sweeps use in place of |x_i|^2, |y_j|^2
   const float* mu = nullptr;
@@ -477,8 +480,8 @@ static int map_y_bias(TcOps* ops, void* base, int64_t m) {
   const int64_t rows = cdiv(m, 256) * 256;
   ops->yb_base = base;
   int rc = make_map(&ops->yb, base, rows, 16, ops->bn);
-  if (!rc && !ops->gscale && ops->nkb == 1) rc = make_map(&ops->yb128, base, rows, 16, 128);
-  if (!rc && !ops->gscale && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb))
+  if (!rc && !ops->words && ops->nkb == 1) rc = make_map(&ops->yb128, base, rows, 16, 128);
+  if (!rc && !ops->words && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb))
     rc = make_map(&ops->yb_mt, base, rows, 16, map_tc_onepass_tile_cols());
   return rc;
 }
@@ -528,12 +531,13 @@ enum class Operands { kAuto, kMoved, kGridTwoParts };
 // for every centre.
 static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t d, double eps, int32_t precision,
                    const Workspace& ws, TcOps* ops, cudaStream_t s, const float* f_cur = nullptr,
-                   const float* g_cur = nullptr, bool loop = false, Operands kind = Operands::kAuto) {
+                   const float* g_cur = nullptr, bool loop = false, Operands kind = Operands::kAuto,
+                   int32_t step = 1) {
   const bool two = kind == Operands::kGridTwoParts, grid = precision == PROGOT_FP32 || two;
   ops->on = precision != PROGOT_FP32 || ws.grid;
   ops->lse_ready = false;
   ops->loop = false;
-  ops->gscale = grid ? ws.gscale : nullptr;
+  ops->words = grid ? ws.words : nullptr;
   if (!ops->on) return PROGOT_OK;
   const int32_t dp = pad64(d);
   ops->nkb = dp / 64;
@@ -547,9 +551,9 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   ops->ync = ws.ync;
   const bool hull = grid && kind == Operands::kMoved;
   if (two)
-    CK(cudaMemsetAsync(ws.gmax, 0, 2 * sizeof(float), s));
+    CK(cudaMemsetAsync(ws.words->norm2_max, 0, sizeof(GridWords) - offsetof(GridWords, norm2_max), s));
   else if (!hull)
-    CK(launch_center(x, n, y, m, d, ws.rpart, ws.ticket, ws.mu, grid ? ws.gmax : nullptr, s));
+    CK(launch_center(x, n, y, m, d, ws.rpart, ws.ticket, ws.mu, grid ? ws.words : nullptr, s));
   OperandPrep op;
   memset(&op, 0, sizeof(op));
   op.x = x;
@@ -564,8 +568,8 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   op.mu = ws.mu;
   op.xnc = ws.xnc;
   op.ync = ws.ync;
-  op.gmax = ws.gmax;
-  op.gscale = ws.gscale;
+  op.words = ws.words;
+  op.step = step;
   op.xp[0] = ws.xh;
   op.xp[1] = ops->parts > 1 ? ws.xl : nullptr;
   op.xp[2] = ops->parts > 2 ? ws.xr : nullptr;
@@ -714,12 +718,12 @@ static int lse_sweep(const SweepParams& p, cudaStream_t s, const TcOps* ops = nu
     TcMaps maps;
     maps.a[0] = a_is_x ? &ops->xh_a : &ops->yh_a;
     maps.a[1] = a_is_x ? &ops->xl_a : &ops->yl_a;
-    maps.a[2] = ops->gscale ? (a_is_x ? &ops->xr_a : &ops->yr_a) : maps.a[1];
+    maps.a[2] = ops->words ? (a_is_x ? &ops->xr_a : &ops->yr_a) : maps.a[1];
     maps.b[0] = a_is_x ? &ops->yh_b : &ops->xh_b;
     maps.b[1] = a_is_x ? &ops->yl_b : &ops->xl_b;
-    maps.b[2] = ops->gscale ? (a_is_x ? &ops->yr_b : &ops->xr_b) : maps.b[1];
+    maps.b[2] = ops->words ? (a_is_x ? &ops->yr_b : &ops->xr_b) : maps.b[1];
     maps.bias = a_is_x ? &ops->yb : &ops->xb;
-    const bool bf16 = ops->gscale == nullptr && ws != nullptr;
+    const bool bf16 = ops->words == nullptr && ws != nullptr;
     maps.a_part[0] = !bf16 ? nullptr : a_is_x ? ws->xh : ws->yh;
     maps.a_part[1] = !bf16 ? nullptr : ops->parts < 2 ? maps.a_part[0] : a_is_x ? ws->xl : ws->yl;
     void* bias_out = (p.mode == kModePotential && ws) ? (a_is_x ? ws->xb : ws->yb) : nullptr;
@@ -730,7 +734,7 @@ static int lse_sweep(const SweepParams& p, cudaStream_t s, const TcOps* ops = nu
     // the operands are centred: the row constants of the epilogue are the centred norms
     if (q.An != nullptr) q.An = a_is_x ? ops->xnc : ops->ync;
     if (q.Bn != nullptr) q.Bn = a_is_x ? ops->ync : ops->xnc;
-    CK(launch_lse_sweep_tc(q, maps, ops->nkb, ops->parts, ops->gscale, ops->bn, G, maxseg, ws ? ws->fault : nullptr,
+    CK(launch_lse_sweep_tc(q, maps, ops->nkb, ops->parts, ops->words, ops->bn, G, maxseg, ws ? ws->fault : nullptr,
                            bias_out, s));
   } else {
     CK(launch_lse_sweep_fp32(p, s));
@@ -746,11 +750,12 @@ static int lse_sweep(const SweepParams& p, cudaStream_t s, const TcOps* ops = nu
 // descriptions built by sinkhorn_core; ops describes the prepared operands, with whose
 // bias rows prep_tc has written the loop's tables, flags and state. On return the current f
 // is in f_a, g in g, and (map_follows) the y-side bias rows ops describes hold g for a map
-// step at the same eps, ws.L its row log-sum-exps.
+// step at the same eps, ws.L its row log-sum-exps. *bad: the clouds are out of the integer
+// grid's range and nothing ran.
 static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, int64_t m, int32_t max_iter,
                                     double tau, float* f_a, float* f_b, float* g, const Workspace& ws,
                                     TcOps& ops, bool map_follows, int32_t* iters_out, double* err_out,
-                                    cudaStream_t s) {
+                                    cudaStream_t s, bool* bad) {
   pf.An = ops.xnc;
   pf.Bn = ops.ync;
   pg.An = ops.ync;
@@ -796,14 +801,14 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   Gs.cslot = ws.ltab_cslot + ws.lslots;
   Gs.crow = ws.ltab_crow + rb;
   Gs.nseg = ws.ltab_nseg + num_sms();
-  const bool grid = ops.gscale != nullptr;
+  const bool grid = ops.words != nullptr;
   const CUtensorMap* maps[16] = {&ops.xh_a, &ops.xl_a, &ops.yh_a, &ops.yl_a, &ops.xh_b, &ops.xl_b,
                                  &ops.yh_b, &ops.yl_b,
                                  grid ? &ops.xr_a : &ops.xl_a, grid ? &ops.yr_a : &ops.yl_a,
                                  grid ? &ops.xr_b : &ops.xl_b, grid ? &ops.yr_b : &ops.yl_b,
                                  &ops.xb,   &xb2_map,   &ops.yb,   &yb2_map};
   for (int q = 0; q < 16; ++q) L.maps[q] = maps[q];
-  L.gscale = ops.gscale;
+  L.words = ops.words;
   L.errpart = ws.lerr;
   L.state = ws.state;
   L.fault = ws.fault;
@@ -833,8 +838,15 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   CK(cudaMemcpyAsync(t_host.hs, ws.state, kStateBytes, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   const SolverState fin = t_host.hs[0];
-  const int32_t fault = *reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(t_host.hs) + 128);
-  if (fault) return fail(PROGOT_ERR_TIMEOUT, "the persistent Sinkhorn loop hit its bounded wait and aborted");
+  if (t_host.fault()) return fail(PROGOT_ERR_TIMEOUT, "the persistent Sinkhorn loop hit its bounded wait and aborted");
+  *bad = grid && t_host.words().bad != 0;
+  if (*bad) {
+    if (t_prof.on) {
+      pr.counted = false;
+      t_prof.recs.push_back(pr);
+    }
+    return PROGOT_OK;
+  }
   // every iteration up to the stop ran both sweeps (the last g-update without writes)
   const int64_t sweeps = 2 * ((int64_t)fin.it + 1);
   if (t_prof.on) {
@@ -877,6 +889,39 @@ static int sinkhorn_loop_persistent(SweepParams pf, SweepParams pg, int64_t n, i
   }
 }
 
+static int zero_counters(const Workspace& ws, cudaStream_t s) {
+  // cnt, mcnt and the small words (fault, raised by a tensor-core kernel's expired wait)
+  // follow one another
+  CK(cudaMemsetAsync(ws.cnt, 0, (size_t)((char*)ws.state + 256 - (char*)ws.cnt), s));
+  return PROGOT_OK;
+}
+
+// PROGOT_ERR_TIMEOUT when a tensor-core kernel of this call raised the fault flag
+// (synchronises the stream).
+// *bad (optional): the step whose clouds the integer grid's kernels found out of their range
+// and left alone (0: none).
+static int check_fault(const Workspace& ws, cudaStream_t s, int32_t* bad = nullptr) {
+  const int rc = t_host.init();
+  if (rc) return rc;
+  CK(cudaMemcpyAsync(t_host.hs, ws.state, kStateBytes, cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (t_host.fault()) return fail(PROGOT_ERR_TIMEOUT, "a tensor-core kernel hit its bounded wait (2 s) and aborted");
+  if (bad) *bad = t_host.words().bad;
+  return PROGOT_OK;
+}
+
+// After grid kernels found the clouds out of their range (words->bad): the word cleared, the
+// norms the CUDA cores read, and in *w a view of the workspace without the grid's operands.
+static int leave_grid(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const Workspace& ws, Workspace* w,
+                      cudaStream_t s) {
+  *w = ws;
+  w->grid = false;
+  CK(cudaMemsetAsync(&ws.words->bad, 0, sizeof(int32_t), s));
+  CK(launch_row_sqnorm(x, n, d, ws.xn, s));
+  CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  return PROGOT_OK;
+}
+
 // Sinkhorn loop (Alg. 1) on device-resident state. f lives in {f_a, f_b} (ping-pong);
 // on return the current f is copied into f_a. Norms xn, yn must be ready.
 // ops_out (optional) receives the tensor-core operand descriptions, valid for a map
@@ -892,6 +937,14 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
                          const Cost& cost = Cost(), Operands kind = Operands::kAuto) {
   int rc = t_host.init();
   if (rc) return rc;
+  // the same on CUDA cores, for clouds that the grid kernels found out of their range
+  auto on_cuda_cores = [&]() -> int {
+    Workspace w;
+    int r = leave_grid(x, n, y, m, d, ws, &w, s);
+    if (r) return r;
+    return sinkhorn_core(x, a, n, y, b, m, d, eps, tau, max_iter, precision, f_a, f_b, g, w.xn, w.yn, w, iters_out,
+                         err_out, s, ops_out, symmetric, cost);
+  };
   TcOps ops_local;
   TcOps& ops = ops_out ? *ops_out : ops_local;
   if (cost.pnorm()) {
@@ -935,9 +988,15 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
   pf.lag = pg.lag = lag ? 1 : 0;
   if (ops.loop) {
     pf.lag = pg.lag = 0;
-    return sinkhorn_loop_persistent(pf, pg, n, m, max_iter, tau, f_a, f_b, g, ws, ops, ops_out != nullptr, iters_out,
-                                    err_out, s);
+    bool bad = false;
+    rc = sinkhorn_loop_persistent(pf, pg, n, m, max_iter, tau, f_a, f_b, g, ws, ops, ops_out != nullptr, iters_out,
+                                  err_out, s, &bad);
+    return bad ? on_cuda_cores() : rc;
   }
+  const bool grid = ops.on && ops.words != nullptr;
+  int32_t* bad = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(t_host.hs) + 248);
+  *bad = 0;
+  if (grid) CK(cudaMemcpyAsync(bad, &ws.words->bad, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
 
   int64_t sym_sweeps = 0;
   int64_t launched = 0;  // iterations enqueued so far
@@ -1006,6 +1065,13 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
       pending = true;
     }
     CK(cudaEventSynchronize(t_host.ev[cur]));
+    if (*bad) {
+      for (ProfRec& rr : chunk_recs) {
+        rr.counted = false;
+        t_prof.recs.push_back(rr);
+      }
+      return on_cuda_cores();
+    }
     const SolverState now = t_host.hs[cur];
     if (now.done) {
       fin = now;
@@ -1085,7 +1151,7 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
     TcMaps maps = {{&ops.xh_a, &ops.xl_a, &ops.xr_a}, {&ops.yh_b, &ops.yl_b, &ops.yr_b}, &ops.yb, {nullptr, nullptr}};
     int G = 0, maxseg = 0;
     tc_plan(rows, m, ops.bn, num_sms(), &G, &maxseg);
-    CK(launch_lse_sweep_tc(p, maps, ops.nkb, ops.parts, ops.gscale, ops.bn, G, maxseg, ws.fault, nullptr, s,
+    CK(launch_lse_sweep_tc(p, maps, ops.nkb, ops.parts, ops.words, ops.bn, G, maxseg, ws.fault, nullptr, s,
                            ws.L + row0, ws.prob, row0));
     PvLaunch pv;
     pv.X = X + row0 * d;
@@ -1093,7 +1159,7 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
     pv.rsum = ws.rsum + row0;
     pv.prob = ws.prob;
     for (int q = 0; q < 3; ++q) pv.mapY[q] = &ymap[q];
-    pv.gscale = ops.gscale;
+    pv.words = ops.words;
     pv.mu = ops.mu;
     pv.rows = rows;
     pv.m = m;
@@ -1128,7 +1194,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
            : tc                   ? lse_sweep(pl, s, ops, true, &ws)
                                   : lse_sweep(pl, s);
   if (rc) return rc;
-  if (tc && !ops->gscale && ops->nkb == 1 && g_map_tc.load()) {
+  if (tc && !ops->words && ops->nkb == 1 && g_map_tc.load()) {
     // d <= 64: S and P Y both on the tensor cores (P Y reuses the centred, scaled y operand)
     int G = 0, maxseg = 0;
     tc_plan(n, m, 128, num_sms(), &G, &maxseg);
@@ -1141,7 +1207,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
   }
-  if (tc && !ops->gscale && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb) && g_map_tc.load()) {
+  if (tc && !ops->words && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb) && g_map_tc.load()) {
     // 64 < d <= 256: one launch, S once per tile, all output coordinates in TMEM
     int G = 0, maxseg = 0;
     tc_plan(n, m, map_tc_onepass_tile_cols(), num_sms(), &G, &maxseg);
@@ -1154,18 +1220,28 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
   }
+  TcOps gops;
   if (tc && g_map_tc.load()) {
     // float32 path, and the bf16x3 path for d > 256 (its operands give way to the
     // integer-grid ones, whose accuracy the CUDA-core map it replaces had): P a chunk of
     // row blocks at a time, then P Y
-    TcOps gops;
     const TcOps* go = ops;
-    if (!ops->gscale) {
+    if (!ops->words) {
       rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g, false, Operands::kGridTwoParts);
       if (rc) return rc;
       go = &gops;
     }
-    return grid_map_step(X, n, m, d, eps, alpha, ws, s, *go);
+    rc = grid_map_step(X, n, m, d, eps, alpha, ws, s, *go);
+    if (rc || ops->words) return rc;  // the float32 path's callers look at words->bad
+    int32_t bad = 0;
+    rc = check_fault(ws, s, &bad);
+    if (rc || !bad) return rc;
+    // out of the grid's range: the operands and L of before again, then the CUDA cores
+    Workspace w;
+    rc = leave_grid(X, n, y, m, d, ws, &w, s);
+    if (!rc) rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g);
+    if (!rc) rc = lse_sweep(pl, s, &gops, true, &ws);
+    if (rc) return rc;
   }
   if (tc) {
     // the float32 map sweep below forms t_ij from the uncentred X and Y: move L there
@@ -1208,23 +1284,6 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     CK(launch_map_sweep_fp32(mp, s));
   if (rec) prof_end(r, s, kProfMap, (double)n * (double)m);
   if (t_prof.on) t_prof.worked[kProfMap] += 1;
-  return PROGOT_OK;
-}
-
-static int zero_counters(const Workspace& ws, cudaStream_t s) {
-  // cnt, mcnt and the small words (fault, raised by a tensor-core kernel's expired wait)
-  // follow one another
-  CK(cudaMemsetAsync(ws.cnt, 0, (size_t)((char*)ws.state + 256 - (char*)ws.cnt), s));
-  return PROGOT_OK;
-}
-
-// PROGOT_ERR_TIMEOUT when a tensor-core kernel of this call raised the fault flag
-// (synchronises the stream).
-static int check_fault(const Workspace& ws, cudaStream_t s) {
-  int32_t fault = 0;
-  CK(cudaMemcpyAsync(&fault, ws.fault, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (fault) return fail(PROGOT_ERR_TIMEOUT, "a tensor-core kernel hit its bounded wait (2 s) and aborted");
   return PROGOT_OK;
 }
 
@@ -1275,8 +1334,14 @@ static int metrics_core(const float* x, const float* a, int64_t n, const float* 
   CK(cudaMemcpyAsync(t_host.hd, ws.metout, sizeof(double) * 2 * kMetricSums, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (ops.on) {
-    rc = check_fault(ws, s);
+    int32_t bad = 0;
+    rc = check_fault(ws, s, &bad);
     if (rc) return rc;
+    if (bad) {
+      Workspace w;
+      rc = leave_grid(x, n, y, m, d, ws, &w, s);
+      return rc ? rc : metrics_core(x, a, n, y, b, m, d, f, g, eps, w, s, out, cost, x_cost);
+    }
   }
   const double* R = t_host.hd;                // row sweep: pot = f, w = a
   const double* Cs = t_host.hd + kMetricSums;  // column sweep: pot = g, w = b
@@ -1288,6 +1353,54 @@ static int metrics_core(const float* x, const float* a, int64_t n, const float* 
   out->dual = R[kSumPotW] + Cs[kSumPotW] - eps * R[kSumMass];
   if (!std::isfinite(out->transport_cost) || !std::isfinite(out->entropy) || !std::isfinite(out->dual))
     return fail(PROGOT_ERR_NUMERIC, "non-finite coupling metric");
+  return PROGOT_OK;
+}
+
+// Row and column sums of P = exp((f (+) g - C)/eps) and their distance to the weights, with
+// float32 accuracy at every precision setting: the integer-grid operands where the workspace
+// has room for them, else CUDA cores. The arrival counters must be zero.
+static int marginals_core(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const float* f,
+                          const float* g, double eps, float* row, float* col, const float* a, const float* b,
+                          double* err_l1_out, const Workspace& ws, cudaStream_t s) {
+  if (!ws.grid) {
+    CK(launch_row_sqnorm(x, n, d, ws.xn, s));
+    CK(launch_row_sqnorm(y, m, d, ws.yn, s));
+  }
+  TcOps ops;
+  int rc = prep_tc(x, n, y, m, d, eps, PROGOT_FP32, ws, &ops, s, f, g);
+  if (rc) return rc;
+  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws, ops.on ? 1 : 2);
+  pr.wA = a;
+  pr.potB = g;
+  pr.potA_old = f;
+  pr.out = row;
+  pr.mode = kModeMarginal;
+  rc = lse_sweep(pr, s, &ops, true, &ws);
+  if (rc) return rc;
+  const int64_t rbr = cdiv(n, fp32_tile_rows());
+  CK(cudaMemcpyAsync(&t_host.hd[0], ws.errpart + rbr, sizeof(double), cudaMemcpyDeviceToHost, s));
+  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws, ops.on ? 1 : 2);
+  pc.wA = b;
+  pc.potB = f;
+  pc.potA_old = g;
+  pc.out = col;
+  pc.mode = kModeMarginal;
+  rc = lse_sweep(pc, s, &ops, false, &ws);
+  if (rc) return rc;
+  const int64_t rbc = cdiv(m, fp32_tile_rows());
+  CK(cudaMemcpyAsync(&t_host.hd[1], ws.errpart + rbc, sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (ops.on) {
+    int32_t bad = 0;
+    rc = check_fault(ws, s, &bad);
+    if (rc) return rc;
+    if (bad) {
+      Workspace w;
+      rc = leave_grid(x, n, y, m, d, ws, &w, s);
+      return rc ? rc : marginals_core(x, n, y, m, d, f, g, eps, row, col, a, b, err_l1_out, w, s);
+    }
+  }
+  if (err_l1_out) *err_l1_out = t_host.hd[0] + t_host.hd[1];
   return PROGOT_OK;
 }
 
@@ -1531,17 +1644,28 @@ int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, i
     }
   }
   if ((precision == PROGOT_FP32 && !ws.grid) || !g_map_tc.load()) CK(launch_row_sqnorm(y, m, d, ws.yn, s));
-  TcOps ops;
-  for (int k = 0; k < K; ++k) {
-    const double al = (k == K - 1) ? 1.0 : alpha[k];
-    const float* gk = g_all + (int64_t)k * m;
-    rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
-                 k ? Operands::kMoved : Operands::kAuto);
+  for (int k0 = 0;;) {
+    TcOps ops;
+    for (int k = k0; k < K; ++k) {
+      const double al = (k == K - 1) ? 1.0 : alpha[k];
+      const float* gk = g_all + (int64_t)k * m;
+      rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
+                   k > k0 ? Operands::kMoved : Operands::kAuto, k + 1);
+      if (rc) return rc;
+      rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
+      if (rc) return rc;
+    }
+    if (!ops.on) return PROGOT_OK;
+    int32_t bad = 0;
+    rc = check_fault(ws, s, &bad);
+    if (rc || !bad) return rc;
+    // steps bad .. K - 1 did nothing: the same on CUDA cores
+    k0 = bad - 1;
+    Workspace w;
+    rc = leave_grid(out, nq, y, m, d, ws, &w, s);
     if (rc) return rc;
-    rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
-    if (rc) return rc;
+    ws = w;
   }
-  return ops.on ? check_fault(ws, s) : PROGOT_OK;
 }
 
 int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const float* f,
@@ -1560,40 +1684,8 @@ int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int
   cudaStream_t s = (cudaStream_t)stream;
   rc = zero_counters(ws, s);
   if (rc) return rc;
-  if (!ws.grid) {
-    CK(launch_row_sqnorm(x, n, d, ws.xn, s));
-    CK(launch_row_sqnorm(y, m, d, ws.yn, s));
-  }
-  // float32 accuracy at every precision setting: the integer-grid operands where the
-  // workspace has room for them, else CUDA cores
-  TcOps ops;
-  rc = prep_tc(x, n, y, m, d, eps, PROGOT_FP32, ws, &ops, s, f, g);
-  if (rc) return rc;
-  SweepParams pr = make_sweep(x, n, y, m, d, ws.xn, ws.yn, eps, ws, ops.on ? 1 : 2);
-  pr.wA = a;
-  pr.potB = g;
-  pr.potA_old = f;
-  pr.out = row;
-  pr.mode = kModeMarginal;
-  rc = lse_sweep(pr, s, &ops, true, &ws);
-  if (rc) return rc;
-  const int64_t rbr = cdiv(n, fp32_tile_rows());
-  CK(cudaMemcpyAsync(&t_host.hd[0], ws.errpart + rbr, sizeof(double), cudaMemcpyDeviceToHost, s));
-  SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws, ops.on ? 1 : 2);
-  pc.wA = b;
-  pc.potB = f;
-  pc.potA_old = g;
-  pc.out = col;
-  pc.mode = kModeMarginal;
-  rc = lse_sweep(pc, s, &ops, false, &ws);
-  if (rc) return rc;
-  const int64_t rbc = cdiv(m, fp32_tile_rows());
-  CK(cudaMemcpyAsync(&t_host.hd[1], ws.errpart + rbc, sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (err_l1_out) *err_l1_out = t_host.hd[0] + t_host.hd[1];
-  return ops.on ? check_fault(ws, s) : PROGOT_OK;
+  return marginals_core(x, n, y, m, d, f, g, eps, row, col, a, b, err_l1_out, ws, s);
 }
-
 int progot_solve(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m, int32_t d,
                  int32_t K, const double* alpha, const double* eps, const double* tau, int32_t max_iter,
                  int32_t precision, float* x_out, float* g_all, float* f_last, float* x_last, int32_t* iters,
@@ -1945,6 +2037,18 @@ int progot_schedule_eps(const float* x, int64_t n, const float* y, const float* 
     if (rc) return rc;
     rc = map_step(ws.T, mt, y, m, d, ws.gaux, ws.yn, eps, 1.0, precision, ws, s, &ops);
     if (rc) return rc;
+    if (ops.on) {
+      int32_t bad = 0;
+      rc = check_fault(ws, s, &bad);
+      if (rc) return rc;
+      if (bad) {  // the held-out points are still in place: the same on CUDA cores
+        Workspace w;
+        rc = leave_grid(ws.T, mt, y, m, d, ws, &w, s);
+        ops.on = false;
+        if (!rc) rc = map_step(ws.T, mt, y, m, d, ws.gaux, w.yn, eps, 1.0, precision, w, s, &ops);
+        if (rc) return rc;
+      }
+    }
     CK(launch_sq_error(y_test, ws.T, mt, d, ws.rpart, reduce_parts(), ws.rout, s));
     rc = t_host.init();
     if (rc) return rc;

@@ -10,6 +10,20 @@ constexpr double kLog2e = 1.4426950408889634;  // log2(e)
 constexpr double kLn2 = 0.6931471805599453;    // ln(2)
 constexpr int kGridParts = 3;  // operand parts of the integer-grid split (grid_split.cuh)
 
+// Words of the integer-grid operands (grid_split.cuh) in the workspace, written with the
+// operands and read by every kernel on them.
+struct GridWords {
+  float s2;                // 2^(ex + ey): units of the accumulators per log2 unit
+  float inv;               // 2^-(ex + ey)
+  float inv_ey;            // 2^-ey
+  int32_t bad;             // nonzero (the step that found it, counted from 1): the clouds are out of the split's
+                           //   range, kernels on these operands and on later steps' return at entry
+  float norm2_max[2];      // largest squared norm of the centred x and y
+  uint32_t nonzero[2];     // rows with a nonzero norm, and the sums of their squared norms' exponents
+  long long exp_sum[2];    //   about the centre and
+  long long raw_sum[2];    //   about the origin
+};
+
 // Epilogue of a row log-sum-exp sweep, applied once per row after the
 // deterministic combine of the column splits. L_i = log2 sum_j 2^{t_ij}.
 enum SweepMode : int32_t {

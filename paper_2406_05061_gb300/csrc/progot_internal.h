@@ -83,9 +83,9 @@ struct TcMaps {
   const void* bias;   // bias rows of the columns' side (bn-row boxes)
   const void* a_part[2];  // the rows' side bf16 hi, lo operand rows (NULL: grid operands)
 };
-// parts: operand parts in use (1 bf16, 2 bf16x3); gscale non-NULL: the integer-grid split
-// (grid_split.cuh; parts 2 or 3, bn = 128) with its device scales.
-cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const float* gscale,
+// parts: operand parts in use (1 bf16, 2 bf16x3); words non-NULL: the integer-grid split
+// (grid_split.cuh; parts 2 or 3, bn = 128) with its device words.
+cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const GridWords* words,
                                 int bn, int G, int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream,
                                 const float* lrow = nullptr, void* prob = nullptr, int64_t a_row0 = 0);
 // x <- x + alpha (T(x) - x) for rows [row0, row0 + rows) from the P tiles and row sums a
@@ -96,7 +96,7 @@ struct PvLaunch {
   const float* rsum;   // [rows]
   const void* prob;
   const void* mapY[3];
-  const float* gscale;
+  const GridWords* words;
   const float* mu;
   int64_t rows, m;
   int32_t d, parts;
@@ -108,15 +108,15 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream);
 // Tensor-core operands (operands.cu).
 // mu = (mean of the rows of X + mean of the rows of Y) / 2, the sums carried beyond float64
 // rounding of their order; partial: reduce_parts() * d doubles of scratch; ticket: a zero
-// word, zero again afterwards; gmax (or NULL): two words zeroed for launch_operands.
+// word, zero again afterwards; words (or NULL): their norms and counts zeroed for launch_operands.
 cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial,
-                          unsigned* ticket, float* mu, float* gmax, cudaStream_t s);
+                          unsigned* ticket, float* mu, GridWords* words, cudaStream_t s);
 // Both clouds: parts of sqrt(c) (x - mu), rows of dp 16-bit elements (zeros past d): bf16
 // hi, lo, or the integer grid's two or three half-precision parts (grid_split.cuh); unused
 // parts are NULL. Centred squared norms, and bias rows of both sides from the potentials f
 // (x side) and g (y side) where given, into one or two buffers each, rows padded to a
-// multiple of 256. Grid: gmax = the largest squared norms, gscale = {2^(ex + ey),
-// 2^-(ex + ey), 2^-ey}.
+// multiple of 256. Grid: the words of the split; step is what words->bad becomes (when zero)
+// if the clouds are out of its range.
 struct OperandPrep {
   const float* x;
   const float* y;
@@ -126,8 +126,8 @@ struct OperandPrep {
   const float* mu;
   float* xnc;
   float* ync;
-  float* gmax;
-  float* gscale;
+  GridWords* words;
+  int32_t step;
   void* xp[3];
   void* yp[3];
   const float* f;           // NULL: no x-side bias rows
@@ -156,7 +156,7 @@ struct LoopSetup {
   int32_t aligned;          // every CTA on one row block (tc::aligned_segment)
 };
 // kGridHull: the integer grid for clouds inside the hull of the two that the last kGrid call
-// on this workspace saw (same mu and gmax).
+// on this workspace saw (same mu and words).
 enum class OperandKind { kBf16, kGrid, kGridHull };
 cudaError_t launch_operands(const OperandPrep& op, OperandKind kind, const LoopSetup* loop, cudaStream_t s);
 cudaError_t launch_loop_finish(const float* f_new, const float* an, const float* w, double log_w_uniform, double eps,
@@ -216,7 +216,7 @@ struct LoopLaunch {
   // boxes); third parts of the grid split: X, Y (128-row), X, Y (bn-row; any map without
   // the grid split); bias rows X[0], X[1], Y[0], Y[1] (bn-row boxes)
   const void* maps[16];
-  const float* gscale;       // grid split: its device scales (NULL: bf16 operands)
+  const GridWords* words;    // grid split: its device words (NULL: bf16 operands)
   double* errpart;           // [2][row blocks of X]
   SolverState* state;
   int32_t* fault;

@@ -47,7 +47,7 @@ struct PvParams {
   float* out;
   const float* rsum;
   const unsigned char* prob;
-  const float* gscale;
+  const GridWords* words;
   const float* mu;
   int32_t* fault;
   int64_t rows;
@@ -89,6 +89,10 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
     pv_tc(const __grid_constant__ CUtensorMap mapY0, const __grid_constant__ CUtensorMap mapY1,
           const __grid_constant__ CUtensorMap mapY2, const PvParams pp) {
   constexpr int N = 64 * NB, NH = N / 2;  // coordinates of the CTA and of one warpgroup
+  if (__ldg(&pp.words->bad) != 0) {  // no P was written
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
     const int r0 = rank * BM / pp.splits, r1 = (rank + 1) * BM / pp.splits;
     const int64_t left = pp.rows - (int64_t)rb * BM;
     const int rend = left < r1 ? (int)left : r1;
-    const float scale = pp.inv_sc * __ldg(pp.gscale + 2);
+    const float scale = pp.inv_sc * __ldg(&pp.words->inv_ey);
     const uint32_t base = smem_u32(osum);
     for (int q = r0 * N + threadIdx.x; q < rend * N; q += PV_NTHREADS) {
       const int r = q / N, k = q % N, kk = chunk * N + k;
@@ -315,7 +319,7 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream) {
   pp.out = p.out;
   pp.rsum = p.rsum;
   pp.prob = (const unsigned char*)p.prob;
-  pp.gscale = p.gscale;
+  pp.words = p.words;
   pp.mu = p.mu;
   pp.fault = p.fault;
   pp.rows = p.rows;

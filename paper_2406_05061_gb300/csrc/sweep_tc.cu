@@ -91,7 +91,7 @@ struct TcParams {
   int32_t maxseg;     // partial slots per CTA
   int32_t* fault;     // set to 1 by a CTA whose bounded wait expired
   __nv_bfloat16* bias_out;  // potential mode: beta rows of the updated side (rows x 16), or nullptr
-  const float* gscale;      // grid split: {2^(ex + ey), 2^-(ex + ey)} (device)
+  const GridWords* words;   // grid split: its words
   // kModeProb: row L (log2 units) of this launch's rows, which start at operand row a_row0,
   // and the P tiles (see pv_tc.cu): [row block][64-column unit][hi, lo][128 rows x 64]
   const uint4* a_part[2];   // A in TMEM: bf16 hi, lo rows of A (nA x 64 nkb)
@@ -370,7 +370,7 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
       e[h] = row_epilogue(p, i, Lr, rin[h], out_target, &val);
       if (tp.bias_out != nullptr && p.mode == kModePotential) {
         if constexpr (GRID)
-          write_bias_row_grid(tp.bias_out + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), __ldg(tp.gscale));
+          write_bias_row_grid(tp.bias_out + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), __ldg(&tp.words->s2));
         else
           write_bias_row(tp.bias_out + i * 16, (val - rin[h].an) * p.bscale);
       }
@@ -427,6 +427,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // Programmatic dependent launch: let the next sweep's CTAs be scheduled as soon as
   // SMs free up; this kernel's own reads of the previous sweep's results wait below.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (GRID) {
+    // out of the split's range: the host runs this sweep on CUDA cores (the wait keeps the
+    // order of what follows behind what came before)
+    if (__ldg(&tp.words->bad) != 0) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      return;
+    }
+  }
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -727,7 +735,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     constexpr int CW = GRID ? 64 : 128;  // columns folded at a time (registers)
     constexpr int NC = CW / 32;
     int tl = 0, jt = 0;
-    const float inv2 = GRID ? __ldg(tp.gscale + 1) : 1.f;
+    const float inv2 = GRID ? __ldg(&tp.words->inv) : 1.f;
     const uint64_t inv22 = pack2(inv2, inv2);
     const bool prob = GRID && p.mode == kModeProb;
     // potentials, weights and the solver state below are the previous sweep's results
@@ -1068,10 +1076,10 @@ static cudaError_t launch_tc(const tc::TcParams& tp, size_t smem, const TcMaps& 
                             at(m.b[1]), at(m.b[2]), at(m.bias), tp);
 }
 
-cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const float* gscale,
+cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const GridWords* words,
                                 int bn, int G, int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream,
                                 const float* lrow, void* prob, int64_t a_row0) {
-  const bool grid = gscale != nullptr;
+  const bool grid = words != nullptr;
   int stages, a_bufs;
   tc_shape(bn, nkb, parts, grid, &stages, &a_bufs);
   // 128-column bf16 tiles of up to four K blocks and many of them per CTA: A in TMEM, all of
@@ -1097,7 +1105,7 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
   tp.maxseg = maxseg;
   tp.fault = fault;
   tp.bias_out = (__nv_bfloat16*)bias_out;
-  tp.gscale = gscale;
+  tp.words = words;
   tp.lrow = lrow;
   tp.prob = (unsigned char*)prob;
   tp.a_row0 = a_row0;
