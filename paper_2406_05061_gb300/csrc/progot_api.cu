@@ -156,8 +156,22 @@ static int plan_splits(int64_t nA, int64_t nB, int ctas_per_sm, int extra_mult =
 // d = 126, 17 iterations). The grid loops do not drift, and results callers already hold for
 // such clouds would change by as much, so these loops stay on CUDA cores.
 constexpr int32_t kGridSolveDim = 64;
-// Least rows x columns x coordinates of a float32 map step on the tensor cores.
-constexpr double kGridMapWork = 2.5e7;
+// Whether a float32 map of K steps runs on the tensor cores: where their estimated time for the
+// whole call is the smaller. The fixed 77 us are the first step's preparation (the later steps'
+// takes one launch) and the read of the fault word at the end; t the 128 x 128 tiles of a step,
+// in microseconds fitted to both paths measured over 300 shapes (500 to 20000 points, d = 2 to
+// 256, K = 1, 2, 8): CUDA cores / tensor cores 69 / 126 at 2000 x 2000, d = 16, K = 1; 204 / 191
+// at 3000 x 3000, K = 2, and 770 / 544 at K = 8; 110 / 130 there at d = 64, 2000 x 2000, K = 1,
+// and 206 / 185 at K = 2; 5264 / 632 at 8000 x 8000, d = 256, K = 1. The eighth on top covers the
+// fit's error: of those shapes none is more than 3 % slower than its CUDA-core call.
+static bool grid_map_pays(int64_t n, int64_t m, int32_t d, int32_t K) {
+  const double rb = (double)((n + 127) / 128), ct = (double)((m + 127) / 128), t = rb * ct;
+  const double dd = std::max<int32_t>(d, 16), wide = std::max<int32_t>(d - 64, 0);
+  const double cuda_cores = 16.0 + K * (15.0 + 0.36 * dd + t * (0.070 + 0.0021 * dd + 0.0033 * wide) + 0.57 * ct);
+  const double tensor_cores =
+      77.0 + K * (32.0 + 0.081 * std::min(t, 256.0) + 0.063 * std::max(t - 256.0, 0.0) + 0.0005 * t * wide + 0.062 * rb);
+  return 1.12 * tensor_cores < cuda_cores;
+}
 // P of a chunk of rows stays in L2 between the sweep that writes it and the product that
 // reads it; a p-norm cost up to about the size of L2 is kept for its loop.
 constexpr int64_t kProbChunk = (int64_t)64 << 20;
@@ -1629,11 +1643,7 @@ int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, i
   rc = zero_counters(ws, s);
   if (rc) return rc;
   if (out != xq) CK(cudaMemcpyAsync(out, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
-  // Small queries of the float32 path stay on CUDA cores, whose two launches a step cost less
-  // than the grid's four: 28 us against 35 a step at 500 x 500, d = 2; both 39 at 1000 x 2048,
-  // d = 16; 69 against 40 at 1000 x 2048, d = 64; 94 against 62 at 3000 x 3000, d = 16.
-  if (precision == PROGOT_FP32 && (double)nq * (double)m * (double)std::max<int32_t>(d, 16) < kGridMapWork)
-    ws.grid = false;
+  if (precision == PROGOT_FP32 && !grid_map_pays(nq, m, d, K)) ws.grid = false;
   // A capture cannot read the fault word of the tensor-core kernels back; the CUDA cores wait
   // for nothing.
   if (precision == PROGOT_FP32 && ws.grid) {

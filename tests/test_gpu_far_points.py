@@ -54,11 +54,14 @@ def row_terms(x, y, g, eps):
 
 
 @pytest.mark.parametrize("far_x,far_y", [(3e4, 1.0), (1e5, 3e4), (1.0, 1e5)])
-@pytest.mark.parametrize("n,m,d", [(1900, 1700, 24), (2500, 2049, 64)])
+@pytest.mark.parametrize("n,m,d", [(5300, 5200, 24), (3500, 3049, 64)])
 def test_map_of_ordinary_points_beside_very_far_ones(n, m, d, far_x, far_y):
     x, y = clouds(n, m, d, seed=d, far_x=far_x, far_y=far_y)
     eps = 0.05 * 2.0 * d
     g = far_potential(x, y, eps)
+    # the far target weighs nothing: its own t is off by far more than one in float32, so that
+    # whether it has a weight is not a float32 result
+    g[0] -= 1e13 if far_y > 1 else 0.0
     out = nat.entropic_map_apply(dev(x), dev(y), dev(g[None]), [eps], [1.0]).cpu().numpy()
     w, _ = row_terms(x, y, g, eps)
     ref = w @ y.astype(np.float64)
@@ -71,7 +74,7 @@ def test_map_of_ordinary_points_beside_very_far_ones(n, m, d, far_x, far_y):
 
 
 def test_map_rows_that_are_not_finite_stay_alone():
-    n, m, d = 1900, 1700, 24
+    n, m, d = 2500, 2300, 64
     x, y = clouds(n, m, d, seed=1)
     eps = 0.1 * 2.0 * d
     g = np.stack([far_potential(x, y, e) for e in (2 * eps, eps)])

@@ -15,8 +15,8 @@ def dev(a):
 
 
 def problem():
-    p = W.gmm_pair(2500, 2300, 16, seed=2, k=3)
-    eps = 0.2 * float(np.mean((p.x - p.y[: len(p.x)].mean(0)) ** 2) * 16)
+    p = W.gmm_pair(2500, 2300, 64, seed=2, k=3)
+    eps = 0.2 * float(np.mean((p.x - p.y[: len(p.x)].mean(0)) ** 2) * 64)
     g = np.random.default_rng(0).standard_normal((2, 2300)).astype(np.float32) * np.float32(eps)
     return dev(p.x), dev(p.y), dev(g), [2 * eps, eps], [0.5, 1.0]
 
@@ -35,7 +35,7 @@ def test_expired_wait_of_a_float32_map_is_reported():
 
 def test_captured_float32_map_replays_on_new_points():
     x, y, g, eps, alpha = problem()
-    ws = nat.Workspace(2500, 2300, 16)
+    ws = nat.Workspace(2500, 2300, 64)
     out = torch.empty_like(x)
     nat.entropic_map_apply(x, y, g, eps, alpha, out=out, workspace=ws)  # kernels are loaded
     graph = torch.cuda.CUDAGraph()
