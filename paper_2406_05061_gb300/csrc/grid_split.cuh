@@ -11,7 +11,8 @@
 //   l = half(v - h), r = half(v - h - l)  (what is left is below 2^-24),
 // so that every partial sum of h . h' is an integer below 2^22 and accumulates without any
 // rounding. The other products (h l', l h', l l', h r', r h': 2^-11 of the first and less)
-// go to a second accumulator, whose own truncation is 2^-24 of that; the bias is split
+// go to a second accumulator, whose own truncation is 2^-24 of that, and so do l r' and r l'
+// where far points leave the ordinary ones a small part of the grid (grid_reach); the bias is split
 // into its integer part (first accumulator, exact) and its fraction (second). The LSE
 // warps add the two accumulators with one rounding to nearest. So t_ij carries half an
 // ulp, less than the float32 chain of any d, and nothing depends on the order of the
@@ -54,17 +55,24 @@ __device__ __forceinline__ GridScale grid_scale(const GridWords& w, float sc, bo
   return g;
 }
 
-// Whether the split carries these clouds. A point's parts resolve 2^-25 units, 2^-36 of its cloud's
-// largest norm, so a pair of ordinary points has t to 2^-36 max|x~| |y~| c (and the same with the
-// sides swapped), where the CUDA cores' float32 chain has 2^-24 |x||y| c, uncentred: when far points
-// set the grid (or pull the centre away) by more than 2^10 the CUDA cores are the more exact. Norms
-// of ordinary points: geometric means (of powers of two). Below ex + ey = 0 t exceeds 2^22 and float32 log-sum-exps of it lose whole
-// units; a norm that is not finite has no grid at all. Such clouds are left to the CUDA cores.
-constexpr float kGridReach = 10.f;
-__device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const GridScale& g, bool hull) {
+// What the split loses on these clouds beside the CUDA cores' float32 chain, which carries a pair
+// of ordinary points to 2^-24 |x||y| c (uncentred; norms of ordinary points are geometric means, to
+// powers of two). A point's parts resolve 2^-25 units, 2^-36 of its cloud's largest norm, so the
+// grid has t to 2^-36 max|x~| |y~| c, and the same with the sides swapped: when far points set the
+// grid (or pull the centre away) by more than 2^10, x2 below, the CUDA cores are the more exact and
+// the clouds are left to them. Without the products l r' and r l' (2^-14 units a coordinate) it has
+// 2^-39 sqrt(d) max|x~| max|y~| c: they are formed beyond 2^8, x1 below, where that reaches the
+// chain's. (300 x 300, d = 64, one point of each cloud moved out by k spreads, relative error of
+// the other rows' sums: k = 100 2.8e-6 without them and 3e-7 with, k = 300 2.4e-5 and 3e-7, the
+// chain 3e-7.) Below ex + ey = 0 t exceeds 2^22 and float32 log-sum-exps of it lose whole units;
+// a norm that is not finite has no grid at all: both are left to the CUDA cores too.
+struct GridReach {
+  float x1, x2;  // log2
+};
+__device__ __forceinline__ GridReach grid_reach(const GridWords& w, int d, bool hull) {
   const float a = w.norm2_max[0], b = w.norm2_max[1];
-  if (!isfinite(a) || !isfinite(b) || g.ex + g.ey < 0) return true;
-  if (w.nonzero[0] == 0u || w.nonzero[1] == 0u || !(a > 0.f) || !(b > 0.f)) return false;
+  GridReach r = {0.f, 0.f};
+  if (w.nonzero[0] == 0u || w.nonzero[1] == 0u || !(a > 0.f) || !(b > 0.f)) return r;
   // log2 of: largest norms, ordinary norms about the centre and about the origin
   float ax = 0.5f * (float)ilogbf(a);
   const float ay = 0.5f * (float)ilogbf(b);
@@ -77,7 +85,13 @@ __device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const Grid
     cx = fmaxf(cx, cy);
     rx = fminf(rx, ry);
   }
-  return fmaxf(ax + cy, ay + cx) - (rx + ry) > kGridReach;
+  r.x1 = ax + ay - (rx + ry) + fmaxf(0.f, 0.5f * log2f((float)d) - 3.f);
+  r.x2 = fmaxf(ax + cy, ay + cx) - (rx + ry);
+  return r;
+}
+constexpr float kGridCross = 8.f, kGridReach = 10.f;
+__device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const GridScale& g, const GridReach& r) {
+  return !isfinite(w.norm2_max[0]) || !isfinite(w.norm2_max[1]) || g.ex + g.ey < 0 || r.x2 > kGridReach;
 }
 
 // beta = (pot - norm) bscale as an unevaluated sum of two floats (hi + lo): a float32 beta
@@ -167,6 +181,14 @@ __device__ __forceinline__ void issue_grid_part(int part, uint32_t d1, uint32_t 
 #pragma unroll
     for (int kk = 0; kk < KS; ++kk) umma_id(d2, ah + kk * 2, bp + kk * 2, kId, 1u);
   }
+}
+// The products r l' and l r' of a K block (GridWords::cross) by the elected lane (on). Out of line:
+// in the issue loop their mere presence costs the persistent loop 11 % (1150 us against 1032 for
+// 21 updates at 8192^2, d = 64), a call that is not taken nothing.
+template <int BN>
+__device__ __noinline__ void issue_grid_cross(int ksteps, uint64_t a, uint64_t b, uint32_t d2, bool on) {
+  if (!on) return;
+  for (int kk = 0; kk < ksteps; ++kk) umma_id(d2, a + kk * 2, b + kk * 2, make_idesc_f16(BM, BN), 1u);
 }
 template <int BN, int PARTS>
 __device__ __forceinline__ void issue_grid_part(int ksteps, int part, uint32_t d1, uint32_t d2, uint64_t ah,

@@ -606,6 +606,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     if (CONV || lane == 0) {
       const uint64_t abias = desc_sw32(smem_u32(smem + L.a_bias));
       const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
+      const bool cross = GRID && __ldg(&P.words->cross) != 0;
       bool ok = true;
       int tl = 0, ka = 0;
       int s_cur = 0;          // stage of the next B block (ring position, kept without division)
@@ -650,6 +651,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                   if (issuer())
                     issue_grid_part<BN, GRID, kGridParts>(
                         part, d_tmem, d2, ah, al, ar, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)), 0u);
+                  if (part > 0 && __builtin_expect(cross, 0))
+                    issue_grid_cross<BN>(GRID, part == 1 ? ar : al, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)),
+                                         d2, issuer());
                   if (issuer()) umma_commit(&sh.empty[s]);
                 }
               }

@@ -18,6 +18,8 @@ struct GridWords {
   float inv_ey;            // 2^-ey
   int32_t bad;             // nonzero (the step that found it, counted from 1): the clouds are out of the split's
                            //   range, kernels on these operands and on later steps' return at entry
+  int32_t cross;           // nonzero: the products l r' and r l' are formed too
+  int32_t pad_;
   float norm2_max[2];      // largest squared norm of the centred x and y
   uint32_t nonzero[2];     // rows with a nonzero norm, and the sums of their squared norms' exponents
   long long exp_sum[2];    //   about the centre and

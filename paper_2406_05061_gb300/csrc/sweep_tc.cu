@@ -610,6 +610,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
     const uint64_t abias = desc_sw32(smem_u32(smem + L.a_bias));
     const uint64_t abias2 = desc_sw32(smem_u32(smem + L.a_bias + (GRID ? A_BIAS_BYTES : 0)));
+    const bool cross = GRID && __ldg(&tp.words->cross) != 0;
     bool ok = true;
     int u = 0, tl = 0;
     int s_cur = 0;       // ring position and fill parity of unit u, kept without division
@@ -662,6 +663,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                 issue_grid_part<BN, 2>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
                 issue_grid_part<BN, 2>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
               }
+            }
+            if (parts > 2 && __builtin_expect(cross, 0)) {
+              issue_grid_cross<BN>(ksteps, ar, bl, d2, elect_one());
+              issue_grid_cross<BN>(ksteps, al, br, d2, elect_one());
             }
           } else if constexpr (ATM) {
             const uint32_t th = tmem_base + 256 + (uint32_t)(kb * 32), tlo = th + (uint32_t)(nkb * 32);

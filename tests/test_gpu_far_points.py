@@ -121,3 +121,36 @@ def test_marginals_and_metrics_beside_very_far_points():
     assert (err <= tol[1:]).all(), (err / tol[1:]).max()
     met = nat.coupling_metrics(dev(x), dev(y), dev(f), dev(g), eps)
     assert abs(met["mass"] - P.sum()) <= (tol[1:] * P.sum(1)[1:]).sum()
+
+
+@pytest.mark.parametrize("far", [100.0, 300.0, 1000.0])
+@pytest.mark.parametrize("n,m,d", [(300, 300, 64), (500, 450, 16), (260, 390, 33)])
+def test_far_points_in_both_clouds_leave_the_others_float32_accuracy(n, m, d, far):
+    x, y = clouds(n, m, d, seed=n + d, far_x=far, far_y=far)
+    eps = 0.05 * 2.0 * d
+    g = far_potential(x, y, eps)
+    g[0] -= 1e12  # as above
+    w, lse = row_terms(x, y, g, eps)
+    f = (-eps * lse - eps * np.log(n)).astype(np.float32)
+    P = np.exp((f[:, None].astype(np.float64) + g[None, :] - sq_cost(x, y)) / eps)
+    row, _, _ = nat.coupling_marginals(dev(x), dev(y), dev(f), dev(g), eps)
+    xn = (x.astype(np.float64) ** 2).sum(1)
+    dt = pair_error(x, y, g, eps)
+    tol = (w * dt).sum(1) + 2.0 ** -21 * (np.abs(f) + xn) / eps + 2.0 ** -20
+    err = np.abs(row.cpu().numpy()[1:] / P.sum(1)[1:] - 1)
+    assert (err <= tol[1:] / 4).all(), (err / tol[1:]).max()  # two roundings a term, not eight
+
+
+@pytest.mark.parametrize("far", [100.0, 300.0, 1000.0])
+@pytest.mark.parametrize("n,m,d", [(300, 300, 64), (1500, 1450, 16)])
+def test_one_loop_update_beside_far_points(n, m, d, far):
+    """f of one iteration from g = 0 (the far column weighs nothing in the other rows)."""
+    x, y = clouds(n, m, d, seed=n + 2 * d, far_x=far, far_y=far)
+    eps = 0.05 * 2.0 * d
+    r = nat.sinkhorn_potentials(dev(x), dev(y), eps, 0.0, 1)
+    g0 = np.zeros(m, np.float32)
+    w, lse = row_terms(x, y, g0, eps)
+    xn = (x.astype(np.float64) ** 2).sum(1)
+    tol = eps * ((w * pair_error(x, y, g0, eps)).sum(1) + 2.0 ** -21 * xn / eps + 2.0 ** -20)
+    err = np.abs(r.f.cpu().numpy() - (-eps * lse - eps * np.log(n)))
+    assert (err[1:] <= tol[1:] / 4).all(), (err[1:] / tol[1:]).max()
