@@ -90,8 +90,9 @@ __device__ __forceinline__ GridReach grid_reach(const GridWords& w, int d, bool 
   return r;
 }
 constexpr float kGridCross = 8.f, kGridReach = 10.f;
-__device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const GridScale& g, const GridReach& r) {
-  return !isfinite(w.norm2_max[0]) || !isfinite(w.norm2_max[1]) || g.ex + g.ey < 0 || r.x2 > kGridReach;
+__device__ __forceinline__ bool grid_out_of_range(const GridWords& w, const GridScale& g, const GridReach& r,
+                                                  int min_exp) {
+  return !isfinite(w.norm2_max[0]) || !isfinite(w.norm2_max[1]) || g.ex + g.ey < min_exp || r.x2 > kGridReach;
 }
 
 // beta = (pot - norm) bscale as an unevaluated sum of two floats (hi + lo): a float32 beta

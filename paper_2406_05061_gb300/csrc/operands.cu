@@ -309,7 +309,7 @@ __global__ void operands_kernel(OperandPrep op, LoopSetup ls, int row_blocks) {
       op.words->inv_ey = ldexpf(1.f, -gs.ey);
       const GridReach gr = grid_reach(*op.words, op.d, GRID == 2);
       op.words->cross = gr.x1 > kGridCross;
-      if (op.words->bad == 0 && grid_out_of_range(*op.words, gs, gr)) op.words->bad = op.step;
+      if (op.words->bad == 0 && grid_out_of_range(*op.words, gs, gr, op.min_exp)) op.words->bad = op.step;
     }
   }
   float nv = 0.f;

@@ -584,6 +584,10 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   op.ync = ws.ync;
   op.words = ws.words;
   op.step = step;
+  // L of the bf16x3 operands against P of the grid's: P = 2^{t - L + 14} in half precision has
+  // room for two bits of difference. bf16x3 has t to 2^-16 |x~||y~| c (three omitted terms of
+  // 2^-18 and the truncated sums of a few thousand coordinates), which is 2^(6 - ex - ey).
+  op.min_exp = two && precision != PROGOT_BF16 ? 6 : 0;
   op.xp[0] = ws.xh;
   op.xp[1] = ops->parts > 1 ? ws.xl : nullptr;
   op.xp[2] = ops->parts > 2 ? ws.xr : nullptr;
@@ -1203,12 +1207,17 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
   pl.out = ws.L;
   pl.mode = kModeLse;
   apply_cost(pl, cost, eps);
+  const bool map_tc = tc && g_map_tc.load();
+  // the mixed precisions' map beyond d = 256 gets integer-grid operands of its own; their t
+  // can differ by many bits from a hi-only t, so L is then taken from them
+  const bool remake = map_tc && !ops->words && ops->nkb > 1 && !map_tc_onepass_supported(ops->nkb);
+  const bool own_l = remake && ops->parts < 2;
   // the persistent loop that produced g may already have left L in ws.L
-  int rc = (tc && ops->lse_ready) ? PROGOT_OK
-           : tc                   ? lse_sweep(pl, s, ops, true, &ws)
-                                  : lse_sweep(pl, s);
+  int rc = own_l || (tc && ops->lse_ready) ? PROGOT_OK
+           : tc                            ? lse_sweep(pl, s, ops, true, &ws)
+                                           : lse_sweep(pl, s);
   if (rc) return rc;
-  if (tc && !ops->words && ops->nkb == 1 && g_map_tc.load()) {
+  if (map_tc && !ops->words && ops->nkb == 1) {
     // d <= 64: S and P Y both on the tensor cores (P Y reuses the centred, scaled y operand)
     int G = 0, maxseg = 0;
     tc_plan(n, m, 128, num_sms(), &G, &maxseg);
@@ -1221,7 +1230,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
   }
-  if (tc && !ops->words && ops->nkb > 1 && map_tc_onepass_supported(ops->nkb) && g_map_tc.load()) {
+  if (map_tc && !ops->words && !remake) {
     // 64 < d <= 256: one launch, S once per tile, all output coordinates in TMEM
     int G = 0, maxseg = 0;
     tc_plan(n, m, map_tc_onepass_tile_cols(), num_sms(), &G, &maxseg);
@@ -1235,18 +1244,19 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     return PROGOT_OK;
   }
   TcOps gops;
-  if (tc && g_map_tc.load()) {
-    // float32 path, and the bf16x3 path for d > 256 (its operands give way to the
+  if (map_tc) {
+    // float32 path, and the mixed precisions for d > 256 (their operands give way to the
     // integer-grid ones, whose accuracy the CUDA-core map it replaces had): P a chunk of
     // row blocks at a time, then P Y
     const TcOps* go = ops;
-    if (!ops->words) {
+    if (remake) {
       rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g, false, Operands::kGridTwoParts);
+      if (!rc && own_l) rc = lse_sweep(pl, s, &gops, true, &ws);
       if (rc) return rc;
       go = &gops;
     }
     rc = grid_map_step(X, n, m, d, eps, alpha, ws, s, *go);
-    if (rc || ops->words) return rc;  // the float32 path's callers look at words->bad
+    if (rc || !remake) return rc;  // the float32 path's callers look at words->bad
     int32_t bad = 0;
     rc = check_fault(ws, s, &bad);
     if (rc || !bad) return rc;

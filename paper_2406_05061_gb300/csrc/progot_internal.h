@@ -128,6 +128,7 @@ struct OperandPrep {
   float* ync;
   GridWords* words;
   int32_t step;
+  int32_t min_exp;          // least ex + ey within range
   void* xp[3];
   void* yp[3];
   const float* f;           // NULL: no x-side bias rows
