@@ -160,7 +160,7 @@ namespace tc {
 // meet it, KS steps of K = 16: only h h' goes to the first accumulator d1. Unrolled, so
 // that the descriptors are constants apart from their base (at N = 128 a product lasts 64
 // cycles, about what a loop around it costs the issuing thread).
-template <int BN, int KS, int PARTS>
+template <int BN, int KS>
 __device__ __forceinline__ void issue_grid_part(int part, uint32_t d1, uint32_t d2, uint64_t ah, uint64_t al,
                                                 uint64_t ar, uint64_t bp, uint32_t more) {
   constexpr uint32_t kId = make_idesc_f16(BM, BN);
@@ -170,7 +170,7 @@ __device__ __forceinline__ void issue_grid_part(int part, uint32_t d1, uint32_t 
       // +32 bytes per K = 16 step inside the 128-byte swizzle atom (encoded >> 4)
       umma_id(d1, ah + kk * 2, bp + kk * 2, kId, kk > 0 ? 1u : more);
       umma_id(d2, al + kk * 2, bp + kk * 2, kId, kk > 0 ? 1u : more);
-      if (PARTS > 2) umma_id(d2, ar + kk * 2, bp + kk * 2, kId, 1u);
+      umma_id(d2, ar + kk * 2, bp + kk * 2, kId, 1u);
     }
   } else if (part == 1) {
 #pragma unroll
@@ -191,17 +191,17 @@ __device__ __noinline__ void issue_grid_cross(int ksteps, uint64_t a, uint64_t b
   if (!on) return;
   for (int kk = 0; kk < ksteps; ++kk) umma_id(d2, a + kk * 2, b + kk * 2, make_idesc_f16(BM, BN), 1u);
 }
-template <int BN, int PARTS>
+template <int BN>
 __device__ __forceinline__ void issue_grid_part(int ksteps, int part, uint32_t d1, uint32_t d2, uint64_t ah,
                                                 uint64_t al, uint64_t ar, uint64_t bp, uint32_t more) {
   if (ksteps == 4)
-    issue_grid_part<BN, 4, PARTS>(part, d1, d2, ah, al, ar, bp, more);
+    issue_grid_part<BN, 4>(part, d1, d2, ah, al, ar, bp, more);
   else if (ksteps == 3)
-    issue_grid_part<BN, 3, PARTS>(part, d1, d2, ah, al, ar, bp, more);
+    issue_grid_part<BN, 3>(part, d1, d2, ah, al, ar, bp, more);
   else if (ksteps == 2)
-    issue_grid_part<BN, 2, PARTS>(part, d1, d2, ah, al, ar, bp, more);
+    issue_grid_part<BN, 2>(part, d1, d2, ah, al, ar, bp, more);
   else
-    issue_grid_part<BN, 1, PARTS>(part, d1, d2, ah, al, ar, bp, more);
+    issue_grid_part<BN, 1>(part, d1, d2, ah, al, ar, bp, more);
 }
 
 }  // namespace tc

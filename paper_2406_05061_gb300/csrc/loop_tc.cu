@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                   if (!ok) break;
                   tc_fence_after();
                   if (issuer())
-                    issue_grid_part<BN, GRID, kGridParts>(
+                    issue_grid_part<BN, GRID>(
                         part, d_tmem, d2, ah, al, ar, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)), 0u);
                   if (part > 0 && __builtin_expect(cross, 0))
                     issue_grid_cross<BN>(GRID, part == 1 ? ar : al, desc_sw128(smem_u32(smem + L.stage0 + s * L.stage_bytes)),

@@ -333,21 +333,27 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
   ws.ltab_crow = (int2*)take(w.tc ? sizeof(int2) * 2 * (size_t)w.rbmax : 0);
   ws.ltab_nseg = (int32_t*)take(w.tc ? sizeof(int32_t) * 2 * (size_t)num_sms() : 0);
   ws.lerr = (double*)take(w.tc ? sizeof(double) * 2 * (size_t)w.rbmax : 0);
-  ws.xr = take(w.grid ? opb : 0);
-  ws.yr = take(w.grid ? opb : 0);
-  // Map steps on integer-grid operands keep P for a chunk of row blocks (kProbChunk; one row
-  // block at least, less when all of P is smaller); p-norm loops their cost (kCostBytes). The bf16x3 path needs them for d > 256, where
-  // the partial buffers of the CUDA-core map are idle and larger than one row block's P.
+  // Third parts of integer-grid operands; their map steps keep P for a chunk of row blocks
+  // (kProbChunk; one row block at least, less when all of P is smaller), p-norm loops their
+  // cost (kCostBytes).
   if (w.grid) {
+    ws.xr = take(opb);
+    ws.yr = take(opb);
     const int64_t block = pv_prob_bytes_per_block(w.nmax);
     ws.prob_bytes = std::max<int64_t>(block, std::min<int64_t>(block * w.rbmax, kCostBytes));
     ws.prob = take((size_t)ws.prob_bytes);
-    ws.rsum = ws.Rpart;
   } else {
-    ws.prob = (char*)ws.Opart;
-    ws.prob_bytes = (int64_t)sizeof(float) * w.opart_elems;
-    ws.rsum = ws.Rpart;
+    // The mixed precisions need them for d > 256, in the partial buffer of the CUDA-core map,
+    // which is idle then: it has 4 d bytes for more than 2 nmax + 128 rows, the third parts take
+    // 4 dp < 4 (d + 64) for nmax of them, and one row block's P, 512 bytes a row, fits in the rest.
+    const size_t third = align256(opb), have = sizeof(float) * (size_t)w.opart_elems;
+    const bool room = w.tc && have > 2 * third;
+    ws.xr = room ? (char*)ws.Opart : nullptr;
+    ws.yr = room ? (char*)ws.Opart + third : nullptr;
+    ws.prob = room ? (char*)ws.Opart + 2 * third : nullptr;
+    ws.prob_bytes = room ? (int64_t)(have - 2 * third) : 0;
   }
+  ws.rsum = ws.Rpart;
   ws.grid = w.grid;
   ws.bytes = off;
   if (out) *out = ws;
@@ -527,13 +533,13 @@ static LoopSetup loop_setup_params(int64_t n, int64_t m, const TcOps& ops, const
   return ls;
 }
 
-// What prep_tc prepares: bf16 operands of the precision setting, the integer grid's three
-// parts (the float32 path) or two of them on a centre already in ws.mu (the bf16x3 path's
-// map step for d > 256).
+// What prep_tc prepares: bf16 operands of the precision setting or the integer grid's three
+// parts (the float32 path); kGridMap: the latter on a centre already in ws.mu, without regard to
+// the precision setting (the mixed precisions' map step for d > 256).
 // kMoved: as kAuto after an earlier kAuto of the same solve or map, the x cloud having moved
 // by map steps only: the integer grid then keeps its centre and its norms' bound, and needs
 // one launch (the bf16 operands are centred anew).
-enum class Operands { kAuto, kMoved, kGridTwoParts };
+enum class Operands { kAuto, kMoved, kGridMap };
 
 // Tensor-core operands of both clouds at this eps (operands.cu) and their TMA descriptions;
 // bias rows of both sides from the current potentials (f on x, g on y) and the centred
@@ -547,7 +553,7 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
                    const Workspace& ws, TcOps* ops, cudaStream_t s, const float* f_cur = nullptr,
                    const float* g_cur = nullptr, bool loop = false, Operands kind = Operands::kAuto,
                    int32_t step = 1) {
-  const bool two = kind == Operands::kGridTwoParts, grid = precision == PROGOT_FP32 || two;
+  const bool remake = kind == Operands::kGridMap, grid = precision == PROGOT_FP32 || remake;
   ops->on = precision != PROGOT_FP32 || ws.grid;
   ops->lse_ready = false;
   ops->loop = false;
@@ -556,7 +562,7 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   const int32_t dp = pad64(d);
   ops->nkb = dp / 64;
   ops->split3 = precision != PROGOT_BF16 ? 1 : 0;
-  ops->parts = grid ? (two ? 2 : kGridParts) : 1 + ops->split3;
+  ops->parts = grid ? kGridParts : 1 + ops->split3;
   if (!grid && tc_stages(ops->nkb, ops->split3) < 2)
     return fail(PROGOT_ERR_INVALID_ARG, "d = %d is too large for the tensor-core sweep", d);
   ops->bn = grid ? 128 : tc_tile_cols(ops->nkb, ops->split3);
@@ -564,7 +570,7 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   ops->xnc = ws.xnc;
   ops->ync = ws.ync;
   const bool hull = grid && kind == Operands::kMoved;
-  if (two)
+  if (remake)
     CK(cudaMemsetAsync(ws.words->norm2_max, 0, sizeof(GridWords) - offsetof(GridWords, norm2_max), s));
   else if (!hull)
     CK(launch_center(x, n, y, m, d, ws.rpart, ws.ticket, ws.mu, grid ? ws.words : nullptr, s));
@@ -587,13 +593,13 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   // L of the bf16x3 operands against P of the grid's: P = 2^{t - L + 14} in half precision has
   // room for two bits of difference. bf16x3 has t to 2^-16 |x~||y~| c (three omitted terms of
   // 2^-18 and the truncated sums of a few thousand coordinates), which is 2^(6 - ex - ey).
-  op.min_exp = two && precision != PROGOT_BF16 ? 6 : 0;
+  op.min_exp = remake && precision != PROGOT_BF16 ? 6 : 0;
   op.xp[0] = ws.xh;
   op.xp[1] = ops->parts > 1 ? ws.xl : nullptr;
-  op.xp[2] = ops->parts > 2 ? ws.xr : nullptr;
+  op.xp[2] = grid ? ws.xr : nullptr;
   op.yp[0] = ws.yh;
   op.yp[1] = ops->parts > 1 ? ws.yl : nullptr;
-  op.yp[2] = ops->parts > 2 ? ws.yr : nullptr;
+  op.yp[2] = grid ? ws.yr : nullptr;
   op.f = f_cur;
   op.g = g_cur;
   op.bscale = (float)(kLog2e / eps);
@@ -623,8 +629,8 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   if (!rc) rc = make_map(&ops->yh_a, ws.yh, m, dp, 128);
   if (!rc) rc = make_map(&ops->yl_a, yl, m, dp, 128);
   if (!rc && grid) {
-    rc = make_map(&ops->xr_a, ops->parts > 2 ? ws.xr : xl, n, dp, 128);
-    if (!rc) rc = make_map(&ops->yr_a, ops->parts > 2 ? ws.yr : yl, m, dp, 128);
+    rc = make_map(&ops->xr_a, ws.xr, n, dp, 128);
+    if (!rc) rc = make_map(&ops->yr_a, ws.yr, m, dp, 128);
   }
   if (ops->bn == 128) {
     // the same boxes serve both roles
@@ -1148,9 +1154,9 @@ static int sinkhorn_core(const float* x, const float* a, int64_t n, const float*
 // ws.prob holds, a sweep writes P and its row sums (ws.L the stabiliser), then P Y.
 static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, double alpha, const Workspace& ws,
                          cudaStream_t s, const TcOps& ops) {
-  CUtensorMap ymap[3];
-  void* const yparts[3] = {ws.yh, ws.yl, ops.parts > 2 ? ws.yr : ws.yl};
-  for (int q = 0; q < 3; ++q) {
+  CUtensorMap ymap[kGridParts];
+  void* const yparts[kGridParts] = {ws.yh, ws.yl, ws.yr};
+  for (int q = 0; q < kGridParts; ++q) {
     const int rc = make_map(&ymap[q], yparts[q], m, pad64(d), 64);
     if (rc) return rc;
   }
@@ -1176,13 +1182,12 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
     pv.out = X + row0 * d;
     pv.rsum = ws.rsum + row0;
     pv.prob = ws.prob;
-    for (int q = 0; q < 3; ++q) pv.mapY[q] = &ymap[q];
+    for (int q = 0; q < kGridParts; ++q) pv.mapY[q] = &ymap[q];
     pv.words = ops.words;
     pv.mu = ops.mu;
     pv.rows = rows;
     pv.m = m;
     pv.d = d;
-    pv.parts = ops.parts;
     pv.alpha = (float)alpha;
     pv.inv_sc = (float)std::sqrt(eps / (2.0 * kLog2e));
     pv.fault = ws.fault;
@@ -1250,7 +1255,7 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     // row blocks at a time, then P Y
     const TcOps* go = ops;
     if (remake) {
-      rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g, false, Operands::kGridTwoParts);
+      rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g, false, Operands::kGridMap);
       if (!rc && own_l) rc = lse_sweep(pl, s, &gops, true, &ws);
       if (rc) return rc;
       go = &gops;

@@ -84,7 +84,7 @@ struct TcMaps {
   const void* a_part[2];  // the rows' side bf16 hi, lo operand rows (NULL: grid operands)
 };
 // parts: operand parts in use (1 bf16, 2 bf16x3); words non-NULL: the integer-grid split
-// (grid_split.cuh; parts 2 or 3, bn = 128) with its device words.
+// (grid_split.cuh; three parts, bn = 128) with its device words.
 cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nkb, int parts, const GridWords* words,
                                 int bn, int G, int maxseg, int32_t* fault, void* bias_out, cudaStream_t stream,
                                 const float* lrow = nullptr, void* prob = nullptr, int64_t a_row0 = 0);
@@ -95,11 +95,11 @@ struct PvLaunch {
   float* out;
   const float* rsum;   // [rows]
   const void* prob;
-  const void* mapY[3];
+  const void* mapY[kGridParts];
   const GridWords* words;
   const float* mu;
   int64_t rows, m;
-  int32_t d, parts;
+  int32_t d;
   float alpha, inv_sc; // inv_sc = 1 / sqrt(c)
   int32_t* fault;
 };

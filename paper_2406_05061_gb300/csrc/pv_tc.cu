@@ -51,7 +51,7 @@ struct PvParams {
   const float* mu;
   int32_t* fault;
   int64_t rows;
-  int32_t d, parts, units, chunks, splits, stages;
+  int32_t d, units, chunks, splits, stages;
   float alpha, inv_sc;
 };
 
@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ PvShared sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int parts = pp.parts, S = pp.stages;
-  const uint32_t st_bytes = PV_P_BYTES + (uint32_t)parts * NB * PV_Y_BYTES;
+  const int S = pp.stages;
+  constexpr uint32_t st_bytes = PV_P_BYTES + kGridParts * NB * PV_Y_BYTES;
   const int rank = blockIdx.x % pp.splits, tile = blockIdx.x / pp.splits;
   const int chunk = tile % pp.chunks, rb = tile / pp.chunks;
   const int u0 = (int)((int64_t)rank * pp.units / pp.splits), u1 = (int)((int64_t)(rank + 1) * pp.units / pp.splits);
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
       if (elect_one()) {
         mbar_arrive_expect_tx(&sh.full[s], st_bytes);
         bulk_load(st, pp.prob + ((int64_t)rb * pp.units + u0 + u) * PV_P_BYTES, PV_P_BYTES, &sh.full[s]);
-        for (int q = 0; q < parts; ++q) {
+        for (int q = 0; q < kGridParts; ++q) {
           const CUtensorMap* mY = q == 0 ? &mapY0 : q == 1 ? &mapY1 : &mapY2;
           // coordinates past the operand's width are filled with zeros
           for (int b = 0; b < NB; ++b)
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
           umma_id(d2, ph + adv, y1 + bdv, kId, more);
           umma_id(d2, pl + adv, y0 + bdv, kId, 1u);
           umma_id(d2, pl + adv, y1 + bdv, kId, 1u);
-          if (parts > 2) umma_id(d2, ph + adv, y2 + bdv, kId, 1u);
+          umma_id(d2, ph + adv, y2 + bdv, kId, 1u);
         }
         umma_commit(&sh.empty[s]);
         umma_commit(&sh.acc_full[b]);
@@ -324,7 +324,6 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream) {
   pp.fault = p.fault;
   pp.rows = p.rows;
   pp.d = p.d;
-  pp.parts = p.parts;
   pp.alpha = p.alpha;
   pp.inv_sc = p.inv_sc;
   const int nb = p.d > 64 ? 2 : 1;
@@ -342,12 +341,11 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream) {
       pp.splits = s;
     }
   }
-  const uint32_t st_bytes = tc::PV_P_BYTES + (uint32_t)p.parts * nb * tc::PV_Y_BYTES;
+  const uint32_t st_bytes = tc::PV_P_BYTES + (uint32_t)kGridParts * nb * tc::PV_Y_BYTES;
   pp.stages = std::min<int>(tc::PV_MAXST, (int)((225 * 1024) / st_bytes));
   const size_t smem = std::max<size_t>((size_t)pp.stages * st_bytes, (size_t)128 * (64 * nb + 1) * 4) + 1024;
-  const void* maps[3] = {p.mapY[0], p.mapY[1], p.parts > 2 ? p.mapY[2] : p.mapY[1]};
-  const int grid = (int)(tiles * pp.splits);
-  const cudaError_t e = nb == 2 ? launch_pv<2>(pp, grid, smem, maps, stream) : launch_pv<1>(pp, grid, smem, maps, stream);
+    const int grid = (int)(tiles * pp.splits);
+  const cudaError_t e = nb == 2 ? launch_pv<2>(pp, grid, smem, p.mapY, stream) : launch_pv<1>(pp, grid, smem, p.mapY, stream);
   count_launch();
   return e;
 }

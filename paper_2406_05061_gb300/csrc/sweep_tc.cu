@@ -82,7 +82,7 @@ struct TcShared {
 struct TcParams {
   SweepParams p;
   int32_t nkb;        // K blocks of 64
-  int32_t parts;      // operand parts: 1 bf16 (hi only), 2 bf16x3 (hi, lo), or the grid split's 2 or 3
+  int32_t parts;      // operand parts: 1 bf16 (hi only), 2 bf16x3 (hi, lo), 3 the grid split
   int32_t stages;     // B pipeline depth (units of one K block of one tile)
   int32_t a_bufs;     // 1 or 2 resident A-operand buffers, or 0: A K blocks stream with B
   int32_t G;          // CTAs
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             tma_load_2d(abuf + kb * A_TILE_BYTES, &mapAh, &sh.a_full[ai], kb * KB, a_row);
             if (parts > 1)
               tma_load_2d(abuf + L.a_lo_off + kb * A_TILE_BYTES, &mapAl, &sh.a_full[ai], kb * KB, a_row);
-            if (GRID && parts > 2)
+            if constexpr (GRID)
               tma_load_2d(abuf + 2 * L.a_lo_off + kb * A_TILE_BYTES, &mapAr, &sh.a_full[ai], kb * KB, a_row);
           }
         }
@@ -579,12 +579,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             mbar_arrive_expect_tx(&sh.full[s], bbytes + sabytes + (bias_now ? BIAS_TILE_BYTES : 0u));
             tma_load_2d(st, &mapBh, &sh.full[s], kb * KB, t * BN);
             if (parts > 1) tma_load_2d(st + L.b_lo_off, &mapBl, &sh.full[s], kb * KB, t * BN);
-            if (GRID && parts > 2) tma_load_2d(st + 2 * L.b_lo_off, &mapBr, &sh.full[s], kb * KB, t * BN);
+            if constexpr (GRID) tma_load_2d(st + 2 * L.b_lo_off, &mapBr, &sh.full[s], kb * KB, t * BN);
             if (bias_now) tma_load_2d(st + L.bias_off, &mapBbias, &sh.full[s], 0, t * BN);
             if (!ATM && NA == 0) {
               tma_load_2d(st + L.a_stage_off, &mapAh, &sh.full[s], kb * KB, a_row);
               if (parts > 1) tma_load_2d(st + L.a_stage_off + A_TILE_BYTES, &mapAl, &sh.full[s], kb * KB, a_row);
-              if (GRID && parts > 2)
+              if constexpr (GRID)
                 tma_load_2d(st + L.a_stage_off + 2 * A_TILE_BYTES, &mapAr, &sh.full[s], kb * KB, a_row);
             }
             if (waited || kb != 0) mbar_arrive(&sh.bias_full[s]);
@@ -655,16 +655,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t d2 = d_tmem + 256;
             if (elect_one()) {
               const uint32_t more = kb > 0 ? 1u : 0u;
-              if (parts > 2) {
-                issue_grid_part<BN, 3>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
-                issue_grid_part<BN, 3>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
-                issue_grid_part<BN, 3>(ksteps, 2, d_tmem, d2, ah, al, ar, br, more);
-              } else {
-                issue_grid_part<BN, 2>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
-                issue_grid_part<BN, 2>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
-              }
+              issue_grid_part<BN>(ksteps, 0, d_tmem, d2, ah, al, ar, bh, more);
+              issue_grid_part<BN>(ksteps, 1, d_tmem, d2, ah, al, ar, bl, more);
+              issue_grid_part<BN>(ksteps, 2, d_tmem, d2, ah, al, ar, br, more);
             }
-            if (parts > 2 && __builtin_expect(cross, 0)) {
+            if (__builtin_expect(cross, 0)) {
               issue_grid_cross<BN>(ksteps, ar, bl, d2, elect_one());
               issue_grid_cross<BN>(ksteps, al, br, d2, elect_one());
             }
@@ -1095,7 +1090,7 @@ cudaError_t launch_lse_sweep_tc(const SweepParams& p, const TcMaps& maps, int nk
     a_bufs = 0;
     stages = tc_stages_atm(nkb, parts);
   }
-  if (stages < 2 || (bn != 128 && bn != 256) || (grid && (bn != 128 || parts < 2)) || parts < 1 || parts > 3)
+  if (stages < 2 || (bn != 128 && bn != 256) || parts != (grid ? kGridParts : std::clamp(parts, 1, 2)) || (grid && bn != 128))
     return cudaErrorInvalidValue;
   const size_t smem = tc::smem_layout(bn, nkb, parts, stages, a_bufs, grid, atm).total;
   tc::TcParams tp;

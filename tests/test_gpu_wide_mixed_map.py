@@ -65,3 +65,28 @@ def test_map_far_below_the_cost_stays_finite(n, m, d, cloud, precision, scale):
     tol = 8 * bound(x, y, eps)
     if tol < 0.5:
         np.testing.assert_allclose(out, exact_map(x, y, g, eps), rtol=0, atol=tol * spread)
+
+
+@pytest.mark.parametrize("d,far", [(300, 1.0), (300, 16.0), (1000, 1.0), (1000, 16.0), (1024, 4.0)])
+@pytest.mark.parametrize("precision", ["bf16x3", "bf16", "fp32"])
+def test_map_is_no_further_from_float64_than_float32_products(d, far, precision):
+    """The CUDA-core map (float32 throughout) is the measure; a quarter on top for the sample."""
+    rng = np.random.default_rng(d)
+    x, y = rng.standard_normal((1500, d)), rng.standard_normal((1400, d))
+    y[0] *= far
+    x, y = x.astype(np.float32), y.astype(np.float32)
+    eps = 0.1 * d
+    g = (rng.standard_normal(1400) * eps).astype(np.float32)
+    if far > 1:
+        g[0] = -1e9 * eps  # without weight: its own score is no float32 result
+    ref = exact_map(x, y, g, eps)
+    args = (dev(x), dev(y), dev(g[None]), [eps], [1.0])
+    err = {}
+    for tc in (True, False):
+        nat.set_map_tc(tc)
+        try:
+            out = nat.entropic_map_apply(*args, precision=precision if tc else "bf16x3")
+        finally:
+            nat.set_map_tc(True)
+        err[tc] = float(np.sqrt(((out.cpu().numpy() - ref) ** 2).mean()))
+    assert err[True] <= 1.25 * err[False], err
