@@ -59,12 +59,17 @@ __device__ __forceinline__ GridScale grid_scale(const GridWords& w, float sc, bo
 // of ordinary points to 2^-24 |x||y| c (uncentred; norms of ordinary points are geometric means, to
 // powers of two). A point's parts resolve 2^-25 units, 2^-36 of its cloud's largest norm, so the
 // grid has t to 2^-36 max|x~| |y~| c, and the same with the sides swapped: when far points set the
-// grid (or pull the centre away) by more than 2^10, x2 below, the CUDA cores are the more exact and
+// grid (or pull the centre away) by more than 2^10 (d <= 64), x2 below, the CUDA cores are the more exact and
 // the clouds are left to them. Without the products l r' and r l' (2^-14 units a coordinate) it has
 // 2^-39 sqrt(d) max|x~| max|y~| c: they are formed beyond 2^8, x1 below, where that reaches the
 // chain's. (300 x 300, d = 64, one point of each cloud moved out by k spreads, relative error of
 // the other rows' sums: k = 100 2.8e-6 without them and 3e-7 with, k = 300 2.4e-5 and 3e-7, the
-// chain 3e-7.) Below ex + ey = 0 t exceeds 2^22 and float32 log-sum-exps of it lose whole units;
+// chain 3e-7.) With many coordinates an ordinary point beside a far one has its leading parts near
+// zero, so that the second accumulator carries the sums and truncates them at every K step: 1.2 bits
+// of reach for every doubling of d beyond 64 (a map beside one far y, rms error of the others against
+// the CUDA cores': d = 300, 64 spreads 6.0e-8 against 7.5e-8 and 300 spreads 2.1e-7; d = 1000, 32
+// spreads 4.7e-8 against 4.4e-8 and 64 spreads 1.1e-7; d = 3000, 16 spreads 5.1e-8 against 4.3e-8
+// and 64 spreads 2.3e-7), at most 7.5, so that clouds without far points stay. Below ex + ey = 0 t exceeds 2^22 and float32 log-sum-exps of it lose whole units;
 // a norm that is not finite has no grid at all: both are left to the CUDA cores too.
 struct GridReach {
   float x1, x2;  // log2
@@ -86,7 +91,7 @@ __device__ __forceinline__ GridReach grid_reach(const GridWords& w, int d, bool 
     rx = fminf(rx, ry);
   }
   r.x1 = ax + ay - (rx + ry) + fmaxf(0.f, 0.5f * log2f((float)d) - 3.f);
-  r.x2 = fmaxf(ax + cy, ay + cx) - (rx + ry);
+  r.x2 = fmaxf(ax + cy, ay + cx) - (rx + ry) + fminf(7.5f, 1.2f * fmaxf(0.f, log2f((float)d) - 6.f));
   return r;
 }
 constexpr float kGridCross = 8.f, kGridReach = 10.f;

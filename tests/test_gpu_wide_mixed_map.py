@@ -67,7 +67,8 @@ def test_map_far_below_the_cost_stays_finite(n, m, d, cloud, precision, scale):
         np.testing.assert_allclose(out, exact_map(x, y, g, eps), rtol=0, atol=tol * spread)
 
 
-@pytest.mark.parametrize("d,far", [(300, 1.0), (300, 16.0), (1000, 1.0), (1000, 16.0), (1024, 4.0)])
+@pytest.mark.parametrize("d,far", [(300, 1.0), (300, 16.0), (1000, 1.0), (1000, 16.0), (1024, 4.0), (300, 300.0),
+                                   (1000, 100.0), (3000, 40.0), (3000, 1000.0)])
 @pytest.mark.parametrize("precision", ["bf16x3", "bf16", "fp32"])
 def test_map_is_no_further_from_float64_than_float32_products(d, far, precision):
     """The CUDA-core map (float32 throughout) is the measure; a quarter on top for the sample."""
