@@ -920,18 +920,27 @@ static int zero_counters(const Workspace& ws, cudaStream_t s) {
   return PROGOT_OK;
 }
 
-// PROGOT_ERR_TIMEOUT when a tensor-core kernel of this call raised the fault flag
-// (synchronises the stream).
+// The fault word and the integer grid's words on their way to the host (t_host.init() was
+// called); the caller synchronises the stream before seen_fault.
+static int fetch_words(const Workspace& ws, cudaStream_t s) {
+  CK(cudaMemcpyAsync(t_host.hs, ws.state, kStateBytes, cudaMemcpyDeviceToHost, s));
+  return PROGOT_OK;
+}
+// PROGOT_ERR_TIMEOUT when a tensor-core kernel of this call raised the fault flag.
 // *bad (optional): the step whose clouds the integer grid's kernels found out of their range
 // and left alone (0: none).
-static int check_fault(const Workspace& ws, cudaStream_t s, int32_t* bad = nullptr) {
-  const int rc = t_host.init();
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(t_host.hs, ws.state, kStateBytes, cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+static int seen_fault(int32_t* bad = nullptr) {
   if (t_host.fault()) return fail(PROGOT_ERR_TIMEOUT, "a tensor-core kernel hit its bounded wait (2 s) and aborted");
   if (bad) *bad = t_host.words().bad;
   return PROGOT_OK;
+}
+// Both, and the synchronisation between them.
+static int check_fault(const Workspace& ws, cudaStream_t s, int32_t* bad = nullptr) {
+  int rc = t_host.init();
+  if (!rc) rc = fetch_words(ws, s);
+  if (rc) return rc;
+  CK(cudaStreamSynchronize(s));
+  return seen_fault(bad);
 }
 
 // After grid kernels found the clouds out of their range (words->bad): the word cleared, the
@@ -1361,10 +1370,11 @@ static int metrics_core(const float* x, const float* a, int64_t n, const float* 
   if (rc) return rc;
   CK(launch_sum_parts(ws.metpart, (int)cdiv(m, fp32_tile_rows()), kMetricSums, ws.metout + kMetricSums, s));
   CK(cudaMemcpyAsync(t_host.hd, ws.metout, sizeof(double) * 2 * kMetricSums, cudaMemcpyDeviceToHost, s));
+  if (ops.on && (rc = fetch_words(ws, s)) != PROGOT_OK) return rc;
   CK(cudaStreamSynchronize(s));
   if (ops.on) {
     int32_t bad = 0;
-    rc = check_fault(ws, s, &bad);
+    rc = seen_fault(&bad);
     if (rc) return rc;
     if (bad) {
       Workspace w;
@@ -1395,6 +1405,10 @@ static int marginals_core(const float* x, int64_t n, const float* y, int64_t m, 
     CK(launch_row_sqnorm(x, n, d, ws.xn, s));
     CK(launch_row_sqnorm(y, m, d, ws.yn, s));
   }
+  // both errors in the solver states' place, unused here: one copy brings them and the words
+  // (a copy between the sweeps cost 10 us)
+  double* const sums = reinterpret_cast<double*>(ws.state);
+  const double* const errs = reinterpret_cast<const double*>(t_host.hs);
   TcOps ops;
   int rc = prep_tc(x, n, y, m, d, eps, PROGOT_FP32, ws, &ops, s, f, g);
   if (rc) return rc;
@@ -1404,24 +1418,23 @@ static int marginals_core(const float* x, int64_t n, const float* y, int64_t m, 
   pr.potA_old = f;
   pr.out = row;
   pr.mode = kModeMarginal;
+  pr.err_total = sums;
   rc = lse_sweep(pr, s, &ops, true, &ws);
   if (rc) return rc;
-  const int64_t rbr = cdiv(n, fp32_tile_rows());
-  CK(cudaMemcpyAsync(&t_host.hd[0], ws.errpart + rbr, sizeof(double), cudaMemcpyDeviceToHost, s));
   SweepParams pc = make_sweep(y, m, x, n, d, ws.yn, ws.xn, eps, ws, ops.on ? 1 : 2);
   pc.wA = b;
   pc.potB = f;
   pc.potA_old = g;
   pc.out = col;
   pc.mode = kModeMarginal;
+  pc.err_total = sums + 1;
   rc = lse_sweep(pc, s, &ops, false, &ws);
   if (rc) return rc;
-  const int64_t rbc = cdiv(m, fp32_tile_rows());
-  CK(cudaMemcpyAsync(&t_host.hd[1], ws.errpart + rbc, sizeof(double), cudaMemcpyDeviceToHost, s));
+  if ((rc = fetch_words(ws, s)) != PROGOT_OK) return rc;
   CK(cudaStreamSynchronize(s));
   if (ops.on) {
     int32_t bad = 0;
-    rc = check_fault(ws, s, &bad);
+    rc = seen_fault(&bad);
     if (rc) return rc;
     if (bad) {
       Workspace w;
@@ -1429,7 +1442,7 @@ static int marginals_core(const float* x, int64_t n, const float* y, int64_t m, 
       return rc ? rc : marginals_core(x, n, y, m, d, f, g, eps, row, col, a, b, err_l1_out, w, s);
     }
   }
-  if (err_l1_out) *err_l1_out = t_host.hd[0] + t_host.hd[1];
+  if (err_l1_out) *err_l1_out = errs[0] + errs[1];
   return PROGOT_OK;
 }
 

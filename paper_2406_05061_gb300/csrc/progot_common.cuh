@@ -82,6 +82,7 @@ struct SweepParams {
   const float* Acn;    // |ac_i|^2 (squared Euclidean cost)
   float* cpart;        // [splits][nA] sums_j 2^{t_ij - max} c(ac_i, b_j) (when Ac is given)
   double* errpart;     // [row blocks] float64 error partials
+  double* err_total;   // the sweep's error (NULL: in errpart[row blocks])
   unsigned int* cnt;   // [row blocks + 1] arrival counters (zero between launches)
   SolverState* state;  // nullptr when the sweep is not part of a Sinkhorn loop
   int64_t nA, nB;

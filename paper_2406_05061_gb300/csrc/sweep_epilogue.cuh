@@ -70,7 +70,7 @@ __device__ __forceinline__ void f_update_transition(SolverState& st, double err,
 __device__ __forceinline__ void finish_sweep_warp(const SweepParams& p, int nblocks) {
   const double err = sum_errpart_warp(p.errpart, nblocks);
   if ((threadIdx.x & 31) != 0) return;
-  p.errpart[nblocks] = err;
+  *(p.err_total != nullptr ? p.err_total : p.errpart + nblocks) = err;
   if (p.state == nullptr || !(p.role == 1 || p.role == 3)) return;
   SolverState st = *p.state;
   f_update_transition(st, err, p);
