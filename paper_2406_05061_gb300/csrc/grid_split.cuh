@@ -112,21 +112,25 @@ __device__ __forceinline__ float2 grid_beta(float pot, float norm, float bscale,
   return make_float2(h, fmaf(d, bscale, -h) + fmaf(d, bscale_lo, de * bscale));
 }
 
+// Below this (units of the accumulators) a score is no score: a padded column's, or one of a point
+// masked out by its potential (-inf, zero weight, the type's lowest value). The folds skip a running
+// maximum below it, since differences of such values times a sum would overflow.
+constexpr float kGridEmpty = -1e30f;
+
 // Bias row (16 bf16 slots) of beta: slots 0-2 the integer part of beta s2 in bf16 pieces
-// (added to the first accumulator), slots 8-10 its fraction (second accumulator). -inf
-// (padding, a zero weight) becomes a large negative finite value, since the other
-// accumulator's product meets it with a zero; NaN and +inf stay NaN.
+// (added to the first accumulator), slots 8-10 its fraction (second accumulator). What lies
+// below kGridEmpty becomes a large negative finite value, since the other accumulator's
+// product meets it with a zero; NaN and +inf stay NaN.
 __device__ __forceinline__ void write_bias_row_grid(__nv_bfloat16* row16, float2 beta2, float s2) {
-  const float beta = beta2.x;
+  const float bs = beta2.x * s2;
   uint32_t w[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) w[q] = 0u;
-  if (beta == -INFINITY) {
+  if (bs < kGridEmpty) {
     w[0] = 0xFF7Fu;  // -3.39e38
-  } else if (!isfinite(beta)) {
+  } else if (!isfinite(bs)) {
     w[0] = 0x7FC0u;
   } else {
-    const float bs = beta * s2;
     const float bi = rintf(bs), bf = (bs - bi) + beta2.y * s2;
     const __nv_bfloat16 i1 = __float2bfloat16_rn(bi);
     const float r1 = bi - __bfloat162float(i1);

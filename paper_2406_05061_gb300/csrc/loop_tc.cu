@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int q = 1; q < 2 * NC; ++q) tmax = fmaxf(tmax, mx[q]);
             const float mnew = fmaxf(m_run, tmax);
-            if (mnew != -INFINITY) {
+            if (GRID ? mnew > kGridEmpty : mnew != -INFINITY) {
               // grid split: the accumulators hold t 2^(ex + ey); (t - m) 2^-(ex + ey) is exact
               const float nm = GRID ? -mnew * inv2 : -mnew;
               const uint64_t negm = pack2(nm, nm);
