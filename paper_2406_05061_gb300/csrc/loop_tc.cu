@@ -362,7 +362,7 @@ __device__ __forceinline__ float loop_row_potential_grid(const Side& Sd, int sd,
 // Combine of two partial (max, sum) pairs in log2 units with the hardware exp2.
 __device__ __forceinline__ float2 combine_fast(float2 p, float2 q) {
   const float M = fmaxf(p.x, q.x);
-  if (M == -INFINITY) return make_float2(-INFINITY, 0.f);
+  if (M == -INFINITY) return make_float2(-INFINITY, p.y + q.y);
   return make_float2(M, p.y * fast_exp2(p.x - M) + q.y * fast_exp2(q.x - M));
 }
 

@@ -124,10 +124,11 @@ struct SweepParams {
 // with p = 1.5 (|z| sqrt|z|) specialised.
 enum CostKind : int32_t { kCostSqEuclid = 0, kCostP15 = 1, kCostPGeneral = 2 };
 
-// Combine two partial log-sum-exps (max, sum) in log2 units.
+// Combine two partial log-sum-exps (max, sum) in log2 units. A NaN sum stays one, whatever the
+// other part (fmaxf passes over a NaN maximum).
 __device__ __forceinline__ float2 lse_combine(float2 p, float2 q) {
   float M = fmaxf(p.x, q.x);
-  if (M == -INFINITY) return make_float2(-INFINITY, 0.f);
+  if (M == -INFINITY) return make_float2(-INFINITY, p.y + q.y);
   float s = p.y * exp2f(p.x - M) + q.y * exp2f(q.x - M);
   return make_float2(M, s);
 }

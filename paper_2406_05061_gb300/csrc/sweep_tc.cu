@@ -212,7 +212,7 @@ __device__ __forceinline__ SolverState sweep_state(const SweepParams& p) {
 // and W = sum 2^{t - M} (t - M).
 __device__ __forceinline__ float3 tilt_merge(float3 p, float3 q) {
   const float M = fmaxf(p.x, q.x);
-  if (M == -INFINITY) return make_float3(-INFINITY, 0.f, 0.f);
+  if (M == -INFINITY) return make_float3(-INFINITY, p.y + q.y, p.z + q.z);
   float s = 0.f, w = 0.f;
   if (p.x != -INFINITY) {
     const float c = exp2f(p.x - M);

@@ -92,3 +92,22 @@ def test_loop_from_a_masked_start(n, m, value):
         r2 = max((x.astype(np.float64) ** 2).sum(1).max(), (y.astype(np.float64) ** 2).sum(1).max())
         np.testing.assert_allclose(r.f.cpu().numpy(), f, rtol=0, atol=eps * 2.0 ** -21 * (4 * 1.2 * r2 / eps + 16))
         assert bool(torch.isfinite(r.g).all())
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("n,m,d,j", [(200, 500, 16, 70), (200, 500, 16, 133), (1500, 2500, 16, 3), (1500, 2500, 16, 2311),
+                                     (900, 700, 64, 650)])
+def test_potentials_that_are_not_finite_show(n, m, d, j, value):
+    """One NaN (or infinite) g_j belongs to every row sum."""
+    rng = np.random.default_rng(j)
+    x, y = rng.standard_normal((n, d)), rng.standard_normal((m, d))
+    f, g = np.zeros(n), np.zeros(m)
+    g[j] = value
+    eps = 0.2 * d
+    row, _, err = nat.coupling_marginals(dev(x), dev(y), dev(f), dev(g), eps)
+    assert not bool(torch.isfinite(row).any()) and not np.isfinite(err)
+    _, col, err = nat.coupling_marginals(dev(y), dev(x), dev(g), dev(f), eps)
+    assert not bool(torch.isfinite(col).any()) and not np.isfinite(err)
+    with pytest.raises(nat.ProgOTError) as ei:
+        nat.sinkhorn_potentials(dev(x), dev(y), eps, 0.0, 3, f=dev(f), g=dev(g))
+    assert ei.value.code == nat.PROGOT_ERR_NUMERIC
