@@ -18,8 +18,8 @@
  *   frees them. Arrays named as "host" are host memory.
  * - Potentials follow the dual convention of eq. (5): the coupling is
  *   P_ij = exp((f_i + g_j - c(x_i, y_j)) / eps); g absorbs eps log b_j.
- * - workspace / ws_bytes: device scratch owned by the caller, at least
- *   progot_workspace_size(...) bytes, 256-byte aligned. Its contents need not be
+ * - workspace / ws_bytes: device scratch owned by the caller, progot_workspace_size(...)
+ *   bytes (at least progot_workspace_size_min(...)), 256-byte aligned. Its contents need not be
  *   initialised and are garbage after the call. Two calls in flight at the same time
  *   must not share a workspace.
  * - stream: a cudaStream_t (NULL = legacy default stream). Entry points that return
@@ -29,7 +29,7 @@
  *   map steps, marginals and metrics form the cross term x . y on the tcgen05 tensor cores
  *   from half-precision parts whose leading products add exactly (error at or below a
  *   float32 FMA chain's); loops beyond d = 64, small map queries and workspaces smaller than
- *   progot_workspace_size (down to what the CUDA cores need) use float32 FMAs.
+ *   a mixed precision's (down to what the CUDA cores need) use float32 FMAs.
  *   PROGOT_BF16X3 uses tcgen05 tensor cores on a bf16 hi/lo split of both operands
  *   (x.y ~ xh.yh + xh.yl + xl.yh, float32 accumulation; map steps beyond d = 256 as
  *   PROGOT_FP32's); PROGOT_BF16 uses the hi parts only. Log-sum-exps and potentials are
@@ -75,6 +75,12 @@ const char* progot_version(void);
 /* Bytes of device workspace that every entry point below needs for a problem with at
  * most n rows, m columns and dimension d (for entropic_map_apply pass nq as n). */
 size_t progot_workspace_size(int64_t n, int64_t m, int32_t d, int32_t precision);
+
+/* Bytes below which an entry point refuses the workspace. Less than progot_workspace_size
+ * only at PROGOT_FP32, which runs on the tensor cores in a mixed precision's workspace too
+ * (up to about 29,000 points at d <= 64, more beyond; p-norm loops then keep no cost) and on
+ * CUDA cores in a smaller one. */
+size_t progot_workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision);
 
 /*
  * sinkhorn_potentials - Sink(a, X, b, Y, eps, tau, f_init, g_init) of Alg. 1.

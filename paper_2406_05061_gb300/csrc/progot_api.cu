@@ -229,6 +229,7 @@ struct Workspace {
   unsigned* ticket;
   char* prob;       // P tiles of the map step, a chunk of rows at a time (integer-grid operands)
   int64_t prob_bytes;
+  int64_t kept_bytes;  // of prob, for a p-norm cost that outlasts a map step
   float* rsum;      // their row sums
   bool grid;        // the workspace holds the float32 path's tensor-core operands
   size_t bytes;
@@ -342,16 +343,19 @@ static size_t ws_layout(const WsDims& w, Workspace* out, char* base) {
     const int64_t block = pv_prob_bytes_per_block(w.nmax);
     ws.prob_bytes = std::max<int64_t>(block, std::min<int64_t>(block * w.rbmax, kCostBytes));
     ws.prob = take((size_t)ws.prob_bytes);
+    ws.kept_bytes = ws.prob_bytes;
   } else {
-    // The mixed precisions need them for d > 256, in the partial buffer of the CUDA-core map,
-    // which is idle then: it has 4 d bytes for more than 2 nmax + 128 rows, the third parts take
-    // 4 dp < 4 (d + 64) for nmax of them, and one row block's P, 512 bytes a row, fits in the rest.
+    // The mixed precisions' layout has them in the partial buffer of the CUDA-core map, which is
+    // idle in such a step. Beyond d = 256, where the mixed precisions need them, that buffer has
+    // 4 d bytes for more than 2 nmax + 128 rows, the third parts take 4 dp < 4 (d + 64) for nmax
+    // of them, and one row block's P, 512 bytes a row, fits in the rest.
     const size_t third = align256(opb), have = sizeof(float) * (size_t)w.opart_elems;
     const bool room = w.tc && have > 2 * third;
     ws.xr = room ? (char*)ws.Opart : nullptr;
     ws.yr = room ? (char*)ws.Opart + third : nullptr;
     ws.prob = room ? (char*)ws.Opart + 2 * third : nullptr;
     ws.prob_bytes = room ? (int64_t)(have - 2 * third) : 0;
+    ws.kept_bytes = 0;
   }
   ws.rsum = ws.Rpart;
   ws.grid = w.grid;
@@ -366,9 +370,14 @@ static int carve(int64_t n, int64_t m, int32_t d, void* workspace, size_t ws_byt
   if ((reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
     return fail(PROGOT_ERR_WORKSPACE, "workspace is not 256-byte aligned");
   size_t need = ws_layout(ws_dims(n, m, d, precision), ws, (char*)workspace);
-  // a float32 workspace without room for the tensor-core operands still serves, on CUDA cores
-  if (ws_bytes < need && precision == PROGOT_FP32)
-    need = ws_layout(ws_dims(n, m, d, precision, false), ws, (char*)workspace);
+  // A float32 call takes a smaller workspace too: a mixed precision's, whose layout has room for
+  // the grid's third parts and a row block of P in the CUDA-core map's buffer (up to about 29,000
+  // points at d <= 64), or what the CUDA cores need.
+  if (ws_bytes < need && precision == PROGOT_FP32) {
+    need = ws_layout(ws_dims(n, m, d, PROGOT_BF16X3), ws, (char*)workspace);
+    ws->grid = ws->prob_bytes >= pv_prob_bytes_per_block(std::max<int64_t>(n, m));
+    if (ws_bytes < need || !ws->grid) need = ws_layout(ws_dims(n, m, d, precision, false), ws, (char*)workspace);
+  }
   if (ws_bytes < need)
     return fail(PROGOT_ERR_WORKSPACE, "workspace has %zu bytes, %zu needed", ws_bytes, need);
   return PROGOT_OK;
@@ -725,7 +734,7 @@ static int keep_cost(const float* x, int64_t n, const float* y, int64_t m, int32
                      cudaStream_t s) {
   const int64_t ld = cdiv(m, 128) * 128;
   c->C = nullptr;
-  if (!c->pnorm() || !ws.grid || n > ws.prob_bytes / (int64_t)sizeof(float) / ld) return PROGOT_OK;
+  if (!c->pnorm() || !ws.grid || n > ws.kept_bytes / (int64_t)sizeof(float) / ld) return PROGOT_OK;
   CK(launch_pnorm_cost(x, n, y, m, d, c->kind, c->p, (float*)ws.prob, ld, s));
   c->C = (const float*)ws.prob;
   c->ldc = ld;
@@ -1553,14 +1562,10 @@ const char* progot_last_error_string(void) { return t_last_error.c_str(); }
 
 const char* progot_version(void) { return "0.1.0"; }
 
-}  // extern "C"
-
-size_t progot::workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision) {
+size_t progot_workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision) {
   if (n <= 0 || m <= 0 || d <= 0) return 0;
   return ws_layout(ws_dims(n, m, d, precision, false), nullptr, nullptr);
 }
-
-extern "C" {
 
 size_t progot_workspace_size(int64_t n, int64_t m, int32_t d, int32_t precision) {
   if (n <= 0 || m <= 0 || d <= 0) return 0;

@@ -234,8 +234,6 @@ int encode_operand_map(void* map, void* base, int64_t rows, int32_t dp, int box_
 int32_t stall_window_setting();
 unsigned long long wait_limit_setting();
 int device_sm_count();
-// Least workspace a solve accepts (the float32 path then runs on CUDA cores).
-size_t workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision);
 int fail_message(int code, const char* msg);  // sets the last-error text, returns code
 bool loop_tc_supported(int bn, int nkb, int split3, bool grid);
 

@@ -393,7 +393,7 @@ int64_t progot_server_submit(progot_server* S, const progot_problem* req) {
   // a request that fits the budget only with the smallest workspace runs with that
   size_t wsb = progot::round_up256(progot_workspace_size(req->n, req->m, req->d, S->precision));
   if (progot::request_bytes(*req, wsb) > S->arena->size())
-    wsb = progot::round_up256(progot::workspace_size_min(req->n, req->m, req->d, S->precision));
+    wsb = progot::round_up256(progot_workspace_size_min(req->n, req->m, req->d, S->precision));
   const size_t bytes = progot::request_bytes(*req, wsb);
   if (bytes > S->arena->size()) {
     set_last_error_message("request needs more device memory than the server's budget");

@@ -40,6 +40,7 @@ SIGNATURES = [
     ("progot_last_error_string", ctypes.c_char_p, []),
     ("progot_version", ctypes.c_char_p, []),
     ("progot_workspace_size", _SZ, [_I64, _I64, _I32, _I32]),
+    ("progot_workspace_size_min", _SZ, [_I64, _I64, _I32, _I32]),
     ("sinkhorn_potentials", ctypes.c_int,
      [_P, _P, _I64, _P, _P, _I64, _I32, _D, _D, _I32, _I32, _P, _P, _I32, _P, _P, _P, _SZ, _P]),
     ("entropic_map_apply", ctypes.c_int, [_P, _I64, _P, _I64, _I32, _I32, _P, _P, _P, _I32, _P, _P, _SZ, _P]),
@@ -166,21 +167,25 @@ def workspace_size(n: int, m: int, d: int, precision="fp32") -> int:
 class Workspace:
     """A reusable device workspace (torch uint8 buffer, 256-byte aligned)."""
 
-    def __init__(self, n: int, m: int, d: int, precision="fp32", device=None):
+    def __init__(self, n: int, m: int, d: int, precision="fp32", device=None, stream=None):
         torch = _torch()
         self.bytes = workspace_size(n, m, d, precision)
-        self.buf = torch.empty(self.bytes + 256, dtype=torch.uint8, device=device or "cuda")
+        # the allocator may hand the buffer on once it is dropped: in the order of its own stream
+        with torch.cuda.stream(stream if isinstance(stream, torch.cuda.Stream) else None):
+            self.buf = torch.empty(self.bytes + 256, dtype=torch.uint8, device=device or "cuda")
         base = self.buf.data_ptr()
         self.ptr = (base + 255) & ~255
         self.dims = (n, m, d, _prec(precision))
 
     def covers(self, n, m, d, precision) -> bool:
-        return workspace_size(n, m, d, precision) <= self.bytes
+        """Whether the library takes this buffer for such a call (a mixed precision's serves a
+        float32 call too)."""
+        return int(lib().progot_workspace_size_min(n, m, d, _prec(precision))) <= self.bytes
 
 
-def _ws(ws, n, m, d, precision):
+def _ws(ws, n, m, d, precision, stream=None):
     if ws is None or not ws.covers(n, m, d, precision):
-        ws = Workspace(n, m, d, precision)
+        ws = Workspace(n, m, d, precision, stream=stream)
     return ws
 
 
@@ -219,7 +224,7 @@ def sinkhorn_potentials(x, y, eps, tau, max_iter=10000, a=None, b=None, f=None, 
         f = alloc(n, dtype=torch.float32, device=x.device)
     if g is None:
         g = alloc(m, dtype=torch.float32, device=x.device)
-    ws = _ws(workspace, n, m, d, precision)
+    ws = _ws(workspace, n, m, d, precision, stream)
     it = ctypes.c_int32(0)
     err = ctypes.c_double(0.0)
     rc = lib().sinkhorn_potentials(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d,
@@ -241,7 +246,7 @@ def entropic_map_apply(xq, y, g_all, eps, alpha, precision="fp32", out=None, wor
     al_h = _host_f64(alpha, K)
     if out is None:
         out = torch.empty_like(xq)
-    ws = _ws(workspace, nq, m, d, precision)
+    ws = _ws(workspace, nq, m, d, precision, stream)
     rc = lib().entropic_map_apply(_dev(xq, "xq"), nq, _dev(y, "y"), m, d, K, _dev(g_all.contiguous(), "g_all"),
                                   _hp(eps_h), _hp(al_h), _prec(precision), _dev(out, "out", (nq, d)),
                                   ctypes.c_void_p(ws.ptr), ws.bytes, _stream(stream))
@@ -258,7 +263,7 @@ def coupling_marginals(x, y, f, g, eps, a=None, b=None, precision="fp32", worksp
     row = torch.empty(n, dtype=torch.float32, device=x.device)
     col = torch.empty(m, dtype=torch.float32, device=x.device)
     err = ctypes.c_double(0.0)
-    ws = _ws(workspace, n, m, d, precision)
+    ws = _ws(workspace, n, m, d, precision, stream)
     rc = lib().coupling_marginals(_dev(x, "x"), n, _dev(y, "y"), m, d, _dev(f, "f", (n,)), _dev(g, "g", (m,)),
                                   float(eps), _prec(precision), _dev(row, "row"), _dev(col, "col"),
                                   _opt(a, "a", (n,)), _opt(b, "b", (m,)), ctypes.byref(err),
@@ -292,7 +297,7 @@ def progot_solve(x, y, alpha, eps, tau, max_iter=10000, a=None, b=None, precisio
                    f_last=torch.empty(n, dtype=torch.float32, device=x.device), x_last=torch.empty_like(x))
     iters = np.zeros(K, dtype=np.int32)
     errs = np.zeros(K, dtype=np.float64)
-    ws = _ws(workspace, n, m, d, precision)
+    ws = _ws(workspace, n, m, d, precision, stream)
     rc = lib().progot_solve(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d, K,
                             _hp(al_h), _hp(eps_h), _hp(tau_h), int(max_iter), _prec(precision),
                             _dev(out["x_out"], "x_out", (n, d)), _dev(out["g_all"], "g_all", (K, m)),
@@ -319,7 +324,7 @@ def progot_solve_theta(x, y, alpha, theta, tau, max_iter=10000, a=None, b=None, 
     iters = np.zeros(K, dtype=np.int32)
     errs = np.zeros(K, dtype=np.float64)
     eps_out = np.zeros(K, dtype=np.float64)
-    ws = _ws(workspace, n, m, d, precision)
+    ws = _ws(workspace, n, m, d, precision, stream)
     rc = lib().progot_solve_theta(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d, K,
                                   _hp(al_h), float(theta), _hp(tau_h), int(max_iter), _prec(precision),
                                   _dev(out["x_out"], "x_out", (n, d)), _dev(out["g_all"], "g_all", (K, m)),
@@ -348,7 +353,7 @@ def coupling_metrics(x, y, f, g, eps, a=None, b=None, x_cost=None, workspace=Non
     _dev(x, "x"), _dev(y, "y")
     n, d = x.shape
     m = y.shape[0]
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     res = CouplingMetricsStruct()
     rc = lib().coupling_metrics(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d,
                                 _dev(f, "f", (n,)), _dev(g, "g", (m,)), _opt(x_cost, "x_cost", (n, d)), float(eps),
@@ -365,7 +370,7 @@ def sinkhorn_divergence(x, y, eps, tau, max_iter=10000, a=None, b=None, precisio
     n, d = x.shape
     m = y.shape[0]
     k = max(n, m)
-    ws = _ws(workspace, k, k, d, precision)
+    ws = _ws(workspace, k, k, d, precision, stream)
     val = ctypes.c_double(0.0)
     parts = np.zeros(3, dtype=np.float64)
     its = np.zeros(3, dtype=np.int32)
@@ -382,7 +387,7 @@ def coupling_diagonal(x, y, f, g, eps, log_diag=None, workspace=None, stream=Non
     n, d = x.shape
     if y.shape != x.shape:
         raise ValueError("coupling_diagonal needs x and y of the same shape")
-    ws = _ws(workspace, n, n, d, "fp32")
+    ws = _ws(workspace, n, n, d, "fp32", stream)
     tr = ctypes.c_double(0.0)
     kl = ctypes.c_double(0.0)
     rc = lib().coupling_diagonal(_dev(x, "x"), _dev(y, "y"), n, d, _dev(f, "f", (n,)), _dev(g, "g", (n,)),
@@ -406,7 +411,7 @@ def sinkhorn_potentials_pnorm(x, y, p, eps, tau, max_iter=10000, a=None, b=None,
         f = alloc(n, dtype=torch.float32, device=x.device)
     if g is None:
         g = alloc(m, dtype=torch.float32, device=x.device)
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     it = ctypes.c_int32(0)
     err = ctypes.c_double(0.0)
     rc = lib().sinkhorn_potentials_pnorm(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d,
@@ -436,7 +441,7 @@ def progot_solve_pnorm(x, y, p, alpha, tau, eps=None, theta=None, max_iter=10000
     iters = np.zeros(K, dtype=np.int32)
     errs = np.zeros(K, dtype=np.float64)
     eps_out = np.zeros(K, dtype=np.float64)
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     rc = lib().progot_solve_pnorm(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d,
                                   float(p), K, _hp(al_h), None if eps_h is None else _hp(eps_h),
                                   float(theta or 0.0), _hp(tau_h), int(max_iter), _dev(out["x_out"], "x_out", (n, d)),
@@ -458,7 +463,7 @@ def entropic_map_apply_pnorm(xq, y, p, g_all, eps, alpha, out=None, workspace=No
     eps_h, al_h = _host_f64(eps, K), _host_f64(alpha, K)
     if out is None:
         out = torch.empty_like(xq)
-    ws = _ws(workspace, nq, m, d, "fp32")
+    ws = _ws(workspace, nq, m, d, "fp32", stream)
     rc = lib().entropic_map_apply_pnorm(_dev(xq, "xq"), nq, _dev(y, "y"), m, d, float(p), K,
                                         _dev(g_all.contiguous(), "g_all"), _hp(eps_h), _hp(al_h),
                                         _dev(out, "out", (nq, d)), ctypes.c_void_p(ws.ptr), ws.bytes, _stream(stream))
@@ -471,7 +476,7 @@ def coupling_metrics_pnorm(x, y, p, f, g, eps, a=None, b=None, x_cost=None, work
     _dev(x, "x"), _dev(y, "y")
     n, d = x.shape
     m = y.shape[0]
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     res = CouplingMetricsStruct()
     rc = lib().coupling_metrics_pnorm(_dev(x, "x"), _opt(a, "a", (n,)), n, _dev(y, "y"), _opt(b, "b", (m,)), m, d,
                                       float(p), _dev(f, "f", (n,)), _dev(g, "g", (m,)), _opt(x_cost, "x_cost", (n, d)),
@@ -484,7 +489,7 @@ def coupling_metrics_pnorm(x, y, p, f, g, eps, a=None, b=None, x_cost=None, work
 def progot_mean_cost_pnorm(x, y, p, workspace=None, stream=None) -> float:
     n, d = x.shape
     m = y.shape[0]
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     out = ctypes.c_double(0.0)
     _check(lib().progot_mean_cost_pnorm(_dev(x, "x"), n, _dev(y, "y"), m, d, float(p), ctypes.byref(out),
                                         ctypes.c_void_p(ws.ptr), ws.bytes, _stream(stream)), allow_not_converged=False)
@@ -501,7 +506,7 @@ def progot_schedule_alpha(K: int, kind="constant") -> np.ndarray:
 def progot_mean_cost(x, y, workspace=None, stream=None) -> float:
     n, d = x.shape
     m = y.shape[0]
-    ws = _ws(workspace, n, m, d, "fp32")
+    ws = _ws(workspace, n, m, d, "fp32", stream)
     out = ctypes.c_double(0.0)
     _check(lib().progot_mean_cost(_dev(x, "x"), n, _dev(y, "y"), m, d, ctypes.byref(out), ctypes.c_void_p(ws.ptr),
                                   ws.bytes, _stream(stream)), allow_not_converged=False)
@@ -523,7 +528,7 @@ def progot_schedule_eps(x, y, y_test, alpha, s_grid=None, beta0=5.0, tau=1e-6, m
     errors = np.zeros(P)
     pstar = ctypes.c_int32(0)
     nmax = max(n, m, mt)
-    ws = _ws(workspace, nmax, nmax, d, precision)
+    ws = _ws(workspace, nmax, nmax, d, precision, stream)
     _check(lib().progot_schedule_eps(_dev(x, "x"), n, _dev(y, "y"), _opt(b, "b", (m,)), m,
                                      _dev(y_test, "y_test", (mt, d)), mt, d, K, _hp(al_h), _hp(sg_h), P,
                                      float(beta0), float(tau), int(max_iter), _prec(precision), _hp(eps_out),
