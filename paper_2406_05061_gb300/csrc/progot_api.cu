@@ -1562,6 +1562,15 @@ const char* progot_last_error_string(void) { return t_last_error.c_str(); }
 
 const char* progot_version(void) { return "0.1.0"; }
 
+}  // extern "C"
+
+size_t progot::solve_workspace_size(int64_t n, int64_t m, int32_t d, int32_t precision) {
+  return precision == PROGOT_FP32 && d > kGridSolveDim ? progot_workspace_size_min(n, m, d, precision)
+                                                       : progot_workspace_size(n, m, d, precision);
+}
+
+extern "C" {
+
 size_t progot_workspace_size_min(int64_t n, int64_t m, int32_t d, int32_t precision) {
   if (n <= 0 || m <= 0 || d <= 0) return 0;
   return ws_layout(ws_dims(n, m, d, precision, false), nullptr, nullptr);

@@ -234,6 +234,8 @@ int encode_operand_map(void* map, void* base, int64_t rows, int32_t dp, int box_
 int32_t stall_window_setting();
 unsigned long long wait_limit_setting();
 int device_sm_count();
+// Workspace that progot_solve makes use of (float32 solves beyond d = 64 run on CUDA cores).
+size_t solve_workspace_size(int64_t n, int64_t m, int32_t d, int32_t precision);
 int fail_message(int code, const char* msg);  // sets the last-error text, returns code
 bool loop_tc_supported(int bn, int nkb, int split3, bool grid);
 

@@ -34,16 +34,15 @@ static int check_problem(const progot_problem& p) {
   return PROGOT_OK;
 }
 
-// Per-worker workspace for the largest problem of a batch.
-static size_t slice_bytes(const progot_problem* probs, int32_t count, int32_t precision) {
-  int64_t n = 1, m = 1;
-  int32_t d = 1;
+// Per-worker workspace for every problem of a batch; least: what a solve accepts.
+static size_t slice_bytes(const progot_problem* probs, int32_t count, int32_t precision, bool least = false) {
+  size_t need = 0;
   for (int i = 0; i < count; ++i) {
-    n = std::max<int64_t>(n, probs[i].n);
-    m = std::max<int64_t>(m, probs[i].m);
-    d = std::max<int32_t>(d, probs[i].d);
+    const progot_problem& p = probs[i];
+    need = std::max(need, least ? progot_workspace_size_min(p.n, p.m, p.d, precision)
+                                : solve_workspace_size(p.n, p.m, p.d, precision));
   }
-  return round_up256(progot_workspace_size(n, m, d, precision));
+  return round_up256(need);
 }
 
 // Engine of progot_solve_batched: 1 = one persistent launch over the whole batch
@@ -105,14 +104,13 @@ int progot_solve_batched(progot_problem* problems, int32_t count, int32_t max_it
     progot_batch_plan_destroy(plan);
     return rc;
   }
-  const size_t slice = slice_bytes(problems, count, precision);
-  if (ws_bytes < slice * (size_t)n_streams) {
-    set_last_error_message("batched workspace too small (see progot_batched_workspace_size)");
-    return PROGOT_ERR_WORKSPACE;
-  }
+  // slices of what there is, up to what the solves make use of
   char* base = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(workspace) + 255) & ~uintptr_t(255));
-  if (base + slice * (size_t)n_streams > reinterpret_cast<char*>(workspace) + ws_bytes) {
-    set_last_error_message("batched workspace too small after 256-byte alignment");
+  const size_t skip = (size_t)(base - reinterpret_cast<char*>(workspace));
+  const size_t have = ws_bytes > skip ? (ws_bytes - skip) / (size_t)n_streams & ~size_t(255) : 0;
+  const size_t slice = std::min(slice_bytes(problems, count, precision), have);
+  if (slice < slice_bytes(problems, count, precision, true)) {
+    set_last_error_message("batched workspace too small (see progot_batched_workspace_size)");
     return PROGOT_ERR_WORKSPACE;
   }
   int dev = 0;
@@ -391,7 +389,7 @@ int64_t progot_server_submit(progot_server* S, const progot_problem* req) {
     return -PROGOT_ERR_INVALID_ARG;
   }
   // a request that fits the budget only with the smallest workspace runs with that
-  size_t wsb = progot::round_up256(progot_workspace_size(req->n, req->m, req->d, S->precision));
+  size_t wsb = progot::round_up256(progot::solve_workspace_size(req->n, req->m, req->d, S->precision));
   if (progot::request_bytes(*req, wsb) > S->arena->size())
     wsb = progot::round_up256(progot_workspace_size_min(req->n, req->m, req->d, S->precision));
   const size_t bytes = progot::request_bytes(*req, wsb);

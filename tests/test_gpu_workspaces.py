@@ -83,3 +83,54 @@ def test_private_workspace_belongs_to_the_calls_stream(monkeypatch):
     nat.sinkhorn_potentials(x, x, 1.0, 0.0, 2, stream=s)
     torch.cuda.synchronize()
     assert seen == [s.cuda_stream] * 2
+
+
+def schedule(x, y, K=2):
+    c = float((x ** 2).sum(1).mean() + (y ** 2).sum(1).mean())
+    return [1.0 / (K - k) for k in range(K)], [0.2 * c * (K - k) for k in range(K)]
+
+
+def test_a_server_reserves_for_wide_float32_solves_what_they_use():
+    """They run on CUDA cores: two requests fit where their tensor-core parts would leave one."""
+    n, d = 2048, 200
+    rng = np.random.default_rng(0)
+    x, y = rng.standard_normal((n, d)).astype(np.float32), rng.standard_normal((n, d)).astype(np.float32)
+    al, eps = schedule(x, y)
+    io = 4 * (3 * n * d + 2 * n + n) + 8 * 256
+    least = int(nat.lib().progot_workspace_size_min(n, n, d, 0)) + 256
+    budget = 2 * (least + io)
+    assert budget < 2 * nat.workspace_size(n, n, d)
+    srv = nat.Server(budget, n_workers=2, precision="fp32", max_iter=30)
+    try:
+        ids = [srv.submit(x, y, al, eps, [0.0] * 2) for _ in range(4)]
+        outs = [srv.wait(i) for i in ids]
+        assert srv.stats()["peak_bytes"] > least + io  # two at a time
+    finally:
+        srv.close()
+    solo = nat.progot_solve(dev(x), dev(y), al, eps, [0.0] * 2, max_iter=30)
+    for o in outs:
+        np.testing.assert_array_equal(o["x_out"], solo.x_out.cpu().numpy())
+
+
+@pytest.mark.parametrize("d", [16, 200])
+def test_batched_float32_solves_in_the_least_workspace(d):
+    rng = np.random.default_rng(d)
+    probs = []
+    for n, m in ((700, 600), (300, 900), (1100, 130)):
+        x, y = rng.standard_normal((n, d)).astype(np.float32), rng.standard_normal((m, d)).astype(np.float32)
+        al, eps = schedule(x, y)
+        probs.append(dict(x=dev(x), y=dev(y), alpha=al, eps=eps, tau=[0.0] * 2))
+    full = nat.progot_solve_batched(probs, max_iter=5, precision="fp32", n_streams=2)
+    arr, outs = nat._batch_structs(probs)
+    least = max(int(nat.lib().progot_workspace_size_min(p["x"].shape[0], p["y"].shape[0], d, 0)) for p in probs)
+    size = 2 * ((least + 255) // 256 * 256)
+    for give, status in ((size, nat.PROGOT_ERR_NOT_CONVERGED), (size - 256, nat.PROGOT_ERR_WORKSPACE)):
+        buf = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        base = (buf.data_ptr() + 255) // 256 * 256
+        rc = nat.lib().progot_solve_batched(arr, len(probs), 5, 0, 2, base, give, None)
+        torch.cuda.synchronize()
+        assert rc == status
+    for a, b, p in zip(nat._batch_results(arr, outs), full, probs):
+        r2 = float(max((p["x"] ** 2).sum(1).max(), (p["y"] ** 2).sum(1).max()))
+        tol = 2 * 2 * 5 * 2.0 ** -21 * (4 * 1.2 * r2 / p["eps"][-1] + 16)
+        torch.testing.assert_close(a["x_out"], b["x_out"], rtol=0, atol=tol * r2 ** 0.5)
