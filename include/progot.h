@@ -25,11 +25,13 @@
  * - stream: a cudaStream_t (NULL = legacy default stream). Entry points that return
  *   host results (iteration counts, errors) synchronise that stream before
  *   returning; the others are asynchronous.
- * - precision: PROGOT_FP32 has float32 accuracy throughout. Sinkhorn loops up to d = 64,
- *   map steps, marginals and metrics form the cross term x . y on the tcgen05 tensor cores
- *   from half-precision parts whose leading products add exactly (error at or below a
- *   float32 FMA chain's); loops beyond d = 64, small map queries and workspaces smaller than
- *   a mixed precision's (down to what the CUDA cores need) use float32 FMAs.
+ * - precision: PROGOT_FP32 has float32 accuracy throughout. Solves up to d = 64 (loops and
+ *   map steps), entropic maps, marginals and metrics form the cross term x . y on the tcgen05
+ *   tensor cores from half-precision parts whose leading products add exactly (error at or
+ *   below a float32 FMA chain's). Solves beyond d = 64, small map queries, clouds whose far
+ *   points or whose cost over eps leave the parts' range, and workspaces smaller than a mixed
+ *   precision's (down to what the CUDA cores need) use float32 FMAs; a loop of tens of
+ *   iterations on them moves a g that is small beside the norms by up to 2e-5 of its size.
  *   PROGOT_BF16X3 uses tcgen05 tensor cores on a bf16 hi/lo split of both operands
  *   (x.y ~ xh.yh + xh.yl + xl.yh, float32 accumulation; map steps beyond d = 256 as
  *   PROGOT_FP32's); PROGOT_BF16 uses the hi parts only. Log-sum-exps and potentials are

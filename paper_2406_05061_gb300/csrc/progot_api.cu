@@ -149,12 +149,12 @@ static int plan_splits(int64_t nA, int64_t nB, int ctas_per_sm, int extra_mult =
   return (int)cdiv(ct, tps);
 }
 
-// Float32 Sinkhorn loops use the integer-grid operands up to this dimension. The CUDA-core
-// sweeps round eps' products against unequal norms and so shift mass between f and g by a
-// little every iteration (the plan is unaffected); on wide normalised clouds, where g is
-// small, tens of iterations move it by 1e-5 of its size (1.3e-5 measured at 839 x 726,
-// d = 126, 17 iterations). The grid loops do not drift, and results callers already hold for
-// such clouds would change by as much, so these loops stay on CUDA cores.
+// Float32 solves use the integer-grid operands up to this dimension: the persistent loop on them
+// holds one K block. Beyond it the loops and the map steps of a solve run on CUDA cores, whose sweeps
+// round eps' products against unequal norms and so shift mass between f and g by a little every
+// iteration (the plan is unaffected): on wide normalised clouds, where g is small, tens of
+// iterations move it by 1e-5 of its size (1.3e-5 at 839 x 726, d = 126, 17 iterations), where
+// grid sweeps, one launch an update, do not drift and take a tenth of the time.
 constexpr int32_t kGridSolveDim = 64;
 // Whether a float32 map of K steps runs on the tensor cores: where their estimated time for the
 // whole call is the smaller. The fixed 77 us are the first step's preparation (the later steps'
@@ -515,8 +515,8 @@ static int map_y_bias(TcOps* ops, void* base, int64_t m) {
   return rc;
 }
 
-// Test hook (progot_test_withhold_initial_betas): the persistent loop starts without the
-// initial g's ready flags, so the first f-update's bounded wait expires.
+// What the operand preparation writes for a persistent loop besides the operands: the work
+// split's tables, the flags, counters and states.
 static LoopSetup loop_setup_params(int64_t n, int64_t m, const TcOps& ops, const Workspace& ws) {
   LoopSetup ls;
   memset(&ls, 0, sizeof(ls));
@@ -533,7 +533,8 @@ static LoopSetup loop_setup_params(int64_t n, int64_t m, const TcOps& ops, const
     S.nseg = ws.ltab_nseg + sd * num_sms();
     S.crow = ws.ltab_crow + sd * ws.lrb;
     S.cslot = ws.ltab_cslot + sd * ws.lslots;
-    // flags: nothing published, then the initial g's row blocks as 1
+    // flags: nothing published, then the initial g's row blocks as 1 (the test hook
+    // progot_test_withhold_initial_betas leaves them out: the first f-update's bounded wait expires)
     S.flag = ws.lflag + sd * ws.lrb;
     S.flag_init = sd == 1 && !g_withhold_betas.load() ? 1u : 0u;
     S.cnt = ws.lcnt + sd * ws.lrb;
@@ -1480,7 +1481,6 @@ static int mean_cost_dev(const float* x, int64_t n, const float* y, int64_t m, i
   return PROGOT_OK;
 }
 
-
 // Alg. 2 with eps_k from `eps` (host, K) or, when eps is NULL, from the theta rule
 // eps_k = theta mean cost(X^(k), Y) / 20 on the cloud each solve transports.
 static int solve_impl(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m, int32_t d,
@@ -1738,6 +1738,7 @@ int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int
   if (rc) return rc;
   return marginals_core(x, n, y, m, d, f, g, eps, row, col, a, b, err_l1_out, ws, s);
 }
+
 int progot_solve(const float* x, const float* a, int64_t n, const float* y, const float* b, int64_t m, int32_t d,
                  int32_t K, const double* alpha, const double* eps, const double* tau, int32_t max_iter,
                  int32_t precision, float* x_out, float* g_all, float* f_last, float* x_last, int32_t* iters,

@@ -112,7 +112,7 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream);
 cudaError_t launch_center(const float* X, int64_t n, const float* Y, int64_t m, int32_t d, double* partial,
                           unsigned* ticket, float* mu, GridWords* words, cudaStream_t s);
 // Both clouds: parts of sqrt(c) (x - mu), rows of dp 16-bit elements (zeros past d): bf16
-// hi, lo, or the integer grid's two or three half-precision parts (grid_split.cuh); unused
+// hi, lo, or the integer grid's three half-precision parts (grid_split.cuh); unused
 // parts are NULL. Centred squared norms, and bias rows of both sides from the potentials f
 // (x side) and g (y side) where given, into one or two buffers each, rows padded to a
 // multiple of 256. Grid: the words of the split; step is what words->bad becomes (when zero)
@@ -163,8 +163,6 @@ cudaError_t launch_operands(const OperandPrep& op, OperandKind kind, const LoopS
 cudaError_t launch_loop_finish(const float* f_new, const float* an, const float* w, double log_w_uniform, double eps,
                                int64_t n, float* L, const float* f_cur, float* f_out, cudaStream_t s);
 cudaError_t launch_warm_start(float* g, const float* g_prev, int64_t m, float* f, int64_t n, float c, cudaStream_t s);
-cudaError_t launch_bias_prep(const float* potB, const float* Bn, int64_t nB, int64_t nB_pad, float bscale, void* out,
-                             cudaStream_t s);
 void tc_plan(int64_t nA, int64_t nB, int bn, int sms, int* G, int* maxseg);
 // Barycentric displacement on the tensor cores for d <= 64 (map_tc.cu): x <- x + alpha
 // (T(x) - x) in place (out may alias X), L from a log-sum-exp pass of the same t; the

@@ -207,7 +207,6 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
   } else {
     // ------------------------------------------------------------ float32 sums of the units
     const int wg = (warp - 2) >> 2, quarter = warp & 3;
-    const int row = quarter * 32 + lane;
 #pragma unroll
     for (int e = 0; e < NH; ++e) o[e] = 0.f;
     bool ok = true;
@@ -234,7 +233,6 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
 #pragma unroll
       for (int e = 0; e < NH; ++e) o[e] = NAN;
     }
-    (void)row;
   }
   // every role of this CTA is done with the stages: they hold the sums now (row pitch N + 1
   // words: conflict-free in both directions)

@@ -15,8 +15,9 @@
 //   T_i = sum_j 2^{t_ij - L_i} y_j / sum_j 2^{t_ij - L_i},
 //   x_i <- x_i + alpha (T_i - x_i).
 //
-// With the squared cost these serve float32 loops beyond d = 64, small float32 queries and
-// workspaces without room for the tensor-core operands; the p-norm costs always run here.
+// With the squared cost these serve float32 solves beyond d = 64, small float32 queries, clouds
+// out of the integer grid's range and workspaces without room for the tensor-core operands; the
+// p-norm costs always run here.
 #include <algorithm>
 
 #include "progot_common.cuh"

@@ -143,30 +143,6 @@ __device__ __forceinline__ void seg_bar() {
     asm volatile("bar.sync 3, 64;" ::: "memory");
 }
 
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Two 16-byte chunks (w[0..3], w[4..7]) as one 32-byte store, in swapped order on odd rows.
 __device__ __forceinline__ void store_pair32(unsigned char* dst, const uint32_t (&w)[8], int swap) {
   uint32_t q[8];
@@ -199,15 +175,6 @@ __device__ __forceinline__ SolverState sweep_state(const SweepParams& p) {
   return st;
 }
 
-// Epilogue of segment k of CTA c, run by NT threads (LSE warpgroup 0 with NT = 128 for
-// the CTA's last segment, the epilogue warps with NT = 64 for the others); thread tid
-// owns rows row0 + NT h of the row block. Publishes the segment's (max, sum) partials,
-// arrives on the row block's counter and, on the last arrival, combines the row
-// block's partials in CTA order, writes the rows' epilogue (and bias rows) and the
-// block's error term, summed in the same float32 tree for either NT (a shuffle sum per
-// 32 rows, then (q0 + q1) + (q2 + q3)); the last row block of the sweep finishes it.
-// The g-update of a Sinkhorn loop (role 2) measures no error and changes no solver
-// state, so its row blocks skip the sweep-level arrival altogether.
 // (max, sum, tilted sum) of two parts of a row in log2 units: with M the max, S = sum 2^{t - M}
 // and W = sum 2^{t - M} (t - M).
 __device__ __forceinline__ float3 tilt_merge(float3 p, float3 q) {
@@ -227,6 +194,15 @@ __device__ __forceinline__ float3 tilt_merge(float3 p, float3 q) {
   return make_float3(M, s, w);
 }
 
+// Epilogue of segment k of CTA c, run by NT threads (LSE warpgroup 0 with NT = 128 for
+// the CTA's last segment, the epilogue warps with NT = 64 for the others); thread tid
+// owns rows row0 + NT h of the row block. Publishes the segment's (max, sum) partials,
+// arrives on the row block's counter and, on the last arrival, combines the row
+// block's partials in CTA order, writes the rows' epilogue (and bias rows) and the
+// block's error term, summed in the same float32 tree for either NT (a shuffle sum per
+// 32 rows, then (q0 + q1) + (q2 + q3)); the last row block of the sweep finishes it.
+// The g-update of a Sinkhorn loop (role 2) measures no error and changes no solver
+// state, so its row blocks skip the sweep-level arrival altogether.
 template <int NT, int GRID>
 __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int k, const Seg& sg, const Split& sp,
                                                  int tid, int row0, const float2 (&mv)[BM / NT],
@@ -355,66 +331,66 @@ __device__ __forceinline__ void segment_epilogue(const TcParams& tp, int c, int 
     seg_bar<NT>();
   } else {
 #pragma unroll
-  for (int h = 0; h < RPT; ++h) {
-    e[h] = 0.f;
-    const int rl = row0 + NT * h;
-    const int64_t i = (int64_t)sg.r * BM + rl;
-    if (i < p.nA) {
-      const float2 acc = accs[h];
-      const double Lr = GRID ? (double)acc.x + (double)log2f(acc.y) : (double)(acc.x + __log2f(acc.y));
-      if (GRID && p.mode == kModeProb) {
-        out_target[i] = acc.y;
-        continue;
-      }
-      float val;
-      e[h] = row_epilogue(p, i, Lr, rin[h], out_target, &val);
-      if (tp.bias_out != nullptr && p.mode == kModePotential) {
-        if constexpr (GRID)
-          write_bias_row_grid(tp.bias_out + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), __ldg(&tp.words->s2));
-        else
-          write_bias_row(tp.bias_out + i * 16, (val - rin[h].an) * p.bscale);
+    for (int h = 0; h < RPT; ++h) {
+      e[h] = 0.f;
+      const int rl = row0 + NT * h;
+      const int64_t i = (int64_t)sg.r * BM + rl;
+      if (i < p.nA) {
+        const float2 acc = accs[h];
+        const double Lr = GRID ? (double)acc.x + (double)log2f(acc.y) : (double)(acc.x + __log2f(acc.y));
+        if (GRID && p.mode == kModeProb) {
+          out_target[i] = acc.y;
+          continue;
+        }
+        float val;
+        e[h] = row_epilogue(p, i, Lr, rin[h], out_target, &val);
+        if (tp.bias_out != nullptr && p.mode == kModePotential) {
+          if constexpr (GRID)
+            write_bias_row_grid(tp.bias_out + i * 16, grid_beta(val, rin[h].an, p.bscale, p.bscale_lo), __ldg(&tp.words->s2));
+          else
+            write_bias_row(tp.bias_out + i * 16, (val - rin[h].an) * p.bscale);
+        }
       }
     }
-  }
-  // a g-update and the passes of a map step measure no error
-  if (p.role == 2 || (p.state == nullptr && (p.mode == kModeLse || p.mode == kModeProb))) {
-    seg_bar<NT>();  // the slots are free for the next segment
-    if (tid == 0) p.cnt[sg.r] = 0;
-    return;  // the counter is read again only by the next sweep, after this grid ends
-  }
-  // block sum of the error terms, in a fixed order
-#pragma unroll
-  for (int h = 0; h < RPT; ++h) {
-    float v = e[h];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if ((tid & 31) == 0) red[(row0 + NT * h) >> 5] = v;
-  }
-  seg_bar<NT>();
-  if (tid == 0) {
-    const float tot = (red[0] + red[1]) + (red[2] + red[3]);
-    p.errpart[sg.r] = (double)tot;
-    p.cnt[sg.r] = 0;
-    s_fin = 0;
-    // a lagged loop's stop test runs in the next sweep, which reads the error partials
-    // once this grid has ended
-    if (!(p.lag && p.role == 1)) {
-      const unsigned prev = atomic_add_acq_rel_gpu(&p.cnt[tp.R], 1u);
-      s_fin = (prev == (unsigned)(tp.R - 1));
+    // a g-update and the passes of a map step measure no error
+    if (p.role == 2 || (p.state == nullptr && (p.mode == kModeLse || p.mode == kModeProb))) {
+      seg_bar<NT>();  // the slots are free for the next segment
+      if (tid == 0) p.cnt[sg.r] = 0;
+      return;  // the counter is read again only by the next sweep, after this grid ends
     }
-  }
-  seg_bar<NT>();
-  if (s_fin && tid < 32) {
-    finish_sweep_warp(p, tp.R);
-    if (tid == 0) p.cnt[tp.R] = 0;
-  }
-  seg_bar<NT>();
+    // block sum of the error terms, in a fixed order
+#pragma unroll
+    for (int h = 0; h < RPT; ++h) {
+      float v = e[h];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      if ((tid & 31) == 0) red[(row0 + NT * h) >> 5] = v;
+    }
+    seg_bar<NT>();
+    if (tid == 0) {
+      const float tot = (red[0] + red[1]) + (red[2] + red[3]);
+      p.errpart[sg.r] = (double)tot;
+      p.cnt[sg.r] = 0;
+      s_fin = 0;
+      // a lagged loop's stop test runs in the next sweep, which reads the error partials
+      // once this grid has ended
+      if (!(p.lag && p.role == 1)) {
+        const unsigned prev = atomic_add_acq_rel_gpu(&p.cnt[tp.R], 1u);
+        s_fin = (prev == (unsigned)(tp.R - 1));
+      }
+    }
+    seg_bar<NT>();
+    if (s_fin && tid < 32) {
+      finish_sweep_warp(p, tp.R);
+      if (tid == 0) p.cnt[tp.R] = 0;
+    }
+    seg_bar<NT>();
   }
 }
 
 // GRID = 0: bf16 operands, one accumulator (two buffers of BN columns). GRID = 1, 2 (2 with
-// the tilted sums of the coupling metrics): the integer-grid split (grid_split.cuh), BN = 128, two accumulators per tile (leading
-// products at TMEM columns [0, 256), the others at [256, 512)).
+// the tilted sums of the coupling metrics): the integer-grid split (grid_split.cuh), BN = 128,
+// two accumulators per tile (leading products at TMEM columns [0, 256), the others at [256, 512)).
 // ATM: the bf16 A row block sits in TMEM (hi at columns [256, 256 + 32 nkb), lo after it),
 // as in the persistent loop: 128 < d <= 256.
 template <int BN, int GRID, int ATM>
@@ -975,15 +951,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
-// beta_j = (potB_j - |b_j|^2) log2(e)/eps for j < nB, -inf for nB <= j < nB_pad.
-__global__ void bias_prep_kernel(const float* __restrict__ potB, const float* __restrict__ Bn, int64_t nB,
-                                 int64_t nB_pad, float bscale, __nv_bfloat16* __restrict__ out) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= nB_pad) return;
-  const float beta = (j < nB) ? (potB[j] - Bn[j]) * bscale : -INFINITY;
-  write_bias_row(out + j * 16, beta);
-}
-
 }  // namespace tc
 
 // ---------------------------------------------------------------- host side
@@ -1030,14 +997,6 @@ int tc_stages(int nkb, int split3) {
   int s, na;
   tc_shape(tc_tile_cols(nkb, split3), nkb, 1 + split3, false, &s, &na);
   return s;
-}
-
-cudaError_t launch_bias_prep(const float* potB, const float* Bn, int64_t nB, int64_t nB_pad, float bscale, void* out,
-                             cudaStream_t s) {
-  tc::bias_prep_kernel<<<(unsigned)((nB_pad + 255) / 256), 256, 0, s>>>(potB, Bn, nB, nB_pad, bscale,
-                                                                        (__nv_bfloat16*)out);
-  count_launch();
-  return cudaGetLastError();
 }
 
 // Number of persistent CTAs and partial slots per CTA for a sweep of nA x nB with
