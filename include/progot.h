@@ -119,10 +119,10 @@ int sinkhorn_potentials(const float* x, const float* a, int64_t n, const float* 
  *
  * xq (device, nq x d) query points; y (device, m x d); g_all (device, K x m) the stored
  * g^(k); eps (host, K) and alpha (host, K) float64; out (device, nq x d) may alias xq.
- * Where tensor-core kernels run (the mixed precisions, and PROGOT_FP32 beyond small sizes)
- * the call synchronises the stream to report a bounded wait that ran out
- * (PROGOT_ERR_TIMEOUT). A PROGOT_FP32 call may be captured into a CUDA graph: it then runs on
- * CUDA cores and reads nothing back.
+ * The mixed precisions synchronise the stream to report a bounded wait that ran out
+ * (PROGOT_ERR_TIMEOUT). A PROGOT_FP32 call is asynchronous and may be captured into a CUDA
+ * graph: what its tensor-core kernels give up, or leave alone because of far points, is done
+ * again by float32 FMAs behind them.
  */
 int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, int32_t d, int32_t K,
                        const float* g_all, const double* eps, const double* alpha, int32_t precision, float* out,
@@ -499,7 +499,8 @@ int progot_set_stall_window(int32_t iters);
  * precisions, d <= 256: P and the centred, scaled Y in bf16 hi/lo, three products with
  * PROGOT_BF16X3 and one with PROGOT_BF16, in one kernel; PROGOT_FP32, and d > 256 at the
  * mixed precisions: half-precision parts, P through memory a chunk of rows at a time); 0
- * runs P Y on float32 CUDA cores after the tensor-core LSE pass. Process-wide setting.
+ * runs P Y on float32 CUDA cores, after the tensor-core LSE pass (mixed precisions) or a
+ * float32 one (PROGOT_FP32). Process-wide setting.
  */
 int progot_set_map_tc(int32_t on);
 
@@ -532,7 +533,8 @@ int progot_set_wait_limit_ns(uint64_t ns);
  * (their row blocks' ready flags stay at "nothing published"), so the first f-update
  * waits for words that no sweep provides until the bounded wait
  * (progot_set_wait_limit_ns) expires and the entry point returns PROGOT_ERR_TIMEOUT; a map
- * step in two passes raises the fault word as if a wait had run out.
+ * step in two passes raises the fault word as if a wait had run out (a float32 map then
+ * does its steps again).
  * Nothing faults or hangs; the context stays usable. 0 (default) restores normal
  * operation. Process-wide setting.
  */

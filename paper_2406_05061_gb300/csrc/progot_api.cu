@@ -581,7 +581,7 @@ static int prep_tc(const float* x, int64_t n, const float* y, int64_t m, int32_t
   ops->ync = ws.ync;
   const bool hull = grid && kind == Operands::kMoved;
   if (remake)
-    CK(cudaMemsetAsync(ws.words->norm2_max, 0, sizeof(GridWords) - offsetof(GridWords, norm2_max), s));
+    CK(cudaMemsetAsync(&ws.words->bad, 0, sizeof(GridWords) - offsetof(GridWords, bad), s));
   else if (!hull)
     CK(launch_center(x, n, y, m, d, ws.rpart, ws.ticket, ws.mu, grid ? ws.words : nullptr, s));
   OperandPrep op;
@@ -1225,13 +1225,15 @@ static int grid_map_step(float* X, int64_t n, int64_t m, int32_t d, double eps, 
 static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, const float* g, const float* yn,
                     double eps, double alpha, int32_t precision, const Workspace& ws, cudaStream_t s,
                     const TcOps* ops = nullptr, const Cost& cost = Cost()) {
-  const bool tc = !cost.pnorm() && ops != nullptr && ops->on;
+  // grid operands serve both passes or none: a CUDA-core map does not look at words->bad
+  const bool map_on = g_map_tc.load() != 0;
+  const bool tc = !cost.pnorm() && ops != nullptr && ops->on && (map_on || !ops->words);
   SweepParams pl = make_sweep(X, n, y, m, d, nullptr, yn, eps, ws, tc ? 1 : 2);
   pl.potB = g;
   pl.out = ws.L;
   pl.mode = kModeLse;
   apply_cost(pl, cost, eps);
-  const bool map_tc = tc && g_map_tc.load();
+  const bool map_tc = tc && map_on;
   // the mixed precisions' map beyond d = 256 gets integer-grid operands of its own; their t
   // can differ by many bits from a hi-only t, so L is then taken from them
   const bool remake = map_tc && !ops->words && ops->nkb > 1 && !map_tc_onepass_supported(ops->nkb);
@@ -1267,8 +1269,8 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     if (t_prof.on) t_prof.worked[kProfMap] += 1;
     return PROGOT_OK;
   }
-  TcOps gops;
   if (map_tc) {
+    TcOps gops;
     // float32 path, and the mixed precisions for d > 256 (their operands give way to the
     // integer-grid ones, whose accuracy the CUDA-core map it replaces had): P a chunk of
     // row blocks at a time, then P Y
@@ -1281,15 +1283,9 @@ static int map_step(float* X, int64_t n, const float* y, int64_t m, int32_t d, c
     }
     rc = grid_map_step(X, n, m, d, eps, alpha, ws, s, *go);
     if (rc || !remake) return rc;  // the float32 path's callers look at words->bad
-    int32_t bad = 0;
-    rc = check_fault(ws, s, &bad);
-    if (rc || !bad) return rc;
-    // out of the grid's range: the operands and L of before again, then the CUDA cores
-    Workspace w;
-    rc = leave_grid(X, n, y, m, d, ws, &w, s);
-    if (!rc) rc = prep_tc(X, n, y, m, d, eps, precision, ws, &gops, s, nullptr, g);
-    if (!rc) rc = lse_sweep(pl, s, &gops, true, &ws);
-    if (rc) return rc;
+    const MapRedo redo = {nullptr, X, y, g, ws.Opart, go->words, nullptr, n, m, d, 1, &eps, &alpha, false};
+    CK(launch_map_redo(redo, s));
+    return PROGOT_OK;
   }
   if (tc) {
     // the float32 map sweep below forms t_ij from the uncentred X and Y: move L there
@@ -1685,39 +1681,29 @@ int entropic_map_apply(const float* xq, int64_t nq, const float* y, int64_t m, i
   rc = zero_counters(ws, s);
   if (rc) return rc;
   if (out != xq) CK(cudaMemcpyAsync(out, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
-  if (precision == PROGOT_FP32 && !grid_map_pays(nq, m, d, K)) ws.grid = false;
-  // A capture cannot read the fault word of the tensor-core kernels back; the CUDA cores wait
-  // for nothing.
-  if (precision == PROGOT_FP32 && ws.grid) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      (void)cudaGetLastError();
-      ws.grid = false;
-    }
-  }
+  if (precision == PROGOT_FP32 && (!grid_map_pays(nq, m, d, K) || !g_map_tc.load())) ws.grid = false;
   if ((precision == PROGOT_FP32 && !ws.grid) || !g_map_tc.load()) CK(launch_row_sqnorm(y, m, d, ws.yn, s));
-  for (int k0 = 0;;) {
-    TcOps ops;
-    for (int k = k0; k < K; ++k) {
-      const double al = (k == K - 1) ? 1.0 : alpha[k];
-      const float* gk = g_all + (int64_t)k * m;
-      rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
-                   k > k0 ? Operands::kMoved : Operands::kAuto, k + 1);
-      if (rc) return rc;
-      rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
-      if (rc) return rc;
-    }
-    if (!ops.on) return PROGOT_OK;
-    int32_t bad = 0;
-    rc = check_fault(ws, s, &bad);
-    if (rc || !bad) return rc;
-    // steps bad .. K - 1 did nothing: the same on CUDA cores
-    k0 = bad - 1;
-    Workspace w;
-    rc = leave_grid(out, nq, y, m, d, ws, &w, s);
-    if (rc) return rc;
-    ws = w;
+  const bool grid = precision == PROGOT_FP32 && ws.grid;
+  const float* start = xq;
+  if (grid && out == xq) {
+    CK(cudaMemcpyAsync(ws.T, xq, sizeof(float) * nq * d, cudaMemcpyDeviceToDevice, s));
+    start = ws.T;
   }
+  TcOps ops;
+  for (int k = 0; k < K; ++k) {
+    const double al = (k == K - 1) ? 1.0 : alpha[k];
+    const float* gk = g_all + (int64_t)k * m;
+    rc = prep_tc(out, nq, y, m, d, eps[k], precision, ws, &ops, s, nullptr, gk, false,
+                 k ? Operands::kMoved : Operands::kAuto, k + 1);
+    if (rc) return rc;
+    rc = map_step(out, nq, y, m, d, gk, ws.yn, eps[k], al, precision, ws, s, &ops);
+    if (rc) return rc;
+  }
+  if (!grid) return ops.on ? check_fault(ws, s) : PROGOT_OK;
+  // the call does not wait: what the grid's kernels left or gave up is done again behind them
+  const MapRedo redo = {start, out, y, g_all, ws.Opart, ws.words, ws.fault, nq, m, d, K, eps, alpha, true};
+  CK(launch_map_redo(redo, s));
+  return PROGOT_OK;
 }
 
 int coupling_marginals(const float* x, int64_t n, const float* y, int64_t m, int32_t d, const float* f,

@@ -105,6 +105,23 @@ struct PvLaunch {
 };
 int64_t pv_prob_bytes_per_block(int64_t m);  // P bytes of one 128-row block
 cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream);
+// The steps of a map that the grid's kernels left alone or gave up, in one launch (sweep_fp32.cu);
+// nothing to do when words->bad and *fault are zero. eps, alpha: host, K values, read by the call.
+struct MapRedo {
+  const float* src;     // the points before step 0 (a fault starts again from them), NULL: only words->bad counts
+  float* x;             // n x d, in place
+  const float* y;
+  const float* g;       // K x m
+  float* T;             // n x d of scratch
+  const GridWords* words;
+  const int32_t* fault;
+  int64_t n, m;
+  int32_t d, K;
+  const double* eps;
+  const double* alpha;
+  bool alpha_last_one;  // the last step's alpha is 1 whatever alpha says (Alg. 3)
+};
+cudaError_t launch_map_redo(const MapRedo& q, cudaStream_t stream);
 // Tensor-core operands (operands.cu).
 // mu = (mean of the rows of X + mean of the rows of Y) / 2, the sums carried beyond float64
 // rounding of their order; partial: reduce_parts() * d doubles of scratch; ticket: a zero

@@ -31,8 +31,10 @@ constexpr int DCH = 64;  // columns of d handled per CTA by the map sweep
 
 // Load one BK-wide chunk of `rows` rows (starting at r0) of a row-major (nrows x d)
 // matrix into registers; zero outside [0, nrows) x [0, d).
-struct ChunkLoader {
+template <bool kMoved>  // kMoved: the matrix changes during the kernel (read through L2)
+struct ChunkLoaderT {
   float4 v[2];
+  static __device__ __forceinline__ float one(const float* p) { return kMoved ? __ldcg(p) : __ldg(p); }
   // Element e = threadIdx.x + NT * q maps to row r = e % BM and 4-wide k group
   // kq = e / BM, so that consecutive threads store consecutive rows of the transposed
   // shared tile (conflict-free stores).
@@ -48,12 +50,12 @@ struct ChunkLoader {
       if (gr < nrows) {
         const float* src = M + gr * (int64_t)d + k;
         if (vec_ok) {
-          if (k < d) val = __ldg(reinterpret_cast<const float4*>(src));
+          if (k < d) val = kMoved ? __ldcg(reinterpret_cast<const float4*>(src)) : __ldg(reinterpret_cast<const float4*>(src));
         } else {
-          if (k + 0 < d) val.x = __ldg(src + 0);
-          if (k + 1 < d) val.y = __ldg(src + 1);
-          if (k + 2 < d) val.z = __ldg(src + 2);
-          if (k + 3 < d) val.w = __ldg(src + 3);
+          if (k + 0 < d) val.x = one(src + 0);
+          if (k + 1 < d) val.y = one(src + 1);
+          if (k + 2 < d) val.z = one(src + 2);
+          if (k + 3 < d) val.w = one(src + 3);
         }
       }
       v[q] = val;
@@ -72,6 +74,8 @@ struct ChunkLoader {
     }
   }
 };
+
+using ChunkLoader = ChunkLoaderT<false>;
 
 struct GemmSmem {
   float As[2][BK][BM];
@@ -103,7 +107,7 @@ __device__ __forceinline__ float pair_term(float a, float b, float acc, float cp
 // 128 x 128 tile (a_row . b_col for the squared Euclidean cost). Rows of the thread:
 // ty*4 + {0..3} and 64 + ty*4 + {0..3}; columns likewise with tx. Coordinates beyond d
 // are zero on both sides and add nothing.
-template <int kCost>
+template <int kCost, bool kMoved = false>
 __device__ __forceinline__ void tile_accumulate(GemmSmem& sm, const float* __restrict__ A, int64_t nA,
                                                 const float* __restrict__ B, int64_t nB, int d, int64_t row0,
                                                 int64_t col0, bool vec_ok, float cp, float (&acc)[8][8]) {
@@ -113,7 +117,8 @@ __device__ __forceinline__ void tile_accumulate(GemmSmem& sm, const float* __res
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
   const int nk = (d + BK - 1) / BK;
-  ChunkLoader la, lb;
+  ChunkLoaderT<kMoved> la;
+  ChunkLoader lb;
   la.load(A, nA, d, row0, 0, vec_ok);
   lb.load(B, nB, d, col0, 0, vec_ok);
   __syncthreads();  // previous users of buffer 0 are done
@@ -595,6 +600,232 @@ __global__ void __launch_bounds__(NT, 1) map_sweep_fp32(MapParams p) {
 }
 
 // ---------------------------------------------------------------- launchers
+// ---------------------------------------------------------------- map done again
+// The steps of a map that the integer grid's kernels left alone (words->bad: the clouds are out of
+// their range from that step on) or gave up (fault: a bounded wait ran out), in float32 FMAs and one
+// launch that asynchronous calls can enqueue unseen: 5 to 8 us when there is nothing to do, where
+// a read of those words by the host costs a queue of calls 75 us each (11308 x 416, d = 58, K = 7:
+// 526 us a call with it, 461 so, 452 with neither). A row's path depends on y and itself only, so a
+// CTA takes its 128 rows through all steps: log-sum-exps, then P Y in chunks of 64 coordinates.
+// Without column splits a few row blocks leave the chip idle; such clouds are rare.
+constexpr int kRedoSteps = 32;
+struct RedoParams {
+  const float* src;      // the points before the first step (for a fault), or NULL: faults are left
+  float* x;              // n x d, in place
+  const float* y;
+  const float* g;        // [k1 - k0][m]
+  float* T;              // n x d of scratch
+  const GridWords* words;
+  const int32_t* fault;
+  int64_t n, m;
+  int32_t d, k0, k1;
+  float scale[kRedoSteps], bscale[kRedoSteps], alpha[kRedoSteps];
+};
+
+// beta of a tile's columns: (g_j - |y_j|^2) bscale, a warp a column.
+__device__ __forceinline__ void redo_betas(const RedoParams& p, const float* g, float bscale, int64_t col0, float* beta_s) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int c = warp; c < BN; c += NT / 32) {
+    const int64_t j = col0 + c;
+    float v = 0.f, e = 0.f;  // the norm without loss, as row_sqnorm's
+    auto add = [&](float q) {
+      const float t = v + q, b = t - v;
+      e += (v - (t - b)) + (q - b);
+      v = t;
+    };
+    if (j < p.m)
+      for (int k = lane; k < p.d; k += 32) {
+        const float u = __ldg(p.y + j * (int64_t)p.d + k), q = u * u;
+        add(q);
+        e += fmaf(u, u, -q);
+      }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const float vo = __shfl_xor_sync(0xffffffffu, v, off), eo = __shfl_xor_sync(0xffffffffu, e, off);
+      add(vo);
+      e += eo;
+    }
+    if (isfinite(v)) v += e;
+    if (lane == 0) beta_s[c] = j < p.m ? (__ldg(g + j) - v) * bscale : -INFINITY;
+  }
+}
+
+__global__ void __launch_bounds__(NT, 1) map_redo_fp32(const __grid_constant__ RedoParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // launched while P Y drains
+  const bool faulted = p.src != nullptr && *p.fault != 0;
+  const int bad = p.words->bad;
+  if (bad == 0 && !faulted) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MapSmem& sm = *reinterpret_cast<MapSmem*>(smem_raw);
+  __shared__ float beta_s[BN];
+  __shared__ float Lrow[BM];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int64_t row0 = (int64_t)blockIdx.x * BM;
+  const int64_t elems = min((int64_t)BM, p.n - row0) * p.d;
+  float* const X = p.x + row0 * p.d;
+  float* const T = p.T + row0 * p.d;
+  const bool vec_ok = ((p.d & 3) == 0) && ((reinterpret_cast<uintptr_t>(p.x) & 15) == 0) &&
+                      ((reinterpret_cast<uintptr_t>(p.y) & 15) == 0);
+  const int ntiles = (int)((p.m + BN - 1) / BN);
+  const int first = faulted ? 0 : bad - 1;
+  if (faulted && p.k0 == 0)
+    for (int64_t e = threadIdx.x; e < elems; e += NT) X[e] = __ldcg(p.src + row0 * p.d + e);
+  for (int k = max(first, p.k0); k < p.k1; ++k) {
+    const float* g = p.g + (int64_t)(k - p.k0) * p.m;
+    const float scale = p.scale[k - p.k0], bscale = p.bscale[k - p.k0], alpha = p.alpha[k - p.k0];
+    float acc[8][8];
+    float2 run[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) run[r] = make_float2(-INFINITY, 0.f);
+    for (int tile = 0; tile < ntiles; ++tile) {
+      __syncthreads();  // X is in place; the previous tile's beta_s is no longer read
+      redo_betas(p, g, bscale, (int64_t)tile * BN, beta_s);
+      tile_accumulate<kCostSqEuclid, true>(sm.g, p.x, p.n, p.y, p.m, p.d, row0, (int64_t)tile * BN, vec_ok, 0.f, acc);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float t[8], mx = -INFINITY;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          t[c] = fmaf(acc[r][c], scale, beta_s[thread_col(c)]);
+          mx = fmaxf(mx, t[c]);
+        }
+        float2 part = make_float2(mx, 0.f);
+        if (mx != -INFINITY)
+#pragma unroll
+          for (int c = 0; c < 8; ++c) part.y += fast_exp2(t[c] - mx);
+        run[r] = lse_combine(run[r], part);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) {
+        const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, run[r].x, off), __shfl_xor_sync(0xffffffffu, run[r].y, off));
+        run[r] = lse_combine(run[r], o);
+      }
+      if (tx == 0) Lrow[thread_row(r)] = run[r].x + log2f(run[r].y);
+    }
+    for (int dch0 = 0; dch0 < p.d; dch0 += DCH) {
+      float o[8][4], rs[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        rs[r] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[r][c] = 0.f;
+      }
+      for (int tile = 0; tile < ntiles; ++tile) {
+        const int64_t col0 = (int64_t)tile * BN;
+        __syncthreads();  // Lrow is written; the previous tile's Ps / Ys / beta_s are no longer read
+        redo_betas(p, g, bscale, col0, beta_s);
+        for (int e = threadIdx.x; e < BN * DCH; e += NT) {
+          const int c = e / DCH, kk = dch0 + e % DCH;
+          const int64_t j = col0 + c;
+          sm.Ys[c][e % DCH] = (j < p.m && kk < p.d) ? __ldg(p.y + j * (int64_t)p.d + kk) : 0.f;
+        }
+        tile_accumulate<kCostSqEuclid, true>(sm.g, p.x, p.n, p.y, p.m, p.d, row0, col0, vec_ok, 0.f, acc);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int rr = thread_row(r);
+          const float Lr = Lrow[rr];
+          float part = 0.f;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const int cc = thread_col(c);
+            const float pv = fast_exp2(fmaf(acc[r][c], scale, beta_s[cc]) - Lr);
+            sm.Ps[cc][rr] = pv;
+            part += pv;
+          }
+          rs[r] += part;
+        }
+        __syncthreads();
+        // a tile's sums on their own: one chain over all columns would be less exact than the sweeps'
+        float ot[8][4];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) ot[r][q] = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < BN; ++c) {
+          const float4 p0 = *reinterpret_cast<const float4*>(&sm.Ps[c][ty * 4]);
+          const float4 p1 = *reinterpret_cast<const float4*>(&sm.Ps[c][64 + ty * 4]);
+          const float4 yv = *reinterpret_cast<const float4*>(&sm.Ys[c][tx * 4]);
+          const float pr[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+          const float yk[4] = {yv.x, yv.y, yv.z, yv.w};
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ot[r][q] = fmaf(pr[r], yk[q], ot[r][q]);
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) o[r][q] += ot[r][q];
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float v = rs[r];
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (row0 + thread_row(r) >= p.n) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int kk = dch0 + tx * 4 + q;
+          if (kk < p.d) T[(int64_t)thread_row(r) * p.d + kk] = o[r][q] / v;
+        }
+      }
+    }
+    __syncthreads();  // every chunk has read X and written T
+    for (int64_t e = threadIdx.x; e < elems; e += NT) {
+      const float x = __ldcg(X + e);
+      X[e] = fmaf(alpha, __ldcg(T + e) - x, x);
+    }
+  }
+}
+
+cudaError_t launch_map_redo(const MapRedo& q, cudaStream_t stream) {
+  static thread_local bool attr_set = false;
+  if (!attr_set) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(map_redo_fp32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MapSmem));
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  for (int k0 = 0; k0 < q.K; k0 += kRedoSteps) {
+    RedoParams p;
+    p.src = q.src;
+    p.x = q.x;
+    p.y = q.y;
+    p.g = q.g + (int64_t)k0 * q.m;
+    p.T = q.T;
+    p.words = q.words;
+    p.fault = q.fault;
+    p.n = q.n;
+    p.m = q.m;
+    p.d = q.d;
+    p.k0 = k0;
+    p.k1 = std::min(q.K, k0 + kRedoSteps);
+    for (int k = k0; k < p.k1; ++k) {
+      p.scale[k - k0] = (float)(2.0 * kLog2e / q.eps[k]);
+      p.bscale[k - k0] = (float)(kLog2e / q.eps[k]);
+      p.alpha[k - k0] = (float)(q.alpha_last_one && k == q.K - 1 ? 1.0 : q.alpha[k]);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((q.n + BM - 1) / BM));
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = sizeof(MapSmem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, map_redo_fp32, p);
+    count_launch();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // ------------------------------------------------------- p-norm map and cost sum
 // grad h of the p-norm cost, one coordinate: sign(z) |z|^(p-1).
 template <int kCost>

@@ -154,3 +154,27 @@ def test_one_loop_update_beside_far_points(n, m, d, far):
     tol = eps * ((w * pair_error(x, y, g0, eps)).sum(1) + 2.0 ** -21 * xn / eps + 2.0 ** -20)
     err = np.abs(r.f.cpu().numpy() - (-eps * lse - eps * np.log(n)))
     assert (err[1:] <= tol[1:] / 4).all(), (err[1:] / tol[1:]).max()
+
+
+@pytest.mark.parametrize("n,m,d,K", [(2500, 2300, 64, 3), (1100, 1000, 250, 2), (777, 901, 300, 35)])
+def test_map_steps_beside_very_far_queries(n, m, d, K):
+    """Several steps done again by float32 FMAs: ragged rows, columns and coordinates, more steps than
+    one launch takes."""
+    x, y = clouds(n, m, d, seed=K, far_x=1e6)
+    eps = 0.1 * 2.0 * d
+    g = np.random.default_rng(d).standard_normal((K, m)).astype(np.float32) * np.float32(eps)
+    alpha = [1.0 / (K - k) for k in range(K)]
+    for tc in (True, False):
+        nat.set_map_tc(tc)
+        try:
+            out = nat.entropic_map_apply(dev(x), dev(y), dev(g), [eps] * K, alpha).cpu().numpy()
+        finally:
+            nat.set_map_tc(True)
+        rows = np.r_[1:20, n - 20:n]
+        ref, y64 = x[rows].astype(np.float64), y.astype(np.float64)
+        for gk, al in zip(g.astype(np.float64), alpha):
+            t = (gk - ((ref ** 2).sum(1)[:, None] + (y64 ** 2).sum(1) - 2 * ref @ y64.T)) / eps
+            p = np.exp(t - t.max(1, keepdims=True))
+            ref = ref + al * (p @ y64 / p.sum(1, keepdims=True) - ref)
+        r2 = (y64 ** 2).sum(1).max()
+        np.testing.assert_allclose(out[rows], ref, rtol=0, atol=K * 2.0 ** -21 * (4 * r2 / eps + 16) * r2 ** 0.5)
