@@ -157,20 +157,27 @@ static int plan_splits(int64_t nA, int64_t nB, int ctas_per_sm, int extra_mult =
 // grid sweeps, one launch an update, do not drift and take a tenth of the time.
 constexpr int32_t kGridSolveDim = 64;
 // Whether a float32 map of K steps runs on the tensor cores: where their estimated time for the
-// whole call is the smaller. The fixed 77 us are the first step's preparation (the later steps'
-// takes one launch) and the read of the fault word at the end; t the 128 x 128 tiles of a step,
-// in microseconds fitted to both paths measured over 300 shapes (500 to 20000 points, d = 2 to
-// 256, K = 1, 2, 8): CUDA cores / tensor cores 69 / 126 at 2000 x 2000, d = 16, K = 1; 204 / 191
-// at 3000 x 3000, K = 2, and 770 / 544 at K = 8; 110 / 130 there at d = 64, 2000 x 2000, K = 1,
-// and 206 / 185 at K = 2; 5264 / 632 at 8000 x 8000, d = 256, K = 1. The eighth on top covers the
-// fit's error: of those shapes none is more than 3 % slower than its CUDA-core call.
+// whole call is the smaller. Microseconds fitted to both paths over 968 shapes (300 to 20000
+// points, d = 2 to 256, K = 1 to 8), calls queued behind one another: for the CUDA cores the waves
+// of both launches (two and one CTA an SM) times the tiles of a CTA and their coordinates, and the
+// splits a row block adds up; for the tensor cores the tiles of a CTA, the row blocks and the bytes
+// of the operands, twice at the first step, whose preparation takes two launches more. Tensor cores /
+// CUDA cores: 66 / 46 at 1000 x 1000, d = 2, K = 1; 69 / 103 there at d = 128; 131 / 121 at
+// 2000 x 2000, d = 16, K = 2; 87 / 106 at 3000 x 3000, d = 8, K = 1; 98 / 134 at 11308 x 416, d = 64.
+// With the 3 % on top none of those calls is more than 11 % slower than on the other path, on the
+// mean 0.1 %.
 static bool grid_map_pays(int64_t n, int64_t m, int32_t d, int32_t K) {
-  const double rb = (double)((n + 127) / 128), ct = (double)((m + 127) / 128), t = rb * ct;
-  const double dd = std::max<int32_t>(d, 16), wide = std::max<int32_t>(d - 64, 0);
-  const double cuda_cores = 16.0 + K * (15.0 + 0.36 * dd + t * (0.070 + 0.0021 * dd + 0.0033 * wide) + 0.57 * ct);
-  const double tensor_cores =
-      77.0 + K * (32.0 + 0.081 * std::min(t, 256.0) + 0.063 * std::max(t - 256.0, 0.0) + 0.0005 * t * wide + 0.062 * rb);
-  return 1.12 * tensor_cores < cuda_cores;
+  const int64_t sms = num_sms(), rb = cdiv(n, fp32_tile_rows()), ct = cdiv(m, fp32_tile_cols()), t = rb * ct;
+  const double nk = (double)cdiv(d, 16), nkb = (double)cdiv(d, 64), dch = (double)cdiv(d, map_dchunk());
+  const double x1 = (double)cdiv(ct, plan_splits(n, m, 2)), x2 = (double)cdiv(ct, plan_splits(n, m, 1, (int)dch));
+  const double s1 = std::ceil(ct / x1), s2 = std::ceil(ct / x2);
+  const double w1 = std::ceil(rb * s1 / (2.0 * sms)), w2 = std::ceil(rb * s2 * dch / sms);
+  const double cuda_cores = 14.0 + K * (12.0 + 3.7 * w1 * x1 * nk + w2 * x2 * (13.0 + 1.73 * nk) + 0.32 * s1 + 0.018 * s2 * d);
+  const int64_t G = std::min(t, sms);
+  const double tp = (double)cdiv(t, G), mb = 1e-6 * ((double)n + (double)m) * d;
+  const double tensor_cores = 28.0 + 7.3 * mb + K * (23.6 + 2.86 * std::min(tp, 3.0) + 4.72 * std::max(tp - 3.0, 0.0) +
+                                                     3.64 * tp * nkb + 0.163 * rb + 0.5 * cdiv(G, rb) + 6.7 * mb);
+  return 1.03 * tensor_cores < cuda_cores;
 }
 // P of a chunk of rows stays in L2 between the sweep that writes it and the product that
 // reads it; a p-norm cost up to about the size of L2 is kept for its loop.

@@ -45,13 +45,14 @@ def run(n, m, d, K, rows=40):
     return launches
 
 
-@pytest.mark.parametrize("n,m,d,K", [(1000, 2048, 3, 1), (2000, 2000, 16, 1), (3000, 3000, 8, 1), (2400, 750, 17, 8),
-                                     (12000, 500, 2, 7), (1000, 1000, 64, 2), (500, 500, 100, 1)])
+@pytest.mark.parametrize("n,m,d,K", [(1000, 2048, 3, 1), (1500, 1500, 16, 1), (700, 700, 32, 1), (500, 500, 16, 2),
+                                     (128, 20000, 2, 3), (1000, 1000, 16, 4), (300, 300, 2, 8)])
 def test_short_and_small_float32_maps_stay_on_cuda_cores(n, m, d, K):
     assert run(n, m, d, K) == CUDA_CORES * K + 1
 
 
-@pytest.mark.parametrize("n,m,d,K", [(6000, 5777, 3, 1), (4099, 4300, 16, 4), (3001, 3070, 48, 3), (129, 383, 130, 8),
-                                     (130, 500, 80, 16), (2001, 127, 250, 2), (1, 640, 256, 6), (777, 901, 192, 2)])
+@pytest.mark.parametrize("n,m,d,K", [(6000, 5777, 3, 1), (3000, 3000, 8, 1), (500, 500, 100, 1), (1000, 1000, 64, 2),
+                                     (4099, 4300, 16, 4), (3001, 3070, 48, 3), (129, 383, 130, 8), (130, 500, 80, 16),
+                                     (2001, 127, 250, 2), (1, 640, 256, 6), (777, 901, 192, 2)])
 def test_float32_maps_on_the_tensor_cores(n, m, d, K):
     assert run(n, m, d, K) > CUDA_CORES * K + 1
