@@ -285,28 +285,72 @@ __global__ void __launch_bounds__(PV_NTHREADS, 1)
 int64_t pv_prob_bytes_per_block(int64_t m) { return (m + 127) / 128 * 2 * (int64_t)tc::PV_P_BYTES; }
 
 template <int NB>
-static cudaError_t launch_pv(const tc::PvParams& pp, int grid, size_t smem, const void* const* maps,
-                             cudaStream_t stream) {
+static cudaError_t pv_attributes(size_t smem) {
   static thread_local size_t attr_bytes = 0;
-  if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(tc::pv_tc<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_bytes = smem;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(tc::PV_NTHREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  if (smem <= attr_bytes) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(tc::pv_tc<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) attr_bytes = smem;
+  return e;
+}
+
+static void pv_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int grid, int splits, size_t smem,
+                      cudaStream_t stream) {
+  *cfg = {};
+  cfg->gridDim = dim3(grid);
+  cfg->blockDim = dim3(tc::PV_NTHREADS);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = pp.splits;
+  attr[0].val.clusterDim.x = splits;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 2;
+}
+
+// Clusters of `splits` CTAs that run at once: fewer than the SMs allow, since a cluster stays inside
+// one GPC (15 of eight and 36 of four on a GB300).
+template <int NB>
+static int pv_clusters(int splits, size_t smem, int sms) {
+  static thread_local int cached[9] = {};
+  if (cached[splits] == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    pv_config(&cfg, attr, splits * sms, splits, smem, nullptr);
+    cfg.numAttrs = 1;
+    int c = 0;
+    if (cudaOccupancyMaxActiveClusters(&c, tc::pv_tc<NB>, &cfg) != cudaSuccess || c < 1) {
+      (void)cudaGetLastError();
+      c = std::max(1, sms / splits);
+    }
+    cached[splits] = c;
+  }
+  return cached[splits];
+}
+
+template <int NB>
+static cudaError_t launch_pv(tc::PvParams pp, int64_t tiles, size_t smem, const void* const* maps, int sms,
+                             cudaStream_t stream) {
+  cudaError_t e = pv_attributes<NB>(smem);
+  if (e != cudaSuccess) return e;
+  // CTAs per tile: the share that finishes first in waves of the clusters that run at once, a CTA
+  // costing about three units besides its own (2368 x 753, d = 17: 45.4 us a map step with waves of
+  // SMs, which took eight CTAs for each of the 19 row blocks and so a second wave, 40.4 so)
+  double best = 0.0;
+  pp.splits = 1;
+  for (int s = 1; s <= 8 && s <= pp.units; s *= 2) {
+    const int c = pv_clusters<NB>(s, smem, sms);
+    const double cost = (double)((tiles + c - 1) / c) * ((double)((pp.units + s - 1) / s) + 3.0);
+    if (s == 1 || cost < best) {
+      best = cost;
+      pp.splits = s;
+    }
+  }
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  pv_config(&cfg, attr, (int)(tiles * pp.splits), pp.splits, smem, stream);
   auto at = [](const void* p) -> const CUtensorMap& { return *reinterpret_cast<const CUtensorMap*>(p); };
   return cudaLaunchKernelEx(&cfg, tc::pv_tc<NB>, at(maps[0]), at(maps[1]), at(maps[2]), pp);
 }
@@ -328,22 +372,11 @@ cudaError_t launch_pv_tc(const PvLaunch& p, int sms, cudaStream_t stream) {
   pp.units = (int)((p.m + 127) / 128 * 2);
   pp.chunks = (p.d + 64 * nb - 1) / (64 * nb);
   const int64_t tiles = (p.rows + 127) / 128 * pp.chunks;
-  // CTAs per tile: the share that finishes first in waves of one CTA per SM, a CTA costing
-  // about three units besides its own
-  double best = 0.0;
-  pp.splits = 1;
-  for (int s = 1; s <= 8 && s <= pp.units; s *= 2) {
-    const double cost = (double)((tiles * s + sms - 1) / sms) * ((double)((pp.units + s - 1) / s) + 3.0);
-    if (s == 1 || cost < best) {
-      best = cost;
-      pp.splits = s;
-    }
-  }
   const uint32_t st_bytes = tc::PV_P_BYTES + (uint32_t)kGridParts * nb * tc::PV_Y_BYTES;
   pp.stages = std::min<int>(tc::PV_MAXST, (int)((225 * 1024) / st_bytes));
   const size_t smem = std::max<size_t>((size_t)pp.stages * st_bytes, (size_t)128 * (64 * nb + 1) * 4) + 1024;
-    const int grid = (int)(tiles * pp.splits);
-  const cudaError_t e = nb == 2 ? launch_pv<2>(pp, grid, smem, p.mapY, stream) : launch_pv<1>(pp, grid, smem, p.mapY, stream);
+  const cudaError_t e = nb == 2 ? launch_pv<2>(pp, tiles, smem, p.mapY, sms, stream)
+                                : launch_pv<1>(pp, tiles, smem, p.mapY, sms, stream);
   count_launch();
   return e;
 }
