@@ -162,10 +162,9 @@ constexpr int32_t kGridSolveDim = 64;
 // of both launches (two and one CTA an SM) times the tiles of a CTA and their coordinates, and the
 // splits a row block adds up; for the tensor cores the tiles of a CTA, the row blocks and the bytes
 // of the operands, twice at the first step, whose preparation takes two launches more. Tensor cores /
-// CUDA cores: 66 / 46 at 1000 x 1000, d = 2, K = 1; 69 / 103 there at d = 128; 131 / 121 at
-// 2000 x 2000, d = 16, K = 2; 87 / 106 at 3000 x 3000, d = 8, K = 1; 98 / 134 at 11308 x 416, d = 64.
-// With the 3 % on top none of those calls is more than 11 % slower than on the other path, on the
-// mean 0.1 %.
+// CUDA cores: 64 / 46 at 1000 x 1000, d = 2, K = 1; 68 / 103 there at d = 128; 122 / 121 at
+// 2000 x 2000, d = 16, K = 2; 87 / 106 at 3000 x 3000, d = 8, K = 1; 96 / 134 at 11308 x 416, d = 64.
+// None of those calls is more than 5 % slower than on the other path (8 % where the caller waits).
 static bool grid_map_pays(int64_t n, int64_t m, int32_t d, int32_t K) {
   const int64_t sms = num_sms(), rb = cdiv(n, fp32_tile_rows()), ct = cdiv(m, fp32_tile_cols()), t = rb * ct;
   const double nk = (double)cdiv(d, 16), nkb = (double)cdiv(d, 64), dch = (double)cdiv(d, map_dchunk());
@@ -175,9 +174,9 @@ static bool grid_map_pays(int64_t n, int64_t m, int32_t d, int32_t K) {
   const double cuda_cores = 14.0 + K * (12.0 + 3.7 * w1 * x1 * nk + w2 * x2 * (13.0 + 1.73 * nk) + 0.32 * s1 + 0.018 * s2 * d);
   const int64_t G = std::min(t, sms);
   const double tp = (double)cdiv(t, G), mb = 1e-6 * ((double)n + (double)m) * d;
-  const double tensor_cores = 28.0 + 7.3 * mb + K * (23.6 + 2.86 * std::min(tp, 3.0) + 4.72 * std::max(tp - 3.0, 0.0) +
-                                                     3.64 * tp * nkb + 0.163 * rb + 0.5 * cdiv(G, rb) + 6.7 * mb);
-  return 1.03 * tensor_cores < cuda_cores;
+  const double tensor_cores = 28.7 + 5.4 * mb + K * (23.0 + 2.97 * std::min(tp, 3.0) + 4.96 * std::max(tp - 3.0, 0.0) +
+                                                     3.73 * tp * nkb + 0.16 * rb + 0.5 * cdiv(G, rb) + 7.4 * mb);
+  return tensor_cores < cuda_cores;
 }
 // P of a chunk of rows stays in L2 between the sweep that writes it and the product that
 // reads it; a p-norm cost up to about the size of L2 is kept for its loop.
